@@ -2,7 +2,8 @@
 
 ``listed()`` names the standing cases, ``draw(rng)`` makes one more of the same ranges, ``prepare`` builds
 what a program holds before the call, ``run`` makes one pass through the public entry points, ``work`` counts
-what the pass cannot do without and ``tolerance`` says how far two correct implementations may differ.
+what the pass cannot do without, ``tolerance`` says how far two correct implementations may differ and ``exact``
+gives the same outputs in binary64.
 
 Kinds of work:
 
@@ -255,3 +256,84 @@ def tolerance(case):
         return {"rel": 4e-7}
     # whole numbers are exact, y is a scale product away from an exact integer: the output type decides
     return {"rel": 4e-7 if f32 else 7e-3}
+
+
+# ---- the same outputs in binary64 ----------------------------------------------------------------------
+
+# alpha*(b) of the uniform grids and of the FP4 grid (minimisers of the Gaussian quantization error)
+_ALPHA = {1: 0.7978846, 2: 1.4935300, 3: 2.0510680, 4: 2.5140045, 5: 2.9161513, 6: 3.2779846, 7: 3.6110970, 8: 3.9222038}
+_ALPHA_FP4 = 2.9224751
+_E2M1 = (0.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, 6.0)
+
+
+def _rotated(t, g):
+    """Orthonormal Walsh-Hadamard transform of every block of g consecutive elements of a row (its own inverse)."""
+    v = t.double().reshape(t.shape[0], -1, g)
+    h = 1
+    while h < g:
+        v = v.reshape(t.shape[0], -1, g // (2 * h), 2, h)
+        v = torch.stack((v[..., 0, :] + v[..., 1, :], v[..., 0, :] - v[..., 1, :]), dim=-2)
+        h *= 2
+    return (v / math.sqrt(g)).reshape(t.shape[0], -1)
+
+
+def _projected(t, bits, g, trust):
+    """(grid values 2k - (2^b - 1), row scales, trusted elements)."""
+    u = _rotated(t, g)
+    top = 2.0 ** bits - 1.0
+    alpha = _ALPHA[bits]
+    rms = u.square().mean(1).sqrt()
+    pos = u * (top / (2.0 * alpha)) / rms.clamp_min(1e-300)[:, None] + top / 2.0
+    k = pos.clamp(0.0, top).round()
+    return 2.0 * k - top, alpha * rms / top, (pos - k).abs() <= trust / 2.0
+
+
+def _projected_fp4(t, g):
+    u = _rotated(t, g)
+    rms = u.square().mean(1).sqrt()
+    pos = u * (6.0 / _ALPHA_FP4) / rms.clamp_min(1e-300)[:, None]
+    mag = pos.abs().clamp_max(6.0)
+    step = torch.where(mag < 2.0, 0.5, torch.where(mag < 4.0, 1.0, 2.0))
+    return torch.sign(pos) * (mag / step).round() * step, _ALPHA_FP4 * rms / 6.0
+
+
+def exact(case, seed):
+    """What ``run`` returns, in binary64 from the definition; codes and masks are whole numbers and have no such value."""
+    gen = _gen(seed)
+    kind, M, N, K, bits, g, trust = (case[k] for k in ("kind", "M", "N", "K", "bits", "g", "trust"))
+    dt = _DTYPES[case["dtype"]]
+    x = _activations(M, K, gen, dt)
+    if kind == "quantize":
+        return {"codes": None, "scales": _projected(x, bits, g, trust)[1], "mask": None}
+    if kind == "mlp":
+        wg, wu = _weights(N, K, gen, dt), _weights(N, K, gen, dt)
+        wd = _weights(K, N, gen, dt)
+        qx, sx, _ = _projected(x, bits, g, trust)
+        qg, sg, _ = _projected(wg, bits, g, trust)
+        qu, su, _ = _projected(wu, bits, g, trust)
+        gate = (qx @ qg.T) * sx[:, None] * sg
+        h = (gate / (1.0 + torch.exp(-gate)) * ((qx @ qu.T) * sx[:, None] * su)).to(torch.bfloat16)   # h is a bfloat16 tensor
+        qh, sh, _ = _projected(h, bits, g, trust)
+        qd, sd, _ = _projected(wd, bits, g, trust)
+        out = dict.fromkeys(("xq", "mx", "wgq", "mwg", "wuq", "mwu", "hq", "mh", "wdq", "mwd"))
+        return {**out, "h": h.double(), "y": (qh @ qd.T) * sh[:, None] * sd, "sx": sx, "swg": sg, "swu": su, "sh": sh, "swd": sd}
+    w = _weights(N, K, gen, dt)
+    if kind == "weight_only":
+        xh = _rotated(x, g)
+        qw, sw, _ = _projected(w, bits, g, trust)
+        return {"y": (xh @ qw.T) * sw, "xh": xh, "wq": None, "sw": sw, "mw": None}
+    if kind == "fp4":
+        (qx, sx), (qw, sw) = _projected_fp4(x, g), _projected_fp4(w, g)
+    else:
+        (qx, sx, mx), (qw, sw, mw) = _projected(x, bits, g, trust), _projected(w, bits, g, trust)
+    y = (qx @ qw.T) * sx[:, None] * sw
+    if kind == "gemm":
+        return y
+    if kind == "infer":
+        return {"y": y, "xq": None, "sx": sx}
+    out = {"xq": None, "sx": sx, "mx": None, "wq": None, "sw": sw, "mw": None, "y": y}
+    if kind == "train":
+        dy = torch.randn((M, N), generator=gen, device="cuda").mul_(1e-3).to(torch.bfloat16).double()
+        out["dx"] = _rotated((dy @ (qw * sw[:, None])) * mx, g)
+        out["dw"] = _rotated((dy.T @ (qx * sx[:, None])) * mw, g)
+    return out
