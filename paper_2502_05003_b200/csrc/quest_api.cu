@@ -272,18 +272,25 @@ int quest_lowbit_gemm(const uint8_t *xq, const float *sx, int bits_x,
     if ((s = check_device())) return s;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     Workspace ws = carve_workspace(workspace, M, N, K);
-    const bool need_rs_a = bits_w == 8;    // sum of x operand values multiplies the offset of the w codes
-    const bool need_rs_b = bits_x == 8;
+    // codes of 8 bits are tensor-core operands as they are (unsigned bytes, every value of the byte is a level);
+    // narrower ones are unpacked into the workspace
+    const bool x_codes = bits_x == 8, w_codes = bits_w == 8;
+    const bool need_rs_a = w_codes;        // the sum of x operand values multiplies the offset of the w codes
+    const bool need_rs_b = x_codes;
+    const int8_t *a8 = x_codes ? reinterpret_cast<const int8_t *>(xq) : ws.a8;
+    const int8_t *b8 = w_codes ? reinterpret_cast<const int8_t *>(wq) : ws.b8;
     {
         StageScope scope(QUEST_STAGE_UNPACK, st);
-        const bool e4 = e2m1_operands(bits_x, bits_w);
-        if ((s = launch_unpack_pair(xq, bits_x, M, ws.a8, need_rs_a ? ws.rs_a : nullptr, wq, bits_w, N, ws.b8,
-                                    need_rs_b ? ws.rs_b : nullptr, K, e4, st)))
+        if ((s = launch_unpack_pair(xq, bits_x, M, x_codes ? nullptr : ws.a8, wq, bits_w, N, w_codes ? nullptr : ws.b8, K,
+                                    e2m1_operands(bits_x, bits_w), st)))
+            return s;
+        if ((s = launch_rowsum_pair(a8, M, x_codes, need_rs_a ? ws.rs_a : nullptr, b8, N, w_codes,
+                                    need_rs_b ? ws.rs_b : nullptr, K, st)))
             return s;
     }
     StageScope scope(QUEST_STAGE_GEMM, st);
-    return launch_gemm(ws.a8, ws.b8, ws.rs_a, ws.rs_b, bits_x, bits_w, sx, sw, M, N, K, y, y_dtype, ldy_elems, acc,
-                       st);
+    return launch_gemm(a8, b8, ws.rs_a, ws.rs_b, bits_x, bits_w, sx, sw, M, N, K, y, y_dtype, ldy_elems, acc, st,
+                       x_codes, w_codes);
 }
 
 int quest_linear_fwd_quantize(const void *x, const void *w, int dtype, int64_t M, int64_t N, int64_t K,

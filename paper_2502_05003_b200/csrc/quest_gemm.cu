@@ -9,6 +9,8 @@
 // c = 2k-(2^b-1) (quest_operand.cuh) and the epilogue shifts the exact power of two back out;
 // for b = 8 (|c| up to 255) it is v = k - 128 and the epilogue restores
 // c_x . c_w = 4 v_x.v_w + 2 sum(v_x) + 2 sum(v_w) + K exactly from per-row sums.
+// A packed tensor of 8-bit codes is itself an operand: kind::i8 takes unsigned bytes, c = 2k - 255, and the
+// epilogue restores the product from the row sums of the codes (quest_lowbit_gemm; nothing is unpacked).
 //
 // The FP4 grid (Section 4.4) has a native operand type: its packed E2M1 codes feed tcgen05.mma
 // kind::mxf4 directly (MODE 5 below), with all block scales 2^0.  So do the one- and two-bit uniform
@@ -62,6 +64,7 @@ struct GemmParams {
     const int32_t *rs_b;   // row sums of the B operand values (nullable)
     int mul;               // acc' = (mul*acc + ca*rs_a[i] + cb*rs_b[j] + ck) >> sh   (exact)
     int ca, cb, ck, sh;
+    uint32_t u8_ops = 0;   // MODE 1: instruction-descriptor bits to clear, one per operand that holds unsigned bytes
     void *y;
     int y_dtype;
     long long ldy;
@@ -544,9 +547,10 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         __syncwarp();
     } else if (warp == 1) {
         if (lane == 0 && leader) {
-            constexpr uint32_t idesc = MX ? make_idesc_mxf4(TILE_M, BN)
+            constexpr uint32_t idesc_c = MX ? make_idesc_mxf4(TILE_M, BN)
                                           : F16 ? (make_idesc_bf16(TILE_M, BN) | (AMN ? 1u << 15 : 0u) | (BMN ? 1u << 16 : 0u))
                                                 : make_idesc_i8(TILE_M, BN);
+            const uint32_t idesc = CORR ? idesc_c & ~p.u8_ops : idesc_c;
             int stage = 0;
             uint32_t phase = 0;
             int t = 0;
@@ -1077,6 +1081,43 @@ __global__ void rowsum_i8_kernel(const int8_t *__restrict__ a, long long rows, i
     if (lane == 0) out[row] = s;
 }
 
+// Row sums of the byte operands of a contraction, x and w in one launch: unsigned bytes where the packed codes
+// are the operand, signed where they were unpacked.  Bound by HBM: each operand is read once (and stays in L2
+// for the contraction that follows).  A row belongs to the smallest power-of-two group of lanes that covers it
+// with 16-byte loads, at most a warp; eight loads per lane are in flight on long rows.
+// 16384 x 4096 + 4096 x 4096 8-bit codes: the whole contraction 273 -> 211 us against an unpack pass (29 us) and two
+// launches of 4-byte loads (13 + 7 us).
+__global__ void __launch_bounds__(256)
+rowsum_pair_kernel(const uint8_t *__restrict__ a, long long rows_a, int unsigned_a, int32_t *__restrict__ out_a,
+                   const uint8_t *__restrict__ b, long long rows_b, int unsigned_b, int32_t *__restrict__ out_b,
+                   int K, int lanes_log2) {
+    pdl_launch_dependents();
+    pdl_wait();
+    const int lanes = 1 << lanes_log2;
+    long long row = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> lanes_log2;
+    const int l = threadIdx.x & (lanes - 1);
+    const bool second = row >= rows_a;
+    if (second) row -= rows_a;
+    const bool live = !second || row < rows_b;
+    const bool uns = (second ? unsigned_b : unsigned_a) != 0;
+    int s = 0;
+    if (live) {
+        const uint4 *r = reinterpret_cast<const uint4 *>((second ? b : a) + row * (long long)K);
+        const uint32_t flip = uns ? 0x80808080u : 0u;            // u = s + 128 after flipping the top bit
+        const int nc = K >> 4;
+#pragma unroll 8
+        for (int c = l; c < nc; c += lanes) {
+            const uint4 w = __ldg(r + c);
+            s = __dp4a((int)(w.x ^ flip), 0x01010101, s);
+            s = __dp4a((int)(w.y ^ flip), 0x01010101, s);
+            s = __dp4a((int)(w.z ^ flip), 0x01010101, s);
+            s = __dp4a((int)(w.w ^ flip), 0x01010101, s);
+        }
+    }
+    for (int o = lanes >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (live && l == 0) (second ? out_b : out_a)[row] = uns ? s + 128 * K : s;
+}
+
 // Self-test of the bounded wait: one warp waits, with a short limit, on a barrier that nothing will ever
 // complete.  The wait must give up, record its code in the status word, raise the abort flag, and a second
 // wait must then return at once because the CTA is aborting: the path every kernel of the library takes
@@ -1268,18 +1309,27 @@ int launch_unpack(const uint8_t *codes, int bits, int64_t rows, int64_t K, int8_
     return QUEST_OK;
 }
 
-int launch_unpack_pair(const uint8_t *xq, int bits_x, int64_t M, int8_t *a8, int32_t *rs_a,
-                       const uint8_t *wq, int bits_w, int64_t N, int8_t *b8, int32_t *rs_b, int64_t K, bool e2m1,
-                       cudaStream_t st) {
-    const long long gx = M * K / 32, gw = N * K / 32;
+int launch_unpack_pair(const uint8_t *xq, int bits_x, int64_t M, int8_t *a8, const uint8_t *wq, int bits_w, int64_t N,
+                       int8_t *b8, int64_t K, bool e2m1, cudaStream_t st) {
+    const long long gx = a8 ? M * K / 32 : 0, gw = b8 ? N * K / 32 : 0;
     if (gx + gw == 0) return QUEST_OK;
     cudaError_t e = launch_pdl(unpack_pair_kernel, dim3((unsigned)((gx + gw + 127) / 128)), dim3(128), 0, st, 1, xq, bits_x, gx,
                                reinterpret_cast<uint8_t *>(a8), wq, bits_w, gw, reinterpret_cast<uint8_t *>(b8), e2m1 ? 1 : 0);
-    if (e != cudaSuccess) return cuda_fail(e);
-    int s = QUEST_OK;
-    if (rs_a) s = launch_rowsum(a8, M, K, rs_a, st);
-    if (!s && rs_b) s = launch_rowsum(b8, N, K, rs_b, st);
-    return s;
+    return e == cudaSuccess ? QUEST_OK : cuda_fail(e);
+}
+
+int launch_rowsum_pair(const void *a, int64_t rows_a, bool unsigned_a, int32_t *out_a,
+                       const void *b, int64_t rows_b, bool unsigned_b, int32_t *out_b, int64_t K, cudaStream_t st) {
+    if (!out_a) rows_a = 0;
+    if (!out_b) rows_b = 0;
+    if (rows_a + rows_b == 0) return QUEST_OK;
+    int lg = 0;
+    while (lg < 5 && (16ll << lg) < K) ++lg;
+    const long long threads = (long long)(rows_a + rows_b) << lg;
+    cudaError_t e = launch_pdl(rowsum_pair_kernel, dim3((unsigned)((threads + 255) / 256)), dim3(256), 0, st, 1,
+                               reinterpret_cast<const uint8_t *>(a), (long long)rows_a, unsigned_a ? 1 : 0, out_a,
+                               reinterpret_cast<const uint8_t *>(b), (long long)rows_b, unsigned_b ? 1 : 0, out_b, (int)K, lg);
+    return e == cudaSuccess ? QUEST_OK : cuda_fail(e);
 }
 
 int launch_rowsum(const int8_t *a8, int64_t rows, int64_t K, int32_t *rowsum, cudaStream_t st) {
@@ -1292,20 +1342,23 @@ int launch_rowsum(const int8_t *a8, int64_t rows, int64_t K, int32_t *rowsum, cu
 int launch_gemm(const int8_t *a8, const int8_t *b8, const int32_t *rs_a, const int32_t *rs_b,
                 int bits_x, int bits_w, const float *sx, const float *sw,
                 int64_t M, int64_t N, int64_t K, void *y, int y_dtype, int64_t ldy,
-                int32_t *acc, cudaStream_t st) {
+                int32_t *acc, cudaStream_t st, bool x_codes, bool w_codes) {
     if (M == 0 || N == 0) return QUEST_OK;
     if (e2m1_operands(bits_x, bits_w))               // both operands are E2M1 nibbles of the grid values
         return launch_gemm_e2m1(reinterpret_cast<const uint8_t *>(a8), reinterpret_cast<const uint8_t *>(b8), sx, sw, M, N, K,
                                 y, y_dtype, ldy, acc, 1, st);
-    // operand value v relates to the grid value c by v = 2^(7-b) c below 8 bits and c = 2v + 1 at 8 bits
+    // operand value v relates to the grid value c by v = 2^(7-b) c below 8 bits and by c = 2v + o at 8 bits (o = 1
+    // for the signed bytes k - 128, o = -255 for the unsigned codes themselves)
     const bool x8 = bits_x == 8, w8 = bits_w == 8;
+    const int ox = x_codes ? -255 : 1, ow = w_codes ? -255 : 1;
     GemmParams p;
     p.M = (int)M; p.N = (int)N; p.K = (int)K;
     p.sx = sx; p.sw = sw;
+    p.u8_ops = (x_codes ? 1u << 7 : 0u) | (w_codes ? 1u << 10 : 0u);
     if (!x8 && !w8) { p.mul = 1; p.ca = 0; p.cb = 0; p.ck = 0; p.sh = 14 - bits_x - bits_w; }
-    else if (x8 && w8) { p.mul = 4; p.ca = 2; p.cb = 2; p.ck = (int)K; p.sh = 0; }
-    else if (x8) { p.mul = 2; p.ca = 0; p.cb = 1; p.ck = 0; p.sh = 7 - bits_w; }   // 2 sum v_x op_w + sum op_w
-    else { p.mul = 2; p.ca = 1; p.cb = 0; p.ck = 0; p.sh = 7 - bits_x; }
+    else if (x8 && w8) { p.mul = 4; p.ca = 2 * ow; p.cb = 2 * ox; p.ck = (int)K * ox * ow; p.sh = 0; }
+    else if (x8) { p.mul = 2; p.ca = 0; p.cb = ox; p.ck = 0; p.sh = 7 - bits_w; }   // 2 sum v_x op_w + o_x sum op_w
+    else { p.mul = 2; p.ca = ow; p.cb = 0; p.ck = 0; p.sh = 7 - bits_x; }
     p.rs_a = p.ca ? rs_a : nullptr;                      // row sums of the x operand bytes
     p.rs_b = p.cb ? rs_b : nullptr;                      // row sums of the w operand bytes
     p.y = y; p.y_dtype = y_dtype; p.ldy = ldy; p.acc = acc; p.mask = nullptr; p.sw2 = nullptr; p.up_row0 = 0;

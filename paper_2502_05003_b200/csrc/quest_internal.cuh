@@ -135,15 +135,17 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                     float trust_factor, cudaStream_t st, int grid = GRID_UNIFORM);
 int launch_unpack(const uint8_t *codes, int bits, int64_t rows, int64_t K, int8_t *out,
                   int32_t *rowsum, cudaStream_t st, bool e2m1 = false);
-// Both operands of one contraction in a single launch (row sums follow where asked for).
-int launch_unpack_pair(const uint8_t *xq, int bits_x, int64_t M, int8_t *a8, int32_t *rs_a,
-                       const uint8_t *wq, int bits_w, int64_t N, int8_t *b8, int32_t *rs_b, int64_t K, bool e2m1,
-                       cudaStream_t st);
+// Packed codes -> tensor-core operands of one contraction in a single launch (an operand that is NULL is left out).
+int launch_unpack_pair(const uint8_t *xq, int bits_x, int64_t M, int8_t *a8, const uint8_t *wq, int bits_w, int64_t N,
+                       int8_t *b8, int64_t K, bool e2m1, cudaStream_t st);
+// Row sums of two byte operands with the same row length, signed or unsigned, in one launch (NULL: not wanted).
+int launch_rowsum_pair(const void *a, int64_t rows_a, bool unsigned_a, int32_t *out_a,
+                       const void *b, int64_t rows_b, bool unsigned_b, int32_t *out_b, int64_t K, cudaStream_t st);
 int launch_rowsum(const int8_t *a8, int64_t rows, int64_t K, int32_t *rowsum, cudaStream_t st);
 int launch_gemm(const int8_t *a8, const int8_t *b8, const int32_t *rs_a, const int32_t *rs_b,
                 int bits_x, int bits_w, const float *sx, const float *sw,
                 int64_t M, int64_t N, int64_t K, void *y, int y_dtype, int64_t ldy,
-                int32_t *acc, cudaStream_t st);
+                int32_t *acc, cudaStream_t st, bool x_codes = false, bool w_codes = false);   // *_codes: 8-bit codes as they are
 
 int launch_gemm_swiglu(const int8_t *a8, const int8_t *b8, const int32_t *rs_a, const int32_t *rs_b, int bits,
                        const float *sx, const float *sw_gate, const float *sw_up, int64_t M, int64_t I, int64_t K,

@@ -83,6 +83,24 @@ def test_bit_width_combinations(bx, bw):
     run_case(200, 328, K, bx, bw, torch.float32, seed=bx * 9 + bw)
 
 
+@pytest.mark.parametrize("M,N,K", [(1, 8, 32), (37, 29, 96), (130, 260, 544), (300, 264, 2080)])
+@pytest.mark.parametrize("bx,bw", [(8, 8), (8, 3), (1, 8), (7, 8)])
+def test_eight_bit_codes_as_unsigned_operands(M, N, K, bx, bw):
+    # rows of fewer lanes than a warp, a partial last pass of the row sums, one operand unpacked and the other not
+    run_case(M, N, K, bx, bw, torch.float32, seed=M + K + bx)
+
+
+def test_extreme_eight_bit_codes():
+    import paper_2502_05003_b200 as quest
+    K = 16384                                            # 255 * 255 * K: half of what int32 holds
+    for lx, lw in ((255, 255), (0, 255), (255, 0), (0, 0)):
+        xq = torch.full((130, K), lx, dtype=torch.uint8, device="cuda")
+        wq = torch.full((136, K), lw, dtype=torch.uint8, device="cuda")
+        ones = torch.ones(136, dtype=torch.float32, device="cuda")
+        _, acc = quest.quest_lowbit_gemm(xq, ones[:130], 8, wq, ones, 8, K, want_y=False, want_acc=True)
+        assert bool((acc == (2 * lx - 255) * (2 * lw - 255) * K).all())
+
+
 def test_extreme_codes_do_not_overflow():
     import paper_2502_05003_b200 as quest
     K = 4096
