@@ -162,6 +162,125 @@ iht_rows_kernel(const void *__restrict__ d, int in_dtype, long long ld_in, long 
     }
 }
 
+// The same transform for blocks of g = 2^L = 256 .. 4096, 64 elements per thread.  Phase A: the g/64 threads of a
+// block take pairs of neighbouring elements 2p + 64 j apart (2p + 128 j at g = 4096), so that the strides g/2 .. 64
+// (.. 128) stay in a thread's registers and a warp reads consecutive memory.  The result goes through shared memory
+// in row order (16 bytes of padding per 64 elements: no bank conflicts either way); phase B takes 64 contiguous
+// elements (at g = 4096 first stride 64 against the neighbouring thread's), strides 32 .. 1, and the scaled output
+// goes back through the same shared memory so that it leaves in consecutive 16-byte stores.  The order of the stages
+// and every operand are those of the kernel above: identical results.
+// Bound by memory traffic (the masked product is read from L2, where the contraction left it).
+template <int L>
+__global__ void __launch_bounds__(128, 4)
+iht_wide_kernel(const float *__restrict__ d, long long rows, int cols, float inv_sqrt_g, void *__restrict__ out,
+                int out_dtype, long long ld, int S, int R) {
+    extern __shared__ __align__(16) float tbuf[];              // [R][cols + cols / 16]
+    constexpr int NA = L == 12 ? 5 : L - 6;                    // strides of phase A
+    constexpr int NL = 5 - NA;
+    constexpr int HI = L == 12 ? 128 : 64;                     // elements between the pairs that phase A combines
+    constexpr int TB = 1 << (L - 6);                           // threads per rotation block
+    pdl_launch_dependents();
+    pdl_wait();
+    const int tid = threadIdx.x;
+    const int r_local = tid / S;
+    const int tr = tid - r_local * S;
+    const long long row0 = (long long)blockIdx.x * R;
+    const long long row = row0 + r_local;
+    const bool active = row < rows && tr < (cols >> 6);
+    const int pitch = cols + (cols >> 4);
+    float *trow = tbuf + (size_t)r_local * pitch;
+    float2 v[32];
+    const float2 neg1 = make_float2(-1.0f, -1.0f);
+    if (active) {
+        const int p = tr & (TB - 1);
+        const int i0 = (tr / TB) * (1 << L) + 2 * p;           // first element of this thread's pairs
+        const float *src = d + row * cols + i0;
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+            v[j] = __ldg(reinterpret_cast<const float2 *>(src + (j >> NL) * HI + 2 * ((j & ((1 << NL) - 1)) << NA)));
+#pragma unroll
+        for (int s = 16; s >= (1 << NL); s >>= 1)
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if ((j & s) == 0) {
+                    const float2 a = v[j], b = v[j + s];
+                    v[j] = __fadd2_rn(a, b);
+                    v[j + s] = __ffma2_rn(b, neg1, a);
+                }
+        float *dst = trow + i0 + ((i0 >> 6) << 2);
+#pragma unroll
+        for (int j = 0; j < 32; ++j)
+            *reinterpret_cast<float2 *>(dst + (j >> NL) * (HI + HI / 16) + 2 * ((j & ((1 << NL) - 1)) << NA)) = v[j];
+    }
+    __syncthreads();
+    if (active) {
+        const float4 *own = reinterpret_cast<const float4 *>(trow + tr * 68);
+        if constexpr (L == 12) {
+            const float4 *oth = reinterpret_cast<const float4 *>(trow + (tr ^ 1) * 68);
+            const float sg = (tr & 1) ? -1.0f : 1.0f;
+            const float2 sg2 = make_float2(sg, sg);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const float4 a = own[q], b = oth[q];
+                v[2 * q] = __ffma2_rn(make_float2(a.x, a.y), sg2, make_float2(b.x, b.y));
+                v[2 * q + 1] = __ffma2_rn(make_float2(a.z, a.w), sg2, make_float2(b.z, b.w));
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const float4 a = own[q];
+                v[2 * q] = make_float2(a.x, a.y);
+                v[2 * q + 1] = make_float2(a.z, a.w);
+            }
+        }
+#pragma unroll
+        for (int s = 16; s >= 1; s >>= 1)
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if ((j & s) == 0) {
+                    const float2 a = v[j], b = v[j + s];
+                    v[j] = __fadd2_rn(a, b);
+                    v[j + s] = __ffma2_rn(b, neg1, a);
+                }
+        const float2 sc = make_float2(inv_sqrt_g, inv_sqrt_g);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = __fmul2_rn(make_float2(v[j].x + v[j].y, v[j].x - v[j].y), sc);
+    }
+    if constexpr (L == 12) __syncthreads();                    // the neighbour has read this thread's elements
+    if (active) {
+        if (out_dtype == QUEST_F32) {
+            float4 *o = reinterpret_cast<float4 *>(trow + tr * 68);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) o[q] = make_float4(v[2 * q].x, v[2 * q].y, v[2 * q + 1].x, v[2 * q + 1].y);
+        } else {
+            uint4 *o = reinterpret_cast<uint4 *>(trow + tr * 68);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                uint32_t w[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const __nv_bfloat162 h = __floats2bfloat162_rn(v[4 * q + j].x, v[4 * q + j].y);
+                    w[j] = *reinterpret_cast<const uint32_t *>(&h);
+                }
+                o[q] = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+        }
+    }
+    __syncthreads();
+    // coalesced stores: 16-byte chunk c of a row belongs to thread c / 16 (binary32) or c / 8 (bfloat16) of the row
+    const int sh = out_dtype == QUEST_F32 ? 4 : 3;
+    const int chunks = cols >> (6 - sh);
+    const long long left = rows - row0;
+    const int rows_here = left < R ? (int)left : R;
+    const size_t row_bytes = (size_t)ld * (out_dtype == QUEST_F32 ? 4 : 2);
+    for (int r = 0; r < rows_here; ++r) {
+        uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(out) + (size_t)(row0 + r) * row_bytes);
+        const float *from = tbuf + (size_t)r * pitch;
+        for (int c = tid; c < chunks; c += (int)blockDim.x)
+            dst[c] = *reinterpret_cast<const uint4 *>(from + (c >> sh) * 68 + (c & ((1 << sh) - 1)) * 4);
+    }
+}
+
 struct BwdWorkspace {
     uint16_t *wh, *xh;      // dequantised operands [N x K], [M x K]
     float *d1, *d2;         // masked products when the inverse transform is a separate kernel
@@ -180,8 +299,32 @@ BwdWorkspace carve_bwd(void *base, int64_t M, int64_t N, int64_t K) {
     return w;
 }
 
+template <int L>
+cudaError_t launch_iht_wide(const float *d, int64_t rows, int64_t cols, int had_block, void *out, int out_dtype, int64_t ld,
+                            cudaStream_t st) {
+    const int T = (int)(cols >> 6);                            // at most 128 (cols <= 8192)
+    int S = 1;
+    while (S < T) S <<= 1;
+    const int R = 128 / S;
+    const size_t smem = sizeof(float) * (size_t)R * (size_t)(cols + cols / 16);      // at most 34 KB
+    return launch_pdl(iht_wide_kernel<L>, dim3((unsigned)((rows + R - 1) / R)), dim3(128), smem, st, 1, d, (long long)rows,
+                      (int)cols, 1.0f / sqrtf((float)had_block), out, out_dtype, (long long)ld, S, R);
+}
+
 int launch_iht(const float *d, int64_t rows, int64_t cols, int had_block, void *out, int out_dtype, int64_t ld,
                cudaStream_t st) {
+    // blocks of 256 .. 4096 in rows that one CTA holds with 64 elements per thread
+    if (rows > 0 && had_block >= 256 && had_block <= 4096 && cols <= 8192) {
+        cudaError_t e;
+        switch (had_block) {
+            case 256: e = launch_iht_wide<8>(d, rows, cols, had_block, out, out_dtype, ld, st); break;
+            case 512: e = launch_iht_wide<9>(d, rows, cols, had_block, out, out_dtype, ld, st); break;
+            case 1024: e = launch_iht_wide<10>(d, rows, cols, had_block, out, out_dtype, ld, st); break;
+            case 2048: e = launch_iht_wide<11>(d, rows, cols, had_block, out, out_dtype, ld, st); break;
+            default: e = launch_iht_wide<12>(d, rows, cols, had_block, out, out_dtype, ld, st); break;
+        }
+        return e == cudaSuccess ? QUEST_OK : cuda_fail(e);
+    }
     return launch_hadamard_rows(d, QUEST_F32, cols, rows, cols, had_block, out, out_dtype, ld, st);
 }
 

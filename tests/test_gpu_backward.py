@@ -113,6 +113,14 @@ def test_hadamard_block_sizes(g):
     run_case(gauss(200, 2048, 5), gauss(256, 2048, 6, 0.02), 4, g, seed=g)
 
 
+@pytest.mark.parametrize("M,N,K,g", [(40, 24, 768, 256),        # eight rows per CTA of the transform, four slots of padding
+                                     (24, 136, 2560, 512),      # one row per CTA, 40 of 64 threads
+                                     (136, 8, 3072, 1024), (48, 40, 6144, 2048), (8, 72, 4096, 4096), (24, 16, 8192, 4096)])
+@pytest.mark.parametrize("out_dtype", [torch.float32, torch.bfloat16])
+def test_wide_blocks(M, N, K, g, out_dtype):
+    run_case(gauss(M, K, 31), gauss(N, K, 32, 0.02), 4, g, seed=K + g, out_dtype=out_dtype)
+
+
 def _drop_rows_and_blocks(mx, mw):
     """Extreme bitmaps: a row that trusts nothing, a fully masked rotation block of 128, an isolated
     masked element, and alternating bits."""
