@@ -11,9 +11,9 @@
 //   1. dequant_codes_kernel   wq_h [N x K], xq_h [M x K] from the packed codes and scales
 //   2. gemm (bfloat16 mode)   d1[m][k] = M_x[m][k] sum_n dy[m][n] wq_h[n][k]   (dy K-major, wq_h MN-major)
 //                             d2[n][k] = M_w[n][k] sum_m dy[m][n] xq_h[m][k]   (dy and xq_h MN-major)
-//   3. iht_rows_kernel        block Hadamard transform, 1/sqrt(g), store in the output type
-//      (for blocks of 128 stages 2 and 3 are one kernel: the transform runs in the GEMM epilogue,
-//      where a thread holds exactly one block of its output row)
+//   3. iht_wide / iht_rows    block Hadamard transform, 1/sqrt(g), store in the output type
+//      (for blocks of up to 128 stages 2 and 3 are one kernel: the transform runs in the GEMM epilogue,
+//      where a thread holds 128 aligned columns of its output row)
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -411,24 +411,26 @@ extern "C" int quest_linear_bwd(const void *dy, int64_t M, int64_t N, int64_t K,
         }
         if (e != cudaSuccess) return cuda_fail(e);
     }
+    // blocks of up to 128 in rows of whole 128-column groups: the inverse transform runs in the contraction's epilogue,
+    // the masked product never reaches memory
+    const bool fuse = had_block <= 128 && K % 128 == 0 && K > 128;
     if (dx) {
         Stage gemm_stage(QUEST_STAGE_GEMM, st);
         // activation gradient of Algorithm 2 with its trust mask: d1[m][k] = M_x[m][k] * sum_n dy[m][n] wq_h[n][k]
-        // (blocks of 128: the inverse transform is fused into the contraction's epilogue)
-        if (had_block == 128 && M > 128 && K > 128) {
-            if ((s = launch_gemm_bf16_masked(dy, ws.wh, M, K, N, mx, dx, out_dtype, true, 1, st))) return s;
+        if (fuse && M > 128) {
+            if ((s = launch_gemm_bf16_masked(dy, ws.wh, M, K, N, mx, dx, out_dtype, had_block, 1, st))) return s;
         } else {
-            if ((s = launch_gemm_bf16_masked(dy, ws.wh, M, K, N, mx, ws.d1, QUEST_F32, false, 1, st))) return s;
+            if ((s = launch_gemm_bf16_masked(dy, ws.wh, M, K, N, mx, ws.d1, QUEST_F32, 0, 1, st))) return s;
             if ((s = launch_iht(ws.d1, M, K, had_block, dx, out_dtype, K, st))) return s;
         }
     }
     if (dw) {
         Stage gemm_stage(QUEST_STAGE_GEMM, st);
         // weight gradient of Algorithm 2 with its trust mask: d2[n][k] = M_w[n][k] * sum_m dy[m][n] xq_h[m][k]
-        if (had_block == 128 && N > 128 && K > 128) {
-            if ((s = launch_gemm_bf16_masked(dy, ws.xh, N, K, M, mw, dw, out_dtype, true, 2, st))) return s;
+        if (fuse && N > 128) {
+            if ((s = launch_gemm_bf16_masked(dy, ws.xh, N, K, M, mw, dw, out_dtype, had_block, 2, st))) return s;
         } else {
-            if ((s = launch_gemm_bf16_masked(dy, ws.xh, N, K, M, mw, ws.d2, QUEST_F32, false, 2, st))) return s;
+            if ((s = launch_gemm_bf16_masked(dy, ws.xh, N, K, M, mw, ws.d2, QUEST_F32, 0, 2, st))) return s;
             if ((s = launch_iht(ws.d2, N, K, had_block, dw, out_dtype, K, st))) return s;
         }
     }

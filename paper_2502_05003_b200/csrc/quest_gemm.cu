@@ -75,6 +75,9 @@ struct GemmParams {
     // index the gate rows, sw2 the up rows (rs_b is one array over all rows of B)
     const float *sw2;
     int up_row0;
+    // fused inverse transform (MODE 6): block size, at most 128, and 1 / sqrt of it
+    int iht_g = 0;
+    float iht_scale = 0.0f;
 };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -333,7 +336,9 @@ struct SmemLayout {
 // codes.  MODE 2 (backward pass, Algorithm 2): bfloat16 operands (kind::f16, binary32 accumulators);
 // the epilogue zeroes the elements the trust mask rejects and stores binary32.  MODE 3: MODE 2 plus
 // the inverse Hadamard transform for blocks of 128 fused into the epilogue (BN = 256: the 128
-// columns a thread holds are exactly one block), output in the caller's type.  MODE 4 (weight-only
+// columns a thread holds are exactly one block), output in the caller's type.  MODE 6: the same for smaller blocks
+// (several to a thread); an instantiation of its own because the branches around the stages that a smaller block does
+// not have cost 4 % of the forward and backward pass of 4096 x 2048 x 2048 at g = 128 (105 -> 109.6 us).  MODE 4 (weight-only
 // variant): bfloat16 operands, y = sw[n] * accumulator.  MODE 5 (FP4 grid): packed E2M1 operands on
 // kind::mxf4 with unit block scales; the binary32 accumulators hold sum v_x v_w exactly (multiples of
 // 1/4 below 2^22), reported as acc4 = 4 * sum; tensor memory holds one accumulator buffer of 256
@@ -356,15 +361,16 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                const __grid_constant__ CUtensorMap tmY, GemmParams p) {
     using L = SmemLayout<BN, TWO, MODE == 1>;
     constexpr bool CORR = MODE == 1;
-    constexpr bool BWD = MODE == 2 || MODE == 3;
+    constexpr bool BWD = MODE == 2 || MODE == 3 || MODE == 6;
     constexpr bool F16 = MODE >= 2;               // bfloat16 operands, binary32 accumulators
     constexpr bool WO = MODE == 4;
     constexpr bool MX = MODE == 5;
     constexpr int NBUF = (MX && BN == 256) ? 1 : 2;   // accumulator buffers in tensor memory
     constexpr uint32_t SF_COL = 256;              // MX: 32 columns of scale bytes after the accumulators
-    constexpr bool IHT128 = MODE == 3;
+    constexpr bool IHT_SMALL = MODE == 6;
+    constexpr bool IHT128 = MODE == 3 || IHT_SMALL;
     constexpr bool AMN = OPL == 2, BMN = OPL >= 1;
-    static_assert(OPL == 0 || MODE == 2 || MODE == 3, "MN-major operands: bfloat16 backward modes only");
+    static_assert(OPL == 0 || BWD, "MN-major operands: bfloat16 backward modes only");
     static_assert(!IHT128 || BN == 256, "the fused inverse transform needs 128 columns per thread");
     static_assert(!SWIGLU || (BN == 256 && YT && (MODE == 0 || MODE == 1 || MODE == 5)), "SwiGLU epilogue: integer modes, 256 columns, TMA stores");
     static_assert(!SHORT || (TWO && MODE == 0 && YT && !SWIGLU && OPL == 0), "the short-launch form: plain int8 pair kernel");
@@ -696,8 +702,9 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 release_tmem();
             }
             if constexpr (IHT128) {
-                // trust mask and inverse transform of Algorithm 2 on this thread's block of 128: mask, then the inverse
-                // orthonormal Hadamard transform in registers (descending stride, packed binary32)
+                // trust mask and inverse transform of Algorithm 2 on this thread's 128 columns: mask, then the inverse
+                // orthonormal Hadamard transform of their blocks in registers (descending stride, packed binary32; the
+                // strides of a whole block of 128 that a smaller block does not have are skipped)
                 if (n0 + cbase < p.N) {
                     uint4 mb = make_uint4(0u, 0u, 0u, 0u);
                     if (row_ok) mb = __ldg(reinterpret_cast<const uint4 *>(p.mask + (long long)row * (p.N >> 3) + ((n0 + cbase) >> 3)));
@@ -707,6 +714,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     const float2 neg1 = make_float2(-1.0f, -1.0f);
 #pragma unroll
                     for (int s2 = 32; s2 >= 1; s2 >>= 1) {          // strides 64 .. 2 in pairs of columns
+                        if (IHT_SMALL && 2 * s2 >= p.iht_g) continue;
 #pragma unroll
                         for (int i = 0; i < 64; ++i)
                             if ((i & s2) == 0) {
@@ -717,13 +725,16 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                                 r[2 * (i + s2)] = __float_as_uint(di.x); r[2 * (i + s2) + 1] = __float_as_uint(di.y);
                             }
                     }
-                    const float2 sc = make_float2(0.08838834764831845f, 0.08838834764831845f);    // 1 / sqrt(128)
+                    if (!IHT_SMALL || p.iht_g > 1) {
+                        const float scf = IHT_SMALL ? p.iht_scale : 0.08838834764831845f;     // 1 / sqrt(128)
+                        const float2 sc = make_float2(scf, scf);
 #pragma unroll
-                    for (int i = 0; i < 64; ++i) {                  // stride 1, then the normalisation
-                        const float a = __uint_as_float(r[2 * i]), b = __uint_as_float(r[2 * i + 1]);
-                        const float2 o = __fmul2_rn(make_float2(a + b, a - b), sc);
-                        r[2 * i] = __float_as_uint(o.x);
-                        r[2 * i + 1] = __float_as_uint(o.y);
+                        for (int i = 0; i < 64; ++i) {              // stride 1, then the normalisation
+                            const float a = __uint_as_float(r[2 * i]), b = __uint_as_float(r[2 * i + 1]);
+                            const float2 o = __fmul2_rn(make_float2(a + b, a - b), sc);
+                            r[2 * i] = __float_as_uint(o.x);
+                            r[2 * i + 1] = __float_as_uint(o.y);
+                        }
                     }
                 }
             }
@@ -1438,10 +1449,10 @@ int launch_gemm_swiglu(const int8_t *a8, const int8_t *b8, const int32_t *rs_a, 
 //   0: a [I x Kc], b [J x Kc], the contraction index contiguous (K-major);
 //   1: a [I x Kc] K-major, b [Kc x J] (memory rows run along the contraction: MN-major);
 //   2: a [Kc x I] and b [Kc x J], both MN-major.
-// With fuse_iht128 (J % 128 == 0, I > 128, J > 128) the epilogue also applies the inverse Hadamard
-// transform on blocks of 128 columns and stores out_dtype; otherwise out is binary32.
+// With fuse_iht = g in 1 .. 128 (J % 128 == 0, I > 128, J > 128) the epilogue also applies the inverse Hadamard
+// transform on blocks of g columns and stores out_dtype; with 0 out is the masked product in binary32.
 int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, int64_t Kc,
-                            const uint8_t *mask, void *out, int out_dtype, bool fuse_iht128, int opl, cudaStream_t st) {
+                            const uint8_t *mask, void *out, int out_dtype, int fuse_iht, int opl, cudaStream_t st) {
     if (I == 0 || J == 0) return QUEST_OK;
     GemmParams p;
     p.M = (int)I; p.N = (int)J; p.K = (int)(2 * Kc);
@@ -1468,9 +1479,12 @@ int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, 
     (opl == 2 ? launch_gemm_bn<BNV, MODEV, TWOV, true, 2>(tmA, tmB, tmY, p, st)           \
               : opl == 1 ? launch_gemm_bn<BNV, MODEV, TWOV, true, 1>(tmA, tmB, tmY, p, st) \
                          : launch_gemm_bn<BNV, MODEV, TWOV, true, 0>(tmA, tmB, tmY, p, st))
-    if (fuse_iht128) {
-        if (!pair || J % 128 != 0) return QUEST_ERR_SHAPE;
-        return QUEST_GEMM_BWD(256, 3, true);
+    if (fuse_iht) {
+        if (!pair || J % 128 != 0 || fuse_iht > 128) return QUEST_ERR_SHAPE;
+        p.iht_g = fuse_iht;
+        p.iht_scale = 1.0f / sqrtf((float)fuse_iht);
+        if (fuse_iht == 128) return QUEST_GEMM_BWD(256, 3, true);
+        return QUEST_GEMM_BWD(256, 6, true);
     }
     if (out_dtype != QUEST_F32) return QUEST_ERR_DTYPE;
     if (pair) return QUEST_GEMM_BWD(256, 2, true);

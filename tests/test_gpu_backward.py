@@ -121,6 +121,12 @@ def test_wide_blocks(M, N, K, g, out_dtype):
     run_case(gauss(M, K, 31), gauss(N, K, 32, 0.02), 4, g, seed=K + g, out_dtype=out_dtype)
 
 
+@pytest.mark.parametrize("g", [1, 2, 16, 64])
+@pytest.mark.parametrize("K", [256, 640])                       # the last tile whole, then half empty
+def test_small_blocks_in_the_epilogue(g, K):
+    run_case(gauss(264, K, 41), gauss(136, K, 42, 0.02), 4, g, seed=K + g, edit_masks=_drop_rows_and_blocks)
+
+
 def _drop_rows_and_blocks(mx, mw):
     """Extreme bitmaps: a row that trusts nothing, a fully masked rotation block of 128, an isolated
     masked element, and alternating bits."""
