@@ -1,7 +1,8 @@
 """Builds the CUDA library in-tree: ``python -m paper_2502_05003_b200.build``.
 
 nvcc cross-compiles for sm_100a without a GPU.  The quantizer is compiled with ``-fmad=false``
-(its binary32 operation order is part of the contract); everything else with defaults.
+(its binary32 operation order is part of the contract), and so is the decoding layer that repeats it; everything
+else with defaults.
 """
 from __future__ import annotations
 
@@ -20,6 +21,7 @@ COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", INCLUDE
 UNITS = {
     "quest_api.cu": [],
     "quest_quantize.cu": ["-fmad=false"],
+    "quest_decode.cu": ["-fmad=false"],
     "quest_gemm.cu": [],
     "quest_static.cu": [],
     "quest_backward.cu": [],

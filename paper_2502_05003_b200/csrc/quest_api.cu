@@ -125,6 +125,41 @@ static int validate_gemm_shape(int64_t M, int64_t N, int64_t K, int bits_x, int 
     return QUEST_OK;
 }
 
+static int check_linear_fwd(const void *x, const void *w, int dtype, int64_t M, int64_t N, int64_t K, int bits, int had_block,
+                            float trust_factor, const uint8_t *xq, const float *sx, const uint8_t *mx, const uint8_t *wq,
+                            const float *sw, const uint8_t *mw, int w_is_cached, const void *workspace, size_t workspace_bytes) {
+    if (!xq || !sx || !wq || !sw) return QUEST_ERR_NULL;
+    if (!w_is_cached && !w) return QUEST_ERR_NULL;
+    if (w_is_cached < 0 || w_is_cached > 2) return QUEST_ERR_SHAPE;
+    int s = validate_gemm_shape(M, N, K, bits, bits);
+    if (s) return s;
+    if ((s = validate_quantize(x, dtype, M, K, K, bits, had_block, trust_factor, xq, mx))) return s;
+    if (!w_is_cached && (s = validate_quantize(w, dtype, N, K, K, bits, had_block, trust_factor, wq, mw))) return s;
+    if (!aligned(wq, 16)) return QUEST_ERR_ALIGN;
+    if (!workspace || !aligned(workspace, 256) || workspace_bytes < quest_workspace_bytes(M, N, K, bits, bits))
+        return QUEST_ERR_WORKSPACE;
+    return check_device();
+}
+
+// quest_linear_fwd with cached weights and few rows of x: one launch, or the quantizer and one launch.
+static int linear_fwd_decode(const void *x, int dtype, int64_t M, int64_t N, int64_t K, int bits, int had_block,
+                             float trust_factor, void *y, int y_dtype, uint8_t *xq, float *sx, uint8_t *mx,
+                             uint8_t *wq, float *sw, int w_is_cached, void *workspace, size_t workspace_bytes, cudaStream_t st) {
+    int s = check_linear_fwd(x, nullptr, dtype, M, N, K, bits, had_block, trust_factor, xq, sx, mx, wq, sw, nullptr, w_is_cached,
+                             workspace, workspace_bytes);
+    if (s) return s;
+    Workspace ws = carve_workspace(workspace, M, N, K);
+    const QuantJob jx = {x, M, K, xq, sx, mx, ws.a8, bits == 8 ? ws.rs_a : nullptr};
+    const bool fused = decode_fuses_quantizer(M, K);
+    if (!fused) {
+        StageScope scope(QUEST_STAGE_QUANT_X, st);
+        if ((s = launch_quantize(&jx, 1, dtype, K, bits, had_block, trust_factor, st, GRID_UNIFORM, true))) return s;
+    }
+    StageScope scope(QUEST_STAGE_GEMM, st);
+    return launch_decode(jx, dtype, fused, wq, ws.b8, ws.rs_b, sw, w_is_cached == 1, N, K, bits, had_block, trust_factor, y,
+                         y_dtype, st);
+}
+
 }  // namespace quest
 
 using namespace quest;
@@ -298,17 +333,9 @@ int quest_linear_fwd_quantize(const void *x, const void *w, int dtype, int64_t M
                               uint8_t *xq, float *sx, uint8_t *mx,
                               uint8_t *wq, float *sw, uint8_t *mw, int w_is_cached,
                               void *workspace, size_t workspace_bytes, void *stream) {
-    if (!xq || !sx || !wq || !sw) return QUEST_ERR_NULL;
-    if (!w_is_cached && !w) return QUEST_ERR_NULL;
-    if (w_is_cached < 0 || w_is_cached > 2) return QUEST_ERR_SHAPE;
-    int s = validate_gemm_shape(M, N, K, bits, bits);
+    int s = check_linear_fwd(x, w, dtype, M, N, K, bits, had_block, trust_factor, xq, sx, mx, wq, sw, mw, w_is_cached, workspace,
+                             workspace_bytes);
     if (s) return s;
-    if ((s = validate_quantize(x, dtype, M, K, K, bits, had_block, trust_factor, xq, mx))) return s;
-    if (!w_is_cached && (s = validate_quantize(w, dtype, N, K, K, bits, had_block, trust_factor, wq, mw))) return s;
-    if (!aligned(wq, 16)) return QUEST_ERR_ALIGN;
-    if (!workspace || !aligned(workspace, 256) || workspace_bytes < quest_workspace_bytes(M, N, K, bits, bits))
-        return QUEST_ERR_WORKSPACE;
-    if ((s = check_device())) return s;
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     Workspace ws = carve_workspace(workspace, M, N, K);
     const bool need_rs = bits == 8;
@@ -358,6 +385,9 @@ int quest_linear_fwd(const void *x, const void *w, int dtype, int64_t M, int64_t
     if (!y) return QUEST_ERR_NULL;
     if (y_dtype != QUEST_F32 && y_dtype != QUEST_BF16) return QUEST_ERR_DTYPE;
     if (!aligned(y, y_dtype == QUEST_F32 ? 4 : 2)) return QUEST_ERR_ALIGN;
+    if ((w_is_cached == 1 || w_is_cached == 2) && decode_serves(M, N, K, bits))
+        return linear_fwd_decode(x, dtype, M, N, K, bits, had_block, trust_factor, y, y_dtype, xq, sx, mx, wq, sw, w_is_cached,
+                                 workspace, workspace_bytes, reinterpret_cast<cudaStream_t>(stream));
     int s = quest_linear_fwd_quantize(x, w, dtype, M, N, K, bits, had_block, trust_factor, xq, sx, mx, wq, sw, mw,
                                       w_is_cached, workspace, workspace_bytes, stream);
     if (s) return s;

@@ -63,6 +63,11 @@ Workspace carve_workspace(void *base, int64_t M, int64_t N, int64_t K);
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_begin(bool hold_dependents) {
+    if (!hold_dependents) pdl_launch_dependents();
+    pdl_wait();
+    if (hold_dependents) pdl_launch_dependents();
+}
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
@@ -130,9 +135,21 @@ struct QuantJob {
     uint16_t *rot = nullptr;   // [rows x cols] bfloat16 of the orthonormal rotation (no quantization needed for it)
     uint16_t *cbf = nullptr;   // [rows x cols] grid values as bfloat16
 };
-// Up to two tensors with the same row length, dtype and parameters share one launch.
+// Up to two tensors with the same row length, dtype and parameters share one launch.  for_decode: the launch
+// precedes launch_decode.  That kernel may begin only once everything before the quantizer has finished (so that it
+// may read, ahead of its own wait, what the quantizer does not write), and it takes x as signed bytes 2^(7-b) c at
+// every width.
 int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, int bits, int had_block,
-                    float trust_factor, cudaStream_t st, int grid = GRID_UNIFORM);
+                    float trust_factor, cudaStream_t st, int grid = GRID_UNIFORM, bool for_decode = false);
+// The inference layer with cached weights for a few rows of x, where decode_serves it (quest_decode.cu).  With w_codes the
+// packed codes of w are the source and its operand (and row sums at 8 bits) is written to b8 / rs_b; otherwise b8
+// holds it.  fused: x is quantized in the same launch (only if decode_fuses_quantizer), else by a launch_quantize
+// for_decode directly before.
+bool decode_serves(int64_t M, int64_t N, int64_t K, int bits);
+bool decode_fuses_quantizer(int64_t M, int64_t K);
+int launch_decode(const QuantJob &jx, int dtype, bool fused, const uint8_t *wq, int8_t *b8, int32_t *rs_b, const float *sw,
+                  bool w_codes, int64_t N, int64_t K, int bits, int had_block, float trust_factor, void *y, int y_dtype,
+                  cudaStream_t st);
 int launch_unpack(const uint8_t *codes, int bits, int64_t rows, int64_t K, int8_t *out,
                   int32_t *rowsum, cudaStream_t st, bool e2m1 = false);
 // Packed codes -> tensor-core operands of one contraction in a single launch (an operand that is NULL is left out).

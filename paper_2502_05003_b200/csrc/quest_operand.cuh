@@ -101,27 +101,52 @@ __device__ __forceinline__ float e2m1_value(int code) {
 // 0xA (-1), 0x2 (+1), 0x5 (+3).
 __host__ __device__ inline bool e2m1_operands(int bits_x, int bits_w) { return bits_x <= 2 && bits_w <= 2; }
 
+// Eight levels of CB = 1 or 2 bits, level 0 lowest, nothing above them -> eight E2M1 nibbles.
+template <int CB>
+__device__ __forceinline__ uint32_t e2m1_word_from_levels(uint32_t lv) {
+    static_assert(CB == 1 || CB == 2, "only the one- and two-bit grids are E2M1 subsets");
+    if constexpr (CB == 1) {
+        uint32_t t = (lv | (lv << 12)) & 0x000F000Fu;              // spread: bit j -> bit 0 of nibble j
+        t = (t | (t << 6)) & 0x03030303u;
+        t = (t | (t << 3)) & 0x11111111u;
+        return 0xAAAAAAAAu ^ (t << 3);                             // k = 1 clears the sign bit
+    } else {
+        uint32_t t = (lv | (lv << 8)) & 0x00FF00FFu;               // spread: level j -> low bits of nibble j
+        t = (t | (t << 4)) & 0x0F0F0F0Fu;
+        t = (t | (t << 2)) & 0x33333333u;
+        const uint32_t x = (t ^ (t >> 1)) & 0x11111111u;           // k1 ^ k0: set for the inner levels (+-1)
+        const uint32_t k1 = (t >> 1) & 0x11111111u;
+        // sign = !k1; +-3 = 0b101 (bits 0 and 2) when the level bits agree, +-1 = 0b010 otherwise
+        return ((k1 ^ 0x11111111u) << 3) | ((x ^ 0x11111111u) * 5u) | (x << 1);
+    }
+}
+
 // 32 consecutive codes (CB = 1 or 2 words) -> 32 E2M1 nibbles in element order (4 words).
 template <int CB>
 __device__ __forceinline__ void e2m1_operand_from_code_words(const uint32_t (&w)[CB], uint32_t (&o)[4]) {
-    static_assert(CB == 1 || CB == 2, "only the one- and two-bit grids are E2M1 subsets");
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        if constexpr (CB == 1) {
-            const uint32_t b = (w[0] >> (8 * q)) & 0xFFu;          // eight levels, one bit each
-            uint32_t t = (b | (b << 12)) & 0x000F000Fu;            // spread: bit j -> bit 0 of nibble j
-            t = (t | (t << 6)) & 0x03030303u;
-            t = (t | (t << 3)) & 0x11111111u;
-            o[q] = 0xAAAAAAAAu ^ (t << 3);                         // k = 1 clears the sign bit
-        } else {
-            const uint32_t h = (w[q >> 1] >> (16 * (q & 1))) & 0xFFFFu;   // eight levels, two bits each
-            uint32_t t = (h | (h << 8)) & 0x00FF00FFu;             // spread: level j -> low bits of nibble j
-            t = (t | (t << 4)) & 0x0F0F0F0Fu;
-            t = (t | (t << 2)) & 0x33333333u;
-            const uint32_t x = (t ^ (t >> 1)) & 0x11111111u;       // k1 ^ k0: set for the inner levels (+-1)
-            const uint32_t k1 = (t >> 1) & 0x11111111u;
-            // sign = !k1; +-3 = 0b101 (bits 0 and 2) when the level bits agree, +-1 = 0b010 otherwise
-            o[q] = ((k1 ^ 0x11111111u) << 3) | ((x ^ 0x11111111u) * 5u) | (x << 1);
+        if constexpr (CB == 1) o[q] = e2m1_word_from_levels<1>((w[0] >> (8 * q)) & 0xFFu);
+        else o[q] = e2m1_word_from_levels<2>((w[q >> 1] >> (16 * (q & 1))) & 0xFFFFu);
+    }
+}
+
+// 16 consecutive codes of CB = 4 or 8 bits (CB / 2 words) -> 16 operand bytes in element order (4 words).
+template <int CB>
+__device__ __forceinline__ void operand16_from_codes(const uint32_t (&w)[CB / 2], int bits, uint32_t (&o)[4]) {
+    static_assert(CB == 4 || CB == 8, "narrower codes are E2M1 operands");
+    const uint32_t m = (0xFFu << (8 - bits)) & 0xFFu;
+    const uint32_t M = m * 0x01010101u, C = bits == 8 ? 0x80808080u : (0x80u | (1u << (7 - bits))) * 0x01010101u;
+    if constexpr (CB == 8) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) o[q] = lop3_mask_xor_set(w[q] << (8 - bits), M, C);
+    } else {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const uint32_t lo = lop3_mask_xor_set(w[q] << (8 - bits), M, C);   // elements 0, 2, 4, 6 of the word
+            const uint32_t hi = lop3_mask_xor_set(w[q] << (4 - bits), M, C);   // elements 1, 3, 5, 7
+            o[2 * q] = byte_perm(lo, hi, 0x5140);
+            o[2 * q + 1] = byte_perm(lo, hi, 0x7362);
         }
     }
 }

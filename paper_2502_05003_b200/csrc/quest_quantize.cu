@@ -172,6 +172,7 @@ struct QuantArgs {
     QuantConsts qc;
     float inv_sqrt_g;      // 1 / sqrt(had_block) in binary32
     int S, R;
+    int for_decode;        // see launch_quantize
 };
 
 // Eight positions on the E2M1 value axis -> eight 4-bit codes in one word (element 0 in the low
@@ -455,7 +456,13 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
             if constexpr (GRID == GRID_UNIFORM) {              // the FP4 codes are themselves the tensor-core operand
             if constexpr (CB <= 2) {
                 // one- and two-bit grids: E2M1 nibbles for the FP4 tensor-core path, 16 bytes per 32 elements
-                if (tn.op8) {                                   // uniform over the CTA
+                if (tn.op8 && a.for_decode) {                   // uniform over the CTA; the decoding kernel multiplies bytes
+                    uint32_t o[8];
+                    operand_from_code_words<CB>(w, a.bits, o);
+                    uint4 *dst = reinterpret_cast<uint4 *>(tn.op8 + row * (long long)cols + (long long)tr * E + g32 * 32);
+                    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+                    dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+                } else if (tn.op8) {
                     uint32_t o[4];
                     e2m1_operand_from_code_words<CB>(w, o);
                     *reinterpret_cast<uint4 *>(tn.op8 + row * (long long)(cols >> 1) + (long long)tr * (E / 2) + g32 * 16) =
@@ -497,8 +504,7 @@ __global__ void __launch_bounds__(E == 64 ? 256 : 512)
 quantize_rows_kernel(const __grid_constant__ QuantArgs a) {
     extern __shared__ float xsm[];                 // [E][blockDim.x] exchange, then [warps] partial sums
     constexpr int H = E / 2;                       // float2 pairs per thread
-    pdl_launch_dependents();
-    pdl_wait();
+    pdl_begin(a.for_decode != 0);
     const int tid = threadIdx.x;
     const int which = (int)blockIdx.x >= a.blocks0 ? 1 : 0;
     const QuantTensor &tn = a.t[which];
@@ -552,8 +558,7 @@ quantize_stream_kernel(const __grid_constant__ QuantArgs a, int total_groups, in
     constexpr int H = E / 2;
     constexpr int STREAM_SLOT = 2 * E + 16;
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    pdl_launch_dependents();
-    pdl_wait();
+    pdl_begin(a.for_decode != 0);
     float *xsm = reinterpret_cast<float *>(smem_raw);
     uint8_t *stage = smem_raw + exchange_bytes;
     const int tid = threadIdx.x;
@@ -671,8 +676,7 @@ template <int CB, bool FAST, int GRID, int G>
 __global__ void __launch_bounds__(256, 3)
 quantize_wide_kernel(const __grid_constant__ QuantArgs a, int exchange_bytes) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    pdl_launch_dependents();
-    pdl_wait();
+    pdl_begin(a.for_decode != 0);
     const int cols = a.cols, S = a.S, R = a.R;
     static_assert(G == 32 || G == 64 || G == 128, "rotation blocks of 1024, 2048 or 4096 elements");
     constexpr int gshift = G == 32 ? 5 : G == 64 ? 6 : 7;
@@ -804,8 +808,7 @@ quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
     constexpr int CS = COLS / 32;
     const int S = CS ? CS : a.S, R = CS ? 128 / CS : a.R, cols = COLS ? COLS : a.cols;
     extern __shared__ float xsm[];                 // [warps] partial sums
-    pdl_launch_dependents();
-    pdl_wait();
+    pdl_begin(a.for_decode != 0);
     const int tid = threadIdx.x, lane = tid & 31;
     const int which = (int)blockIdx.x >= a.blocks0 ? 1 : 0;
     const QuantTensor &tn = a.t[which];
@@ -956,8 +959,7 @@ quantize_block128_kernel(const __grid_constant__ QuantArgs a) {
     constexpr bool CT_POW2 = CT != 0 && (CT & (CT - 1)) == 0 && CT <= 32;
     constexpr int CR = CT == 0 ? 0 : CT_POW2 ? 64 / CT : (CT >= 128 ? 1 : 128 / CT);     // the host's choice of rows per CTA
     extern __shared__ __align__(16) uint8_t smem_raw[];   // [warps][8 KB] tiles, then [threads] + [rows] floats
-    pdl_launch_dependents();
-    pdl_wait();
+    pdl_begin(a.for_decode != 0);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int bid = (int)blockIdx.x;
     const int which = (bid >= a.bend[0] ? 1 : 0) + (bid >= a.bend[1] ? 1 : 0) + (bid >= a.bend[2] ? 1 : 0);
@@ -1249,7 +1251,7 @@ static cudaError_t launch_stream(int cb, int grid, int threads, size_t smem, cud
 }  // namespace
 
 int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, int bits, int had_block,
-                    float trust_factor, cudaStream_t st, int grid_kind) {
+                    float trust_factor, cudaStream_t st, int grid_kind, bool for_decode) {
     const QuantConsts qc = grid_kind == GRID_FP4 ? make_quant_consts_fp4(had_block, trust_factor)
                                                  : make_quant_consts(bits, had_block, trust_factor);
     if (grid_kind == GRID_FP4 && cols % 32 != 0) return QUEST_ERR_SHAPE;
@@ -1303,6 +1305,7 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                 a.blocks0 = a.bend[0];
                 a.cols = (int)cols; a.bits = bits; a.had_block = had_block; a.qc = qc; a.S = T; a.R = R;
                 a.inv_sqrt_g = 1.0f / sqrtf((float)had_block);
+            a.for_decode = for_decode ? 1 : 0;
                 const dim3 grid((unsigned)total);
                 const cudaError_t e = grid_kind == GRID_FP4 ? launch_block128<GRID_FP4>(cb, grid, threads, smem, st, a)
                                                             : launch_block128<GRID_UNIFORM>(cb, grid, threads, smem, st, a);
@@ -1349,6 +1352,7 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                 a.t[j] = QuantTensor{nullptr, 0, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
             a.cols = (int)cols; a.bits = bits; a.had_block = had_block; a.qc = qc; a.S = S; a.R = R;
             a.inv_sqrt_g = 1.0f / sqrtf((float)had_block);
+            a.for_decode = for_decode ? 1 : 0;
             const dim3 grid((unsigned)(nb[0] + nb[1]));
             cudaError_t e;
             // the specialised tail: codes, scales and masks requested (or the rotation alone), trust_factor >= 1,

@@ -1,0 +1,77 @@
+"""GPU parity of the inference layer with cached weights and few rows of x: bit for bit what the same rows give in a
+call with many rows (the path that the oracle tests cover), and against the oracle directly."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import quest_oracle as qo
+
+pytestmark = pytest.mark.gpu
+
+
+def layer(M, N, K, dtype, seed):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    x = torch.randn((M, K), generator=gen, device="cuda")
+    x[:, 0] *= 30.0                                       # clipped elements
+    if M > 2:
+        x[2] = 0.0                                        # a row whose RMS is zero
+    w = torch.randn((N, K), generator=gen, device="cuda") * 0.02
+    return x.to(dtype), w.to(dtype)
+
+
+def check(M, N, K, bits, g, dtype=torch.bfloat16, out=torch.bfloat16, trust=1.0, seed=0):
+    import paper_2502_05003_b200 as quest
+    big = 40                                              # above the decoding path
+    x, w = layer(big, N, K, dtype, seed)
+    full = quest.quest_linear_fwd(x, w, bits, g, trust, out_dtype=out)
+    cached = {"wq": full["wq"], "sw": full["sw"]}
+    ws = quest.alloc_workspace(big, N, K, bits, bits)
+    ws.fill_(0x5A)
+    for mode in (False, True):                            # packed codes (writes the operand), then the operand
+        cached["operand_in_workspace"] = mode
+        got = quest.quest_linear_fwd(x[:M], None, bits, g, trust, out_dtype=out, w_cached=cached, workspace=ws)
+        torch.cuda.synchronize()
+        assert quest.quest_device_status() == 0
+        for key in ("xq", "sx", "mx", "y"):
+            assert torch.equal(got[key], full[key][:M]), (key, mode)
+        bare = quest.quest_linear_fwd(x[:M], None, bits, g, trust, out_dtype=out, w_cached=cached, workspace=ws,
+                                      want_masks=False)
+        assert torch.equal(bare["y"], full["y"][:M]) and torch.equal(bare["xq"], full["xq"][:M])
+    # the operand that the decoding path left in the workspace serves the general path
+    again = quest.quest_linear_fwd(x, None, bits, g, trust, out_dtype=out, w_cached=cached, workspace=ws)
+    assert torch.equal(again["y"], full["y"])
+
+
+@pytest.mark.parametrize("bits", [1, 2, 3, 4, 6, 8])
+@pytest.mark.parametrize("M", [1, 3, 8, 9, 17, 32])
+def test_rows_and_widths(M, bits):
+    check(M, 264, 544, bits, 32, seed=M + bits)           # ragged tiles of w, a half chunk of K, two tasks a row
+
+
+@pytest.mark.parametrize("N,K,g", [(8, 32, 32), (24, 96, 1), (40, 160, 4), (520, 768, 256), (16, 1024, 512), (2376, 2048, 2048),
+                                   (136, 5504, 128), (2400, 4096, 4096), (72, 8192, 64), (48, 16384, 8192)])
+@pytest.mark.parametrize("M", [1, 4, 24])
+def test_shapes_and_blocks(M, N, K, g):
+    check(M, N, K, 4, g, seed=M + N)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("out", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("trust", [0.0, 0.5, 1.3])
+def test_types_and_trust_factors(dtype, out, trust):
+    for M in (2, 20):
+        check(M, 200, 1024, 4, 128, dtype, out, trust)
+        check(M, 200, 1024, 8, 64, dtype, out, trust)
+
+
+def test_against_the_oracle():
+    import paper_2502_05003_b200 as quest
+    for bits in (1, 4, 8):
+        x, w = layer(5, 96, 1536, torch.float32, bits)
+        ref = qo.linear_fwd(x.cpu().numpy(), w.cpu().numpy(), bits, 512, 1.0)
+        cached = {"wq": torch.from_numpy(ref["wq"]).cuda(), "sw": torch.from_numpy(ref["sw"]).cuda()}
+        got = quest.quest_linear_fwd(x, None, bits, 512, out_dtype=torch.float32, w_cached=cached)
+        assert np.array_equal(got["xq"].cpu().numpy(), ref["xq"]) and np.array_equal(got["mx"].cpu().numpy(), ref["mx"])
+        assert np.allclose(got["sx"].cpu().numpy(), ref["sx"], rtol=1e-6, atol=0)
+        err = np.abs(got["y"].cpu().numpy().astype(np.float64) - ref["y"]).max()
+        assert err <= 1e-5 * np.abs(ref["y"]).max()
