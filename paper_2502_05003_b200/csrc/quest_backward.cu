@@ -413,11 +413,11 @@ extern "C" int quest_linear_bwd(const void *dy, int64_t M, int64_t N, int64_t K,
     }
     // blocks of up to 128 in rows of whole 128-column groups: the inverse transform runs in the contraction's epilogue,
     // the masked product never reaches memory
-    const bool fuse = had_block <= 128 && K % 128 == 0 && K > 128;
+    const bool fuse = had_block <= 128 && K % 128 == 0;
     if (dx) {
         Stage gemm_stage(QUEST_STAGE_GEMM, st);
         // activation gradient of Algorithm 2 with its trust mask: d1[m][k] = M_x[m][k] * sum_n dy[m][n] wq_h[n][k]
-        if (fuse && M > 128) {
+        if (fuse) {
             if ((s = launch_gemm_bf16_masked(dy, ws.wh, M, K, N, mx, dx, out_dtype, had_block, 1, st))) return s;
         } else {
             if ((s = launch_gemm_bf16_masked(dy, ws.wh, M, K, N, mx, ws.d1, QUEST_F32, 0, 1, st))) return s;
@@ -427,7 +427,7 @@ extern "C" int quest_linear_bwd(const void *dy, int64_t M, int64_t N, int64_t K,
     if (dw) {
         Stage gemm_stage(QUEST_STAGE_GEMM, st);
         // weight gradient of Algorithm 2 with its trust mask: d2[n][k] = M_w[n][k] * sum_m dy[m][n] xq_h[m][k]
-        if (fuse && N > 128) {
+        if (fuse) {
             if ((s = launch_gemm_bf16_masked(dy, ws.xh, N, K, M, mw, dw, out_dtype, had_block, 2, st))) return s;
         } else {
             if ((s = launch_gemm_bf16_masked(dy, ws.xh, N, K, M, mw, ws.d2, QUEST_F32, 0, 2, st))) return s;

@@ -17,18 +17,19 @@
 // grids, whose values +-1 and +-3 are E2M1 numbers: when both operands have at most two bits the
 // workspace holds E2M1 nibbles and the same mode runs the contraction at twice the int8 rate.
 //
-// Two launch shapes of one kernel template.  TWO = false: one CTA per SM, persistent over 128 x BN
-// output tiles.  TWO = true: clusters of two CTAs (tcgen05 cta_group::2) persistent over 256 x 256
-// tiles; each CTA stages its own 128 rows of A and its own 128 of the tile's 256 rows of B, the
-// leader CTA issues one M=256 MMA that reads both CTAs' shared memory, and each CTA's TMEM holds
-// its 128 accumulator rows.  That cuts the operand bytes a CTA pulls from L2 per MAC by a third,
-// which is what bounds the single-CTA shape.  No TMA multicast is used: every CTA loads only tiles
-// it alone needs.
+// Clusters of two CTAs (tcgen05 cta_group::2), persistent over output tiles of 256 x BN, BN = 256 or 128; each CTA
+// stages its own 128 rows of A and its own half of the tile's BN rows of B, the leader CTA issues one M=256 MMA
+// that reads both CTAs' shared memory, and each CTA's TMEM holds its 128 accumulator rows.  No TMA multicast is
+// used: every CTA loads only tiles it alone needs.  A k-block of 128 bytes takes 0.27 .. 0.29 us on a 256-column
+// tile (the tensor cores set the pace) and 0.14 us on a 128-column tile with few pairs at work, 0.20 us with all of
+// them (there the loads do), and a launch with one round of the narrow tiles spends 1 us less outside its main loop:
+// narrow_tiles() below holds the rule.  (Single-CTA tiles of 128 x 256 and 128 x 128 served small products before;
+// they lost to the narrow pair tile everywhere but at K = 512, where they are equal.)
 //
 // Kernel structure:
-//   warp 0      TMA producer: 128B-swizzled K-major tiles of A (128 x 128 B) and B (BN or BN/2 rows
-//               x 128 B) into a 3..6-stage shared-memory ring, completion on mbarriers
-//   warp 1      MMA issuer: one thread issues tcgen05.mma (M=128 or 256, N=BN, K=32) x 4 per stage
+//   warp 0      TMA producer: 128B-swizzled K-major tiles of A (128 x 128 B) and B (BN/2 rows
+//               x 128 B) into a 5..6-stage shared-memory ring, completion on mbarriers
+//   warp 1      MMA issuer: one thread issues tcgen05.mma (M=256, N=BN, K=32) x 4 per stage
 //               into one of two TMEM accumulator buffers; tcgen05.commit releases the stage /
 //               signals the epilogue
 //   warps 2..9  epilogue: each warp reads its 32 rows x BN/2 columns with tcgen05.ld, hands the TMEM
@@ -37,6 +38,8 @@
 //               overlaps the next tile's main loop through the second TMEM buffer
 // Every wait is bounded: on expiry the CTA records a status word, stops issuing work and exits
 // through the common tail (which frees its TMEM).
+#include <algorithm>
+
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -49,7 +52,6 @@ namespace {
 constexpr int BM = 128;          // tile rows (TMEM lanes)
 constexpr int BK = 128;          // bytes (= int8 elements) of K per pipeline stage: one swizzle row
 constexpr int UMMA_K = 32;       // K per tcgen05.mma kind::i8
-constexpr int STAGES = 4;
 constexpr int EPI_WARPS = 8;     // two per TMEM lane quarter, each taking half of the tile's columns
 constexpr int NUM_THREADS = 64 + 32 * EPI_WARPS;
 constexpr long long WAIT_LIMIT_CYCLES = 4000000000LL;   // ~2 s at 2 GHz
@@ -88,9 +90,6 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 }
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     uint32_t ok;
@@ -141,13 +140,6 @@ __device__ __forceinline__ bool elect_one() {
     return is != 0;
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *tm, int c0, int c1, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(bar), "r"(c0), "r"(c1)
-        : "memory");
-}
-
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of 128 bytes,
 // 8-row groups 1024 bytes apart.
 __device__ __forceinline__ uint64_t make_smem_desc(uint32_t smem_addr) {
@@ -176,42 +168,15 @@ __device__ __forceinline__ uint64_t make_smem_desc_mn(uint32_t smem_addr) {
 __host__ __device__ constexpr uint32_t make_idesc_i8(int m, int n) {
     return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
-__device__ __forceinline__ void umma_i8(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                        uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
 // kind::f16 with bfloat16 operands (both K-major) and binary32 accumulation
 __host__ __device__ constexpr uint32_t make_idesc_bf16(int m, int n) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
-}
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
 }
 // kind::mxf4 (Section 4.4, FP4): A and B are packed E2M1 (two per byte, K-major, 64 elements of K per
 // instruction), accumulation in binary32, one UE8M0 scale per 32 elements of K read from tensor
 // memory.  The low-bit path uses no block scales, so every scale byte is 2^0.
 __host__ __device__ constexpr uint32_t make_idesc_mxf4(int m, int n) {
     return (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | (1u << 23) | ((uint32_t)(m >> 4) << 24);
-}
-__device__ __forceinline__ void umma_mxf4(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate, uint32_t sfa_tmem, uint32_t sfb_tmem) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], %1, %2, %3, [%5], [%6], p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(sfa_tmem), "r"(sfb_tmem)
-        : "memory");
 }
 __device__ __forceinline__ void umma_mxf4_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                                uint32_t accumulate, uint32_t sfa_tmem, uint32_t sfb_tmem) {
@@ -225,10 +190,6 @@ __device__ __forceinline__ void umma_mxf4_pair(uint32_t d_tmem, uint64_t a_desc,
 // Four columns of this warp's 32 tensor-memory lanes <- one word each.
 __device__ __forceinline__ void tmem_st4(uint32_t taddr, uint32_t v) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v), "r"(v), "r"(v), "r"(v)
-                 : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
                  : "memory");
 }
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -327,15 +288,14 @@ __device__ __forceinline__ void pin(uint32_t &v) { asm volatile("" : "+r"(v)::"m
 // Shared memory of a CTA, from a 1024-byte-aligned base: output staging, barriers, the column-scale tiles (and the
 // column corrections of 8-bit codes, CBT), then the operand ring.  The ring takes as many stages as the launch's
 // dynamic shared memory holds behind the alignment padding, up to MAX_NSTAGES: the kernel counts them at run time
-// (a pair kernel with 256 columns gets six when the base needs no padding and no correction tile is wanted, else
-// five).  A lone pair saturates with four stages; with every pair loading, the fifth is worth 4-9 % and the sixth
+// (256 columns: six when the base needs no padding and no correction tile is wanted, else five; 128 columns: six).  A lone pair saturates with four stages; with every pair loading, the fifth is worth 4-9 % and the sixth
 // another 1-2 %.
 constexpr int SMEM_OPTIN_MAX = 232448;           // largest dynamic shared memory of a CTA on this part
-template <int BN, bool TWO, bool CBT>
+template <int BN, bool CBT>
 struct SmemLayout {
-    static constexpr int MAX_NSTAGES = TWO ? MAX_STAGES : STAGES;     // a single CTA with 256 columns (48 KB stages) gets four when the base needs no padding, else three
+    static constexpr int MAX_NSTAGES = MAX_STAGES;
     static constexpr int A_BYTES = BM * BK;
-    static constexpr int B_ROWS = TWO ? BN / 2 : BN;         // rows of B this CTA stages
+    static constexpr int B_ROWS = BN / 2;                    // rows of B this CTA stages
     static constexpr int B_BYTES = B_ROWS * BK;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
     static constexpr int SLABS = (BN == 128) ? 2 : 1;        // what the stages leave room for
@@ -355,8 +315,8 @@ struct SmemLayout {
 // MODE 0: int8 operands, scaled output.  MODE 1: int8 operands with the exact correction for 8-bit
 // codes.  MODE 2 (backward pass, Algorithm 2): bfloat16 operands (kind::f16, binary32 accumulators);
 // the epilogue zeroes the elements the trust mask rejects and stores binary32.  MODE 3: MODE 2 plus
-// the inverse Hadamard transform for blocks of 128 fused into the epilogue (BN = 256: the 128
-// columns a thread holds are exactly one block), output in the caller's type.  MODE 6: the same for smaller blocks
+// the inverse Hadamard transform for blocks of 128 fused into the epilogue (the 128 columns a
+// thread holds are exactly one block), output in the caller's type.  MODE 6: the same for smaller blocks
 // (several to a thread); an instantiation of its own because the branches around the stages that a smaller block does
 // not have cost 4 % of the forward and backward pass of 4096 x 2048 x 2048 at g = 128 (105 -> 109.6 us).  MODE 4 (weight-only
 // variant): bfloat16 operands, y = sw[n] * accumulator.  MODE 5 (FP4 grid): packed E2M1 operands on
@@ -375,11 +335,11 @@ struct SmemLayout {
 // for launches in which a CTA pair runs at most two tiles, where set-up and exit are a visible share.  Each warp
 // arrives at the two cluster barriers as early as it can and waits as late as it can, and the output type and the
 // absence of the accumulator output are constants.  With many tiles per pair the plain form measured faster.
-template <int BN, int MODE, bool TWO, bool YT, int OPL = 0, bool SWIGLU = false, bool SHORT = false>
+template <int BN, int MODE, bool YT, int OPL = 0, bool SWIGLU = false, bool SHORT = false>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmY, GemmParams p) {
-    using L = SmemLayout<BN, TWO, MODE == 1>;
+    using L = SmemLayout<BN, MODE == 1>;
     constexpr bool CORR = MODE == 1;
     constexpr bool BWD = MODE == 2 || MODE == 3 || MODE == 6;
     constexpr bool F16 = MODE >= 2;               // bfloat16 operands, binary32 accumulators
@@ -391,11 +351,16 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     constexpr bool IHT128 = MODE == 3 || IHT_SMALL;
     constexpr bool AMN = OPL == 2, BMN = OPL >= 1;
     static_assert(OPL == 0 || BWD, "MN-major operands: bfloat16 backward modes only");
-    static_assert(!IHT128 || BN == 256, "the fused inverse transform needs 128 columns per thread");
+    // epilogue: two groups of four warps take the two column halves of every tile, except that the fused inverse
+    // transform needs 128 columns in a thread: on 128-column tiles the groups take whole tiles in turn
+    constexpr bool ALT = IHT128 && BN == 128;
+    constexpr int CW = ALT ? BN : BN / 2;         // columns per epilogue warp
+    constexpr int TILE_STEP = ALT ? 2 : 1;
+    constexpr int GROUP_THREADS = ALT ? 128 : 32 * EPI_WARPS;
     static_assert(!SWIGLU || (BN == 256 && YT && (MODE == 0 || MODE == 1 || MODE == 5)), "SwiGLU epilogue: integer modes, 256 columns, TMA stores");
-    static_assert(!SHORT || (TWO && MODE == 0 && YT && !SWIGLU && OPL == 0), "the short-launch form: plain int8 pair kernel");
+    static_assert(!SHORT || (MODE == 0 && YT && !SWIGLU && OPL == 0), "the short-launch form: plain int8 pair kernel");
     constexpr int BN_OUT = SWIGLU ? BN / 2 : BN;  // output columns per tile
-    constexpr int TILE_M = TWO ? 2 * BM : BM;    // rows of one output tile (both CTAs of a pair)
+    constexpr int TILE_M = 2 * BM;               // rows of one output tile (both CTAs of a pair)
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // 1024-byte aligned, still a shared pointer
     // stages of the operand ring that fit behind the padding (the same in every CTA of the launch: the base is a
@@ -426,9 +391,9 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     constexpr uint32_t TMEM_COLS = MX ? 512 : 2 * BN;       // two accumulator buffers (MX: accumulators + scales)
-    // pair variant: rank of this CTA in its cluster of two; rank 0 leads (issues the MMAs, owns the
-    // full and accumulator-empty barriers that both CTAs signal)
-    const uint32_t rank = TWO ? cluster_ctarank() : 0u;
+    // rank of this CTA in its cluster of two; rank 0 leads (issues the MMAs, owns the full and
+    // accumulator-empty barriers that both CTAs signal)
+    const uint32_t rank = cluster_ctarank();
     const bool leader = rank == 0;
     pdl_launch_dependents();
     if (threadIdx.x == 32) {
@@ -437,8 +402,8 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
         if constexpr (YT) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmY)) : "memory");
     }
-    const int unit = TWO ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;          // tile-loop index
-    const int num_units = TWO ? (int)(gridDim.x >> 1) : (int)gridDim.x;
+    const int unit = (int)(blockIdx.x >> 1);                                  // tile-loop index
+    const int num_units = (int)(gridDim.x >> 1);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -447,7 +412,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(smem_u32(&tfull_bar[b]), 1);
-            mbar_init(smem_u32(&tempty_bar[b]), TWO ? 2 * EPI_WARPS : EPI_WARPS);   // epilogue warps (of both CTAs of a pair)
+            mbar_init(smem_u32(&tempty_bar[b]), 2 * EPI_WARPS / TILE_STEP);         // epilogue warps of both CTAs that read a tile
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -460,22 +425,16 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         cluster_arrive();
     }
     if (warp == 1) {
-        if constexpr (TWO) {      // executed by this warp of both CTAs of the pair
-            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                         "r"(TMEM_COLS)
-                         : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-        } else {
-            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                         "r"(TMEM_COLS)
-                         : "memory");
-            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-        }
+        // executed by this warp of both CTAs of the pair
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"(TMEM_COLS)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
     if constexpr (SHORT) cluster_wait();         // the peer's barriers are initialised before anything signals them
-    else if constexpr (TWO) cluster_sync_all();
+    else cluster_sync_all();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     if constexpr (MX) {
@@ -489,7 +448,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         tc_fence_before();
         __syncthreads();
-        if constexpr (TWO) cluster_sync_all();   // the leader's MMAs read the scales of both CTAs
+        cluster_sync_all();                      // the leader's MMAs read the scales of both CTAs
         tc_fence_after();
     }
     pdl_wait();     // set-up above overlaps the previous kernel; operands and outputs are touched only from here
@@ -521,43 +480,22 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                     uint8_t *sa = ring + stage * L::STAGE_BYTES;
                     // K-major: one box of 128 bytes of K x rows.  MN-major: 64 x 64 chunks (128 bytes of the
                     // M / N dimension x 64 k), 8192 bytes each, in the order of the M / N dimension.
-                    if constexpr (TWO) {
-                        // both CTAs' loads complete on the leader's barrier, which expects the bytes of both
-                        if (leader) mbar_expect_tx(fb, 2 * L::STAGE_BYTES);
-                        const uint32_t lfb = mapa_shared(fb, 0);
-                        if constexpr (AMN) {
+                    // both CTAs' loads complete on the leader's barrier, which expects the bytes of both
+                    if (leader) mbar_expect_tx(fb, 2 * L::STAGE_BYTES);
+                    const uint32_t lfb = mapa_shared(fb, 0);
+                    if constexpr (AMN) {
 #pragma unroll
-                            for (int c = 0; c < BM / 64; ++c)
-                                tma_load_2d_pair(smem_u32(sa + c * 8192), &tmA, (m0 + 64 * c) * 2, kb * 64, lfb);
-                        } else {
-                            tma_load_2d_pair(smem_u32(sa), &tmA, kb * BK, m0, lfb);
-                        }
-                        if constexpr (BMN) {
-#pragma unroll
-                            for (int c = 0; c < L::B_ROWS / 64; ++c)
-                                tma_load_2d_pair(smem_u32(sa + L::A_BYTES + c * 8192), &tmB, (n0 + 64 * c) * 2, kb * 64, lfb);
-                        } else {
-                            tma_load_2d_pair(smem_u32(sa + L::A_BYTES), &tmB, kb * BK, n0, lfb);
-                        }
+                        for (int c = 0; c < BM / 64; ++c)
+                            tma_load_2d_pair(smem_u32(sa + c * 8192), &tmA, (m0 + 64 * c) * 2, kb * 64, lfb);
                     } else {
-                        mbar_expect_tx(fb, L::STAGE_BYTES);
-                        if constexpr (AMN) {
+                        tma_load_2d_pair(smem_u32(sa), &tmA, kb * BK, m0, lfb);
+                    }
+                    if constexpr (BMN) {
 #pragma unroll
-                            for (int c = 0; c < BM / 64; ++c)
-                                tma_load_2d(smem_u32(sa + c * 8192), &tmA, (m0 + 64 * c) * 2, kb * 64, fb);
-                        } else {
-                            tma_load_2d(smem_u32(sa), &tmA, kb * BK, m0, fb);
-                        }
-                        if constexpr (BMN) {
-#pragma unroll
-                            for (int c = 0; c < L::B_ROWS / 64; ++c)
-                                tma_load_2d(smem_u32(sa + L::A_BYTES + c * 8192), &tmB, (n0 + 64 * c) * 2, kb * 64, fb);
-                        } else if constexpr (SWIGLU) {         // two boxes of 128 rows: gate rows, then up rows
-                            tma_load_2d(smem_u32(sa + L::A_BYTES), &tmB, kb * BK, n0, fb);
-                            tma_load_2d(smem_u32(sa + L::A_BYTES + (BN / 2) * BK), &tmB, kb * BK, n0 + p.up_row0, fb);
-                        } else {
-                            tma_load_2d(smem_u32(sa + L::A_BYTES), &tmB, kb * BK, n0, fb);
-                        }
+                        for (int c = 0; c < L::B_ROWS / 64; ++c)
+                            tma_load_2d_pair(smem_u32(sa + L::A_BYTES + c * 8192), &tmB, (n0 + 64 * c) * 2, kb * 64, lfb);
+                    } else {
+                        tma_load_2d_pair(smem_u32(sa + L::A_BYTES), &tmB, kb * BK, n0, lfb);
                     }
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
@@ -603,39 +541,31 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         const uint64_t bd = b_desc + (uint64_t)(kk * (BMN ? 128 : (UMMA_K >> 4)));
                         const uint32_t accum = (kb | kk) != 0 ? 1u : 0u;
                         if constexpr (MX) {       // 32 bytes of K = 64 E2M1 per instruction
-                            if constexpr (TWO) umma_mxf4_pair(d_tmem, ad, bd, idesc, accum, tmem_base + SF_COL, tmem_base + SF_COL + 16);
-                            else umma_mxf4(d_tmem, ad, bd, idesc, accum, tmem_base + SF_COL, tmem_base + SF_COL + 16);
+                            umma_mxf4_pair(d_tmem, ad, bd, idesc, accum, tmem_base + SF_COL, tmem_base + SF_COL + 16);
                         } else if constexpr (F16) {      // 32 bytes of K = 16 bfloat16 per instruction
-                            if constexpr (TWO) umma_bf16_pair(d_tmem, ad, bd, idesc, accum);
-                            else umma_bf16(d_tmem, ad, bd, idesc, accum);
+                            umma_bf16_pair(d_tmem, ad, bd, idesc, accum);
                         } else {
-                            if constexpr (TWO) umma_i8_pair(d_tmem, ad, bd, idesc, accum);
-                            else umma_i8(d_tmem, ad, bd, idesc, accum);
+                            umma_i8_pair(d_tmem, ad, bd, idesc, accum);
                         }
                     }
                     // stage reusable (in both CTAs of a pair) once these MMAs retire
-                    if constexpr (TWO) umma_commit_pair(smem_u32(&empty_bar[stage]));
-                    else umma_commit(smem_u32(&empty_bar[stage]));
+                    umma_commit_pair(smem_u32(&empty_bar[stage]));
                     if (++stage == STAGES) { stage = 0; phase ^= 1u; }
                 }
-                if (ok) {                                          // accumulator complete
-                    if constexpr (TWO) umma_commit_pair(smem_u32(&tfull_bar[buf]));
-                    else umma_commit(smem_u32(&tfull_bar[buf]));
-                }
+                if (ok) umma_commit_pair(smem_u32(&tfull_bar[buf]));          // accumulator complete
             }
         }
         __syncwarp();
     } else {
         // ---- epilogue: 8 warps; warp w reads TMEM lanes [32 (w & 3), +32) = tile rows 32 (w & 3) + lane
         //      and the column half (w - 2) / 4 of the tile ------------------------------------------------
-        constexpr int CW = BN / 2;                     // columns per warp
         const int quarter = warp & 3;
         const int hgrp = (warp - 2) >> 2;              // which half of the tile's (output) columns
-        const int cbase = hgrp * CW;
+        const int cbase = ALT ? 0 : hgrp * CW;
         // plain modes: a warp takes CW consecutive accumulator columns; SwiGLU: gate columns [64 hgrp, +64) and
         // the up columns of the same outputs, 128 further on
         const int ep_tid = threadIdx.x - 64;           // 0..255 over the epilogue warps
-        int t = 0;
+        int t = ALT ? hgrp : 0;
         bool ok = true;
         const bool vec_y = p.y && (((reinterpret_cast<uintptr_t>(p.y) & 15) == 0) &&
                                    (p.ldy % (p.y_dtype == QUEST_BF16 ? 8 : 4) == 0));
@@ -643,7 +573,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const bool y_f32 = !SHORT && p.y_dtype == QUEST_F32;
         uint8_t *slab_base = smem + L::STG_OFFSET + (warp - 2) * (L::SLABS * 4096);
         int slab_count = 0;                            // slabs this warp has handed to TMA
-        for (int tile = unit; tile < num_tiles && ok; tile += num_units, ++t) {
+        for (int tile = unit + t * num_units; tile < num_tiles && ok; tile += TILE_STEP * num_units, t += TILE_STEP) {
             int tm, tn;
             tile_coords(tile, num_m, num_n, tm, tn);
             const int m0 = tm * TILE_M + (int)rank * BM;
@@ -677,17 +607,17 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             int rsa = 0;
             if (CORR) rsa = (row_ok && p.rs_a) ? p.ca * __ldg(p.rs_a + row) + p.ck : p.ck;
             ok = mbar_wait(smem_u32(&tfull_bar[buf]), bphase, abort_flag, p.status, ST_EPILOGUE);
-            // one barrier over the epilogue threads publishes the staged scales and makes the
+            // one barrier over the epilogue threads of the tile publishes the staged scales and makes the
             // continue/abort decision unanimous, so no warp can be left waiting at a later barrier
             {
                 uint32_t all_ok;
                 asm volatile(
                     "{\n\t.reg .pred p, q;\n\t"
                     "setp.ne.u32 q, %1, 0;\n\t"
-                    "bar.red.and.pred p, 1, %2, q;\n\t"
+                    "bar.red.and.pred p, %3, %2, q;\n\t"
                     "selp.u32 %0, 1, 0, p;\n\t}"
                     : "=r"(all_ok)
-                    : "r"((uint32_t)(ok ? 1u : 0u)), "n"(32 * EPI_WARPS)
+                    : "r"((uint32_t)(ok ? 1u : 0u)), "n"(GROUP_THREADS), "r"(ALT ? 1 + hgrp : 1)
                     : "memory");
                 ok = all_ok != 0;
             }
@@ -700,10 +630,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             auto release_tmem = [&]() {
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) {
-                    if constexpr (TWO) mbar_arrive_cluster(mapa_shared(smem_u32(&tempty_bar[buf]), 0));   // the leader's barrier
-                    else mbar_arrive(smem_u32(&tempty_bar[buf]));
-                }
+                if (lane == 0) mbar_arrive_cluster(mapa_shared(smem_u32(&tempty_bar[buf]), 0));   // the leader's barrier
                 if constexpr (SHORT) {
                     if (tile + num_units >= num_tiles) {       // this CTA's last tile: nothing more goes to the peer
                         __syncwarp();
@@ -1004,14 +931,11 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         __syncthreads();
         // a CTA of a pair must stay until its peer can no longer signal its barriers or read its
         // shared memory and tensor memory
-        if constexpr (TWO) cluster_sync_all();
+        cluster_sync_all();
     }
     if (warp == 1) {
         tc_fence_after();
-        if constexpr (TWO)
-            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
-        else
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
     }
 }
 
@@ -1260,30 +1184,37 @@ int make_output_map(CUtensorMap *tm, void *base, int64_t rows, int64_t row_bytes
     return QUEST_OK;
 }
 
-template <int BN, int MODE, bool TWO, bool YT, int OPL = 0, bool SWIGLU = false, bool SHORT = false>
-int launch_gemm_bn(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmY, const GemmParams &p,
-                   cudaStream_t st) {
-    using L = SmemLayout<BN, TWO, MODE == 1>;
-    static DynamicSmemOnce smem_attr;            // per kernel instantiation, per device
-    {
-        cudaError_t e = smem_attr.set(gemm_i8_kernel<BN, MODE, TWO, YT, OPL, SWIGLU, SHORT>, L::TOTAL);
-        if (e != cudaSuccess) return cuda_fail(e);
-    }
+int num_sms() {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int tile_m = TWO ? 2 * BM : BM;
-    const int bn_out = SWIGLU ? BN / 2 : BN;
-    const int tiles = ((p.M + tile_m - 1) / tile_m) * ((p.N + bn_out - 1) / bn_out);
-    int grid;
-    if (TWO) {
-        const int pairs = tiles < sms / 2 ? tiles : sms / 2;
-        grid = 2 * pairs;
-    } else {
-        grid = tiles < sms ? tiles : sms;
+    return sms;
+}
+
+// 128-column tiles or 256-column tiles for an M x N product with rows of `row_bytes` operand bytes.  Narrow tiles where
+// they need no more rounds of the CTA pairs (half the time per round: 777 x 2048 x 5504 bytes 16.3 -> 10.4 us), and up
+// to 3 rounds for 2 while the rows are short (3072 x 2048 x 2048: 13.6 -> 12.8 us; equal at 5504 bytes a row; two
+// rounds for one loses from 1024 bytes on: 512 x 5504 x 5504 17.0 -> 20.8 us).
+bool narrow_tiles(int64_t M, int64_t N, int64_t row_bytes) {
+    const int64_t pairs = num_sms() / 2, tm = (M + 255) / 256;
+    const int64_t r2 = (tm * ((N + 255) / 256) + pairs - 1) / pairs, r1 = (tm * ((N + 127) / 128) + pairs - 1) / pairs;
+    return r1 <= r2 || (row_bytes <= 2048 && 2 * r1 <= 3 * r2);
+}
+
+template <int BN, int MODE, bool YT, int OPL = 0, bool SWIGLU = false, bool SHORT = false>
+int launch_gemm_bn(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmY, const GemmParams &p,
+                   cudaStream_t st) {
+    using L = SmemLayout<BN, MODE == 1>;
+    static DynamicSmemOnce smem_attr;            // per kernel instantiation, per device
+    {
+        cudaError_t e = smem_attr.set(gemm_i8_kernel<BN, MODE, YT, OPL, SWIGLU, SHORT>, L::TOTAL);
+        if (e != cudaSuccess) return cuda_fail(e);
     }
-    cudaError_t e = launch_pdl(gemm_i8_kernel<BN, MODE, TWO, YT, OPL, SWIGLU, SHORT>, dim3((unsigned)grid), dim3(NUM_THREADS), (size_t)L::TOTAL, st,
-                               TWO ? 2 : 1, tmA, tmB, tmY, p);
+    const int bn_out = SWIGLU ? BN / 2 : BN;
+    const int tiles = ((p.M + 2 * BM - 1) / (2 * BM)) * ((p.N + bn_out - 1) / bn_out);
+    const int pairs = std::min(tiles, num_sms() / 2);
+    cudaError_t e = launch_pdl(gemm_i8_kernel<BN, MODE, YT, OPL, SWIGLU, SHORT>, dim3((unsigned)(2 * pairs)), dim3(NUM_THREADS),
+                               (size_t)L::TOTAL, st, 2, tmA, tmB, tmY, p);
     return e == cudaSuccess ? QUEST_OK : cuda_fail(e);
 }
 
@@ -1396,12 +1327,11 @@ int launch_gemm(const int8_t *a8, const int8_t *b8, const int32_t *rs_a, const i
     p.status = device_status_word();
     if (!p.status) return QUEST_ERR_CUDA;
 
-    const bool wide = N > 128;
-    const bool pair = wide && M > 128;             // 256 x 256 tiles on CTA pairs
+    const bool narrow = narrow_tiles(M, N, p.K);
     CUtensorMap tmA, tmB;
     int s = make_operand_map(&tmA, a8, M, K, BM);
     if (s) return s;
-    s = make_operand_map(&tmB, b8, N, K, pair ? 128 : wide ? 256 : 128);
+    s = make_operand_map(&tmB, b8, N, K, narrow ? 64 : 128);
     if (s) return s;
     const bool corr = (bits_x == 8) || (bits_w == 8);
     // y through TMA tile stores when its base and row pitch allow it (16-byte multiples)
@@ -1412,22 +1342,17 @@ int launch_gemm(const int8_t *a8, const int8_t *b8, const int32_t *rs_a, const i
         s = make_output_map(&tmY, y, M, (int64_t)N * (int64_t)esz, (int64_t)ldy * (int64_t)esz);
         if (s) return s;
     }
-#define QUEST_GEMM(BNV, TWOV)                                                                        \
-    (corr ? (yt ? launch_gemm_bn<BNV, 1, TWOV, true>(tmA, tmB, tmY, p, st)                            \
-                : launch_gemm_bn<BNV, 1, TWOV, false>(tmA, tmB, tmY, p, st))                           \
-          : (yt ? launch_gemm_bn<BNV, 0, TWOV, true>(tmA, tmB, tmY, p, st)                            \
-                : launch_gemm_bn<BNV, 0, TWOV, false>(tmA, tmB, tmY, p, st)))
-    if (pair && !corr && yt && y_dtype == QUEST_BF16 && !acc) {
+#define QUEST_GEMM(BNV)                                                                              \
+    (corr ? (yt ? launch_gemm_bn<BNV, 1, true>(tmA, tmB, tmY, p, st) : launch_gemm_bn<BNV, 1, false>(tmA, tmB, tmY, p, st))  \
+          : (yt ? launch_gemm_bn<BNV, 0, true>(tmA, tmB, tmY, p, st) : launch_gemm_bn<BNV, 0, false>(tmA, tmB, tmY, p, st)))
+    if (!corr && yt && y_dtype == QUEST_BF16 && !acc) {
         // at most two tiles per CTA pair: the form that hides the cluster barriers of set-up and exit
-        int dev = 0, sms = 148;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int64_t tiles = ((M + 255) / 256) * ((N + 255) / 256);
-        if (tiles <= 2 * (int64_t)(sms / 2)) return launch_gemm_bn<256, 0, true, true, 0, false, true>(tmA, tmB, tmY, p, st);
+        const int64_t tiles = ((M + 255) / 256) * ((N + (narrow ? 127 : 255)) / (narrow ? 128 : 256));
+        if (tiles <= 2 * (int64_t)(num_sms() / 2))
+            return narrow ? launch_gemm_bn<128, 0, true, 0, false, true>(tmA, tmB, tmY, p, st)
+                          : launch_gemm_bn<256, 0, true, 0, false, true>(tmA, tmB, tmY, p, st);
     }
-    if (pair) return QUEST_GEMM(256, true);
-    if (wide) return QUEST_GEMM(256, false);
-    return QUEST_GEMM(128, false);
+    return narrow ? QUEST_GEMM(128) : QUEST_GEMM(256);
 #undef QUEST_GEMM
 }
 
@@ -1449,19 +1374,14 @@ int launch_gemm_swiglu(const int8_t *a8, const int8_t *b8, const int32_t *rs_a, 
     p.y = h; p.y_dtype = QUEST_BF16; p.ldy = I; p.acc = nullptr; p.mask = nullptr;
     p.status = device_status_word();
     if (!p.status) return QUEST_ERR_CUDA;
-    const bool pair = M > 128;
     CUtensorMap tmA, tmB, tmY;
     int s = make_operand_map(&tmA, a8, M, p.K, BM);
     if (s) return s;
     if ((s = make_operand_map(&tmB, b8, 2 * I, p.K, 128))) return s;       // boxes of 128 rows: gate rows or up rows
     if ((s = make_output_map(&tmY, h, M, I * 2, I * 2))) return s;
-#define QUEST_GEMM_SG(MODEV) \
-    (pair ? launch_gemm_bn<256, MODEV, true, true, 0, true>(tmA, tmB, tmY, p, st) \
-          : launch_gemm_bn<256, MODEV, false, true, 0, true>(tmA, tmB, tmY, p, st))
-    if (mx) return QUEST_GEMM_SG(5);
-    if (b8x) return QUEST_GEMM_SG(1);
-    return QUEST_GEMM_SG(0);
-#undef QUEST_GEMM_SG
+    if (mx) return launch_gemm_bn<256, 5, true, 0, true>(tmA, tmB, tmY, p, st);
+    if (b8x) return launch_gemm_bn<256, 1, true, 0, true>(tmA, tmB, tmY, p, st);
+    return launch_gemm_bn<256, 0, true, 0, true>(tmA, tmB, tmY, p, st);
 }
 
 // Backward-pass contraction (the two products of Algorithm 2): out[i][j] = mask[i][j] * sum_k A(i, k) B(j, k) with
@@ -1469,7 +1389,7 @@ int launch_gemm_swiglu(const int8_t *a8, const int8_t *b8, const int32_t *rs_a, 
 //   0: a [I x Kc], b [J x Kc], the contraction index contiguous (K-major);
 //   1: a [I x Kc] K-major, b [Kc x J] (memory rows run along the contraction: MN-major);
 //   2: a [Kc x I] and b [Kc x J], both MN-major.
-// With fuse_iht = g in 1 .. 128 (J % 128 == 0, I > 128, J > 128) the epilogue also applies the inverse Hadamard
+// With fuse_iht = g in 1 .. 128 (J % 128 == 0) the epilogue also applies the inverse Hadamard
 // transform on blocks of g columns and stores out_dtype; with 0 out is the masked product in binary32.
 int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, int64_t Kc,
                             const uint8_t *mask, void *out, int out_dtype, int fuse_iht, int opl, cudaStream_t st) {
@@ -1482,8 +1402,7 @@ int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, 
     const int64_t esz = out_dtype == QUEST_F32 ? 4 : 2;
     p.status = device_status_word();
     if (!p.status) return QUEST_ERR_CUDA;
-    const bool wide = J > 128;
-    const bool pair = wide && I > 128;
+    const bool narrow = narrow_tiles(I, J, p.K);
     CUtensorMap tmA, tmB, tmY;
     int s;
     // MN-major: the tensor is [Kc rows x I (or J) elements]; a box is 128 bytes of a row x 64 rows
@@ -1491,26 +1410,26 @@ int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, 
     else s = make_operand_map(&tmA, reinterpret_cast<const int8_t *>(a), I, 2 * Kc, BM);
     if (s) return s;
     if (opl >= 1) s = make_operand_map(&tmB, reinterpret_cast<const int8_t *>(b), Kc, 2 * J, 64);
-    else s = make_operand_map(&tmB, reinterpret_cast<const int8_t *>(b), J, 2 * Kc, pair ? 128 : wide ? 256 : 128);
+    else s = make_operand_map(&tmB, reinterpret_cast<const int8_t *>(b), J, 2 * Kc, narrow ? 64 : 128);
     if (s) return s;
     s = make_output_map(&tmY, out, I, J * esz, J * esz);
     if (s) return s;
-#define QUEST_GEMM_BWD(BNV, MODEV, TWOV)                                                  \
-    (opl == 2 ? launch_gemm_bn<BNV, MODEV, TWOV, true, 2>(tmA, tmB, tmY, p, st)           \
-              : opl == 1 ? launch_gemm_bn<BNV, MODEV, TWOV, true, 1>(tmA, tmB, tmY, p, st) \
-                         : launch_gemm_bn<BNV, MODEV, TWOV, true, 0>(tmA, tmB, tmY, p, st))
+#define QUEST_GEMM_BWD2(BNV, MODEV)                                                  \
+    (opl == 2 ? launch_gemm_bn<BNV, MODEV, true, 2>(tmA, tmB, tmY, p, st)           \
+              : opl == 1 ? launch_gemm_bn<BNV, MODEV, true, 1>(tmA, tmB, tmY, p, st) \
+                         : launch_gemm_bn<BNV, MODEV, true, 0>(tmA, tmB, tmY, p, st))
+#define QUEST_GEMM_BWD(MODEV) (narrow ? QUEST_GEMM_BWD2(128, MODEV) : QUEST_GEMM_BWD2(256, MODEV))
     if (fuse_iht) {
-        if (!pair || J % 128 != 0 || fuse_iht > 128) return QUEST_ERR_SHAPE;
+        if (J % 128 != 0 || fuse_iht > 128) return QUEST_ERR_SHAPE;
         p.iht_g = fuse_iht;
         p.iht_scale = 1.0f / sqrtf((float)fuse_iht);
-        if (fuse_iht == 128) return QUEST_GEMM_BWD(256, 3, true);
-        return QUEST_GEMM_BWD(256, 6, true);
+        if (fuse_iht == 128) return QUEST_GEMM_BWD(3);
+        return QUEST_GEMM_BWD(6);
     }
     if (out_dtype != QUEST_F32) return QUEST_ERR_DTYPE;
-    if (pair) return QUEST_GEMM_BWD(256, 2, true);
-    if (wide) return QUEST_GEMM_BWD(256, 2, false);
-    return QUEST_GEMM_BWD(128, 2, false);
+    return QUEST_GEMM_BWD(2);
 #undef QUEST_GEMM_BWD
+#undef QUEST_GEMM_BWD2
 }
 
 // Contraction of E2M1 nibble operands xq [M x K/2], wq [N x K/2] on the FP4 tensor-core path:
@@ -1525,12 +1444,11 @@ int launch_gemm_e2m1(const uint8_t *xq, const uint8_t *wq, const float *sx, cons
     p.y = y; p.y_dtype = y_dtype; p.ldy = ldy; p.acc = acc; p.mask = nullptr; p.sw2 = nullptr; p.up_row0 = 0;
     p.status = device_status_word();
     if (!p.status) return QUEST_ERR_CUDA;
-    const bool wide = N > 128;
-    const bool pair = wide && M > 128;
+    const bool narrow = narrow_tiles(M, N, p.K);
     CUtensorMap tmA, tmB;
     int s = make_operand_map(&tmA, reinterpret_cast<const int8_t *>(xq), M, K / 2, BM);
     if (s) return s;
-    s = make_operand_map(&tmB, reinterpret_cast<const int8_t *>(wq), N, K / 2, pair ? 128 : wide ? 256 : 128);
+    s = make_operand_map(&tmB, reinterpret_cast<const int8_t *>(wq), N, K / 2, narrow ? 64 : 128);
     if (s) return s;
     const size_t esz = y_dtype == QUEST_F32 ? 4 : 2;
     const bool yt = y && (reinterpret_cast<uintptr_t>(y) % 16 == 0) && ((size_t)ldy * esz % 16 == 0);
@@ -1539,12 +1457,9 @@ int launch_gemm_e2m1(const uint8_t *xq, const uint8_t *wq, const float *sx, cons
         s = make_output_map(&tmY, y, M, (int64_t)N * (int64_t)esz, (int64_t)ldy * (int64_t)esz);
         if (s) return s;
     }
-#define QUEST_GEMM_MX(BNV, TWOV) \
-    (yt ? launch_gemm_bn<BNV, 5, TWOV, true>(tmA, tmB, tmY, p, st) : launch_gemm_bn<BNV, 5, TWOV, false>(tmA, tmB, tmY, p, st))
-    if (pair) return QUEST_GEMM_MX(256, true);
-    if (wide) return QUEST_GEMM_MX(256, false);
-    return QUEST_GEMM_MX(128, false);
-#undef QUEST_GEMM_MX
+    if (narrow)
+        return yt ? launch_gemm_bn<128, 5, true>(tmA, tmB, tmY, p, st) : launch_gemm_bn<128, 5, false>(tmA, tmB, tmY, p, st);
+    return yt ? launch_gemm_bn<256, 5, true>(tmA, tmB, tmY, p, st) : launch_gemm_bn<256, 5, false>(tmA, tmB, tmY, p, st);
 }
 
 int launch_gemm_bf16_scaled(const void *a, const void *b, const float *sw, int64_t M, int64_t N, int64_t K,
@@ -1557,12 +1472,11 @@ int launch_gemm_bf16_scaled(const void *a, const void *b, const float *sw, int64
     p.y = y; p.y_dtype = y_dtype; p.ldy = ldy; p.acc = nullptr; p.mask = nullptr; p.sw2 = nullptr; p.up_row0 = 0;
     p.status = device_status_word();
     if (!p.status) return QUEST_ERR_CUDA;
-    const bool wide = N > 128;
-    const bool pair = wide && M > 128;
+    const bool narrow = narrow_tiles(M, N, p.K);
     CUtensorMap tmA, tmB;
     int s = make_operand_map(&tmA, reinterpret_cast<const int8_t *>(a), M, 2 * K, BM);
     if (s) return s;
-    s = make_operand_map(&tmB, reinterpret_cast<const int8_t *>(b), N, 2 * K, pair ? 128 : wide ? 256 : 128);
+    s = make_operand_map(&tmB, reinterpret_cast<const int8_t *>(b), N, 2 * K, narrow ? 64 : 128);
     if (s) return s;
     const size_t esz = y_dtype == QUEST_F32 ? 4 : 2;
     const bool yt = (reinterpret_cast<uintptr_t>(y) % 16 == 0) && ((size_t)ldy * esz % 16 == 0);
@@ -1571,12 +1485,9 @@ int launch_gemm_bf16_scaled(const void *a, const void *b, const float *sw, int64
         s = make_output_map(&tmY, y, M, (int64_t)N * (int64_t)esz, (int64_t)ldy * (int64_t)esz);
         if (s) return s;
     }
-#define QUEST_GEMM_WO(BNV, TWOV) \
-    (yt ? launch_gemm_bn<BNV, 4, TWOV, true>(tmA, tmB, tmY, p, st) : launch_gemm_bn<BNV, 4, TWOV, false>(tmA, tmB, tmY, p, st))
-    if (pair) return QUEST_GEMM_WO(256, true);
-    if (wide) return QUEST_GEMM_WO(256, false);
-    return QUEST_GEMM_WO(128, false);
-#undef QUEST_GEMM_WO
+    if (narrow)
+        return yt ? launch_gemm_bn<128, 4, true>(tmA, tmB, tmY, p, st) : launch_gemm_bn<128, 4, false>(tmA, tmB, tmY, p, st);
+    return yt ? launch_gemm_bn<256, 4, true>(tmA, tmB, tmY, p, st) : launch_gemm_bn<256, 4, false>(tmA, tmB, tmY, p, st);
 }
 
 }  // namespace quest

@@ -127,6 +127,13 @@ def test_small_blocks_in_the_epilogue(g, K):
     run_case(gauss(264, K, 41), gauss(136, K, 42, 0.02), 4, g, seed=K + g, edit_masks=_drop_rows_and_blocks)
 
 
+def test_small_blocks_on_wide_tiles():
+    # enough tiles for the 256-column form of the epilogue with blocks below 128 (dL/dx)
+    run_case(gauss(2560, 2048, 43), gauss(1040, 2048, 44, 0.02), 4, 32, seed=3,
+             rows_x=np.random.default_rng(5).choice(2560, 24, replace=False),
+             rows_w=np.random.default_rng(6).choice(1040, 24, replace=False))
+
+
 def _drop_rows_and_blocks(mx, mw):
     """Extreme bitmaps: a row that trusts nothing, a fully masked rotation block of 128, an isolated
     masked element, and alternating bits."""
