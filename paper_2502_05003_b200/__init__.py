@@ -1,7 +1,9 @@
 """B200 (sm_100a) implementation of the QuEST quantized-linear forward pass (arXiv 2502.05003,
 Algorithm 1).  This module is a thin binding over the C ABI in ``include/quest.h``: it marshals
 torch tensors (device memory, current stream) into pointers and sizes; every step of the path
-runs in the CUDA library.  There is no CPU or PyTorch fallback.
+runs in the CUDA library.  There is no CPU or PyTorch fallback.  The per-layer calls go through a
+CPython binding (``csrc/quest_binding.cpp``) when their arguments are the plain case and through
+ctypes otherwise, with the same outcome.
 """
 from __future__ import annotations
 
@@ -38,6 +40,13 @@ def _require_cuda(*ts):
     for t in ts:
         if t is not None and not t.is_cuda:
             raise ValueError("quest: tensors must live in CUDA device memory")
+
+
+def _result(done):
+    """What the CPython binding returned for a call it made: the result, or the status of a call the library refused."""
+    if done.__class__ is int:
+        _lib.check(done)
+    return done
 
 
 def quest_alpha_star(bits: int) -> float:
@@ -97,6 +106,9 @@ def quest_quantize(x: torch.Tensor, bits: int, had_block: int, trust_factor: flo
                    want_mask: bool = True):
     """Rows of ``x`` [rows, cols] -> (codes uint8 [rows, cols*container/8], scales f32 [rows],
     mask uint8 [rows, cols/8] or None)."""
+    done = _lib.binding().quantize(x, bits, had_block, trust_factor, codes, scales, mask, want_mask)
+    if done is not None:
+        return _result(done)
     _require_cuda(x, codes, scales, mask)
     if x.dim() != 2 or x.stride(1) != 1:
         raise ValueError("quest_quantize: x must be 2-D with unit inner stride")
@@ -133,6 +145,9 @@ def quest_lowbit_gemm(xq: torch.Tensor, sx: torch.Tensor, bits_x: int,
                       out_dtype=torch.bfloat16, y: torch.Tensor = None, want_acc: bool = False,
                       acc: torch.Tensor = None, workspace: torch.Tensor = None, want_y: bool = True):
     """Packed codes -> (y [M, N] or None, acc int32 [M, N] or None)."""
+    done = _lib.binding().lowbit_gemm(xq, sx, bits_x, wq, sw, bits_w, K, out_dtype, y, want_acc, acc, workspace, want_y)
+    if done is not None:
+        return _result(done)
     _require_cuda(xq, sx, wq, sw, y, acc, workspace)
     M, N = xq.shape[0], wq.shape[0]
     if y is None and want_y:
@@ -181,6 +196,10 @@ def quest_linear_fwd(x: torch.Tensor, w: torch.Tensor, bits: int, had_block: int
     ``w_cached["operand_in_workspace"]`` true the call also skips unpacking ``wq``: ``workspace``
     must be the tensor an earlier call for the same w used, untouched since (M may differ).
     """
+    done = _lib.binding().linear_fwd(x, w, bits, had_block, trust_factor, out_dtype, y, saved, w_cached, workspace,
+                                      want_masks)
+    if done is not None:
+        return _result(done)
     _require_cuda(x, w, y, workspace)
     M, K = x.shape
     out = dict(saved or {})
@@ -253,6 +272,9 @@ def quest_linear_bwd(dy: torch.Tensor, fwd: dict, bits: int, had_block: int, K: 
                      workspace: torch.Tensor = None) -> dict:
     """Algorithm 2 from the forward call's saved tensors (``fwd`` holds xq, sx, mx, wq, sw, mw).
     ``dy`` [M, N] bfloat16.  Returns {"dx": [M, K] or None, "dw": [N, K] or None}."""
+    done = _lib.binding().linear_bwd(dy, fwd, bits, had_block, K, out_dtype, dx, dw, want_dx, want_dw, workspace)
+    if done is not None:
+        return _result(done)
     _require_cuda(dy, dx, dw, workspace, *[fwd[k] for k in ("xq", "sx", "mx", "wq", "sw", "mw")])
     if dy.dtype != torch.bfloat16 or not dy.is_contiguous():
         raise ValueError("quest_linear_bwd: dy must be a contiguous bfloat16 tensor")
@@ -308,6 +330,9 @@ def quest_mlp_fwd(x: torch.Tensor, w_gate: torch.Tensor, w_up: torch.Tensor, w_d
                   had_block: int, trust_factor: float = 1.0, buffers: dict = None, out_dtype=torch.bfloat16) -> dict:
     """y = down(silu(gate(x)) * up(x)) with QuEST linear layers.  Returns the ``buffers`` dict: "y" [T, H],
     "h" [T, I] bfloat16 and the codes / scales / masks of x, w_gate, w_up, h, w_down."""
+    done = _lib.binding().mlp_fwd(x, w_gate, w_up, w_down, bits, had_block, trust_factor, buffers)
+    if done is not None:
+        return _result(done)
     _require_cuda(x, w_gate, w_up, w_down)
     T, H = x.shape
     I = w_gate.shape[0]
@@ -335,6 +360,9 @@ def quest_linear_fwd_weight_only(x: torch.Tensor, w: torch.Tensor, bits_w: int, 
                                  workspace: torch.Tensor = None) -> dict:
     """y = HT(x) (kept in bfloat16) times the quantized w.  Returns {"y", "xh", "wq", "sw", "mw"};
     ``out`` may hold preallocated tensors under those keys."""
+    done = _lib.binding().linear_fwd_weight_only(x, w, bits_w, had_block, trust_factor, out_dtype, out, workspace)
+    if done is not None:
+        return _result(done)
     _require_cuda(x, w, workspace)
     if x.dim() != 2 or w.dim() != 2 or x.stride(1) != 1 or w.stride(1) != 1 or x.shape[1] != w.shape[1]:
         raise ValueError("quest_linear_fwd_weight_only: x [M, K] and w [N, K] with unit inner stride")
@@ -403,6 +431,9 @@ def quest_lowbit_gemm_fp4(xq, sx, wq, sw, K: int, out_dtype=torch.bfloat16, want
 def quest_linear_fwd_fp4(x: torch.Tensor, w: torch.Tensor, had_block: int, trust_factor: float = 1.0,
                          out_dtype=None, w_cached: dict = None, workspace: torch.Tensor = None) -> dict:
     """Algorithm 1 with the FP4 grid: returns {"y", "xq", "sx", "mx", "wq", "sw", "mw"}."""
+    done = _lib.binding().linear_fwd_fp4(x, w, had_block, trust_factor, out_dtype, w_cached, workspace)
+    if done is not None:
+        return _result(done)
     _require_cuda(x, w, workspace)
     M, K = x.shape
     dev = x.device

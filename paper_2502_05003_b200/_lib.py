@@ -98,6 +98,24 @@ def load() -> ctypes.CDLL:
     return L
 
 
+_binding = None
+
+
+def binding():
+    """The CPython binding of the per-layer calls (``csrc/quest_binding.cpp``).  Its functions return the result, an int
+    (the status of a refused call) or None (not the plain case: the caller goes through ctypes)."""
+    global _binding
+    if _binding is None:
+        load()
+        try:
+            from . import _binding as module
+        except ImportError as e:
+            raise ImportError(f"the CPython binding is missing or does not load ({e}): build it with "
+                              "`python -m paper_2502_05003_b200.build`") from e
+        _binding = module
+    return _binding
+
+
 def check(status: int) -> None:
     if status != 0:
         L = load()

@@ -7,14 +7,17 @@ else with defaults.
 from __future__ import annotations
 
 import os
+import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 OBJ_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libquest_b200.so")
+BINDING = os.path.join(HERE, "_binding" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
@@ -53,7 +56,30 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + f".{os.getpid()}.tmp"
         subprocess.check_call([nvcc] + ARCH + ["-shared", "-o", tmp] + objs)
         os.replace(tmp, LIB)
+    build_binding(force)
     return LIB
+
+
+def build_binding(force: bool = False) -> str:
+    """The CPython binding of the per-layer calls: host code over the C ABI, compiled against torch's headers."""
+    src = os.path.join(CSRC, "quest_binding.cpp")
+    if not (force or _newer([src, os.path.join(INCLUDE, "quest.h")], BINDING)):
+        return BINDING
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(shutil.which(os.environ.get("NVCC", "nvcc")))))
+    includes = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+                sysconfig.get_paths()["include"], os.path.join(cuda, "include"), INCLUDE]
+    tmp = BINDING + f".{os.getpid()}.tmp"
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+    for inc in includes:
+        cmd += ["-isystem", inc]
+    cmd += [src, "-o", tmp, "-L", HERE, "-l:libquest_b200.so", "-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu",
+            "-lc10_cuda", "-lc10", "-Wl,-rpath,$ORIGIN"]
+    subprocess.check_call(cmd)
+    os.replace(tmp, BINDING)
+    return BINDING
 
 
 if __name__ == "__main__":
