@@ -37,6 +37,7 @@ struct QuantConsts {
     float A;       // (2^b-1)/(2 alpha*): RMS-normalised value -> level-axis slope
     float B;       // alpha*/((2^b-1) sqrt(g)): RMS of the un-normalised rotation -> scale
     float h;       // trust_factor/2: trust bound in level steps (FP4 grid: trust_factor, in E2M1 value units)
+    float hi;      // the largest binary32 number that is at most top + h
 };
 QuantConsts make_quant_consts(int bits, int had_block, float trust_factor);
 

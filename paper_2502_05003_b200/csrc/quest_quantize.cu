@@ -23,6 +23,7 @@ QuantConsts make_quant_consts_fp4(int had_block, float trust_factor) {
     c.A = 6.0f / alpha;                                   // RMS-normalised value -> E2M1 value axis
     c.B = alpha / (6.0f * sqrtf((float)had_block));
     c.h = trust_factor;                                   // largest half-interval of the grid: 1 value unit
+    c.hi = c.top + c.h;                                   // not used on this grid
     return c;
 }
 
@@ -35,6 +36,9 @@ QuantConsts make_quant_consts(int bits, int had_block, float trust_factor) {
     c.A = (float)L1 / (2.0f * alpha);
     c.B = alpha / ((float)L1 * sqrtf((float)had_block));
     c.h = 0.5f * trust_factor;
+    const double hi = (double)c.top + (double)c.h;
+    c.hi = (float)hi;
+    if ((double)c.hi > hi) c.hi = nextafterf(c.hi, 0.0f);
     return c;
 }
 
@@ -191,6 +195,73 @@ __device__ __forceinline__ uint32_t cvt_e2m1x8(const float (&t)[8]) {
     return out;
 }
 
+// Levels, mask bits and packed code words of 32 consecutive rotated elements (16 float2 pairs), for trust_factor >= 1.
+//
+// The levels: rounding by the 1.5 * 2^23 constant leaves rint(t) as a 16-bit two's-complement number in the low half
+// of the sum (|t| stays below 2^13: |u| <= rms sqrt(cols)), and rint commutes with a clamp to integers, so two elements
+// are clamped by one 16-bit instruction and packed two at a time.  The mask: an element inside the grid is within half
+// a step of its level, so trusted = |t - level| <= h means -h <= t <= top + h; both differences are exact or round
+// without changing sign, and their product is negative exactly where one of them is.  Against a binary32 clamp per
+// element this takes 1.6 integer-pipe instructions per element less (that pipe runs at half rate).
+template <int CB, int GRID>
+__device__ __forceinline__ void project32_trusting(const float2 *v, float inv, const QuantConsts &qc, uint32_t (&w)[CB],
+                                                   uint32_t &mask_word) {
+    if constexpr (GRID == GRID_FP4) {
+        // FP4 grid (Section 4.4): t = u * inv on the E2M1 value axis, hardware rounding to E2M1.  Every element inside the
+        // grid is within one value unit of its point (exactly, the difference being exact); only saturated elements can
+        // fail: |t| - 6 > trust_factor
+        const float hh = qc.h;
+        uint32_t mbits = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            float t[8];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                t[2 * j] = __fmul_rn(v[q * 4 + j].x, inv);
+                t[2 * j + 1] = __fmul_rn(v[q * 4 + j].y, inv);
+            }
+            w[q] = cvt_e2m1x8(t);
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                mbits |= (__fsub_rn(fabsf(t[j]), 6.0f) <= hh ? 1u : 0u) << (q * 8 + j);
+        }
+        mask_word = mbits;
+    } else {
+        const float2 neg1 = make_float2(-1.0f, -1.0f);
+        const float2 inv2 = make_float2(inv, inv), c02 = make_float2(qc.c0, qc.c0);
+        const float2 magic2 = make_float2(QUEST_MAGIC_RNE, QUEST_MAGIC_RNE);
+        const float2 h2 = make_float2(qc.h, qc.h), hi2 = make_float2(qc.hi, qc.hi);
+        const uint32_t top2 = (uint32_t)qc.top * 0x00010001u;
+        uint32_t kb[32];                                        // low halves: rint(t)
+        uint32_t mlo = 0, mhi = 0;                              // elements 0..15, 16..31 (two independent shift chains)
+#pragma unroll
+        for (int i = 7; i >= 0; --i) {
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int p = i + 8 * half;
+                const float2 t = __ffma2_rn(v[p], inv2, c02);
+                const float2 km = __fadd2_rn(t, magic2);
+                const float2 d = __fmul2_rn(__fadd2_rn(t, h2), __ffma2_rn(t, neg1, hi2));     // (t + h)(hi - t)
+                uint32_t &m = half ? mhi : mlo;
+                m = __funnelshift_l(__float_as_uint(d.y), m, 1); // sign bit: 1 = masked
+                m = __funnelshift_l(__float_as_uint(d.x), m, 1);
+                kb[2 * p] = __float_as_uint(km.x);
+                kb[2 * p + 1] = __float_as_uint(km.y);
+            }
+        }
+        mask_word = ~__byte_perm(mlo, mhi, 0x5410);
+        constexpr int PER = 32 / CB, HP = PER / 2;              // codes per word; per half word
+#pragma unroll
+        for (int q = 0; q < CB; ++q) {
+            uint32_t acc = 0;
+#pragma unroll
+            for (int j = HP - 1; j >= 0; --j)
+                acc = (acc << CB) + __vimin_s16x2_relu(__byte_perm(kb[q * PER + j], kb[q * PER + HP + j], 0x5410), top2);
+            w[q] = acc;
+        }
+    }
+}
+
 // Everything after the load: rotation from stride s_start downwards (larger strides already
 // applied by the caller), RMS, projection, trust test, packing and stores for the E elements this
 // thread holds.  GFULL: had_block >= E, so every in-register stage runs.  FAST: the common case
@@ -198,8 +269,10 @@ __device__ __forceinline__ uint32_t cvt_e2m1x8(const float (&t)[8]) {
 // one warp, codes, scales and mask requested (the GEMM operand and the bfloat16 outputs of the
 // weight-only variant are optional; a tensor may also ask for the rotation alone), no row sums,
 // trust_factor >= 1 -- so that no per-row loop and only a few uniform branches remain.
+// OPT: any of codes, scales and mask may be missing (FAST without OPT: all are there).
 // CS, CCOLS: threads per row and row length when the kernel is instantiated for one row length (0 = run-time values).
-template <int CB, int E, bool GFULL, bool FAST, int GRID = GRID_UNIFORM, bool XDONE = false, bool RS = false, int CS = 0, int CCOLS = 0>
+template <int CB, int E, bool GFULL, bool FAST, int GRID = GRID_UNIFORM, bool XDONE = false, bool RS = false, int CS = 0, int CCOLS = 0,
+          bool OPT = !FAST>
 __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const QuantArgs &a, const QuantTensor &tn,
                                                      bool active, long long row, int tr, int r_local, float *xsm,
                                                      int s_start) {
@@ -335,7 +408,7 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
     }
     const float rms = __fsqrt_rn(__fdiv_rn(ss, (float)cols));
     const float inv = (rms > 0.0f) ? __fdiv_rn(a.qc.A, rms) : 0.0f;
-    if (active && (FAST || tn.scales) && tr == 0) tn.scales[row] = __fmul_rn(rms, a.qc.B);
+    if (active && (!OPT || tn.scales) && tr == 0) tn.scales[row] = __fmul_rn(rms, a.qc.B);
 
     // ---- project: level axis, clamp, round to nearest even, trust test -----------------------
     const float2 inv2 = make_float2(inv, inv), c02 = make_float2(a.qc.c0, a.qc.c0);
@@ -346,11 +419,11 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
     if (active) {
 #pragma unroll
         for (int g32 = 0; g32 < E / 32; ++g32) {
-            uint32_t kb[32];                                    // MAGIC_BITS + level
             uint32_t mbits = 0;
             uint32_t w[CB];
-            if constexpr (GRID == GRID_FP4) {
-                // FP4 grid (Section 4.4): t = u * inv on the E2M1 value axis, hardware rounding to E2M1,
+            if constexpr (FAST) {
+                project32_trusting<CB, GRID>(&v[g32 * 16], inv, a.qc, w, mbits);
+            } else if constexpr (GRID == GRID_FP4) {
                 // trusted = |t - value| <= trust_factor (the largest half-interval is one value unit)
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
@@ -360,67 +433,50 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                         t[2 * j] = __fmul_rn(v[g32 * 16 + q * 4 + j].x, inv);
                         t[2 * j + 1] = __fmul_rn(v[g32 * 16 + q * 4 + j].y, inv);
                     }
-                    const uint32_t cw = cvt_e2m1x8(t);
-                    if (FAST || hh >= 1.0f) {
-                        // every element inside the grid is within one value unit of its point (exactly, the
-                        // difference being exact); only saturated elements can fail: |t| - 6 > trust_factor
+                    w[q] = cvt_e2m1x8(t);
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            mbits |= (__fsub_rn(fabsf(t[j]), 6.0f) <= hh ? 1u : 0u) << (q * 8 + j);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const float val = e2m1_value((int)((cw >> (4 * j)) & 15u));
-                            const bool trusted = fabsf(__fsub_rn(t[j], val)) <= hh;
-                            mbits |= (trusted ? 1u : 0u) << (q * 8 + j);
-                        }
+                    for (int j = 0; j < 8; ++j) {
+                        const float val = e2m1_value((int)((w[q] >> (4 * j)) & 15u));
+                        mbits |= (fabsf(__fsub_rn(t[j], val)) <= hh ? 1u : 0u) << (q * 8 + j);
                     }
-                    w[q] = cw;
                 }
             } else {
+                uint32_t kb[32];                                // MAGIC_BITS + level
 #pragma unroll
-            for (int i = 15; i >= 0; --i) {
-                const float2 t = __ffma2_rn(v[g32 * 16 + i], inv2, c02);
-                float2 tc;
-                tc.x = fminf(fmaxf(t.x, 0.0f), top);
-                tc.y = fminf(fmaxf(t.y, 0.0f), top);
-                const float2 km = __fadd2_rn(tc, magic2);
-                float2 d;
-                if constexpr (FAST) {
-                    // trust_factor >= 1: an element inside the grid is within half a step of its level (the
-                    // difference is exact), so only clipped elements can fail, and for those level = tc
-                    d = __ffma2_rn(tc, neg1, t);                                // t - clamp(t)
-                } else {
+                for (int i = 15; i >= 0; --i) {
+                    const float2 t = __ffma2_rn(v[g32 * 16 + i], inv2, c02);
+                    float2 tc;
+                    tc.x = fminf(fmaxf(t.x, 0.0f), top);
+                    tc.y = fminf(fmaxf(t.y, 0.0f), top);
+                    const float2 km = __fadd2_rn(tc, magic2);
                     const float2 kf = __fadd2_rn(km, nmagic2);
-                    d = __ffma2_rn(kf, neg1, t);                                // t - level
+                    const float2 d = __ffma2_rn(kf, neg1, t);                       // t - level
+                    const float dy = __fsub_rn(hh, fabsf(d.y));                    // >= +0  <=>  trusted
+                    const float dx = __fsub_rn(hh, fabsf(d.x));
+                    mbits = __funnelshift_l(__float_as_uint(dy), mbits, 1);         // sign bit: 1 = masked
+                    mbits = __funnelshift_l(__float_as_uint(dx), mbits, 1);
+                    kb[2 * i] = __float_as_uint(km.x);
+                    kb[2 * i + 1] = __float_as_uint(km.y);
                 }
-                const float dy = __fsub_rn(hh, fabsf(d.y));                    // >= +0  <=>  trusted
-                const float dx = __fsub_rn(hh, fabsf(d.x));
-                mbits = __funnelshift_l(__float_as_uint(dy), mbits, 1);         // sign bit: 1 = masked
-                mbits = __funnelshift_l(__float_as_uint(dx), mbits, 1);
-                kb[2 * i] = __float_as_uint(km.x);
-                kb[2 * i + 1] = __float_as_uint(km.y);
-            }
-            mbits = ~mbits;
-            }
-            if (FAST || tn.mask)
-                reinterpret_cast<uint32_t *>(tn.mask + row * (long long)(cols >> 3))[tr * (E / 32) + g32] = mbits;
-
-            // pack 32/CB codes per word: sum_j (MAGIC_BITS + k_j) * 2^(CB*j), minus the constant part
-            constexpr int PER = 32 / CB;
-            uint32_t magic_sum = 0;
+                mbits = ~mbits;
+                // pack 32/CB codes per word: sum_j (MAGIC_BITS + k_j) * 2^(CB*j), minus the constant part
+                constexpr int PK = 32 / CB;
+                uint32_t magic_sum = 0;
 #pragma unroll
-            for (int j = 0; j < PER; ++j) magic_sum += QUEST_MAGIC_BITS << (CB * j);
-            if constexpr (GRID != GRID_FP4) {
+                for (int j = 0; j < PK; ++j) magic_sum += QUEST_MAGIC_BITS << (CB * j);
 #pragma unroll
                 for (int q = 0; q < CB; ++q) {
                     uint32_t acc = 0;
 #pragma unroll
-                    for (int j = PER - 1; j >= 0; --j) acc = (acc << CB) + kb[q * PER + j];
+                    for (int j = PK - 1; j >= 0; --j) acc = (acc << CB) + kb[q * PK + j];
                     w[q] = acc - magic_sum;
                 }
             }
-            if (FAST || tn.codes) {
+            constexpr int PER = 32 / CB;
+            if (!OPT || tn.mask)
+                reinterpret_cast<uint32_t *>(tn.mask + row * (long long)(cols >> 3))[tr * (E / 32) + g32] = mbits;
+
+            if (!OPT || tn.codes) {
                 uint8_t *dst = tn.codes + row * (long long)(cols * CB / 8) + ((long long)tr * (E / 32) + g32) * (4 * CB);
                 if constexpr (CB == 8) {
                     reinterpret_cast<uint4 *>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
@@ -674,7 +730,7 @@ __device__ __forceinline__ void butterfly32_in_registers(float2 (&v)[16]) {
 // compile-time offset.
 template <int CB, bool FAST, int GRID, int G>
 __global__ void __launch_bounds__(256, 3)
-quantize_wide_kernel(const __grid_constant__ QuantArgs a, int exchange_bytes) {
+quantize_wide32_kernel(const __grid_constant__ QuantArgs a, int exchange_bytes) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     pdl_begin(a.for_decode != 0);
     const int cols = a.cols, S = a.S, R = a.R;
@@ -765,14 +821,14 @@ quantize_wide_kernel(const __grid_constant__ QuantArgs a, int exchange_bytes) {
 }
 
 template <int GRID, bool FAST, int G>
-static cudaError_t launch_wide_g(int cb, int grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
+static cudaError_t launch_wide32_g(int cb, int grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                  int exchange_bytes) {
 #define QUEST_LAUNCH(CBV)                                                                                   \
     do {                                                                                                    \
         static DynamicSmemOnce once_;                                                                       \
-        cudaError_t e_ = once_.set(quantize_wide_kernel<CBV, FAST, GRID, G>, 160 * 1024);                   \
+        cudaError_t e_ = once_.set(quantize_wide32_kernel<CBV, FAST, GRID, G>, 160 * 1024);                   \
         if (e_ != cudaSuccess) return e_;                                                                   \
-        return launch_pdl(quantize_wide_kernel<CBV, FAST, GRID, G>, dim3((unsigned)grid), dim3(threads), smem, st, 1, a, \
+        return launch_pdl(quantize_wide32_kernel<CBV, FAST, GRID, G>, dim3((unsigned)grid), dim3(threads), smem, st, 1, a, \
                           exchange_bytes);                                                                  \
     } while (0)
     if (GRID == GRID_FP4) QUEST_LAUNCH(4);
@@ -786,13 +842,132 @@ static cudaError_t launch_wide_g(int cb, int grid, int threads, size_t smem, cud
 }
 
 template <int GRID, bool FAST>
-static cudaError_t launch_wide(int cb, int grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
+static cudaError_t launch_wide32(int cb, int grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                int exchange_bytes) {
     switch (a.had_block) {
-        case 1024: return launch_wide_g<GRID, FAST, 32>(cb, grid, threads, smem, st, a, exchange_bytes);
-        case 2048: return launch_wide_g<GRID, FAST, 64>(cb, grid, threads, smem, st, a, exchange_bytes);
-        default: return launch_wide_g<GRID, FAST, 128>(cb, grid, threads, smem, st, a, exchange_bytes);
+        case 1024: return launch_wide32_g<GRID, FAST, 32>(cb, grid, threads, smem, st, a, exchange_bytes);
+        case 2048: return launch_wide32_g<GRID, FAST, 64>(cb, grid, threads, smem, st, a, exchange_bytes);
+        default: return launch_wide32_g<GRID, FAST, 128>(cb, grid, threads, smem, st, a, exchange_bytes);
     }
+}
+
+// The same idea with 64 elements per thread, for had_block = 256 .. 4096 in rows of whole spans of 2048 elements.  Phase
+// A: a warp takes 2048 elements of the row, lane p the 32 pairs of neighbours at 64 j + 2 p, so the strides 1024 .. 64
+// combine pairs it holds (those of had_block and above are left out) and every load of the warp reads consecutive
+// memory.  (had_block = 4096: two warps take 4096 elements, pairs at 128 j + 2 p, strides 2048 .. 128.)  The result goes
+// through shared memory in row order (16 bytes of padding per 64 elements: no bank conflicts either way).  Phase B:
+// every thread reads its 64 contiguous elements (had_block = 4096: and those of its neighbour, for stride 64); the
+// strides 32 .. 1 and everything after the rotation are the common tail.  Identical results again.
+// What bounds the wide kernels is instruction issue and the latency that 16 to 24 warps leave open: pairs halve the
+// loads and the fixed costs and take 12 instead of 20 bytes of shared-memory traffic per element (20 instructions per
+// element instead of 27).  16384 x 4096, g = 4096, 3 bits: 75 -> 64 us; 16384 x 2048, g = 256: 37.7 -> 30.8 us;
+// 4096 x 2048 binary32, g = 2048: 20.5 -> 11.8 us.
+template <bool BF16, int CB, int GRID, bool RS, bool G4096>
+__global__ void __launch_bounds__(128, 4)
+quantize_wide_kernel(const __grid_constant__ QuantArgs a, int exchange_bytes) {
+    extern __shared__ __align__(16) uint8_t smem_raw[];
+    pdl_begin(a.for_decode != 0);
+    constexpr int STEP = G4096 ? 128 : 64;                     // elements between the pairs of a thread
+    const int cols = a.cols, S = a.S, R = a.R;
+    float *xsm = reinterpret_cast<float *>(smem_raw);
+    const int tid = threadIdx.x;
+    const int r_local = tid / S;
+    const int tr = tid - r_local * S;
+    float *trow = reinterpret_cast<float *>(smem_raw + exchange_bytes) + (size_t)r_local * (cols + (cols >> 4));
+    const int which = (int)blockIdx.x >= a.blocks0 ? 1 : 0;
+    const QuantTensor &tn = a.t[which];
+    const long long row = (long long)(which ? (int)blockIdx.x - a.blocks0 : (int)blockIdx.x) * R + r_local;
+    const bool row_ok = row < tn.rows;
+    float2 v[32];
+    {   // phase A
+        const int p = G4096 ? tr & 63 : tr & 31;
+        const int base = G4096 ? (tr >> 6) << 12 : (tr >> 5) << 11;
+        const long long first = row * tn.ld + base + 2 * p;
+        if (row_ok) {                                          // rows are whole spans: no bounds inside
+            const uint32_t *xb = reinterpret_cast<const uint32_t *>(reinterpret_cast<const uint16_t *>(tn.x) + first);
+            const float2 *xf = reinterpret_cast<const float2 *>(reinterpret_cast<const float *>(tn.x) + first);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                if (BF16) {
+                    const uint32_t w = __ldg(xb + j * (STEP / 2));
+                    v[j] = make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+                } else {
+                    v[j] = __ldg(xf + j * (STEP / 2));
+                }
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = make_float2(0.0f, 0.0f);
+        }
+        const float2 neg1 = make_float2(-1.0f, -1.0f);
+#pragma unroll
+        for (int s = 16; s >= 1; s >>= 1)
+            if (G4096 || 64 * s < a.had_block) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    if ((j & s) == 0) {
+                        const float2 x = v[j], y = v[j + s];
+                        v[j] = __fadd2_rn(x, y);
+                        v[j + s] = __ffma2_rn(y, neg1, x);
+                    }
+            }
+        float *dst = trow + base + (base >> 4) + 2 * p + (G4096 ? (p >> 5) << 2 : 0);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) *reinterpret_cast<float2 *>(dst + j * (STEP + STEP / 16)) = v[j];
+    }
+    __syncthreads();
+    {   // phase B
+        const float4 *own = reinterpret_cast<const float4 *>(trow + tr * 68);
+        if constexpr (G4096) {
+            const float4 *oth = reinterpret_cast<const float4 *>(trow + (tr ^ 1) * 68);
+            const float sg = (tr & 1) ? -1.0f : 1.0f;
+            const float2 sg2 = make_float2(sg, sg);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const float4 o = own[q], n = oth[q];
+                v[2 * q] = __ffma2_rn(make_float2(o.x, o.y), sg2, make_float2(n.x, n.y));
+                v[2 * q + 1] = __ffma2_rn(make_float2(o.z, o.w), sg2, make_float2(n.z, n.w));
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const float4 o = own[q];
+                v[2 * q] = make_float2(o.x, o.y);
+                v[2 * q + 1] = make_float2(o.z, o.w);
+            }
+        }
+    }
+    rotate_project_store<CB, 64, true, true, GRID, true, RS, 0, 0, true>(v, a, tn, row_ok, row, tr, r_local, xsm, 32);
+}
+
+template <bool BF16, int GRID, bool G4096>
+static cudaError_t launch_wide_g(int cb, int grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
+                                 int exchange_bytes, bool rowsums) {
+#define QUEST_LAUNCH(CBV, RSV)                                                                                              \
+    return launch_pdl(quantize_wide_kernel<BF16, CBV, GRID, RSV, G4096>, dim3((unsigned)grid), dim3(threads), smem, st, 1, a, \
+                      exchange_bytes)
+    if constexpr (GRID == GRID_FP4) {
+        QUEST_LAUNCH(4, false);
+    } else {
+        if (rowsums) QUEST_LAUNCH(8, true);
+        switch (cb) {
+            case 1: QUEST_LAUNCH(1, false);
+            case 2: QUEST_LAUNCH(2, false);
+            case 4: QUEST_LAUNCH(4, false);
+            default: QUEST_LAUNCH(8, false);
+        }
+    }
+#undef QUEST_LAUNCH
+}
+
+template <int GRID>
+static cudaError_t launch_wide(bool bf16, int cb, int grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
+                               int exchange_bytes, bool rowsums) {
+    if (a.had_block == 4096)
+        return bf16 ? launch_wide_g<true, GRID, true>(cb, grid, threads, smem, st, a, exchange_bytes, rowsums)
+                    : launch_wide_g<false, GRID, true>(cb, grid, threads, smem, st, a, exchange_bytes, rowsums);
+    return bf16 ? launch_wide_g<true, GRID, false>(cb, grid, threads, smem, st, a, exchange_bytes, rowsums)
+                : launch_wide_g<false, GRID, false>(cb, grid, threads, smem, st, a, exchange_bytes, rowsums);
 }
 
 // The specialised case (bfloat16 rows, had_block = 128, 32 elements per thread) with direct loads and
@@ -863,71 +1038,7 @@ quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
 // ---------------------------------------------------------------------------------------------
 constexpr int BLK_TILE_BYTES = 8192;             // per warp: 32 blocks x 256 bytes of bfloat16
 constexpr long long BLOCK_KERNEL_MIN_ELEMS = 32ll << 20;
-
-// Levels, mask bits and packed code words of 32 consecutive rotated elements (16 float2 pairs), for
-// trust_factor >= 1: an element inside the grid is within half a step of its level, so only clipped
-// elements can be masked, and for those the level is the clamp bound itself.
-template <int CB, int GRID>
-__device__ __forceinline__ void project32_trusting(const float2 *v, float inv, const QuantConsts &qc, uint32_t (&w)[CB],
-                                                   uint32_t &mask_word) {
-    const float2 neg1 = make_float2(-1.0f, -1.0f);
-    const float hh = qc.h;
-    uint32_t mbits = 0;
-    if constexpr (GRID == GRID_FP4) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            float t[8];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                t[2 * j] = __fmul_rn(v[q * 4 + j].x, inv);
-                t[2 * j + 1] = __fmul_rn(v[q * 4 + j].y, inv);
-            }
-            w[q] = cvt_e2m1x8(t);
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-                mbits |= (__fsub_rn(fabsf(t[j]), 6.0f) <= hh ? 1u : 0u) << (q * 8 + j);
-        }
-        mask_word = mbits;
-    } else {
-        const float2 inv2 = make_float2(inv, inv), c02 = make_float2(qc.c0, qc.c0);
-        const float2 magic2 = make_float2(QUEST_MAGIC_RNE, QUEST_MAGIC_RNE);
-        const float top = qc.top;
-        uint32_t kb[32];                                        // MAGIC_BITS + level
-        uint32_t mhi = 0;                                       // elements 16..31 (two independent shift chains)
-#pragma unroll
-        for (int i = 7; i >= 0; --i) {
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {
-                const int p = i + 8 * half;
-                const float2 t = __ffma2_rn(v[p], inv2, c02);
-                float2 tc;
-                tc.x = fminf(fmaxf(t.x, 0.0f), top);
-                tc.y = fminf(fmaxf(t.y, 0.0f), top);
-                const float2 km = __fadd2_rn(tc, magic2);
-                const float2 d = __ffma2_rn(tc, neg1, t);       // t - clamp(t)
-                const float dy = __fsub_rn(hh, fabsf(d.y));     // >= +0  <=>  trusted
-                const float dx = __fsub_rn(hh, fabsf(d.x));
-                uint32_t &m = half ? mhi : mbits;
-                m = __funnelshift_l(__float_as_uint(dy), m, 1); // sign bit: 1 = masked
-                m = __funnelshift_l(__float_as_uint(dx), m, 1);
-                kb[2 * p] = __float_as_uint(km.x);
-                kb[2 * p + 1] = __float_as_uint(km.y);
-            }
-        }
-        mask_word = ~__byte_perm(mbits, mhi, 0x5410);           // low halves: elements 0..15 | 16..31
-        constexpr int PER = 32 / CB;
-        uint32_t magic_sum = 0;
-#pragma unroll
-        for (int j = 0; j < PER; ++j) magic_sum += QUEST_MAGIC_BITS << (CB * j);
-#pragma unroll
-        for (int q = 0; q < CB; ++q) {
-            uint32_t acc = 0;
-#pragma unroll
-            for (int j = PER - 1; j >= 0; --j) acc = (acc << CB) + kb[q * PER + j];
-            w[q] = acc - magic_sum;
-        }
-    }
-}
+constexpr long long WIDE64_MIN_ELEMS = 4ll << 20;
 
 // Swizzled position of 16-byte chunk `j` in row `r` of a tile whose rows hold NC chunks (NC = 4, 8 or
 // 16): both the row-wise accesses of one thread per row and the chunk-wise accesses of consecutive
@@ -1318,13 +1429,23 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
         // 32 elements per thread (64 registers, twice the resident warps) for bfloat16 rows up to 8192 elements;
         // wider rows keep 64 per thread
         const bool e32 = dtype == QUEST_BF16 && had_block >= 64 && cols <= 8192;
-        const int E = (cols % 64 == 0 && !e32) ? 64 : 32;
+        // wide rotation blocks, 64 elements per thread: rows of whole spans, and enough of them that a CTA's latency (longer
+        // than with 32 elements per thread: 3.5 against 2.9 us for 300 rows of 2048) does not show
+        bool wide = had_block >= 256 && had_block <= 4096 && cols % 2048 == 0 && (had_block < 4096 || cols % 4096 == 0) &&
+                    cols <= 8192 && trust_factor >= 1.0f;
+        int64_t wide_elems = 0;
+        for (int j = 0; j < njobs; ++j) {
+            wide_elems += jobs[j].rows * cols;
+            if (jobs[j].rowsum && container_bits(bits) != 8) wide = false;
+        }
+        if (wide_elems < WIDE64_MIN_ELEMS) wide = false;
+        const int E = (wide || (cols % 64 == 0 && !e32)) ? 64 : 32;
         const int T = (int)(cols / E);
         int S;
         if (T < 32) { S = 1; while (S < T) S <<= 1; } else { S = (T + 31) / 32 * 32; }
         // rows per CTA: CTAs of 128 threads wherever a row fits (finer work units, fewer warps behind each
         // CTA-wide barrier) except for the persistent 64-per-thread streaming kernel
-        const bool streaming = E == 64 && dtype == QUEST_BF16 && had_block >= 64;
+        const bool streaming = E == 64 && dtype == QUEST_BF16 && had_block >= 64 && !wide;
         const int R = (!streaming && S <= 128) ? 128 / S : (S >= 256 ? 1 : 256 / S);
         const int threads = R * S;
         const int warps = (threads + 31) / 32;
@@ -1371,17 +1492,23 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             const int total = nb[0] + nb[1];
-            if (e32 && S == T && S <= 256 && (had_block == 1024 || had_block == 2048 || had_block == 4096)) {
-                // wide rotation blocks: layout-change kernel, one CTA per row group
+            if (wide) {
+                const int exchange = (int)((sizeof(float) * (size_t)warps + 15) / 16 * 16);
+                const size_t smem2 = (size_t)exchange + (size_t)R * (cols + cols / 16) * 4;      // at most 35 KB
+                e = grid_kind == GRID_FP4 ? launch_wide<GRID_FP4>(dtype == QUEST_BF16, cb, total, threads, smem2, st, a, exchange, false)
+                                          : launch_wide<GRID_UNIFORM>(dtype == QUEST_BF16, cb, total, threads, smem2, st, a, exchange,
+                                                                      any_rowsum);
+            } else if (e32 && S == T && S <= 256 && (had_block == 1024 || had_block == 2048 || had_block == 4096)) {
+                // wide rotation blocks, 32 elements per thread, one CTA per row group
                 const int exchange = (int)((sizeof(float) * (size_t)warps + 15) / 16 * 16);
                 const size_t smem2 = (size_t)exchange + (size_t)R * (cols + cols / 8) * 4;
                 const int g = total;
                 if (grid_kind == GRID_FP4)
-                    e = fast_tail ? launch_wide<GRID_FP4, true>(cb, g, threads, smem2, st, a, exchange)
-                                  : launch_wide<GRID_FP4, false>(cb, g, threads, smem2, st, a, exchange);
+                    e = fast_tail ? launch_wide32<GRID_FP4, true>(cb, g, threads, smem2, st, a, exchange)
+                                  : launch_wide32<GRID_FP4, false>(cb, g, threads, smem2, st, a, exchange);
                 else
-                    e = fast_tail ? launch_wide<GRID_UNIFORM, true>(cb, g, threads, smem2, st, a, exchange)
-                                  : launch_wide<GRID_UNIFORM, false>(cb, g, threads, smem2, st, a, exchange);
+                    e = fast_tail ? launch_wide32<GRID_UNIFORM, true>(cb, g, threads, smem2, st, a, exchange)
+                                  : launch_wide32<GRID_UNIFORM, false>(cb, g, threads, smem2, st, a, exchange);
             } else if (e32 && had_block == 128 && fast_tail_rs && any_rowsum && cb == 8 && grid_kind == GRID_UNIFORM && threads <= 256) {
                 // 8-bit codes with the row sums the GEMM needs
                 e = launch_direct128<GRID_UNIFORM>(cb, grid, threads, smem, st, a, true);

@@ -103,6 +103,35 @@ def test_trust_factors(bits, trust):
     check(rows_of("gauss", 64, 1024, 5, True), bits, 128, trust)
 
 
+@pytest.mark.parametrize("bits", [1, 2, 3, 4, 6, 8])
+@pytest.mark.parametrize("trust", [1.0, 1.3, 7.1, 1e30])
+def test_trust_bounds_of_the_packed_projection(bits, trust):
+    # rows with few distinct values put many elements exactly on rounding and trust bounds; heavy tails are clipped
+    x = rows_of("student", 40, 2048, bits, True)
+    x[1::4] = synth.f32_to_bf16_bits(np.sign(np.random.default_rng(bits).standard_normal((10, 2048))).astype(np.float32))
+    x[2::4, 1:] = 0                                       # one nonzero element per row: equal magnitudes after rotation
+    x[3::4] = synth.f32_to_bf16_bits(np.float32(2.0 ** -70) * np.ones((10, 2048), np.float32))
+    check(x, bits, 128, trust)
+    check(x, bits, 2048, trust)
+
+
+@pytest.mark.parametrize("bits", [1, 4, 8])
+@pytest.mark.parametrize("bf16", [True, False])
+@pytest.mark.parametrize("g,cols", [(256, 2048), (512, 4096), (1024, 2048), (2048, 6144), (4096, 4096), (4096, 8192)])
+def test_wide_blocks_of_large_tensors(bits, bf16, g, cols):
+    # from 4 Mi elements: 64 elements per thread; the last CTA holds fewer rows than the others
+    check(rows_of("student", (4 << 20) // cols + 3, cols, bits + g, bf16), bits, g, repeat=1)
+
+
+def test_row_sums_of_wide_blocks():
+    # the 8-bit layer takes its row sums from the quantizer, the contraction of packed codes sums them itself
+    import paper_2502_05003_b200 as quest
+    x, w = (to_dev(rows_of("gauss", n, 2048, n, True)) for n in (2051, 264))
+    r = quest.quest_linear_fwd(x, w, 8, 2048, out_dtype=torch.float32)
+    y, _ = quest.quest_lowbit_gemm(r["xq"], r["sx"], 8, r["wq"], r["sw"], 8, 2048, out_dtype=torch.float32)
+    assert torch.equal(r["y"], y)
+
+
 def test_edge_rows():
     import paper_2502_05003_b200 as quest
     cols = 512
