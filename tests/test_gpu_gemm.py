@@ -90,6 +90,13 @@ def test_eight_bit_codes_as_unsigned_operands(M, N, K, bx, bw):
     run_case(M, N, K, bx, bw, torch.float32, seed=M + K + bx)
 
 
+@pytest.mark.parametrize("bx,bw", [(8, 8), (8, 3), (1, 8), (1, 1), (2, 2), (4, 3)])
+def test_short_launches_agree_with_the_form_that_returns_accumulators(bx, bw):
+    # bfloat16 output without accumulators takes the short-launch kernels, narrow tiles and wide ones (97 tiles of 256)
+    run_case(300, 200, 288, bx, bw, torch.bfloat16, seed=bx + bw)
+    run_case(24800, 136, 160, bx, bw, torch.bfloat16, seed=bx * bw, sample_rows=np.arange(0, 24800, 517))
+
+
 def test_extreme_eight_bit_codes():
     import paper_2502_05003_b200 as quest
     K = 16384                                            # 255 * 255 * K: half of what int32 holds
