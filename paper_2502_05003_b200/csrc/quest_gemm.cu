@@ -129,7 +129,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // behind elect.sync the compiler knows that a single thread executes them, behind a test of the lane index it does not:
 // then a k-block costs the issuing threads about 620 cycles whatever the tile, more than the 524 the tensor cores need
 // for a 256 x 256 tile.  With it (and the inlined first try of the waits) the main loop runs at 516 cycles per k-block:
-// 4096 x 2048 x 2048 16.1 -> 14.0 us, 8192 x 5504 x 2048 65.5 -> 55.9 us.
+// 4096 x 2048 x 2048 17.4 -> 15.8 us, 8192 x 5504 x 2048 71.9 -> 65.6 us (with zeros for operands, which draw less power,
+// 16.1 -> 14.0 and 65.5 -> 55.9 us).
 __device__ __forceinline__ bool elect_one() {
     uint32_t is;
     asm volatile(
@@ -1196,7 +1197,7 @@ int num_sms() {
 // 128-column tiles or 256-column tiles for an M x N product with rows of `row_bytes` operand bytes.  Narrow tiles where
 // they need no more rounds of the CTA pairs (half the time per round: 777 x 2048 x 5504 bytes 16.3 -> 10.4 us), and up
 // to 3 rounds for 2 while the rows are short (3072 x 2048 x 2048: 13.6 -> 12.8 us; equal at 5504 bytes a row; two
-// rounds for one loses from 1024 bytes on: 512 x 5504 x 5504 17.0 -> 20.8 us).
+// rounds for one loses from 1024 bytes on: 512 x 5504 x 5504 17.0 -> 20.8 us).  Measured with zeros for operands.
 bool narrow_tiles(int64_t M, int64_t N, int64_t row_bytes) {
     const int64_t pairs = num_sms() / 2, tm = (M + 255) / 256;
     const int64_t r2 = (tm * ((N + 255) / 256) + pairs - 1) / pairs, r1 = (tm * ((N + 127) / 128) + pairs - 1) / pairs;
