@@ -269,7 +269,8 @@ __device__ __forceinline__ void quantize_rows_in_cta(const DecodeArgs &a, int8_t
                     for (int j = 0; j < 8; ++j) {
                         const uint32_t k = (kb[j >> 2] >> (8 * (j & 3))) & 0xFFu;
                         const float t = __fmaf_rn(v[i][j], inv, a.qc.c0);
-                        mbits |= (fabsf(__fsub_rn(t, (float)k)) <= a.qc.h ? 1u : 0u) << j;
+                        // not "<=": a position that is not a number counts as trusted, as in the sign tests of quest_quantize.cu
+                        mbits |= (fabsf(__fsub_rn(t, (float)k)) > a.qc.h ? 0u : 1u) << j;
                         packed |= (uint64_t)k << (j * cb);
                     }
                     uint8_t *dst = a.codes + ((long long)row * a.K + e0) / 8 * cb;

@@ -64,6 +64,26 @@ def test_types_and_trust_factors(dtype, out, trust):
         check(M, 200, 1024, 8, 64, dtype, out, trust)
 
 
+def same_values(a, b):
+    if not a.is_floating_point():
+        return torch.equal(a, b)
+    return torch.equal(a.isnan(), b.isnan()) and torch.equal(a[~a.isnan()], b[~b.isnan()])
+
+
+@pytest.mark.parametrize("bits", [1, 4, 8])
+@pytest.mark.parametrize("M,K,g", [(1, 2048, 128), (2, 1024, 1024), (4, 512, 32), (20, 2048, 128)])
+def test_rows_that_are_not_finite(M, K, g, bits):
+    import paper_2502_05003_b200 as quest
+    x, w = layer(40, 64, K, torch.bfloat16, M)
+    x[0, 5] = float("nan")
+    x[1, 7], x[1, K - 1] = float("inf"), float("-inf")
+    x[3, 100] = float("-inf")
+    full = quest.quest_linear_fwd(x, w, bits, g)
+    got = quest.quest_linear_fwd(x[:M], None, bits, g, w_cached={"wq": full["wq"], "sw": full["sw"]})
+    for key in ("xq", "sx", "mx", "y"):
+        assert same_values(got[key], full[key][:M]), key
+
+
 def test_against_the_oracle():
     import paper_2502_05003_b200 as quest
     for bits in (1, 4, 8):
