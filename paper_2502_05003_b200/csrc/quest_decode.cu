@@ -50,7 +50,8 @@ struct DecodeArgs {
     const float *sx;
     void *y;
     int y_f32;
-    float fold;                           // exact power of two of the operand scaling
+    float fold;                           // exact power of two of the operand scaling, applied to the row scale ...
+    int shift;                            // ... or to the sums: where the contraction of many rows does which
     int pitch;                            // FUSED: bytes per row of the operand of x in shared memory
 };
 
@@ -469,6 +470,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
             }
             s = (int)(4u * (uint32_t)s + 2u * (uint32_t)(FUSED ? s_rsa[n] : __ldg(a.rs_a + n)) + 2u * (uint32_t)rb + (uint32_t)a.K);
         }
+        s >>= a.shift;
         const float sxr = __fmul_rn(FUSED ? s_sx[n] : __ldg(a.sx + n), a.fold);
         const float yv = __fmul_rn(__fmul_rn(sxr, __ldg(a.sw + col)), (float)s);
         if (a.y_f32) reinterpret_cast<float *>(a.y)[(long long)n * a.N + col] = yv;
@@ -537,8 +539,11 @@ int launch_decode(const QuantJob &jx, int dtype, bool fused, const uint8_t *wq, 
     a.a8 = jx.op8; a.rs_a = jx.rowsum; a.sx = jx.scales;
     a.y = y; a.y_f32 = y_dtype == QUEST_F32;
     const bool e4 = e2m1_operands(bits, bits);
-    // operand scalings: 2^(7-b) c on both sides, 16 c for w of one or two bits (bytes_of_e2m1)
-    a.fold = bits == 8 ? 1.0f : 1.0f / (float)(1 << (e4 ? 11 - bits : 14 - 2 * bits));
+    // operand scalings: 2^(7-b) c on both sides, 16 c for w of one or two bits (bytes_of_e2m1).  The contraction of
+    // quest_gemm.cu takes its power of two out of the row scale, and has none at one and two bits (E2M1 operands):
+    // there the sums are shifted, or products of scales below 2^-116 would lose bits that it keeps.
+    a.fold = bits == 8 || e4 ? 1.0f : 1.0f / (float)(1 << (14 - 2 * bits));
+    a.shift = e4 ? 11 - bits : 0;
     a.pitch = (int)((K + 127) / 128 * 128 + 64);               // rows 64 bytes apart modulo 128: two rows of a load share no bank
     int src = e4 ? SRC_OP4 : SRC_OP8;
     if (w_codes) {

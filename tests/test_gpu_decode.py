@@ -84,6 +84,17 @@ def test_rows_that_are_not_finite(M, K, g, bits):
         assert same_values(got[key], full[key][:M]), key
 
 
+@pytest.mark.parametrize("bits", [1, 2, 3, 4, 8])
+@pytest.mark.parametrize("M", [1, 20])
+def test_scales_whose_product_is_close_to_the_smallest_normal_number(M, bits):
+    import paper_2502_05003_b200 as quest
+    x, w = layer(40, 64, 2048, torch.float32, bits)
+    x, w = x * 1e-18, w * 5e-17
+    full = quest.quest_linear_fwd(x, w, bits, 128)
+    got = quest.quest_linear_fwd(x[:M], None, bits, 128, w_cached={"wq": full["wq"], "sw": full["sw"]})
+    assert torch.equal(got["y"], full["y"][:M])
+
+
 def test_against_the_oracle():
     import paper_2502_05003_b200 as quest
     for bits in (1, 4, 8):
