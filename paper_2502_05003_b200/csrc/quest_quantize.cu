@@ -434,10 +434,18 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                         t[2 * j + 1] = __fmul_rn(v[g32 * 16 + q * 4 + j].y, inv);
                     }
                     w[q] = cvt_e2m1x8(t);
+                    if (hh >= 1.0f) {
+                        // only saturated elements can fail, as in project32_trusting: without this branch the launches
+                        // that come here with such a bound take a quarter longer (4096 x 2048, g = 32: 8.8 -> 11.8 us)
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float val = e2m1_value((int)((w[q] >> (4 * j)) & 15u));
-                        mbits |= (fabsf(__fsub_rn(t[j], val)) <= hh ? 1u : 0u) << (q * 8 + j);
+                        for (int j = 0; j < 8; ++j)
+                            mbits |= (__fsub_rn(fabsf(t[j]), 6.0f) <= hh ? 1u : 0u) << (q * 8 + j);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const float val = e2m1_value((int)((w[q] >> (4 * j)) & 15u));
+                            mbits |= (fabsf(__fsub_rn(t[j], val)) <= hh ? 1u : 0u) << (q * 8 + j);
+                        }
                     }
                 }
             } else {

@@ -58,6 +58,12 @@ def test_trust_factors(trust):
     check_quantize(rows("gauss", 64, 1024, 5), 128, trust)
 
 
+@pytest.mark.parametrize("trust", [0.5, 0.99, 1.0, 1.3, 3.0])
+@pytest.mark.parametrize("g,cols,bf16", [(32, 1024, True), (256, 768, True), (128, 512, False), (512, 16384, True)])
+def test_trust_factors_of_the_general_kernels(g, cols, bf16, trust):
+    check_quantize(rows("student", 40, cols, g, bf16), g, trust)
+
+
 def test_edge_rows_and_hardware_rounding_on_exact_ties():
     cols = 512
     x = np.zeros((6, cols), np.float32)
