@@ -64,10 +64,14 @@ Workspace carve_workspace(void *base, int64_t M, int64_t N, int64_t K);
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_begin(bool hold_dependents) {
-    if (!hold_dependents) pdl_launch_dependents();
+// HOLD: the next kernel may begin only once everything before this one has finished.  A template parameter: with the
+// choice read from the arguments the first instruction waits for them, and with it every launch behind
+// (back to back, 1024 x 2048 at g = 32: 4.8 -> 5.4 us; 1 % on the median of the quantizer's launches).
+template <bool HOLD>
+__device__ __forceinline__ void pdl_begin() {
+    if (!HOLD) pdl_launch_dependents();
     pdl_wait();
-    if (hold_dependents) pdl_launch_dependents();
+    if (HOLD) pdl_launch_dependents();
 }
 
 template <typename... KArgs, typename... Args>

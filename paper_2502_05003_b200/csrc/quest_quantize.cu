@@ -176,7 +176,6 @@ struct QuantArgs {
     QuantConsts qc;
     float inv_sqrt_g;      // 1 / sqrt(had_block) in binary32
     int S, R;
-    int for_decode;        // see launch_quantize
 };
 
 // Eight positions on the E2M1 value axis -> eight 4-bit codes in one word (element 0 in the low
@@ -270,9 +269,10 @@ __device__ __forceinline__ void project32_trusting(const float2 *v, float inv, c
 // weight-only variant are optional; a tensor may also ask for the rotation alone), no row sums,
 // trust_factor >= 1 -- so that no per-row loop and only a few uniform branches remain.
 // OPT: any of codes, scales and mask may be missing (FAST without OPT: all are there).
+// DECODE: the launch precedes the decoding kernel (see launch_quantize).
 // CS, CCOLS: threads per row and row length when the kernel is instantiated for one row length (0 = run-time values).
 template <int CB, int E, bool GFULL, bool FAST, int GRID = GRID_UNIFORM, bool XDONE = false, bool RS = false, int CS = 0, int CCOLS = 0,
-          bool OPT = !FAST>
+          bool OPT = !FAST, bool DECODE = false>
 __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const QuantArgs &a, const QuantTensor &tn,
                                                      bool active, long long row, int tr, int r_local, float *xsm,
                                                      int s_start) {
@@ -421,6 +421,7 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
         for (int g32 = 0; g32 < E / 32; ++g32) {
             uint32_t mbits = 0;
             uint32_t w[CB];
+            [[maybe_unused]] uint32_t kb[32];                   // MAGIC_BITS + level
             if constexpr (FAST) {
                 project32_trusting<CB, GRID>(&v[g32 * 16], inv, a.qc, w, mbits);
             } else if constexpr (GRID == GRID_FP4) {
@@ -449,7 +450,6 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                     }
                 }
             } else {
-                uint32_t kb[32];                                // MAGIC_BITS + level
 #pragma unroll
                 for (int i = 15; i >= 0; --i) {
                     const float2 t = __ffma2_rn(v[g32 * 16 + i], inv2, c02);
@@ -467,22 +467,23 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                     kb[2 * i + 1] = __float_as_uint(km.y);
                 }
                 mbits = ~mbits;
+            }
+            if (!OPT || tn.mask)
+                reinterpret_cast<uint32_t *>(tn.mask + row * (long long)(cols >> 3))[tr * (E / 32) + g32] = mbits;
+            constexpr int PER = 32 / CB;
+            if constexpr (!FAST && GRID != GRID_FP4) {
                 // pack 32/CB codes per word: sum_j (MAGIC_BITS + k_j) * 2^(CB*j), minus the constant part
-                constexpr int PK = 32 / CB;
                 uint32_t magic_sum = 0;
 #pragma unroll
-                for (int j = 0; j < PK; ++j) magic_sum += QUEST_MAGIC_BITS << (CB * j);
+                for (int j = 0; j < PER; ++j) magic_sum += QUEST_MAGIC_BITS << (CB * j);
 #pragma unroll
                 for (int q = 0; q < CB; ++q) {
                     uint32_t acc = 0;
 #pragma unroll
-                    for (int j = PK - 1; j >= 0; --j) acc = (acc << CB) + kb[q * PK + j];
+                    for (int j = PER - 1; j >= 0; --j) acc = (acc << CB) + kb[q * PER + j];
                     w[q] = acc - magic_sum;
                 }
             }
-            constexpr int PER = 32 / CB;
-            if (!OPT || tn.mask)
-                reinterpret_cast<uint32_t *>(tn.mask + row * (long long)(cols >> 3))[tr * (E / 32) + g32] = mbits;
 
             if (!OPT || tn.codes) {
                 uint8_t *dst = tn.codes + row * (long long)(cols * CB / 8) + ((long long)tr * (E / 32) + g32) * (4 * CB);
@@ -520,7 +521,7 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
             if constexpr (GRID == GRID_UNIFORM) {              // the FP4 codes are themselves the tensor-core operand
             if constexpr (CB <= 2) {
                 // one- and two-bit grids: E2M1 nibbles for the FP4 tensor-core path, 16 bytes per 32 elements
-                if (tn.op8 && a.for_decode) {                   // uniform over the CTA; the decoding kernel multiplies bytes
+                if (DECODE && tn.op8) {                         // uniform over the CTA; the decoding kernel multiplies bytes
                     uint32_t o[8];
                     operand_from_code_words<CB>(w, a.bits, o);
                     uint4 *dst = reinterpret_cast<uint4 *>(tn.op8 + row * (long long)cols + (long long)tr * E + g32 * 32);
@@ -563,12 +564,12 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
     }
 }
 
-template <bool BF16, int CB, int E, int GRID = GRID_UNIFORM>
+template <bool BF16, int CB, int E, int GRID = GRID_UNIFORM, bool DECODE = false>
 __global__ void __launch_bounds__(E == 64 ? 256 : 512)
 quantize_rows_kernel(const __grid_constant__ QuantArgs a) {
     extern __shared__ float xsm[];                 // [E][blockDim.x] exchange, then [warps] partial sums
     constexpr int H = E / 2;                       // float2 pairs per thread
-    pdl_begin(a.for_decode != 0);
+    pdl_begin<DECODE>();
     const int tid = threadIdx.x;
     const int which = (int)blockIdx.x >= a.blocks0 ? 1 : 0;
     const QuantTensor &tn = a.t[which];
@@ -605,7 +606,7 @@ quantize_rows_kernel(const __grid_constant__ QuantArgs a) {
 #pragma unroll
         for (int i = 0; i < H; ++i) v[i] = make_float2(0.0f, 0.0f);
     }
-    rotate_project_store<CB, E, false, false, GRID>(v, a, tn, active, row, tr, r_local, xsm, a.had_block >> 1);
+    rotate_project_store<CB, E, false, false, GRID, false, false, 0, 0, true, DECODE>(v, a, tn, active, row, tr, r_local, xsm, a.had_block >> 1);
 }
 
 // Streaming variant for bfloat16 rows (E = 64, had_block >= 64): a persistent grid in which every
@@ -616,13 +617,13 @@ quantize_rows_kernel(const __grid_constant__ QuantArgs a) {
 // (source size 0), so reads need no predicate.  The first butterfly stage (stride had_block/2)
 // pairs this thread with thread tid ^ dist0 of the same row; both read both raw slots from shared
 // memory, so that stage needs no shuffles.
-template <int CB, int E, bool FAST, int GRID = GRID_UNIFORM>
+template <int CB, int E, bool FAST, int GRID = GRID_UNIFORM, bool DECODE = false>
 __global__ void __launch_bounds__(256, E == 64 ? 2 : 4)
 quantize_stream_kernel(const __grid_constant__ QuantArgs a, int total_groups, int exchange_bytes) {
     constexpr int H = E / 2;
     constexpr int STREAM_SLOT = 2 * E + 16;
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    pdl_begin(a.for_decode != 0);
+    pdl_begin<DECODE>();
     float *xsm = reinterpret_cast<float *>(smem_raw);
     uint8_t *stage = smem_raw + exchange_bytes;
     const int tid = threadIdx.x;
@@ -700,7 +701,7 @@ quantize_stream_kernel(const __grid_constant__ QuantArgs a, int total_groups, in
 #pragma unroll
             for (int q = 0; q < E / 8; ++q) widen(own[q], &v[q * 4]);
         }
-        rotate_project_store<CB, E, true, FAST, GRID>(v, a, tn, active, row, tr, r_local, xsm, s_start);
+        rotate_project_store<CB, E, true, FAST, GRID, false, false, 0, 0, !FAST, DECODE>(v, a, tn, active, row, tr, r_local, xsm, s_start);
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
@@ -736,11 +737,11 @@ __device__ __forceinline__ void butterfly32_in_registers(float2 (&v)[16]) {
 
 // G (threads per rotation block) is a template parameter so that every index of the two layout changes is a
 // compile-time offset.
-template <int CB, bool FAST, int GRID, int G>
+template <int CB, bool FAST, int GRID, int G, bool DECODE>
 __global__ void __launch_bounds__(256, 3)
 quantize_wide32_kernel(const __grid_constant__ QuantArgs a, int exchange_bytes) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    pdl_begin(a.for_decode != 0);
+    pdl_begin<DECODE>();
     const int cols = a.cols, S = a.S, R = a.R;
     static_assert(G == 32 || G == 64 || G == 128, "rotation blocks of 1024, 2048 or 4096 elements");
     constexpr int gshift = G == 32 ? 5 : G == 64 ? 6 : 7;
@@ -824,38 +825,41 @@ quantize_wide32_kernel(const __grid_constant__ QuantArgs a, int exchange_bytes) 
                 }
             }
         }
-        rotate_project_store<CB, 32, true, FAST, GRID, true>(v, a, tn, active, row, tr, r_local, xsm, 16);
+        rotate_project_store<CB, 32, true, FAST, GRID, true, false, 0, 0, !FAST, DECODE>(v, a, tn, active, row, tr, r_local, xsm, 16);
     }
 }
 
-template <int GRID, bool FAST, int G>
+template <int GRID, bool FAST, int G, bool DECODE>
 static cudaError_t launch_wide32_g(int cb, int grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                  int exchange_bytes) {
 #define QUEST_LAUNCH(CBV)                                                                                   \
     do {                                                                                                    \
         static DynamicSmemOnce once_;                                                                       \
-        cudaError_t e_ = once_.set(quantize_wide32_kernel<CBV, FAST, GRID, G>, 160 * 1024);                   \
+        cudaError_t e_ = once_.set(quantize_wide32_kernel<CBV, FAST, GRID, G, DECODE>, 160 * 1024);                   \
         if (e_ != cudaSuccess) return e_;                                                                   \
-        return launch_pdl(quantize_wide32_kernel<CBV, FAST, GRID, G>, dim3((unsigned)grid), dim3(threads), smem, st, 1, a, \
+        return launch_pdl(quantize_wide32_kernel<CBV, FAST, GRID, G, DECODE>, dim3((unsigned)grid), dim3(threads), smem, st, 1, a, \
                           exchange_bytes);                                                                  \
     } while (0)
-    if (GRID == GRID_FP4) QUEST_LAUNCH(4);
-    switch (cb) {
-        case 1: QUEST_LAUNCH(1);
-        case 2: QUEST_LAUNCH(2);
-        case 4: QUEST_LAUNCH(4);
-        default: QUEST_LAUNCH(8);
+    if constexpr (GRID == GRID_FP4) {
+        QUEST_LAUNCH(4);
+    } else {
+        switch (cb) {
+            case 1: QUEST_LAUNCH(1);
+            case 2: QUEST_LAUNCH(2);
+            case 4: QUEST_LAUNCH(4);
+            default: QUEST_LAUNCH(8);
+        }
     }
 #undef QUEST_LAUNCH
 }
 
-template <int GRID, bool FAST>
+template <int GRID, bool FAST, bool DECODE = false>
 static cudaError_t launch_wide32(int cb, int grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                int exchange_bytes) {
     switch (a.had_block) {
-        case 1024: return launch_wide32_g<GRID, FAST, 32>(cb, grid, threads, smem, st, a, exchange_bytes);
-        case 2048: return launch_wide32_g<GRID, FAST, 64>(cb, grid, threads, smem, st, a, exchange_bytes);
-        default: return launch_wide32_g<GRID, FAST, 128>(cb, grid, threads, smem, st, a, exchange_bytes);
+        case 1024: return launch_wide32_g<GRID, FAST, 32, DECODE>(cb, grid, threads, smem, st, a, exchange_bytes);
+        case 2048: return launch_wide32_g<GRID, FAST, 64, DECODE>(cb, grid, threads, smem, st, a, exchange_bytes);
+        default: return launch_wide32_g<GRID, FAST, 128, DECODE>(cb, grid, threads, smem, st, a, exchange_bytes);
     }
 }
 
@@ -874,7 +878,7 @@ template <bool BF16, int CB, int GRID, bool RS, bool G4096>
 __global__ void __launch_bounds__(128, 4)
 quantize_wide_kernel(const __grid_constant__ QuantArgs a, int exchange_bytes) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
-    pdl_begin(a.for_decode != 0);
+    pdl_begin<false>();
     constexpr int STEP = G4096 ? 128 : 64;                     // elements between the pairs of a thread
     const int cols = a.cols, S = a.S, R = a.R;
     float *xsm = reinterpret_cast<float *>(smem_raw);
@@ -988,13 +992,14 @@ static cudaError_t launch_wide(bool bf16, int cb, int grid, int threads, size_t 
 // HB, OPT: blocks of 64 (stride 64 is left out) and launches that do not ask for every output take instantiations of
 // their own with run-time row length (6144 x 2048, g = 64, every output, against the general kernel: 13.6 -> 11.9 us;
 // a whole layer of 777 x 2048 x 5504 without masks 21.8 -> 21.1 us).
-template <int CB, int GRID = GRID_UNIFORM, bool RS = false, int COLS = 0, int HB = 128, bool OPT = false>
+template <int CB, int GRID = GRID_UNIFORM, bool RS = false, int COLS = 0, int HB = 128, bool OPT = false,
+          bool DECODE = false>
 __global__ void __launch_bounds__(256, 4)
 quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
     constexpr int CS = COLS / 32;
     const int S = CS ? CS : a.S, R = CS ? 128 / CS : a.R, cols = COLS ? COLS : a.cols;
     extern __shared__ float xsm[];                 // [warps] partial sums
-    pdl_begin(a.for_decode != 0);
+    pdl_begin<DECODE>();
     const int tid = threadIdx.x, lane = tid & 31;
     const int which = (int)blockIdx.x >= a.blocks0 ? 1 : 0;
     const QuantTensor &tn = a.t[which];
@@ -1029,7 +1034,7 @@ quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
             v[i] = __ffma2_rn(v[i], sgn, p);
         }
     }
-    rotate_project_store<CB, 32, true, true, GRID, false, RS, CS, COLS, OPT>(v, a, tn, active, row, tr, r_local, xsm, 32);
+    rotate_project_store<CB, 32, true, true, GRID, false, RS, CS, COLS, OPT, DECODE>(v, a, tn, active, row, tr, r_local, xsm, 32);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1081,7 +1086,7 @@ quantize_block128_kernel(const __grid_constant__ QuantArgs a) {
     constexpr bool CT_POW2 = CT != 0 && (CT & (CT - 1)) == 0 && CT <= 32;
     constexpr int CR = CT == 0 ? 0 : CT_POW2 ? 64 / CT : (CT >= 128 ? 1 : 128 / CT);     // the host's choice of rows per CTA
     extern __shared__ __align__(16) uint8_t smem_raw[];   // [warps][8 KB] tiles, then [threads] + [rows] floats
-    pdl_begin(a.for_decode != 0);
+    pdl_begin<false>();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int bid = (int)blockIdx.x;
     const int which = (bid >= a.bend[0] ? 1 : 0) + (bid >= a.bend[1] ? 1 : 0) + (bid >= a.bend[2] ? 1 : 0);
@@ -1281,25 +1286,30 @@ static cudaError_t launch_block128(int cb, dim3 grid, int threads, size_t smem, 
     return launch_block128_ct<GRID, 0>(cb, grid, threads, smem, st, a);
 }
 
-template <int GRID, int COLS, int HB, bool OPT>
+template <int GRID, int COLS, int HB, bool OPT, bool DECODE = false>
 static cudaError_t launch_direct128_cols(int cb, dim3 grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                          bool rowsums) {
     if constexpr (GRID == GRID_FP4) {
-        return launch_pdl(quantize_direct128_kernel<4, GRID, false, COLS, HB, OPT>, grid, dim3(threads), smem, st, 1, a);
+        return launch_pdl(quantize_direct128_kernel<4, GRID, false, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
     } else {
-        if (rowsums) return launch_pdl(quantize_direct128_kernel<8, GRID, true, COLS, HB, OPT>, grid, dim3(threads), smem, st, 1, a);
+        if (rowsums) return launch_pdl(quantize_direct128_kernel<8, GRID, true, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
         switch (cb) {
-            case 1: return launch_pdl(quantize_direct128_kernel<1, GRID, false, COLS, HB, OPT>, grid, dim3(threads), smem, st, 1, a);
-            case 2: return launch_pdl(quantize_direct128_kernel<2, GRID, false, COLS, HB, OPT>, grid, dim3(threads), smem, st, 1, a);
-            case 4: return launch_pdl(quantize_direct128_kernel<4, GRID, false, COLS, HB, OPT>, grid, dim3(threads), smem, st, 1, a);
-            default: return launch_pdl(quantize_direct128_kernel<8, GRID, false, COLS, HB, OPT>, grid, dim3(threads), smem, st, 1, a);
+            case 1: return launch_pdl(quantize_direct128_kernel<1, GRID, false, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
+            case 2: return launch_pdl(quantize_direct128_kernel<2, GRID, false, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
+            case 4: return launch_pdl(quantize_direct128_kernel<4, GRID, false, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
+            default: return launch_pdl(quantize_direct128_kernel<8, GRID, false, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
         }
     }
 }
 
 template <int GRID>
 static cudaError_t launch_direct128(int cb, dim3 grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
-                                    bool rowsums, bool every_output) {
+                                    bool rowsums, bool every_output, bool for_decode) {
+    if constexpr (GRID == GRID_UNIFORM) {
+        if (for_decode)
+            return a.had_block == 64 ? launch_direct128_cols<GRID, 0, 64, true, true>(cb, grid, threads, smem, st, a, rowsums)
+                                     : launch_direct128_cols<GRID, 0, 128, true, true>(cb, grid, threads, smem, st, a, rowsums);
+    }
     if (a.had_block == 64) return launch_direct128_cols<GRID, 0, 64, true>(cb, grid, threads, smem, st, a, rowsums);
     if (!every_output) return launch_direct128_cols<GRID, 0, 128, true>(cb, grid, threads, smem, st, a, rowsums);
     // the instantiations for one row length assume the launch geometry chosen for it: cols / 32 threads per row,
@@ -1312,16 +1322,16 @@ static cudaError_t launch_direct128(int cb, dim3 grid, int threads, size_t smem,
     return launch_direct128_cols<GRID, 0, 128, false>(cb, grid, threads, smem, st, a, rowsums);
 }
 
-template <bool BF16, int E>
+template <bool BF16, int E, bool DECODE = false>
 static cudaError_t launch_rows(int cb, dim3 grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a) {
 #define QUEST_LAUNCH(CBV)                                                                                   \
     do {                                                                                                    \
         if (smem > 48 * 1024) {                                                                             \
             static DynamicSmemOnce once_;                                                                   \
-            cudaError_t e_ = once_.set(quantize_rows_kernel<BF16, CBV, E>, 72 * 1024);                      \
+            cudaError_t e_ = once_.set(quantize_rows_kernel<BF16, CBV, E, GRID_UNIFORM, DECODE>, 72 * 1024);                      \
             if (e_ != cudaSuccess) return e_;                                                               \
         }                                                                                                   \
-        cudaError_t l_ = launch_pdl(quantize_rows_kernel<BF16, CBV, E>, grid, dim3(threads), smem, st, 1, a);  \
+        cudaError_t l_ = launch_pdl(quantize_rows_kernel<BF16, CBV, E, GRID_UNIFORM, DECODE>, grid, dim3(threads), smem, st, 1, a);  \
         if (l_ != cudaSuccess) return l_;                                                                   \
     } while (0)
     switch (cb) {
@@ -1355,15 +1365,15 @@ static cudaError_t launch_stream_fp4(int grid, int threads, size_t smem, cudaStr
                       total_groups, exchange_bytes);
 }
 
-template <int E, bool FAST>
+template <int E, bool FAST, bool DECODE = false>
 static cudaError_t launch_stream(int cb, int grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                  int total_groups, int exchange_bytes) {
 #define QUEST_LAUNCH(CBV)                                                                                   \
     do {                                                                                                    \
         static DynamicSmemOnce once_;                                                                       \
-        cudaError_t e_ = once_.set(quantize_stream_kernel<CBV, E, FAST>, 160 * 1024);                       \
+        cudaError_t e_ = once_.set(quantize_stream_kernel<CBV, E, FAST, GRID_UNIFORM, DECODE>, 160 * 1024);                       \
         if (e_ != cudaSuccess) return e_;                                                                   \
-        return launch_pdl(quantize_stream_kernel<CBV, E, FAST>, dim3((unsigned)grid), dim3(threads), smem, st, 1, a, \
+        return launch_pdl(quantize_stream_kernel<CBV, E, FAST, GRID_UNIFORM, DECODE>, dim3((unsigned)grid), dim3(threads), smem, st, 1, a, \
                           total_groups, exchange_bytes);                                                    \
     } while (0)
     switch (cb) {
@@ -1432,7 +1442,6 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                 a.blocks0 = a.bend[0];
                 a.cols = (int)cols; a.bits = bits; a.had_block = had_block; a.qc = qc; a.S = T; a.R = R;
                 a.inv_sqrt_g = 1.0f / sqrtf((float)had_block);
-            a.for_decode = for_decode ? 1 : 0;
                 const dim3 grid((unsigned)total);
                 const cudaError_t e = grid_kind == GRID_FP4 ? launch_block128<GRID_FP4>(cb, grid, threads, smem, st, a)
                                                             : launch_block128<GRID_UNIFORM>(cb, grid, threads, smem, st, a);
@@ -1489,7 +1498,6 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                 a.t[j] = QuantTensor{nullptr, 0, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
             a.cols = (int)cols; a.bits = bits; a.had_block = had_block; a.qc = qc; a.S = S; a.R = R;
             a.inv_sqrt_g = 1.0f / sqrtf((float)had_block);
-            a.for_decode = for_decode ? 1 : 0;
             const dim3 grid((unsigned)(nb[0] + nb[1]));
             cudaError_t e;
             // the specialised tail (trust_factor >= 1): with codes, scales and masks requested (or the rotation alone), with
@@ -1523,14 +1531,17 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                 if (grid_kind == GRID_FP4)
                     e = fast_tail ? launch_wide32<GRID_FP4, true>(cb, g, threads, smem2, st, a, exchange)
                                   : launch_wide32<GRID_FP4, false>(cb, g, threads, smem2, st, a, exchange);
+                else if (for_decode)
+                    e = fast_tail ? launch_wide32<GRID_UNIFORM, true, true>(cb, g, threads, smem2, st, a, exchange)
+                                  : launch_wide32<GRID_UNIFORM, false, true>(cb, g, threads, smem2, st, a, exchange);
                 else
                     e = fast_tail ? launch_wide32<GRID_UNIFORM, true>(cb, g, threads, smem2, st, a, exchange)
                                   : launch_wide32<GRID_UNIFORM, false>(cb, g, threads, smem2, st, a, exchange);
             } else if (e32 && (had_block == 128 || had_block == 64) && fast_tail_opt && (!any_rowsum || (cb == 8 && grid_kind == GRID_UNIFORM)) &&
                        threads <= 256) {
                 // the common case: direct loads, one CTA per row group
-                e = grid_kind == GRID_FP4 ? launch_direct128<GRID_FP4>(cb, grid, threads, smem, st, a, false, every_output)
-                                          : launch_direct128<GRID_UNIFORM>(cb, grid, threads, smem, st, a, any_rowsum, every_output);
+                e = grid_kind == GRID_FP4 ? launch_direct128<GRID_FP4>(cb, grid, threads, smem, st, a, false, every_output, false)
+                                          : launch_direct128<GRID_UNIFORM>(cb, grid, threads, smem, st, a, any_rowsum, every_output, for_decode);
             } else if (streaming) {
                 // rows wider than 8192: persistent streaming kernel, 64 elements per thread, as many CTAs as fit
                 const int exchange = (int)((smem + 15) / 16 * 16);
@@ -1541,6 +1552,9 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                 if (grid_kind == GRID_FP4)
                     e = fast ? launch_stream_fp4<64, true>(g, threads, smem2, st, a, total, exchange)
                              : launch_stream_fp4<64, false>(g, threads, smem2, st, a, total, exchange);
+                else if (for_decode)
+                    e = fast ? launch_stream<64, true, true>(cb, g, threads, smem2, st, a, total, exchange)
+                             : launch_stream<64, false, true>(cb, g, threads, smem2, st, a, total, exchange);
                 else
                     e = fast ? launch_stream<64, true>(cb, g, threads, smem2, st, a, total, exchange)
                              : launch_stream<64, false>(cb, g, threads, smem2, st, a, total, exchange);
@@ -1551,6 +1565,13 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                 else
                     e = dtype == QUEST_BF16 ? launch_rows_fp4<true, 32>(grid, threads, smem, st, a)
                                             : launch_rows_fp4<false, 32>(grid, threads, smem, st, a);
+            } else if (for_decode) {
+                if (E == 64)
+                    e = dtype == QUEST_BF16 ? launch_rows<true, 64, true>(cb, grid, threads, smem, st, a)
+                                            : launch_rows<false, 64, true>(cb, grid, threads, smem, st, a);
+                else
+                    e = dtype == QUEST_BF16 ? launch_rows<true, 32, true>(cb, grid, threads, smem, st, a)
+                                            : launch_rows<false, 32, true>(cb, grid, threads, smem, st, a);
             } else if (E == 64)
                 e = dtype == QUEST_BF16 ? launch_rows<true, 64>(cb, grid, threads, smem, st, a)
                                         : launch_rows<false, 64>(cb, grid, threads, smem, st, a);
