@@ -1392,8 +1392,11 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
     const QuantConsts qc = grid_kind == GRID_FP4 ? make_quant_consts_fp4(had_block, trust_factor)
                                                  : make_quant_consts(bits, had_block, trust_factor);
     if (grid_kind == GRID_FP4 && cols % 32 != 0) return QUEST_ERR_SHAPE;
+    // the kernels that a launch before the decoding kernel may take hold that kernel back and write its operand; the
+    // generic kernel, the FP4 grid and the kernels of large tensors do neither
+    if (for_decode && (cols % 32 != 0 || grid_kind == GRID_FP4)) return QUEST_ERR_SHAPE;
     const int cb = container_bits(bits);
-    if (dtype == QUEST_BF16 && had_block == 128 && cols % 128 == 0 && trust_factor >= 1.0f) {
+    if (!for_decode && dtype == QUEST_BF16 && had_block == 128 && cols % 128 == 0 && trust_factor >= 1.0f) {
         // one thread per rotation block, when every tensor of the call is stored densely and asks for codes,
         // scales and mask (plus, optionally, the GEMM operand)
         bool ok = true;
@@ -1457,7 +1460,7 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
         // wide rotation blocks, 64 elements per thread: rows of whole spans, and enough of them that a CTA's latency (longer
         // than with 32 elements per thread: 3.5 against 2.9 us for 300 rows of 2048) does not show
         bool wide = had_block >= 256 && had_block <= 4096 && cols % 2048 == 0 && (had_block < 4096 || cols % 4096 == 0) &&
-                    cols <= 8192 && trust_factor >= 1.0f;
+                    cols <= 8192 && trust_factor >= 1.0f && !for_decode;
         int64_t wide_elems = 0;
         for (int j = 0; j < njobs; ++j) {
             wide_elems += jobs[j].rows * cols;
