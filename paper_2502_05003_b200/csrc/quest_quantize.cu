@@ -701,7 +701,7 @@ quantize_stream_kernel(const __grid_constant__ QuantArgs a, int total_groups, in
 #pragma unroll
             for (int q = 0; q < E / 8; ++q) widen(own[q], &v[q * 4]);
         }
-        rotate_project_store<CB, E, true, FAST, GRID, false, false, 0, 0, !FAST, DECODE>(v, a, tn, active, row, tr, r_local, xsm, s_start);
+        rotate_project_store<CB, E, true, FAST, GRID, false, false, 0, 0, DECODE || !FAST, DECODE>(v, a, tn, active, row, tr, r_local, xsm, s_start);
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
@@ -1555,9 +1555,10 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                 if (grid_kind == GRID_FP4)
                     e = fast ? launch_stream_fp4<64, true>(g, threads, smem2, st, a, total, exchange)
                              : launch_stream_fp4<64, false>(g, threads, smem2, st, a, total, exchange);
-                else if (for_decode)
-                    e = fast ? launch_stream<64, true, true>(cb, g, threads, smem2, st, a, total, exchange)
-                             : launch_stream<64, false, true>(cb, g, threads, smem2, st, a, total, exchange);
+                else if (for_decode)                       // any of the outputs: the specialised tail serves them all
+                    e = fast_tail_opt && !any_rowsum && had_block == 128
+                            ? launch_stream<64, true, true>(cb, g, threads, smem2, st, a, total, exchange)
+                            : launch_stream<64, false, true>(cb, g, threads, smem2, st, a, total, exchange);
                 else
                     e = fast ? launch_stream<64, true>(cb, g, threads, smem2, st, a, total, exchange)
                              : launch_stream<64, false>(cb, g, threads, smem2, st, a, total, exchange);
