@@ -54,6 +54,13 @@ int check_device() {
     return cached[dev] == 1 ? QUEST_OK : QUEST_ERR_DEVICE;
 }
 
+int num_sms() {
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
 // Optional per-stage timing: CUDA events recorded on the caller's stream around each stage.
 struct StageTimer {
     bool enabled = false;
@@ -150,7 +157,7 @@ static int linear_fwd_decode(const void *x, int dtype, int64_t M, int64_t N, int
     if (s) return s;
     Workspace ws = carve_workspace(workspace, M, N, K);
     const QuantJob jx = {x, M, K, xq, sx, mx, ws.a8, bits == 8 ? ws.rs_a : nullptr};
-    const bool fused = decode_fuses_quantizer(M, K);
+    const bool fused = decode_fuses_quantizer(M, N, K);
     if (!fused) {
         StageScope scope(QUEST_STAGE_QUANT_X, st);
         if ((s = launch_quantize(&jx, 1, dtype, K, bits, had_block, trust_factor, st, GRID_UNIFORM, true))) return s;
@@ -385,7 +392,7 @@ int quest_linear_fwd(const void *x, const void *w, int dtype, int64_t M, int64_t
     if (!y) return QUEST_ERR_NULL;
     if (y_dtype != QUEST_F32 && y_dtype != QUEST_BF16) return QUEST_ERR_DTYPE;
     if (!aligned(y, y_dtype == QUEST_F32 ? 4 : 2)) return QUEST_ERR_ALIGN;
-    if ((w_is_cached == 1 || w_is_cached == 2) && decode_serves(M, N, K, bits))
+    if ((w_is_cached == 1 || w_is_cached == 2) && decode_serves(M, N, K, bits, w_is_cached == 1))
         return linear_fwd_decode(x, dtype, M, N, K, bits, had_block, trust_factor, y, y_dtype, xq, sx, mx, wq, sw, w_is_cached,
                                  workspace, workspace_bytes, reinterpret_cast<cudaStream_t>(stream));
     int s = quest_linear_fwd_quantize(x, w, dtype, M, N, K, bits, had_block, trust_factor, xq, sx, mx, wq, sw, mw,

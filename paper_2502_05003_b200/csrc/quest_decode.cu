@@ -513,19 +513,41 @@ cudaError_t launch_form(int src, const DecodeArgs &a, bool two, cudaStream_t st)
 
 }  // namespace
 
-// The decoding path serves up to 32 rows.  One- and two-bit w is unpacked from nibbles to bytes here but not by the FP4
-// contraction of quest_gemm.cu, which is ahead once many rows meet a large w (32 x 5504 x 5504 at one bit: 16.7 against
-// 14.9 us; 32 x 5504 x 2048: 9.4 against 9.7; 16 x 5504 x 5504: 13.1 against 14.9).
-bool decode_serves(int64_t M, int64_t N, int64_t K, int bits) {
+// Where the decoding path serves.  Its time grows in steps with N, with the CTAs that share an SM (a CTA takes 16 rows of
+// w, 32 above 16 per SM; from 32 rows per SM on CTAs begin to share one, above 64 there is a second round), with the
+// groups of eight rows of x, and at one and two bits with the unpacking of w to bytes, which the FP4 contraction of
+// quest_gemm.cu need not do.  Against that contraction (device time back to back, us, here / there):
+//    4 bits, operand: 8 x 32768 x 4096 27.1 / 41.0; 32 x 4096 x 4096 10.0 / 10.5, 32 x 11008 x 512 1.09 of it, 32 x 16384 x
+//                     2048 14.3 / 12.5;  codes: 32 x 32768 x 2048 32.2 / 42.7  (8 bits behave as 4)
+//    1 bit, operand:  8 x 8192 x 8192 0.9 of it, 8 x 16384 x 2048 10.7 / 10.7, x 4096 15.9 / 12.9; 16 x 5504 x 8192 1.16;
+//                     32 x 2368 x 4096 1.28, 32 x 5504 x 1024 1.09
+//    2 bits, codes:   8 x 9472 x 4096 13.8 / 16.4, 8 x 11008 x 4096 18.7 / 18.2, 8 x 32768 x 4096 39.5 / 42.5
+// (the contraction of a large w varies by a quarter with what L2 holds: a limit is where it is ahead all the same).
+bool decode_serves(int64_t M, int64_t N, int64_t K, int bits, bool w_codes) {
     if (M < 1 || N < 1 || M > 32) return false;
-    return bits > 2 || M <= 16 || N * K <= (8ll << 20);
+    const int64_t sms = num_sms();
+    if (bits > 2) return w_codes || M <= 16 || N <= 64 * sms || (N <= 96 * sms && K >= 1024);
+    if (bits == 2 && w_codes && M <= 8 && N > 96 * sms) return true;
+    // longest rows at one and two bits; columns: up to 8, below 16, 32, 48, up to 64, 96 rows of w per SM, and more
+    constexpr int ALL = 16384;
+    static constexpr int LIMIT[2][3][7] = {
+        // operand in the workspace: up to 8, 16, 32 rows of x
+        {{ALL, ALL, ALL, ALL, ALL, 3072, 1024}, {ALL, ALL, 8192, 5504, 8192, 1536, 0}, {ALL, 2048, 1024, 0, 0, 0, 0}},
+        // packed codes
+        {{ALL, ALL, ALL, ALL, ALL, 4096, 3072}, {ALL, ALL, 8192, 5504, 8192, 2048, 1024}, {ALL, 3072, 2048, 1024, 1024, 0, 0}}};
+    const int col = N <= 8 * sms ? 0 : N < 16 * sms ? 1 : N < 32 * sms ? 2 : N < 48 * sms ? 3 : N <= 64 * sms ? 4 : N <= 96 * sms ? 5 : 6;
+    return K <= LIMIT[w_codes ? 1 : 0][M <= 8 ? 0 : M <= 16 ? 1 : 2][col];
 }
 
-// Quantizing in every CTA saves a launch and pays while each warp has at most two pieces of x (K = 2048, one launch
-// against two, device time: 4.1 and 4.6 us for one row, 5.0 and 4.7 for two, 7.4 and 4.7 for four; the second launch
-// costs the host 2.7 us).
-bool decode_fuses_quantizer(int64_t M, int64_t K) {
-    return M <= FUSED_ROWS && M * ((K + 255) / 256) <= WARPS * MAX_TASKS;
+// Quantizing in every CTA saves a launch: 2.7 us of host time, and the dependency between the two.  It pays on the
+// device while a warp has one piece of x and the CTAs are resident at once (two launches take 1.0 .. 1.2 times as long
+// back to back up to 32 rows of w per SM, 0.85 .. 1.1 up to 64; with a second round of CTAs, which quantize again, 0.65
+// .. 0.9).  With two pieces per warp two launches are the faster device work (0.85 .. 0.9 of one at 1 x 2048 x 4096 and
+// 2 x 2048 x 2048, 0.83 at 4 x 2048 x 1024), which only a replayed graph would see; a program that issues its calls
+// waits for the host (the same three 0.95 .. 1.05, 1.02 and 1.1), so they are fused up to 32 rows per SM.
+bool decode_fuses_quantizer(int64_t M, int64_t N, int64_t K) {
+    const int64_t pieces = M * ((K + 255) / 256), sms = num_sms();
+    return M <= FUSED_ROWS && (pieces <= WARPS ? N <= 64 * sms : pieces <= WARPS * MAX_TASKS && N < 32 * sms);
 }
 
 int launch_decode(const QuantJob &jx, int dtype, bool fused, const uint8_t *wq, int8_t *b8, int32_t *rs_b, const float *sw,
@@ -550,12 +572,9 @@ int launch_decode(const QuantJob &jx, int dtype, bool fused, const uint8_t *wq, 
         const int cb = container_bits(bits);
         src = cb == 1 ? SRC_CODES1 : cb == 2 ? SRC_CODES2 : cb == 4 ? SRC_CODES4 : SRC_CODES8;
     }
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // 32 rows of w per CTA once 16 would give more CTAs than there are SMs: half the reads (or quantizations) of x
     // (32 x 2048 x 2048: 5.7 us with 16 rows, 6.9 with 32; 32 x 5504 x 5504: 15.1 and 14.7 us)
-    const bool two = N > 16ll * sms;
+    const bool two = N > 16ll * num_sms();
     const cudaError_t e = fused ? launch_form<true>(src, a, two, st) : launch_form<false>(src, a, two, st);
     return e == cudaSuccess ? QUEST_OK : cuda_fail(e);
 }

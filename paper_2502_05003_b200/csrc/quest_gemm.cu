@@ -1187,13 +1187,6 @@ int make_output_map(CUtensorMap *tm, void *base, int64_t rows, int64_t row_bytes
     return QUEST_OK;
 }
 
-int num_sms() {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    return sms;
-}
-
 // 128-column tiles or 256-column tiles for an M x N product with rows of `row_bytes` operand bytes.  Narrow tiles where
 // they need no more rounds of the CTA pairs (half the time per round: 777 x 2048 x 5504 bytes 16.3 -> 10.4 us), and up
 // to 3 rounds for 2 while the rows are short (3072 x 2048 x 2048: 13.6 -> 12.8 us; equal at 5504 bytes a row; two

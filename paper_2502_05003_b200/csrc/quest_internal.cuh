@@ -124,6 +124,7 @@ int cuda_fail(cudaError_t e);             // records the message, returns QUEST_
 int cuda_fail_msg(const char *msg);
 int *device_status_word();                // device address of the timeout word (current device)
 int check_device();                       // QUEST_OK iff current device is sm_10x
+int num_sms();                            // of the current device
 
 // Launchers (each returns a quest_status; arguments already validated).
 // One tensor of a quantizer launch: rows of `x` -> any of codes / scales / mask / int8 GEMM
@@ -150,8 +151,8 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
 // packed codes of w are the source and its operand (and row sums at 8 bits) is written to b8 / rs_b; otherwise b8
 // holds it.  fused: x is quantized in the same launch (only if decode_fuses_quantizer), else by a launch_quantize
 // for_decode directly before.
-bool decode_serves(int64_t M, int64_t N, int64_t K, int bits);
-bool decode_fuses_quantizer(int64_t M, int64_t K);
+bool decode_serves(int64_t M, int64_t N, int64_t K, int bits, bool w_codes);
+bool decode_fuses_quantizer(int64_t M, int64_t N, int64_t K);
 int launch_decode(const QuantJob &jx, int dtype, bool fused, const uint8_t *wq, int8_t *b8, int32_t *rs_b, const float *sw,
                   bool w_codes, int64_t N, int64_t K, int bits, int had_block, float trust_factor, void *y, int y_dtype,
                   cudaStream_t st);

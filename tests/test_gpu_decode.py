@@ -55,6 +55,15 @@ def test_shapes_and_blocks(M, N, K, g):
     check(M, N, K, 4, g, seed=M + N)
 
 
+@pytest.mark.parametrize("M,N,K,bits", [(1, 9472, 256, 4), (1, 9480, 256, 4), (4, 9480, 1024, 2), (2, 4728, 2048, 4),
+                                        (2, 4744, 2048, 1), (1, 2048, 3072, 4), (8, 9480, 3104, 1), (16, 9480, 1568, 2),
+                                        (16, 14216, 64, 1), (17, 1192, 2080, 1), (24, 2376, 1056, 2), (24, 9480, 992, 4),
+                                        (32, 9480, 1024, 8), (32, 14216, 1024, 4)])
+def test_both_sides_of_the_routes(M, N, K, bits):
+    # the last size of a route and the first of the next, on 148 SMs
+    check(M, N, K, bits, 32, seed=M + K)
+
+
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("out", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("trust", [0.0, 0.5, 1.3])
