@@ -1187,14 +1187,21 @@ int make_output_map(CUtensorMap *tm, void *base, int64_t rows, int64_t row_bytes
     return QUEST_OK;
 }
 
-// 128-column tiles or 256-column tiles for an M x N product with rows of `row_bytes` operand bytes.  Narrow tiles where
-// they need no more rounds of the CTA pairs (half the time per round: 777 x 2048 x 5504 bytes 16.3 -> 10.4 us), and up
-// to 3 rounds for 2 while the rows are short (3072 x 2048 x 2048: 13.6 -> 12.8 us; equal at 5504 bytes a row; two
-// rounds for one loses from 1024 bytes on: 512 x 5504 x 5504 17.0 -> 20.8 us).  Measured with zeros for operands.
-bool narrow_tiles(int64_t M, int64_t N, int64_t row_bytes) {
+// 128-column tiles or 256-column tiles for an M x N product with rows of `row_bytes` operand bytes.  Rounds of the CTA
+// pairs, narrow : wide, decide, and for short rows what the epilogue costs.  Time with narrow tiles over time with wide
+// ones, random operands, medians over shapes of each kind:
+//   no more rounds (1:1)    int8 0.78 .. 0.58 (256 .. 8192 bytes a row), bfloat16 0.87 .. 0.76, FP4 0.78 .. 0.62
+//   3:2                     0.91 .. 0.97 int8, 0.84 .. 0.91 8-bit codes, 0.89 .. 0.93 FP4, 0.93 .. 0.98 bfloat16, 0.87 ..
+//                           0.95 gradients with the fused transform; nothing longer than 5504 bytes was measured
+//   2:1, 4:2, 14:7          0.95 .. 1.05 up to 1024 bytes, 1.05 .. 1.25 above
+//   5:3, 7:4, 14:8          int8 0.95 .. 0.99 up to 512 bytes and 1.02 .. 1.06 at 1024, 8-bit codes 0.88 .. 0.94, FP4
+//                           0.92 .. 0.99 and gradients with the fused transform 0.89 .. 0.95 up to 1024 (there the two
+//                           groups of epilogue warps take tiles in turn); other bfloat16 1.0 .. 1.07
+// short_rows: up to which length the last line holds for the kind.
+bool narrow_tiles(int64_t M, int64_t N, int64_t row_bytes, int64_t short_rows) {
     const int64_t pairs = num_sms() / 2, tm = (M + 255) / 256;
     const int64_t r2 = (tm * ((N + 255) / 256) + pairs - 1) / pairs, r1 = (tm * ((N + 127) / 128) + pairs - 1) / pairs;
-    return r1 <= r2 || (row_bytes <= 2048 && 2 * r1 <= 3 * r2);
+    return r1 <= r2 || (row_bytes <= 6144 && 2 * r1 <= 3 * r2) || (row_bytes <= short_rows && r1 < 2 * r2);
 }
 
 template <int BN, int MODE, bool YT, int OPL = 0, bool SWIGLU = false, bool SHORT = false>
@@ -1338,7 +1345,7 @@ int launch_gemm(const int8_t *a8, const int8_t *b8, const int32_t *rs_a, const i
     p.status = device_status_word();
     if (!p.status) return QUEST_ERR_CUDA;
 
-    const bool narrow = narrow_tiles(M, N, p.K);
+    const bool narrow = narrow_tiles(M, N, p.K, x8 || w8 ? 1024 : 512);
     CUtensorMap tmA, tmB;
     int s = make_operand_map(&tmA, a8, M, K, BM);
     if (s) return s;
@@ -1402,7 +1409,7 @@ int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, 
     const int64_t esz = out_dtype == QUEST_F32 ? 4 : 2;
     p.status = device_status_word();
     if (!p.status) return QUEST_ERR_CUDA;
-    const bool narrow = narrow_tiles(I, J, p.K);
+    const bool narrow = narrow_tiles(I, J, p.K, fuse_iht ? 1024 : 0);
     CUtensorMap tmA, tmB, tmY;
     int s;
     // MN-major: the tensor is [Kc rows x I (or J) elements]; a box is 128 bytes of a row x 64 rows
@@ -1444,7 +1451,7 @@ int launch_gemm_e2m1(const uint8_t *xq, const uint8_t *wq, const float *sx, cons
     p.y = y; p.y_dtype = y_dtype; p.ldy = ldy; p.acc = acc; p.mask = nullptr; p.sw2 = nullptr; p.up_row0 = 0;
     p.status = device_status_word();
     if (!p.status) return QUEST_ERR_CUDA;
-    const bool narrow = narrow_tiles(M, N, p.K);
+    const bool narrow = narrow_tiles(M, N, p.K, 1024);
     CUtensorMap tmA, tmB;
     int s = make_operand_map(&tmA, reinterpret_cast<const int8_t *>(xq), M, K / 2, BM);
     if (s) return s;
@@ -1470,7 +1477,7 @@ int launch_gemm_bf16_scaled(const void *a, const void *b, const float *sw, int64
     p.y = y; p.y_dtype = y_dtype; p.ldy = ldy; p.acc = nullptr; p.mask = nullptr; p.sw2 = nullptr; p.up_row0 = 0;
     p.status = device_status_word();
     if (!p.status) return QUEST_ERR_CUDA;
-    const bool narrow = narrow_tiles(M, N, p.K);
+    const bool narrow = narrow_tiles(M, N, p.K, 0);
     CUtensorMap tmA, tmB;
     int s = make_operand_map(&tmA, reinterpret_cast<const int8_t *>(a), M, 2 * K, BM);
     if (s) return s;

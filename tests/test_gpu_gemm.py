@@ -92,9 +92,49 @@ def test_eight_bit_codes_as_unsigned_operands(M, N, K, bx, bw):
 
 @pytest.mark.parametrize("bx,bw", [(8, 8), (8, 3), (1, 8), (1, 1), (2, 2), (4, 3)])
 def test_short_launches_agree_with_the_form_that_returns_accumulators(bx, bw):
-    # bfloat16 output without accumulators takes the short-launch kernels, narrow tiles and wide ones (97 tiles of 256)
+    # bfloat16 output without accumulators takes the short-launch kernels up to two tiles per CTA pair (4 narrow tiles), and
+    # the plain ones above (194 narrow tiles); the wide tiles are below
     run_case(300, 200, 288, bx, bw, torch.bfloat16, seed=bx + bw)
     run_case(24800, 136, 160, bx, bw, torch.bfloat16, seed=bx * bw, sample_rows=np.arange(0, 24800, 517))
+
+
+def tiles_of(M, N, row_bytes, short_rows):
+    """(columns of a tile, tiles, CTA pairs) of a contraction with rows of ``row_bytes`` operand bytes: the rule of quest_gemm.cu."""
+    pairs = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    tm, wide, narrow = -(-M // 256), -(-N // 256), -(-N // 128)
+    r2, r1 = -(-tm * wide // pairs), -(-tm * narrow // pairs)
+    if r1 <= r2 or (row_bytes <= 6144 and 2 * r1 <= 3 * r2) or (row_bytes <= short_rows and r1 < 2 * r2):
+        return 128, tm * narrow, pairs
+    return 256, tm * wide, pairs
+
+
+def row_bytes(K, bx, bw):
+    return K // 2 if max(bx, bw) <= 2 else K
+
+
+SHORT_ROWS = {(8, 8): 1024, (8, 3): 1024, (1, 8): 1024, (2, 2): 1024, (1, 1): 1024, (4, 3): 512}
+
+
+@pytest.mark.parametrize("bx,bw", list(SHORT_ROWS))
+@pytest.mark.parametrize("M,N,K,short", [(4090, 2040, 288, True), (4090, 2039, 96, True), (8200, 2040, 160, False)])
+def test_wide_tiles_in_every_form(M, N, K, bx, bw, short):
+    """256-column tiles with ragged edges: short launches (at most two tiles per pair) and longer ones, through TMA stores and,
+    where the pitch of y is not a multiple of 16 bytes, direct ones; binary32 and bfloat16 output, with accumulators and
+    without.  A row of y per tile row, and the last rows."""
+    width, tiles, pairs = tiles_of(M, N, row_bytes(K, bx, bw), SHORT_ROWS[bx, bw])
+    assert width == 256 and (tiles <= 2 * pairs) == short
+    rows = np.unique(np.r_[np.arange(7, M, 251), M - 3:M])
+    for out in (torch.bfloat16, torch.float32):
+        run_case(M, N, K, bx, bw, out, seed=K + bx, sample_rows=rows)
+
+
+@pytest.mark.parametrize("bits,M,N,K,width", [
+    (4, 3000, 2048, 2048, 128), (4, 1024, 5500, 6144, 128), (4, 1024, 5500, 6176, 256),      # 3 rounds for 2, by length
+    (4, 2048, 5504, 512, 128), (4, 2048, 5504, 544, 256),                                    # 5 rounds for 3
+    (8, 2048, 5504, 1024, 128), (8, 2048, 5504, 1056, 256), (2, 2048, 5504, 2048, 128), (2, 2048, 5504, 2112, 256)])
+def test_both_sides_of_the_tile_width(bits, M, N, K, width):
+    assert tiles_of(M, N, row_bytes(K, bits, bits), SHORT_ROWS.get((bits, bits), 512))[0] == width
+    run_case(M, N, K, bits, bits, torch.bfloat16, seed=K, sample_rows=np.arange(0, M, 97))
 
 
 def test_extreme_eight_bit_codes():
