@@ -28,7 +28,8 @@ __device__ __forceinline__ uint16_t bf16_bits(float v) {
 }
 
 // Packed level indices and per-row scales -> dequantised values bf16(scale[r] * c) [rows x K], dense, up to two
-// tensors per launch (CTAs from blocks0 on work on the second).  A CTA converts `rpb` whole rows, eight consecutive
+// tensors per launch (CTAs from blocks0 on work on the second).  A CTA converts `rpb` whole rows, or (SPLIT)
+// `piece` octets of one row, gridDim.y of them: a few long rows would leave most SMs without a CTA.  Eight consecutive
 // elements (one 16-byte store; K % 32 == 0 keeps them in one row) per thread and step, four steps in flight.  Bound by
 // the writes (2 B/element) once the arithmetic is out of the way: the row of an octet comes from a multiplication
 // (`magic` = ceil(2^32 / octets), exact below 2^20 octets per CTA) instead of a 64-bit division, and 2k - (2^b - 1) from
@@ -40,17 +41,18 @@ struct DequantTensor {
     uint16_t *out;
     long long rows;
 };
-template <int CB>
+template <int CB, bool SPLIT>
 __global__ void __launch_bounds__(256)
-dequant_codes_kernel(DequantTensor t0, DequantTensor t1, int blocks0, int rpb, int octets, uint32_t magic, int bits) {
+dequant_codes_kernel(DequantTensor t0, DequantTensor t1, int blocks0, int rpb, int piece, int octets, uint32_t magic, int bits) {
     pdl_launch_dependents();
     pdl_wait();
     const bool second = (int)blockIdx.x >= blocks0;
     const DequantTensor t = second ? t1 : t0;
     const long long row0 = (long long)(second ? (int)blockIdx.x - blocks0 : (int)blockIdx.x) * rpb;
     const int rows_here = t.rows - row0 < rpb ? (int)(t.rows - row0) : rpb;
-    const int n = rows_here * octets;
-    const long long first = row0 * octets;                   // octet index of the CTA's first row
+    const int begin = SPLIT ? (int)blockIdx.y * piece : 0;
+    const int n = SPLIT ? min(octets - begin, piece) : rows_here * octets;
+    const long long first = row0 * octets + begin;           // the CTA's first octet
     const uint32_t *c32 = reinterpret_cast<const uint32_t *>(t.codes);
     const float off = -(8388608.0f + (float)((1 << bits) - 1));
     const float2 two = make_float2(2.0f, 2.0f), off2 = make_float2(off, off);
@@ -431,14 +433,22 @@ extern "C" int quest_linear_bwd(const void *dy, int64_t M, int64_t N, int64_t K,
         while (per_cta > 256 && (tw.rows + tx.rows) * octets < 1184ll * per_cta) per_cta >>= 1;
         const int rpb = (per_cta + octets - 1) / octets;
         const int blocks0 = (int)((tw.rows + rpb - 1) / rpb);
-        const dim3 grid((unsigned)(blocks0 + (tx.rows + rpb - 1) / rpb));
+        const int blocks = blocks0 + (int)((tx.rows + rpb - 1) / rpb);
+        // rows shared by several CTAs only where there are fewer rows than two per SM (64 x 8192: 0.7 us; 1536 x 5504 would
+        // take 2.9 us longer)
+        const int parts = rpb == 1 && blocks < 2 * num_sms() ? (octets + 255) / 256 : 1;
+        const int piece = (octets + parts - 1) / parts;
+        const dim3 grid((unsigned)blocks, (unsigned)parts);
         const uint32_t magic = (uint32_t)((((uint64_t)1 << 32) + octets - 1) / octets);
+        auto dequant = [&](auto whole, auto split) {
+            return launch_pdl(parts > 1 ? split : whole, grid, dim3(256), 0, st, 1, tw, tx, blocks0, rpb, piece, octets, magic, bits);
+        };
         cudaError_t e;
         switch (container_bits(bits)) {
-            case 1: e = launch_pdl(dequant_codes_kernel<1>, grid, dim3(256), 0, st, 1, tw, tx, blocks0, rpb, octets, magic, bits); break;
-            case 2: e = launch_pdl(dequant_codes_kernel<2>, grid, dim3(256), 0, st, 1, tw, tx, blocks0, rpb, octets, magic, bits); break;
-            case 4: e = launch_pdl(dequant_codes_kernel<4>, grid, dim3(256), 0, st, 1, tw, tx, blocks0, rpb, octets, magic, bits); break;
-            default: e = launch_pdl(dequant_codes_kernel<8>, grid, dim3(256), 0, st, 1, tw, tx, blocks0, rpb, octets, magic, bits); break;
+            case 1: e = dequant(dequant_codes_kernel<1, false>, dequant_codes_kernel<1, true>); break;
+            case 2: e = dequant(dequant_codes_kernel<2, false>, dequant_codes_kernel<2, true>); break;
+            case 4: e = dequant(dequant_codes_kernel<4, false>, dequant_codes_kernel<4, true>); break;
+            default: e = dequant(dequant_codes_kernel<8, false>, dequant_codes_kernel<8, true>); break;
         }
         if (e != cudaSuccess) return cuda_fail(e);
     }

@@ -134,6 +134,13 @@ def test_small_blocks_on_wide_tiles():
              rows_w=np.random.default_rng(6).choice(1040, 24, replace=False))
 
 
+@pytest.mark.parametrize("bits", [1, 2, 4, 8])
+@pytest.mark.parametrize("M,N,K,g", [(16, 8, 16384, 128), (8, 24, 4128, 32), (24, 8, 2112, 64), (8, 600, 2080, 32)])
+def test_few_long_rows(M, N, K, g, bits):
+    # the dequantisation deals pieces of a row to its CTAs: whole pieces, and a last one that is shorter
+    run_case(gauss(M, K, 51), gauss(N, K, 52, 0.02), bits, g, seed=K + bits)
+
+
 def _drop_rows_and_blocks(mx, mw):
     """Extreme bitmaps: a row that trusts nothing, a fully masked rotation block of 128, an isolated
     masked element, and alternating bits."""
