@@ -42,6 +42,27 @@ def _require_cuda(*ts):
             raise ValueError("quest: tensors must live in CUDA device memory")
 
 
+def _dense_operands(name: str, x: torch.Tensor, w: torch.Tensor):
+    """x and w as the library reads them: rows one after the other, one dtype, one row length (w None: cached)."""
+    if w is not None:
+        if w.dim() != 2 or w.shape[1] != x.shape[1]:
+            raise ValueError(f"{name}: x [M, K] and w [N, K]")
+        if w.dtype != x.dtype:
+            raise TypeError(f"{name}: x and w share one dtype")
+        w = w.contiguous()
+    return x.contiguous(), w
+
+
+def _require_room(name: str, **tensors):
+    """Every (tensor, bytes) is stored densely in CUDA memory and holds that many bytes (None: not given)."""
+    for key, (t, nbytes) in tensors.items():
+        if t is None:
+            continue
+        _require_cuda(t)
+        if not t.is_contiguous() or t.numel() * t.element_size() < nbytes:
+            raise ValueError(f"{name}: {key} must be contiguous and hold {nbytes} bytes")
+
+
 def _result(done):
     """What the CPython binding returned for a call it made: the result, or the status of a call the library refused."""
     if done.__class__ is int:
@@ -195,6 +216,8 @@ def quest_linear_fwd(x: torch.Tensor, w: torch.Tensor, bits: int, had_block: int
     from an earlier call skips the weight quantization (then ``w`` may be None).  With
     ``w_cached["operand_in_workspace"]`` true the call also skips unpacking ``wq``: ``workspace``
     must be the tensor an earlier call for the same w used, untouched since (M may differ).
+    ``x`` or ``w`` with other strides than those of a dense tensor is copied first; tensors that the
+    call writes to, and cached ones, must be dense.
     """
     done = _lib.binding().linear_fwd(x, w, bits, had_block, trust_factor, out_dtype, y, saved, w_cached, workspace,
                                       want_masks)
@@ -206,8 +229,10 @@ def quest_linear_fwd(x: torch.Tensor, w: torch.Tensor, bits: int, had_block: int
     if w_cached is not None:
         out["wq"], out["sw"] = w_cached["wq"], w_cached["sw"]
         N = out["wq"].shape[0]
+        x, _ = _dense_operands("quest_linear_fwd", x, None)
     else:
         N = w.shape[0]
+        x, w = _dense_operands("quest_linear_fwd", x, w)
     cb = container_bits(bits) if 1 <= bits <= 8 else 8
     dev = x.device
 
@@ -229,6 +254,10 @@ def quest_linear_fwd(x: torch.Tensor, w: torch.Tensor, bits: int, had_block: int
         y = torch.empty((M, N), dtype=out_dtype or x.dtype, device=dev)
     if workspace is None:
         workspace = alloc_workspace(M, N, K, bits, bits, dev)
+    if 1 <= bits <= 8:
+        _require_room("quest_linear_fwd", y=(y, M * N * y.element_size()), xq=(out["xq"], M * (K * cb // 8)), sx=(out["sx"], 4 * M),
+                      mx=(out["mx"], M * (K // 8)), wq=(out["wq"], N * (K * cb // 8)), sw=(out["sw"], 4 * N),
+                      mw=(out["mw"] if w_cached is None else None, N * (K // 8)))
     st = _lib.load().quest_linear_fwd(
         _p(x), _p(w), _dtype_code(x), M, N, K, bits, had_block, ctypes.c_float(trust_factor),
         _p(y), _dtype_code(y), _p(out["xq"]), _p(out["sx"]), _p(out["mx"]),
@@ -247,6 +276,7 @@ def quest_linear_fwd_quantize(x: torch.Tensor, w: torch.Tensor, bits: int, had_b
     _require_cuda(x, w, workspace)
     M, K = x.shape
     N = w.shape[0]
+    x, w = _dense_operands("quest_linear_fwd_quantize", x, w)
     st = _lib.load().quest_linear_fwd_quantize(
         _p(x), _p(w), _dtype_code(x), M, N, K, bits, had_block, ctypes.c_float(trust_factor),
         _p(saved["xq"]), _p(saved["sx"]), _p(saved.get("mx")), _p(saved["wq"]), _p(saved["sw"]), _p(saved.get("mw")), 0,
@@ -441,8 +471,11 @@ def quest_linear_fwd_fp4(x: torch.Tensor, w: torch.Tensor, had_block: int, trust
     if w_cached is not None:
         out["wq"], out["sw"], out["mw"] = w_cached["wq"], w_cached["sw"], None
         N = out["wq"].shape[0]
+        x, _ = _dense_operands("quest_linear_fwd_fp4", x, None)
+        _require_room("quest_linear_fwd_fp4", wq=(out["wq"], N * (K // 2)), sw=(out["sw"], 4 * N))
     else:
         N = w.shape[0]
+        x, w = _dense_operands("quest_linear_fwd_fp4", x, w)
         out["wq"] = torch.empty((N, K // 2), dtype=torch.uint8, device=dev)
         out["sw"] = torch.empty(N, dtype=torch.float32, device=dev)
         out["mw"] = torch.empty((N, K // 8), dtype=torch.uint8, device=dev)

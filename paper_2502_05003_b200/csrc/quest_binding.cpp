@@ -6,7 +6,8 @@
 //   * its result, when the call was made and accepted;
 //   * an int, the quest_status of a call that the library refused;
 //   * None, when the arguments are not the plain case (an argument of another type, a tensor that is not in CUDA
-//     memory, a tensor subclass, an unsupported dtype, a shape the library has no workspace for): nothing has been
+//     memory, a tensor subclass, an unsupported dtype, strides that the C ABI does not take, a buffer that is too small,
+//     a shape the library has no workspace for): nothing has been
 //     done, and the Python function goes on to raise what it raises for such arguments or to handle them.
 #include <Python.h>
 
@@ -42,6 +43,21 @@ const at::Tensor &matrix(PyObject *o) {
     const at::Tensor &t = plain_tensor(o);
     if (t.dim() != 2) throw NotPlain();
     return t;
+}
+const at::Tensor &dense(PyObject *o) {   // a matrix without gaps: the layer calls take no leading dimension
+    const at::Tensor &t = matrix(o);
+    if (!t.is_contiguous()) throw NotPlain();
+    return t;
+}
+const at::Tensor &dense_like(PyObject *o, const at::Tensor &x) {         // w beside x
+    const at::Tensor &t = dense(o);
+    if (t.scalar_type() != x.scalar_type() || t.size(1) != x.size(1)) throw NotPlain();
+    return t;
+}
+void room(PyObject *o, int64_t bytes) {  // a buffer of at least that size, where one was given
+    if (!o || o == Py_None) return;
+    const at::Tensor &t = plain_tensor(o);
+    if (!t.is_contiguous() || (int64_t)t.nbytes() < bytes) throw NotPlain();
 }
 void *ptr(PyObject *o) {                // a tensor, or None
     if (!o || o == Py_None) return nullptr;
@@ -211,7 +227,7 @@ PyObject *lowbit_gemm(PyObject *const *a) {
 
 // x, w, bits, had_block, trust_factor, out_dtype, y, saved, w_cached, workspace, want_masks
 PyObject *linear_fwd(PyObject *const *a) {
-    const at::Tensor &x = matrix(a[0]);
+    const at::Tensor &x = dense(a[0]);
     const int bits = bits_arg(a[2]);
     const int64_t g = int_arg(a[3]), M = x.size(0), K = x.size(1), cb = container(bits);
     const float trust = float_arg(a[4]);
@@ -227,7 +243,7 @@ PyObject *linear_fwd(PyObject *const *a) {
         if (!PyDict_CheckExact(a[8])) throw NotPlain();
         PyObject *wq = item(a[8], k_wq), *sw = item(a[8], k_sw);
         N = matrix(wq).size(0);
-        plain_tensor(sw, false);
+        plain_tensor(sw);
         out.set(k_wq, wq);
         out.set(k_sw, sw);
         PyObject *held = item(a[8], k_operand_in_workspace);
@@ -235,7 +251,7 @@ PyObject *linear_fwd(PyObject *const *a) {
         if (h < 0) throw python_error();
         cached = h ? 2 : 1;
     } else {
-        N = matrix(a[1]).size(0);
+        N = dense_like(a[1], x).size(0);
     }
     out.need(k_xq, {M, K * cb / 8}, at::kByte);
     out.need(k_sx, {M}, at::kFloat);
@@ -251,6 +267,7 @@ PyObject *linear_fwd(PyObject *const *a) {
     if (a[6] != Py_None) {
         y = plain_tensor(a[6]);
         code_of(y.scalar_type());
+        room(a[6], M * N * y.element_size());
     } else {
         y = fresh({M, N}, ot, x.device());
     }
@@ -261,6 +278,12 @@ PyObject *linear_fwd(PyObject *const *a) {
         if (!n) throw NotPlain();
         ws = fresh({(int64_t)n}, at::kByte, x.device());
     }
+    room(out.get(k_xq), M * (K * cb / 8));
+    room(out.get(k_sx), 4 * M);
+    room(out.get(k_mx), M * (K / 8));
+    room(out.get(k_wq), N * (K * cb / 8));
+    room(out.get(k_sw), 4 * N);
+    if (!cached) room(out.get(k_mw), N * (K / 8));
     uint8_t *xq = (uint8_t *)out.at(k_xq), *mx = (uint8_t *)out.at(k_mx), *wq = (uint8_t *)out.at(k_wq), *mw = (uint8_t *)out.at(k_mw);
     float *sx = (float *)out.at(k_sx), *sw = (float *)out.at(k_sw);
     const int ydt = code_of(y.scalar_type());
@@ -327,7 +350,7 @@ PyObject *linear_bwd(PyObject *const *a) {
 
 // x, w, had_block, trust_factor, out_dtype, w_cached, workspace
 PyObject *linear_fwd_fp4(PyObject *const *a) {
-    const at::Tensor &x = matrix(a[0]);
+    const at::Tensor &x = dense(a[0]);
     const int64_t g = int_arg(a[2]), M = x.size(0), K = x.size(1);
     const float trust = float_arg(a[3]);
     const int xdt = code_of(x.scalar_type());
@@ -341,12 +364,13 @@ PyObject *linear_fwd_fp4(PyObject *const *a) {
         if (!PyDict_CheckExact(a[5])) throw NotPlain();
         PyObject *wq = item(a[5], k_wq), *sw = item(a[5], k_sw);
         N = matrix(wq).size(0);
-        plain_tensor(sw, false);
+        room(wq, N * (K / 2));
+        room(sw, 4 * N);
         out.set(k_wq, wq);
         out.set(k_sw, sw);
         out.set(k_mw, Py_None);
     } else {
-        N = matrix(a[1]).size(0);
+        N = dense_like(a[1], x).size(0);
         out.need(k_wq, {N, K / 2}, at::kByte);
         out.need(k_sw, {N}, at::kFloat);
         out.need(k_mw, {N, K / 8}, at::kByte);

@@ -103,3 +103,53 @@ def test_given_outputs_are_used_and_returned():
         r2 = q.quest_linear_fwd(x, x, 4, 128)
     side.synchronize()
     assert torch.equal(r2["y"], y)
+
+
+def test_strided_inputs_are_read_as_what_they_show(monkeypatch):
+    """The last position of every sequence, a slice of wider rows, an expanded row, transposed storage: the same as copies."""
+    import paper_2502_05003_b200 as q
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    hidden = torch.randn((24, 3, 256), generator=gen, device="cuda").bfloat16()
+    wide = torch.randn((256, 512), generator=gen, device="cuda").bfloat16()
+    full = q.quest_linear_fwd(hidden[:, 0].contiguous(), wide[:48, :256].contiguous(), 4, 128)
+    cached = {"wq": full["wq"], "sw": full["sw"]}
+    xs = [hidden[:, -1], hidden[:, 1, 128:], wide[:24, 128:384], hidden[0, :1].expand(8, 256), wide[:, :256].t()]
+    for x in xs:
+        K = x.shape[1]
+        for w in (wide[:48, :K], wide[:K, :48].t()):
+            assert not x.is_contiguous() and not w.is_contiguous()
+            for call in (lambda a, b: q.quest_linear_fwd(a, b, 4, 128), lambda a, b: q.quest_linear_fwd_fp4(a, b, 128, out_dtype=torch.float32)):
+                fast, slow = both(monkeypatch, lambda: call(x, w))
+                same(fast, slow)
+                same(fast, call(x.contiguous(), w.contiguous()))
+        if K == 256:
+            same(q.quest_linear_fwd(x, None, 4, 128, w_cached=cached), q.quest_linear_fwd(x.contiguous(), None, 4, 128, w_cached=cached))
+    saved = {k: torch.zeros_like(v) for k, v in full.items() if k != "y"}
+    ws = q.alloc_workspace(24, 48, 256, 4, 4)
+    q.quest_linear_fwd_quantize(hidden[:, 0], wide[:48, :256], 4, 128, 1.0, saved, ws)
+    same(saved, {k: full[k] for k in saved})
+
+
+def test_arguments_that_do_not_fit_are_refused(monkeypatch):
+    import paper_2502_05003_b200 as q
+    x, w = torch.randn((16, 256), device="cuda").bfloat16(), torch.randn((48, 256), device="cuda").bfloat16()
+    full = q.quest_linear_fwd(x, w, 4, 128)
+    e = lambda *shape, dt=torch.uint8, dev="cuda": torch.empty(shape, dtype=dt, device=dev)
+    fwd = lambda **kw: lambda: q.quest_linear_fwd(x, w, 4, 128, **kw)
+    refused = [
+        (TypeError, lambda: q.quest_linear_fwd(x, w.float(), 4, 128)), (TypeError, lambda: q.quest_linear_fwd_fp4(x.float(), w, 128)),
+        (ValueError, lambda: q.quest_linear_fwd(x, w[:, :128], 4, 128)), (ValueError, lambda: q.quest_linear_fwd_fp4(x, w[:, :128], 128)),
+        (ValueError, fwd(y=e(48, 16, dt=torch.bfloat16).t())), (ValueError, fwd(y=e(16, 40, dt=torch.bfloat16))),
+        (ValueError, fwd(saved={"xq": e(16, 64)})), (ValueError, fwd(saved={"sx": e(16, dt=torch.float32, dev="cpu")})),
+        (ValueError, fwd(saved={"mx": e(16, 64)[:, ::2]})), (ValueError, fwd(saved={"mw": e(40, 32)})),
+        (ValueError, lambda: q.quest_linear_fwd(x, None, 4, 128, w_cached={"wq": full["wq"][:, :64], "sw": full["sw"]})),
+        (ValueError, lambda: q.quest_linear_fwd(x, None, 4, 128, w_cached={"wq": full["wq"], "sw": full["sw"][:40]})),
+        (ValueError, lambda: q.quest_linear_fwd_fp4(x, None, 128, w_cached={"wq": full["wq"][:, :64], "sw": full["sw"]})),
+    ]
+    for i, (error, call) in enumerate(refused):
+        fast, slow = both(monkeypatch, call)
+        assert fast == slow and isinstance(fast, tuple) and fast[0] is error, (i, fast, slow)
+    # room to spare and other shapes of the same bytes stay welcome
+    y, xq = e(20, 48, dt=torch.bfloat16), e(16 * 128, dt=torch.int8)
+    r = q.quest_linear_fwd(x, w, 4, 128, y=y, saved={"xq": xq})
+    assert torch.equal(r["y"][:16], full["y"]) and torch.equal(xq.view(torch.uint8).view(16, 128), full["xq"])
