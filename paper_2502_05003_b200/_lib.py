@@ -2,7 +2,9 @@
 from __future__ import annotations
 
 import ctypes
+import importlib
 import os
+import warnings
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libquest_b200.so")
@@ -101,18 +103,28 @@ def load() -> ctypes.CDLL:
 _binding = None
 
 
+class _NoBinding:
+    """Leaves every call to ctypes."""
+
+    def __getattr__(self, name):
+        return lambda *args: None
+
+
 def binding():
     """The CPython binding of the per-layer calls (``csrc/quest_binding.cpp``).  Its functions return the result, an int
-    (the status of a refused call) or None (not the plain case: the caller goes through ctypes)."""
+    (the status of a refused call) or None (not the plain case: the caller goes through ctypes).  Where there is none
+    for the installed torch, or it does not load, every call goes through ctypes, which costs host time (15 to 35 us a
+    call) and changes nothing else; that is said once."""
     global _binding
     if _binding is None:
         load()
+        from . import build
         try:
-            from . import _binding as module
+            _binding = importlib.import_module("." + build.binding_name(), __package__)
         except ImportError as e:
-            raise ImportError(f"the CPython binding is missing or does not load ({e}): build it with "
-                              "`python -m paper_2502_05003_b200.build`") from e
-        _binding = module
+            warnings.warn(f"the CPython binding for this torch is missing or does not load ({e}): calls go through ctypes; "
+                          "build it with `python -m paper_2502_05003_b200.build`", RuntimeWarning, stacklevel=3)
+            _binding = _NoBinding()
     return _binding
 
 

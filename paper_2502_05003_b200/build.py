@@ -7,6 +7,7 @@ else with defaults.
 from __future__ import annotations
 
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -17,7 +18,6 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 OBJ_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libquest_b200.so")
-BINDING = os.path.join(HERE, "_binding" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
@@ -60,26 +60,40 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
-def build_binding(force: bool = False) -> str:
-    """The CPython binding of the per-layer calls: host code over the C ABI, compiled against torch's headers."""
-    src = os.path.join(CSRC, "quest_binding.cpp")
-    if not (force or _newer([src, os.path.join(INCLUDE, "quest.h")], BINDING)):
-        return BINDING
+def binding_name() -> str:
+    """Module name of the CPython binding for the installed torch: an object compiled against another one is not found."""
     import torch
+    return "_binding_torch_" + re.sub(r"\W", "_", torch.__version__)
+
+
+def build_binding(force: bool = False):
+    """The CPython binding of the per-layer calls: host code over the C ABI, compiled against torch's headers.  Without a
+    CUDA build of torch there is none (None is returned): the package goes through ctypes."""
+    try:
+        import torch
+    except ImportError:
+        return None
+    if torch.version.cuda is None:
+        return None
+    name = binding_name()
+    target = os.path.join(HERE, name + sysconfig.get_config_var("EXT_SUFFIX"))
+    src = os.path.join(CSRC, "quest_binding.cpp")
+    if not (force or _newer([src, os.path.join(INCLUDE, "quest.h")], target)):
+        return target
     root = os.path.dirname(torch.__file__)
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(shutil.which(os.environ.get("NVCC", "nvcc")))))
     includes = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
                 sysconfig.get_paths()["include"], os.path.join(cuda, "include"), INCLUDE]
-    tmp = BINDING + f".{os.getpid()}.tmp"
+    tmp = target + f".{os.getpid()}.tmp"
     cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}"]
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f"-DQUEST_BINDING={name}"]
     for inc in includes:
         cmd += ["-isystem", inc]
     cmd += [src, "-o", tmp, "-L", HERE, "-l:libquest_b200.so", "-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu",
             "-lc10_cuda", "-lc10", "-Wl,-rpath,$ORIGIN"]
     subprocess.check_call(cmd)
-    os.replace(tmp, BINDING)
-    return BINDING
+    os.replace(tmp, target)
+    return target
 
 
 if __name__ == "__main__":

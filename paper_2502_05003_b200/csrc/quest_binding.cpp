@@ -465,16 +465,21 @@ PyObject *mlp_fwd(PyObject *const *a) {
     return a[7];
 }
 
+// QUEST_BINDING: the module's name (build.py: it carries the version of torch)
+#define QUEST_STRING_(X) #X
+#define QUEST_STRING(X) QUEST_STRING_(X)
+#define QUEST_INIT_(X) PyInit_##X
+#define QUEST_INIT(X) QUEST_INIT_(X)
 #define QUEST_METHOD(NAME, N) {#NAME, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(entry<NAME, N>)), METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {
     QUEST_METHOD(quantize, 8), QUEST_METHOD(lowbit_gemm, 13), QUEST_METHOD(linear_fwd, 11), QUEST_METHOD(linear_bwd, 11),
     QUEST_METHOD(linear_fwd_fp4, 7), QUEST_METHOD(linear_fwd_weight_only, 8), QUEST_METHOD(mlp_fwd, 8),
     {nullptr, nullptr, 0, nullptr}};
-PyModuleDef module_def = {PyModuleDef_HEAD_INIT, "_binding", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+PyModuleDef module_def = {PyModuleDef_HEAD_INIT, QUEST_STRING(QUEST_BINDING), nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
 
-PyMODINIT_FUNC PyInit__binding(void) {
+PyMODINIT_FUNC QUEST_INIT(QUEST_BINDING)(void) {
 #define QUEST_KEY_INTERN(name) if (!(k_##name = PyUnicode_InternFromString(#name))) return nullptr;
     QUEST_KEYS(QUEST_KEY_INTERN)
     return PyModule_Create(&module_def);
