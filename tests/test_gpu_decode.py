@@ -73,6 +73,51 @@ def test_types_and_trust_factors(dtype, out, trust):
         check(M, 200, 1024, 8, 64, dtype, out, trust)
 
 
+@pytest.mark.parametrize("bits", [1, 2])
+@pytest.mark.parametrize("K,g", [(1024, 64), (2048, 128), (2048, 1024), (4096, 4096), (8320, 64), (16384, 128)])
+@pytest.mark.parametrize("trust", [0.5, 1.3])
+def test_byte_operands_of_one_and_two_bits(K, g, trust, bits):
+    # every kernel that quantizes x in a launch of its own writes it as bytes here, and as E2M1 nibbles elsewhere
+    check(12, 136, K, bits, g, trust=trust, seed=K + g)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("bits", [1, 4, 8])
+@pytest.mark.parametrize("K,g", [(2048, 64), (2048, 128), (2048, 256), (2048, 2048), (4096, 4096), (16384, 128)])
+def test_weights_that_change_between_calls(K, g, bits, dtype):
+    """The kernel reads w ahead of its wait for the quantizer: what an earlier launch on the stream wrote, with nothing
+    but the stream between them.  New codes in one buffer before every call; the operand that the call before has left;
+    the operand that a call which quantizes w has left."""
+    import paper_2502_05003_b200 as quest
+    M, N, rounds = 24, 1040, 4
+    gen = torch.Generator(device="cuda").manual_seed(K + bits)
+    x = torch.randn((M, K), generator=gen, device="cuda").to(dtype)
+    ws = [torch.randn((N, K), generator=gen, device="cuda").to(dtype) for _ in range(rounds)]
+    want = []
+    for w in ws:
+        want.append(quest.quest_linear_fwd(x, w, bits, g)["y"])
+        torch.cuda.synchronize()
+    saved = quest.quest_linear_fwd(x, ws[0], bits, g, want_masks=False)
+    saved = {k: torch.zeros_like(v) for k, v in saved.items() if k not in ("y", "mx", "mw")}
+    work = quest.alloc_workspace(M, N, K, bits, bits)
+    got = torch.zeros((3, 2, rounds, M, N), dtype=dtype, device="cuda")
+
+    def layer_of(y, w=None, **cached):
+        quest.quest_linear_fwd(x, w, bits, g, y=y, saved=saved, workspace=work, want_masks=False,
+                               w_cached=None if w is not None else {"wq": saved["wq"], "sw": saved["sw"], **cached})
+    torch.cuda.synchronize()
+    for again in range(2):
+        for i, w in enumerate(ws):
+            quest.quest_quantize(w, bits, g, codes=saved["wq"], scales=saved["sw"], want_mask=False)
+            layer_of(got[0, again, i])
+            layer_of(got[1, again, i], operand_in_workspace=True)
+            layer_of(got[2, again, i], w)
+            layer_of(got[2, again, i], operand_in_workspace=True)
+    torch.cuda.synchronize()
+    for i in range(rounds):
+        assert all(torch.equal(got[k, again, i], want[i]) for k in range(3) for again in range(2)), i
+
+
 def same_values(a, b):
     if not a.is_floating_point():
         return torch.equal(a, b)

@@ -32,7 +32,7 @@ def rows(kind, r, c, seed, bf16=True):
     return synth.f32_to_bf16_bits(a) if bf16 else a
 
 
-@pytest.mark.parametrize("g,cols", [(1, 64), (32, 96), (128, 128), (128, 2048), (128, 5504), (512, 512), (2048, 2048),
+@pytest.mark.parametrize("g,cols", [(1, 64), (32, 96), (64, 640), (64, 2048), (64, 8192), (128, 128), (128, 2048), (128, 5504), (512, 512), (2048, 2048),
                                     (4096, 4096)])
 @pytest.mark.parametrize("bf16", [True, False])
 def test_quantize_shapes(g, cols, bf16):

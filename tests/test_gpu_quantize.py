@@ -59,6 +59,16 @@ def test_bf16_rows(bits, g, cols):
     check(rows_of("student", 67, cols, bits * 100 + g, True), bits, g)
 
 
+@pytest.mark.parametrize("bits", [1, 2, 4, 8])
+@pytest.mark.parametrize("cols,trust", [(576, 1.0), (1024, 1.3), (5504, 1.0), (8192, 1.0), (1024, 0.5)])
+def test_blocks_of_64(bits, cols, trust):
+    # rows within a warp, rows of several warps with idle lanes, the widest row; below trust factor 1 the general kernel
+    x = rows_of("outliers", 45, cols, bits + cols, True)
+    x[3] = 0
+    x[4, 1:] = 0
+    check(x, bits, 64, trust)
+
+
 @pytest.mark.parametrize("bits", [1, 2, 3, 4, 8])
 @pytest.mark.parametrize("dtype_bf16", [False, True])
 @pytest.mark.parametrize("g,cols", [(8, 8), (8, 24), (1, 40), (8, 72), (8, 136), (4, 1000), (8, 4104), (2, 16376)])

@@ -61,6 +61,14 @@ def test_tile_edges_ragged_shapes_and_block_sizes(M, N, K, g):
     run_case(gauss(M, K, 3), gauss(N, K, 4, 0.02), 4, g)
 
 
+@pytest.mark.parametrize("bf16", [True, False])
+@pytest.mark.parametrize("K,g", [(2048, 256), (2048, 2048), (4096, 4096)])
+def test_rotation_alone_of_large_tensors_with_wide_blocks(K, g, bf16):
+    # from 4 Mi elements the kernel with 64 elements per thread serves x, of which only the rotation is wanted, and w
+    M = (4 << 20) // K + 3
+    run_case(gauss(M, K, 15, bf16=bf16), gauss(72, K, 16, 0.02, bf16=bf16), 4, g)
+
+
 def test_binary32_inputs_bfloat16_output_and_strided_rows():
     run_case(gauss(260, 384, 5, bf16=False), gauss(136, 384, 6, 0.02, bf16=False), 2, 128, out_dtype=torch.bfloat16)
     run_case(gauss(140, 256, 7), gauss(264, 256, 8, 0.02, bf16=False), 3, 128, ldx=320)
