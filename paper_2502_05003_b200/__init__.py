@@ -242,8 +242,9 @@ def quest_linear_fwd(x: torch.Tensor, w: torch.Tensor, bits: int, had_block: int
 
     need("xq", (M, K * cb // 8), torch.uint8)
     need("sx", (M,), torch.float32)
-    need("wq", (N, K * cb // 8), torch.uint8)
-    need("sw", (N,), torch.float32)
+    if w_cached is None:
+        need("wq", (N, K * cb // 8), torch.uint8)
+        need("sw", (N,), torch.float32)
     if want_masks:
         need("mx", (M, K // 8), torch.uint8)
         if w_cached is None:

@@ -54,10 +54,11 @@ const at::Tensor &dense_like(PyObject *o, const at::Tensor &x) {         // w be
     if (t.scalar_type() != x.scalar_type() || t.size(1) != x.size(1)) throw NotPlain();
     return t;
 }
-void room(PyObject *o, int64_t bytes) {  // a buffer of at least that size, where one was given
-    if (!o || o == Py_None) return;
+void *room(PyObject *o, int64_t bytes) {  // a buffer of at least that size, or None
+    if (!o || o == Py_None) return nullptr;
     const at::Tensor &t = plain_tensor(o);
     if (!t.is_contiguous() || (int64_t)t.nbytes() < bytes) throw NotPlain();
+    return t.data_ptr();
 }
 void *ptr(PyObject *o) {                // a tensor, or None
     if (!o || o == Py_None) return nullptr;
@@ -124,10 +125,18 @@ struct Named {
         return v == Py_None ? nullptr : v;
     }
     void set(PyObject *key, PyObject *v) { if (PyDict_SetItem(d, key, v) < 0) throw python_error(); }
-    void need(PyObject *key, at::IntArrayRef shape, at::ScalarType t) {
-        if (get(key)) return;
-        Ref v(THPVariable_Wrap(fresh(shape, t, dev)));
+    // the tensor under that name, with room for that shape (`any`: as it is), or a new one; its memory
+    void *need(PyObject *key, at::IntArrayRef shape, at::ScalarType t, bool any = false) {
+        if (PyObject *given = get(key)) {
+            if (any) return ptr(given);
+            int64_t n = (int64_t)c10::elementSize(t);
+            for (const int64_t s : shape) n *= s;
+            return room(given, n);
+        }
+        const at::Tensor made = fresh(shape, t, dev);
+        Ref v(THPVariable_Wrap(made));
         set(key, v.p);
+        return made.data_ptr();
     }
     void *at(PyObject *key) const { return ptr(get(key)); }
 };
@@ -253,14 +262,14 @@ PyObject *linear_fwd(PyObject *const *a) {
     } else {
         N = dense_like(a[1], x).size(0);
     }
-    out.need(k_xq, {M, K * cb / 8}, at::kByte);
-    out.need(k_sx, {M}, at::kFloat);
-    out.need(k_wq, {N, K * cb / 8}, at::kByte);
-    out.need(k_sw, {N}, at::kFloat);
-    if (masks) {
-        out.need(k_mx, {M, K / 8}, at::kByte);
-        if (!cached) out.need(k_mw, {N, K / 8}, at::kByte);
-    }
+    uint8_t *xq = (uint8_t *)out.need(k_xq, {M, K * cb / 8}, at::kByte);
+    float *sx = (float *)out.need(k_sx, {M}, at::kFloat);
+    uint8_t *wq = (uint8_t *)out.need(k_wq, {N, K * cb / 8}, at::kByte);
+    float *sw = (float *)out.need(k_sw, {N}, at::kFloat);
+    // masks: those that are wanted, and any that the caller gives
+    uint8_t *mx = nullptr, *mw = nullptr;
+    if (masks || out.get(k_mx)) mx = (uint8_t *)out.need(k_mx, {M, K / 8}, at::kByte);
+    if (!cached && (masks || out.get(k_mw))) mw = (uint8_t *)out.need(k_mw, {N, K / 8}, at::kByte);
     for (PyObject *key : {k_mx, k_mw})
         if (!item(dict.p, key)) out.set(key, Py_None);
     at::Tensor y, ws;
@@ -278,14 +287,6 @@ PyObject *linear_fwd(PyObject *const *a) {
         if (!n) throw NotPlain();
         ws = fresh({(int64_t)n}, at::kByte, x.device());
     }
-    room(out.get(k_xq), M * (K * cb / 8));
-    room(out.get(k_sx), 4 * M);
-    room(out.get(k_mx), M * (K / 8));
-    room(out.get(k_wq), N * (K * cb / 8));
-    room(out.get(k_sw), 4 * N);
-    if (!cached) room(out.get(k_mw), N * (K / 8));
-    uint8_t *xq = (uint8_t *)out.at(k_xq), *mx = (uint8_t *)out.at(k_mx), *wq = (uint8_t *)out.at(k_wq), *mw = (uint8_t *)out.at(k_mw);
-    float *sx = (float *)out.at(k_sx), *sw = (float *)out.at(k_sw);
     const int ydt = code_of(y.scalar_type());
     void *st = stream();
     const int s = unlocked([&] {
@@ -364,17 +365,16 @@ PyObject *linear_fwd_fp4(PyObject *const *a) {
         if (!PyDict_CheckExact(a[5])) throw NotPlain();
         PyObject *wq = item(a[5], k_wq), *sw = item(a[5], k_sw);
         N = matrix(wq).size(0);
-        room(wq, N * (K / 2));
-        room(sw, 4 * N);
+        plain_tensor(sw);
         out.set(k_wq, wq);
         out.set(k_sw, sw);
         out.set(k_mw, Py_None);
     } else {
         N = dense_like(a[1], x).size(0);
-        out.need(k_wq, {N, K / 2}, at::kByte);
-        out.need(k_sw, {N}, at::kFloat);
-        out.need(k_mw, {N, K / 8}, at::kByte);
     }
+    uint8_t *wq = (uint8_t *)out.need(k_wq, {N, K / 2}, at::kByte);
+    float *sw = (float *)out.need(k_sw, {N}, at::kFloat);
+    uint8_t *mw = cached ? nullptr : (uint8_t *)out.need(k_mw, {N, K / 8}, at::kByte);
     void *wsp = nullptr;
     size_t wsn = 0;
     if (a[6] != Py_None) {
@@ -382,13 +382,11 @@ PyObject *linear_fwd_fp4(PyObject *const *a) {
         wsp = t.data_ptr();
         wsn = (size_t)t.numel();
     }
-    out.need(k_xq, {M, K / 2}, at::kByte);
-    out.need(k_sx, {M}, at::kFloat);
-    out.need(k_mx, {M, K / 8}, at::kByte);
+    uint8_t *xq = (uint8_t *)out.need(k_xq, {M, K / 2}, at::kByte);
+    float *sx = (float *)out.need(k_sx, {M}, at::kFloat);
+    uint8_t *mx = (uint8_t *)out.need(k_mx, {M, K / 8}, at::kByte);
     Ref yv(THPVariable_Wrap(fresh({M, N}, ot, x.device())));
     void *yp = ptr(yv.p), *st = stream();
-    uint8_t *xq = (uint8_t *)out.at(k_xq), *mx = (uint8_t *)out.at(k_mx), *wq = (uint8_t *)out.at(k_wq), *mw = (uint8_t *)out.at(k_mw);
-    float *sx = (float *)out.at(k_sx), *sw = (float *)out.at(k_sw);
     const int s = unlocked([&] {
         return quest_linear_fwd_fp4(x.data_ptr(), wp, xdt, M, N, K, (int)g, trust, yp, code_of(ot), xq, sx, mx, wq, sw, mw,
                                     cached ? 1 : 0, wsp, wsn, st);
@@ -415,11 +413,11 @@ PyObject *linear_fwd_weight_only(PyObject *const *a) {
     at::Tensor ws;
     if (a[7] != Py_None) ws = plain_tensor(a[7]);
     else if (!(n = quest_weight_only_workspace_bytes(M, N, K))) throw NotPlain();
-    out.need(k_y, {M, N}, ot);
-    out.need(k_xh, {M, K}, at::kBFloat16);
-    out.need(k_wq, {N, K * container(bits) / 8}, at::kByte);
-    out.need(k_sw, {N}, at::kFloat);
-    out.need(k_mw, {N, K / 8}, at::kByte);
+    out.need(k_y, {M, N}, ot, true);
+    out.need(k_xh, {M, K}, at::kBFloat16, true);
+    out.need(k_wq, {N, K * container(bits) / 8}, at::kByte, true);
+    out.need(k_sw, {N}, at::kFloat, true);
+    out.need(k_mw, {N, K / 8}, at::kByte, true);
     if (n) ws = fresh({(int64_t)n}, at::kByte, x.device());
     const at::Tensor &y = matrix(out.get(k_y));
     const int ydt = code_of(y.scalar_type());

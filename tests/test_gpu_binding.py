@@ -149,6 +149,14 @@ def test_arguments_that_do_not_fit_are_refused(monkeypatch):
     for i, (error, call) in enumerate(refused):
         fast, slow = both(monkeypatch, call)
         assert fast == slow and isinstance(fast, tuple) and fast[0] is error, (i, fast, slow)
+    for w_cached in ({"wq": full["wq"]}, {"wq": full["wq"], "sw": None}):
+        for call in (lambda: q.quest_linear_fwd(x, None, 4, 128, w_cached=w_cached), lambda: q.quest_linear_fwd_fp4(x, None, 128, w_cached=w_cached)):
+            fast, slow = both(monkeypatch, call)
+            assert fast == slow and isinstance(fast, tuple), (fast, slow)
+    # a pitched y stays welcome where the call takes one
+    wide = e(16, 64, dt=torch.bfloat16)
+    r, plain = (q.quest_linear_fwd_weight_only(x, w, 4, 128, out=o) for o in ({"y": wide[:, :48]}, None))
+    assert torch.equal(wide[:, :48], plain["y"]) and r["y"].data_ptr() == wide.data_ptr()
     # room to spare and other shapes of the same bytes stay welcome
     y, xq = e(20, 48, dt=torch.bfloat16), e(16 * 128, dt=torch.int8)
     r = q.quest_linear_fwd(x, w, 4, 128, y=y, saved={"xq": xq})
