@@ -1,7 +1,8 @@
 // The inference layer with cached weights for a handful of rows of x (decoding): y = (xq cw^T) sx sw for M <= 32.
 //
-// The tensor-core kernel of quest_gemm.cu gives such a layer 128 x 256 tiles: eight CTAs for 2048 columns, each
-// streaming half a megabyte of weights alone (12.7 us, quantizer apart).  What bounds the work is reading w once
+// The tensor-core kernel of quest_gemm.cu gives such a layer 256 x 128 tiles of CTA pairs, of which 8 to 32 rows are wanted:
+// 16 pairs for 2048 columns (8.2 us with the quantizer; 11.7 with the single-CTA 128 x 256 tiles it had when this was
+// written).  What bounds the work is reading w once
 // (4 MB at 2048 x 2048: under a microsecond from HBM) and latency, so here a CTA takes 16 or 32 rows of w, its eight
 // warps split K, and every warp multiplies with mma.sync m16n8k32 (w is the 16-row operand, the rows of x are the 8
 // columns): integer sums are exact in any order, so the K positions a lane holds are simply 16 consecutive bytes of
@@ -19,8 +20,8 @@
 // w comes either as the operand that an earlier call left in the workspace, or as packed codes, which are unpacked
 // on the way to the tensor cores and also written to the workspace as the operand that later calls may reuse.
 //
-// Compiled with -fmad=false; the rotation, the row's RMS and the projection follow the operation order stated in
-// quest_quantize.cu bit for bit.
+// Compiled with -fmad=false; the rotation, the row's RMS, the projection and the trust test follow the operation order
+// stated in quest_quantize.cu bit for bit (rows with NaN or infinities included).
 #include <cuda_bf16.h>
 
 #include "quest_internal.cuh"

@@ -1393,8 +1393,7 @@ int launch_gemm_swiglu(const int8_t *a8, const int8_t *b8, const int32_t *rs_a, 
 
 // Backward-pass contraction (the two products of Algorithm 2): out[i][j] = mask[i][j] * sum_k A(i, k) B(j, k) with
 // bfloat16 operands and binary32 output [I x J].  `opl` says how the operands lie in memory:
-//   0: a [I x Kc], b [J x Kc], the contraction index contiguous (K-major);
-//   1: a [I x Kc] K-major, b [Kc x J] (memory rows run along the contraction: MN-major);
+//   1: a [I x Kc] with the contraction index contiguous (K-major), b [Kc x J] (memory rows run along it: MN-major);
 //   2: a [Kc x I] and b [Kc x J], both MN-major.
 // With fuse_iht = g in 1 .. 128 (J % 128 == 0) the epilogue also applies the inverse Hadamard
 // transform on blocks of g columns and stores out_dtype; with 0 out is the masked product in binary32.
@@ -1416,16 +1415,14 @@ int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, 
     if (opl == 2) s = make_operand_map(&tmA, reinterpret_cast<const int8_t *>(a), Kc, 2 * I, 64);
     else s = make_operand_map(&tmA, reinterpret_cast<const int8_t *>(a), I, 2 * Kc, BM);
     if (s) return s;
-    if (opl >= 1) s = make_operand_map(&tmB, reinterpret_cast<const int8_t *>(b), Kc, 2 * J, 64);
-    else s = make_operand_map(&tmB, reinterpret_cast<const int8_t *>(b), J, 2 * Kc, narrow ? 64 : 128);
-    if (s) return s;
+    if ((s = make_operand_map(&tmB, reinterpret_cast<const int8_t *>(b), Kc, 2 * J, 64))) return s;
     s = make_output_map(&tmY, out, I, J * esz, J * esz);
     if (s) return s;
-#define QUEST_GEMM_BWD2(BNV, MODEV)                                                  \
-    (opl == 2 ? launch_gemm_bn<BNV, MODEV, true, 2>(tmA, tmB, tmY, p, st)           \
-              : opl == 1 ? launch_gemm_bn<BNV, MODEV, true, 1>(tmA, tmB, tmY, p, st) \
-                         : launch_gemm_bn<BNV, MODEV, true, 0>(tmA, tmB, tmY, p, st))
-#define QUEST_GEMM_BWD(MODEV) (narrow ? QUEST_GEMM_BWD2(128, MODEV) : QUEST_GEMM_BWD2(256, MODEV))
+#define QUEST_GEMM_BWD(MODEV)                                                                                             \
+    (narrow ? (opl == 2 ? launch_gemm_bn<128, MODEV, true, 2>(tmA, tmB, tmY, p, st)                                       \
+                        : launch_gemm_bn<128, MODEV, true, 1>(tmA, tmB, tmY, p, st))                                      \
+            : (opl == 2 ? launch_gemm_bn<256, MODEV, true, 2>(tmA, tmB, tmY, p, st)                                       \
+                        : launch_gemm_bn<256, MODEV, true, 1>(tmA, tmB, tmY, p, st)))
     if (fuse_iht) {
         if (J % 128 != 0 || fuse_iht > 128) return QUEST_ERR_SHAPE;
         p.iht_g = fuse_iht;
@@ -1436,7 +1433,6 @@ int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, 
     if (out_dtype != QUEST_F32) return QUEST_ERR_DTYPE;
     return QUEST_GEMM_BWD(2);
 #undef QUEST_GEMM_BWD
-#undef QUEST_GEMM_BWD2
 }
 
 // Contraction of E2M1 nibble operands xq [M x K/2], wq [N x K/2] on the FP4 tensor-core path:

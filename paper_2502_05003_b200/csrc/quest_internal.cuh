@@ -180,7 +180,7 @@ int launch_bounded_wait_probe(long long limit_cycles, int *report, cudaStream_t 
 void *stage_begin(int id, cudaStream_t st);
 void stage_end(void *scope);
 
-// opl: 0 both operands K-major ([rows x Kc]); 1 b MN-major ([Kc x J]); 2 a and b MN-major ([Kc x I], [Kc x J]).
+// opl: 1 a [I x Kc], b [Kc x J]; 2 a [Kc x I], b [Kc x J].
 int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, int64_t Kc,
                             const uint8_t *mask, void *out, int out_dtype, int fuse_iht, int opl, cudaStream_t st);
 

@@ -1516,9 +1516,6 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                 if (grid_kind == GRID_FP4 && (t.op8 || t.rot || t.cbf)) every_output = false;
             }
             const bool fast_tail = fast_tail_opt && every_output && !any_rowsum;
-            int dev = 0, sms = 148;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             const int total = nb[0] + nb[1];
             if (wide) {
                 const int exchange = (int)((sizeof(float) * (size_t)warps + 15) / 16 * 16);
@@ -1550,7 +1547,7 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                 const int exchange = (int)((smem + 15) / 16 * 16);
                 const size_t smem2 = (size_t)exchange + 2 * (size_t)threads * (2 * E + 16);
                 const int per_sm = smem2 > 100 * 1024 ? 1 : 2;
-                const int g = total < sms * per_sm ? total : sms * per_sm;
+                const int g = total < num_sms() * per_sm ? total : num_sms() * per_sm;
                 const bool fast = fast_tail && had_block == 128;
                 if (grid_kind == GRID_FP4)
                     e = fast ? launch_stream_fp4<64, true>(g, threads, smem2, st, a, total, exchange)

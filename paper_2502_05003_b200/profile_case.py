@@ -1,6 +1,9 @@
 """Small, bounded workloads to put under ``ncu`` (one kernel, a few launches, a few GB at most).
 
     python -m paper_2502_05003_b200.profile_case linear [calls]      # quest_linear_fwd, X[4096 x 2048] W[2048 x 2048], b = 4
+    python -m paper_2502_05003_b200.profile_case one-bit [calls]     # the same at b = 1
+    python -m paper_2502_05003_b200.profile_case decode [calls]      # cached weights: 1 x 2048 x 2048 and, from codes, 24 x 5504 x 2048
+    python -m paper_2502_05003_b200.profile_case weight-only [calls] # quest_linear_fwd_weight_only on the same tensors
     python -m paper_2502_05003_b200.profile_case quantize-large      # quest_quantize alone: 6144 x 5504 and 8192 x 4096
     python -m paper_2502_05003_b200.profile_case quantize-wide       # quest_quantize alone, 8192 x 4096, one rotation block per row
     python -m paper_2502_05003_b200.profile_case mlp                 # quest_mlp_fwd, 4096 tokens, H = 2048, I = 5504
@@ -19,17 +22,40 @@ import torch
 import paper_2502_05003_b200 as quest
 
 
-def linear(calls: int = 6) -> None:
+def linear(calls: int = 6, bits: int = 4) -> None:
     M, K, N = 4096, 2048, 2048
     dev = torch.device("cuda")
     sets = []
     for _ in range(3):
         x = torch.randn(M, K, device=dev).bfloat16()
         w = (torch.randn(N, K, device=dev) * 0.02).bfloat16()
-        sets.append((x, w, quest.alloc_workspace(M, N, K, 4, 4), quest.quest_linear_fwd(x, w, 4, 128, 1.0)))
+        sets.append((x, w, quest.alloc_workspace(M, N, K, bits, bits), quest.quest_linear_fwd(x, w, bits, 128, 1.0)))
     for i in range(calls):
         x, w, ws, out = sets[i % 3]
-        quest.quest_linear_fwd(x, w, 4, 128, 1.0, y=out["y"], saved=out, workspace=ws)
+        quest.quest_linear_fwd(x, w, bits, 128, 1.0, y=out["y"], saved=out, workspace=ws)
+
+
+def decode(calls: int = 3) -> None:
+    """``calls`` rounds over 40 layers of either size, 850 MB of weights: none of them is in L2 when its turn comes."""
+    for M, N, K, packed in ((1, 2048, 2048, False), (24, 5504, 2048, True)):
+        x = torch.randn(M, K, device="cuda").bfloat16()
+        layers = []
+        for _ in range(40):
+            w = (torch.randn(N, K, device="cuda") * 0.02).bfloat16()
+            ws = quest.alloc_workspace(M, N, K, 4, 4)
+            r = quest.quest_linear_fwd(x, w, 4, 128, workspace=ws, want_masks=False)
+            layers.append((r, ws, {"wq": r["wq"], "sw": r["sw"], "operand_in_workspace": not packed}))
+        for _ in range(calls):
+            for r, ws, cached in layers:
+                quest.quest_linear_fwd(x, None, 4, 128, y=r["y"], saved={"xq": r["xq"], "sx": r["sx"]}, w_cached=cached,
+                                       workspace=ws, want_masks=False)
+
+
+def weight_only(calls: int = 4) -> None:
+    x = torch.randn(4096, 2048, device="cuda").bfloat16()
+    w = (torch.randn(2048, 2048, device="cuda") * 0.02).bfloat16()
+    for _ in range(calls):
+        quest.quest_linear_fwd_weight_only(x, w, 4, 128)
 
 
 def quantize_large() -> None:
@@ -84,6 +110,12 @@ def main() -> None:
     n = int(sys.argv[2]) if len(sys.argv) > 2 else None
     if case == "linear":
         linear(n or 6)
+    elif case == "one-bit":
+        linear(n or 6, bits=1)
+    elif case == "decode":
+        decode(n or 3)
+    elif case == "weight-only":
+        weight_only(n or 4)
     elif case == "quantize-large":
         quantize_large()
     elif case == "quantize-wide":
