@@ -133,10 +133,11 @@ struct Named {
             for (const int64_t s : shape) n *= s;
             return room(given, n);
         }
-        const at::Tensor made = fresh(shape, t, dev);
-        Ref v(THPVariable_Wrap(made));
+        at::Tensor made = fresh(shape, t, dev);
+        void *const p = made.data_ptr();
+        Ref v(THPVariable_Wrap(std::move(made)));
         set(key, v.p);
-        return made.data_ptr();
+        return p;
     }
     void *at(PyObject *key) const { return ptr(get(key)); }
 };
