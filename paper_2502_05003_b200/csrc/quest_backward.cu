@@ -332,14 +332,35 @@ cudaError_t launch_iht_wide(const float *d, int64_t rows, int64_t cols, int had_
     while (S < T) S <<= 1;
     const int R = 128 / S;
     const size_t smem = sizeof(float) * (size_t)R * (size_t)(cols + cols / 16);      // at most 34 KB
-    return launch_pdl(iht_wide_kernel<L>, dim3((unsigned)((rows + R - 1) / R)), dim3(128), smem, st, 1, d, (long long)rows,
-                      (int)cols, 1.0f / sqrtf((float)had_block), out, out_dtype, (long long)ld, S, R);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)((rows + R - 1) / R));
+    cfg.blockDim = dim3(128);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    // Launched ahead, the CTAs settle on the few SMs that the gradient product leaves free and run there several to an SM
+    // while the others idle: an input gradient of 0.3 to 5 Mi elements launched plainly takes 0.72 .. 0.93 of the time
+    // (204 shapes, at most 1.02).  A grid of a few waves levels that and gains the launch, 0.96 from 6 Mi elements on, and so
+    // does one that fits those SMs.
+    const int64_t elements = rows * cols;
+    cfg.numAttrs = elements < (300 << 10) || elements >= (5 << 20);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, iht_wide_kernel<L>, d, (long long)rows, (int)cols, 1.0f / sqrtf((float)had_block),
+                                             out, out_dtype, (long long)ld, S, R);
+    return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 int launch_iht(const float *d, int64_t rows, int64_t cols, int had_block, void *out, int out_dtype, int64_t ld,
                cudaStream_t st) {
-    // blocks of 256 .. 4096 in rows that one CTA holds with 64 elements per thread
-    if (rows > 0 && had_block >= 256 && had_block <= 4096 && cols <= 8192) {
+    // blocks of 256 .. 4096 in rows that one CTA holds with 64 elements per thread.  Small outputs of narrow blocks stay
+    // with the general kernel: its CTAs are many and short, and the fewer strides leave a thread the less there is to gain.
+    // General kernel's time over this one's, contraction and dequantisation included: g = 256 0.7 .. 0.95 below
+    // 9/16 Mi elements, 1.0 at 0.75, 1.1 at 1.5, 1.15 from 4 Mi on, but 0.75 .. 0.85 up to 2 Mi in rows of one block;
+    // g = 512 0.8 .. 0.95 up to half a Mi, 1.05 at 0.75 .. 2, 1.2 from 4 on; g = 1024 0.8 .. 1.0 up to a quarter Mi
+    const int64_t few = cols == 256 ? 4 << 20 : cols > 4096 ? 0 : had_block <= 512 ? 9 << 16 : had_block == 1024 ? 5 << 16 : 0;
+    if (rows * cols >= few && had_block >= 256 && had_block <= 4096 && cols <= 8192) {
         cudaError_t e;
         switch (had_block) {
             case 256: e = launch_iht_wide<8>(d, rows, cols, had_block, out, out_dtype, ld, st); break;

@@ -121,6 +121,17 @@ def test_wide_blocks(M, N, K, g, out_dtype):
     run_case(gauss(M, K, 31), gauss(N, K, 32, 0.02), 4, g, seed=K + g, out_dtype=out_dtype)
 
 
+@pytest.mark.parametrize("M,K,g", [(768, 768, 256), (760, 768, 256),        # at the limit of the general kernel and a row group below
+                                   (1152, 512, 512), (1144, 512, 512), (320, 1024, 1024), (312, 1024, 1024),
+                                   (16384, 256, 256), (16376, 256, 256),        # rows of one block: 32 to a CTA
+                                   (1640, 2560, 512), (8, 8192, 256), (56, 6144, 1024),  # slots of padding; few long rows
+                                   (5464, 768, 256), (10248, 512, 512)])        # either side of the launch ahead of the product's end
+@pytest.mark.parametrize("out_dtype", [torch.float32, torch.bfloat16])
+def test_wide_blocks_of_large_gradients(M, K, g, out_dtype):
+    rows = np.r_[0:M:211, max(M - 9, 0):M]
+    run_case(gauss(M, K, 61), gauss(8, K, 62, 0.02), 4, g, seed=M + K, out_dtype=out_dtype, rows_x=np.unique(rows))
+
+
 @pytest.mark.parametrize("g", [1, 2, 16, 64])
 @pytest.mark.parametrize("K", [256, 640])                       # the last tile whole, then half empty
 def test_small_blocks_in_the_epilogue(g, K):
