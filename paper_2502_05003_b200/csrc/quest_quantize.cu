@@ -167,6 +167,8 @@ struct QuantTensor {
     uint16_t *rot;         // bfloat16 of the orthonormal rotation itself (weight-only variant)
     uint16_t *cbf;         // grid values c = 2k - (2^b - 1) as bfloat16 (weight-only variant)
 };
+// Threads that an SM holds of a kernel, by the registers its launch bounds leave.
+constexpr int DIRECT_THREADS = 1024, WIDE32_THREADS = 768, WIDE_THREADS = 512, ROWS32_THREADS = 1024, ROWS64_THREADS = 512;
 constexpr int MAX_QUANT_TENSORS = 4;   // tensors one launch of the block kernel can serve (the other kernels: two)
 struct QuantArgs {
     QuantTensor t[MAX_QUANT_TENSORS];
@@ -735,10 +737,36 @@ __device__ __forceinline__ void butterfly32_in_registers(float2 (&v)[16]) {
     }
 }
 
+// Dynamic shared memory of a launch of `ctas` CTAs, `fit` of which an SM holds at once, that wants `smem` bytes of it.  The
+// hardware starts the CTAs of a launch while its predecessor drains, and fills the SMs that are free first: of a grid that
+// fits the chip in one round many gather on a few SMs while others get none.  Asking for so much shared memory that an SM
+// holds no more than its even share levels that (device time of whole calls, back to back, before and after): cached
+// weights 777 x 2048 x 2048 12.1 -> 9.8 us, 4096 x 512 x 512 10.6 -> 8.7; forward 1024 x 1024 x 1024 10.1 -> 8.7; 680 calls of
+// every kind 0.98 in the mean, none above 1.02.  It is left alone below one and a half CTAs per SM, where there is little to
+// level and the CTAs could no longer settle beside a contraction that is still running (100 x 640 x 896 6.8 -> 7.1), and
+// where the share is what fits anyway: there it would only take from the L1 (binary32, 64 x 2048 + 2048 x 2048 9.4 -> 9.9).
+size_t even_share_smem(long long ctas, long long fit, size_t smem) {
+    const long long sms = num_sms(), share = (ctas + sms - 1) / sms;
+    if (2 * ctas < 3 * sms || share >= fit) return smem;
+    const size_t least = 233472 / (size_t)(share + 1) - 1024 + 128;   // of 228 KB, 1 KB of which goes to every CTA
+    return smem > least ? smem : least / 128 * 128;
+}
+
+// Launch of a kernel that may ask for more than the 48 KB of dynamic shared memory that need no permission.
+template <auto KERNEL, typename... Args>
+cudaError_t launch_quantizer(dim3 grid, int threads, size_t smem, cudaStream_t st, const Args &...args) {
+    if (smem > 48 * 1024) {
+        static DynamicSmemOnce once;
+        const cudaError_t e = once.set(KERNEL, 160 * 1024);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_pdl(KERNEL, grid, dim3((unsigned)threads), smem, st, 1, args...);
+}
+
 // G (threads per rotation block) is a template parameter so that every index of the two layout changes is a
 // compile-time offset.
 template <int CB, bool FAST, int GRID, int G, bool DECODE>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(256, WIDE32_THREADS / 256)
 quantize_wide32_kernel(const __grid_constant__ QuantArgs a, int exchange_bytes) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     pdl_begin<DECODE>();
@@ -833,13 +861,8 @@ template <int GRID, bool FAST, int G, bool DECODE>
 static cudaError_t launch_wide32_g(int cb, int grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                  int exchange_bytes) {
 #define QUEST_LAUNCH(CBV)                                                                                   \
-    do {                                                                                                    \
-        static DynamicSmemOnce once_;                                                                       \
-        cudaError_t e_ = once_.set(quantize_wide32_kernel<CBV, FAST, GRID, G, DECODE>, 160 * 1024);                   \
-        if (e_ != cudaSuccess) return e_;                                                                   \
-        return launch_pdl(quantize_wide32_kernel<CBV, FAST, GRID, G, DECODE>, dim3((unsigned)grid), dim3(threads), smem, st, 1, a, \
-                          exchange_bytes);                                                                  \
-    } while (0)
+    return launch_quantizer<quantize_wide32_kernel<CBV, FAST, GRID, G, DECODE>>(                            \
+        dim3((unsigned)grid), threads, even_share_smem(grid, WIDE32_THREADS / threads, smem), st, a, exchange_bytes)
     if constexpr (GRID == GRID_FP4) {
         QUEST_LAUNCH(4);
     } else {
@@ -875,7 +898,7 @@ static cudaError_t launch_wide32(int cb, int grid, int threads, size_t smem, cud
 // element instead of 27).  16384 x 4096, g = 4096, 3 bits: 75 -> 64 us; 16384 x 2048, g = 256: 37.7 -> 30.8 us;
 // 4096 x 2048 binary32, g = 2048: 20.5 -> 11.8 us.
 template <bool BF16, int CB, int GRID, bool RS, bool G4096>
-__global__ void __launch_bounds__(128, 4)
+__global__ void __launch_bounds__(128, WIDE_THREADS / 128)
 quantize_wide_kernel(const __grid_constant__ QuantArgs a, int exchange_bytes) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     pdl_begin<false>();
@@ -956,8 +979,8 @@ template <bool BF16, int GRID, bool G4096>
 static cudaError_t launch_wide_g(int cb, int grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                  int exchange_bytes, bool rowsums) {
 #define QUEST_LAUNCH(CBV, RSV)                                                                                              \
-    return launch_pdl(quantize_wide_kernel<BF16, CBV, GRID, RSV, G4096>, dim3((unsigned)grid), dim3(threads), smem, st, 1, a, \
-                      exchange_bytes)
+    return launch_quantizer<quantize_wide_kernel<BF16, CBV, GRID, RSV, G4096>>(                                             \
+        dim3((unsigned)grid), threads, even_share_smem(grid, WIDE_THREADS / threads, smem), st, a, exchange_bytes)
     if constexpr (GRID == GRID_FP4) {
         QUEST_LAUNCH(4, false);
     } else {
@@ -994,7 +1017,7 @@ static cudaError_t launch_wide(bool bf16, int cb, int grid, int threads, size_t 
 // a whole layer of 777 x 2048 x 5504 without masks 21.8 -> 21.1 us).
 template <int CB, int GRID = GRID_UNIFORM, bool RS = false, int COLS = 0, int HB = 128, bool OPT = false,
           bool DECODE = false>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(256, DIRECT_THREADS / 256)
 quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
     constexpr int CS = COLS / 32;
     const int S = CS ? CS : a.S, R = CS ? 128 / CS : a.R, cols = COLS ? COLS : a.cols;
@@ -1289,17 +1312,21 @@ static cudaError_t launch_block128(int cb, dim3 grid, int threads, size_t smem, 
 template <int GRID, int COLS, int HB, bool OPT, bool DECODE = false>
 static cudaError_t launch_direct128_cols(int cb, dim3 grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                          bool rowsums) {
+#define QUEST_LAUNCH(CBV, RSV)                                                                              \
+    return launch_quantizer<quantize_direct128_kernel<CBV, GRID, RSV, COLS, HB, OPT, DECODE>>(grid, threads, smem, st, a)
+    smem = even_share_smem(grid.x, DIRECT_THREADS / threads, smem);
     if constexpr (GRID == GRID_FP4) {
-        return launch_pdl(quantize_direct128_kernel<4, GRID, false, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
+        QUEST_LAUNCH(4, false);
     } else {
-        if (rowsums) return launch_pdl(quantize_direct128_kernel<8, GRID, true, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
+        if (rowsums) QUEST_LAUNCH(8, true);
         switch (cb) {
-            case 1: return launch_pdl(quantize_direct128_kernel<1, GRID, false, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
-            case 2: return launch_pdl(quantize_direct128_kernel<2, GRID, false, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
-            case 4: return launch_pdl(quantize_direct128_kernel<4, GRID, false, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
-            default: return launch_pdl(quantize_direct128_kernel<8, GRID, false, COLS, HB, OPT, DECODE>, grid, dim3(threads), smem, st, 1, a);
+            case 1: QUEST_LAUNCH(1, false);
+            case 2: QUEST_LAUNCH(2, false);
+            case 4: QUEST_LAUNCH(4, false);
+            default: QUEST_LAUNCH(8, false);
         }
     }
+#undef QUEST_LAUNCH
 }
 
 template <int GRID>
@@ -1324,35 +1351,22 @@ static cudaError_t launch_direct128(int cb, dim3 grid, int threads, size_t smem,
 
 template <bool BF16, int E, bool DECODE = false>
 static cudaError_t launch_rows(int cb, dim3 grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a) {
-#define QUEST_LAUNCH(CBV)                                                                                   \
-    do {                                                                                                    \
-        if (smem > 48 * 1024) {                                                                             \
-            static DynamicSmemOnce once_;                                                                   \
-            cudaError_t e_ = once_.set(quantize_rows_kernel<BF16, CBV, E, GRID_UNIFORM, DECODE>, 72 * 1024);                      \
-            if (e_ != cudaSuccess) return e_;                                                               \
-        }                                                                                                   \
-        cudaError_t l_ = launch_pdl(quantize_rows_kernel<BF16, CBV, E, GRID_UNIFORM, DECODE>, grid, dim3(threads), smem, st, 1, a);  \
-        if (l_ != cudaSuccess) return l_;                                                                   \
-    } while (0)
+#define QUEST_LAUNCH(CBV) return launch_quantizer<quantize_rows_kernel<BF16, CBV, E, GRID_UNIFORM, DECODE>>(grid, threads, smem, st, a)
+    smem = even_share_smem(grid.x, (E == 64 ? ROWS64_THREADS : ROWS32_THREADS) / threads, smem);
     switch (cb) {
-        case 1: QUEST_LAUNCH(1); break;
-        case 2: QUEST_LAUNCH(2); break;
-        case 4: QUEST_LAUNCH(4); break;
-        default: QUEST_LAUNCH(8); break;
+        case 1: QUEST_LAUNCH(1);
+        case 2: QUEST_LAUNCH(2);
+        case 4: QUEST_LAUNCH(4);
+        default: QUEST_LAUNCH(8);
     }
 #undef QUEST_LAUNCH
-    return cudaGetLastError();
 }
 
 // FP4 grid: 4-bit containers only.
 template <bool BF16, int E>
 static cudaError_t launch_rows_fp4(dim3 grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a) {
-    if (smem > 48 * 1024) {
-        static DynamicSmemOnce once_;
-        cudaError_t e_ = once_.set(quantize_rows_kernel<BF16, 4, E, GRID_FP4>, 72 * 1024);
-        if (e_ != cudaSuccess) return e_;
-    }
-    return launch_pdl(quantize_rows_kernel<BF16, 4, E, GRID_FP4>, grid, dim3(threads), smem, st, 1, a);
+    smem = even_share_smem(grid.x, (E == 64 ? ROWS64_THREADS : ROWS32_THREADS) / threads, smem);
+    return launch_quantizer<quantize_rows_kernel<BF16, 4, E, GRID_FP4>>(grid, threads, smem, st, a);
 }
 
 template <int E, bool FAST>

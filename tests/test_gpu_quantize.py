@@ -69,6 +69,14 @@ def test_blocks_of_64(bits, cols, trust):
     check(x, bits, 64, trust)
 
 
+@pytest.mark.parametrize("bits", [1, 4, 8])
+@pytest.mark.parametrize("g,cols,rows,bf16", [(128, 1024, 1200, True), (64, 1376, 700, True), (32, 1024, 1000, True),
+                                              (128, 512, 3600, True), (2048, 2048, 500, True), (4096, 4096, 590, False)])
+def test_grids_of_two_and_three_ctas_per_sm(bits, g, cols, rows, bf16):
+    # every kernel family at grids whose CTAs are spread over the SMs by their shared memory (two and three to an SM)
+    check(rows_of("outliers", rows, cols, bits + cols, bf16), bits, g, repeat=1)
+
+
 @pytest.mark.parametrize("bits", [1, 2, 3, 4, 8])
 @pytest.mark.parametrize("dtype_bf16", [False, True])
 @pytest.mark.parametrize("g,cols", [(8, 8), (8, 24), (1, 40), (8, 72), (8, 136), (4, 1000), (8, 4104), (2, 16376)])
