@@ -482,11 +482,18 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
 template <int SRC, bool FUSED, int MT, int NT>
 cudaError_t launch_one(const DecodeArgs &a, cudaStream_t st) {
     size_t smem = Ring<FUSED, MT, NT>::BYTES;
+    const int ctas = (a.N + 16 * MT - 1) / (16 * MT);
     if (FUSED) smem += (size_t)a.M * a.pitch + (a.g >= 512 ? (size_t)a.M * ((a.K + 255) / 256) * 1024 : 0);
+    // One CTA per SM where there are no more of them: started while the quantizer drains, two would share each SM that is
+    // free first.  Bytes of w from the operand or 4- and 8-bit codes: 24 x 2048 x 5504 9.5 -> 7.8 us, from packed codes 12.8
+    // -> 9.3, 24 x 4096 x 4096 at 8 bits 11.0 -> 9.0; equal on short rows.  One and two bits are held by unpacking and lose
+    // a little (24 x 4096 x 4096 at two bits 8.5 -> 8.7); the fused form, whose CTAs are short, gains nothing.
+    constexpr bool BYTES_OR_NIBBLES = SRC == SRC_OP8 || SRC == SRC_CODES4 || SRC == SRC_CODES8;
+    if (!FUSED && BYTES_OR_NIBBLES && ctas <= num_sms() && smem < 116 * 1024) smem = 116 * 1024;
     static DynamicSmemOnce once;
     const cudaError_t e = once.set(decode_kernel<SRC, FUSED, MT, NT>, 144 * 1024);
     if (e != cudaSuccess) return e;
-    return launch_pdl(decode_kernel<SRC, FUSED, MT, NT>, dim3((unsigned)((a.N + 16 * MT - 1) / (16 * MT))), dim3(THREADS), smem, st, 1, a);
+    return launch_pdl(decode_kernel<SRC, FUSED, MT, NT>, dim3((unsigned)ctas), dim3(THREADS), smem, st, 1, a);
 }
 
 template <int SRC, bool FUSED>
