@@ -168,7 +168,11 @@ struct QuantTensor {
     uint16_t *cbf;         // grid values c = 2k - (2^b - 1) as bfloat16 (weight-only variant)
 };
 // Threads that an SM holds of a kernel, by the registers its launch bounds leave.
-constexpr int DIRECT_THREADS = 1024, WIDE32_THREADS = 768, WIDE_THREADS = 512, ROWS32_THREADS = 1024, ROWS64_THREADS = 512;
+// quantize_wide_kernel: five CTAs (96 registers, up to five words spilled) pay for bfloat16 blocks of 4096, whose exchange
+// with the neighbour leaves more to wait for: 16384 x 4096 63.3 -> 60.3 us, 4096 x 4096 18.3 -> 17.6; narrower blocks gain 2 %
+// at 16384 rows and lose 5 % at 1024, binary32 loses 8 %.
+__host__ __device__ constexpr int wide_threads(bool bf16, bool g4096) { return bf16 && g4096 ? 640 : 512; }
+constexpr int DIRECT_THREADS = 1024, WIDE32_THREADS = 768, ROWS32_THREADS = 1024, ROWS64_THREADS = 512;
 constexpr int MAX_QUANT_TENSORS = 4;   // tensors one launch of the block kernel can serve (the other kernels: two)
 struct QuantArgs {
     QuantTensor t[MAX_QUANT_TENSORS];
@@ -898,7 +902,7 @@ static cudaError_t launch_wide32(int cb, int grid, int threads, size_t smem, cud
 // element instead of 27).  16384 x 4096, g = 4096, 3 bits: 75 -> 64 us; 16384 x 2048, g = 256: 37.7 -> 30.8 us;
 // 4096 x 2048 binary32, g = 2048: 20.5 -> 11.8 us.
 template <bool BF16, int CB, int GRID, bool RS, bool G4096>
-__global__ void __launch_bounds__(128, WIDE_THREADS / 128)
+__global__ void __launch_bounds__(128, wide_threads(BF16, G4096) / 128)
 quantize_wide_kernel(const __grid_constant__ QuantArgs a, int exchange_bytes) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     pdl_begin<false>();
@@ -980,7 +984,7 @@ static cudaError_t launch_wide_g(int cb, int grid, int threads, size_t smem, cud
                                  int exchange_bytes, bool rowsums) {
 #define QUEST_LAUNCH(CBV, RSV)                                                                                              \
     return launch_quantizer<quantize_wide_kernel<BF16, CBV, GRID, RSV, G4096>>(                                             \
-        dim3((unsigned)grid), threads, even_share_smem(grid, WIDE_THREADS / threads, smem), st, a, exchange_bytes)
+        dim3((unsigned)grid), threads, even_share_smem(grid, wide_threads(BF16, G4096) / threads, smem), st, a, exchange_bytes)
     if constexpr (GRID == GRID_FP4) {
         QUEST_LAUNCH(4, false);
     } else {
