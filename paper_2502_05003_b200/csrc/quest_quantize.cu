@@ -172,7 +172,12 @@ struct QuantTensor {
 // with the neighbour leaves more to wait for: 16384 x 4096 63.3 -> 60.3 us, 4096 x 4096 18.3 -> 17.6; narrower blocks gain 2 %
 // at 16384 rows and lose 5 % at 1024, binary32 loses 8 %.
 __host__ __device__ constexpr int wide_threads(bool bf16, bool g4096) { return bf16 && g4096 ? 640 : 512; }
-constexpr int DIRECT_THREADS = 1024, WIDE32_THREADS = 768, ROWS32_THREADS = 1024, ROWS64_THREADS = 512;
+// quantize_direct128_kernel: 56 registers with run-time row lengths, so that six CTAs of 192 threads (rows of 5152 .. 6144)
+// fit an SM, not five: 8192 x 5504 + 2048 x 5504 at 8 bits 63.7 -> 60.8 us, without masks 59.0 -> 56.9, cached weights of two
+// bits 4096 x 2048 x 5504 46.7 -> 45.7; 1 % slower on some shorter rows (8192 x 640).  The fixed row lengths, which fill an SM
+// either way, lose 5 % with 48 registers.
+__host__ __device__ constexpr int direct_threads(int cols) { return cols ? 65536 / 64 : 65536 / 56; }
+constexpr int WIDE32_THREADS = 768, ROWS32_THREADS = 1024, ROWS64_THREADS = 512;
 constexpr int MAX_QUANT_TENSORS = 4;   // tensors one launch of the block kernel can serve (the other kernels: two)
 struct QuantArgs {
     QuantTensor t[MAX_QUANT_TENSORS];
@@ -1021,7 +1026,7 @@ static cudaError_t launch_wide(bool bf16, int cb, int grid, int threads, size_t 
 // a whole layer of 777 x 2048 x 5504 without masks 21.8 -> 21.1 us).
 template <int CB, int GRID = GRID_UNIFORM, bool RS = false, int COLS = 0, int HB = 128, bool OPT = false,
           bool DECODE = false>
-__global__ void __launch_bounds__(256, DIRECT_THREADS / 256)
+__global__ void __maxnreg__(COLS ? 64 : 56)
 quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
     constexpr int CS = COLS / 32;
     const int S = CS ? CS : a.S, R = CS ? 128 / CS : a.R, cols = COLS ? COLS : a.cols;
@@ -1318,7 +1323,7 @@ static cudaError_t launch_direct128_cols(int cb, dim3 grid, int threads, size_t 
                                          bool rowsums) {
 #define QUEST_LAUNCH(CBV, RSV)                                                                              \
     return launch_quantizer<quantize_direct128_kernel<CBV, GRID, RSV, COLS, HB, OPT, DECODE>>(grid, threads, smem, st, a)
-    smem = even_share_smem(grid.x, DIRECT_THREADS / threads, smem);
+    smem = even_share_smem(grid.x, direct_threads(COLS) / threads, smem);
     if constexpr (GRID == GRID_FP4) {
         QUEST_LAUNCH(4, false);
     } else {
