@@ -70,7 +70,7 @@ def test_blocks_of_64(bits, cols, trust):
 
 
 @pytest.mark.parametrize("bits", [1, 4, 8])
-@pytest.mark.parametrize("g,cols,rows,bf16", [(128, 1024, 1200, True), (64, 1376, 700, True), (32, 1024, 1000, True),
+@pytest.mark.parametrize("g,cols,rows,bf16", [(128, 1024, 1200, True), (64, 1344, 700, True), (32, 1024, 1000, True),
                                               (128, 512, 3600, True), (2048, 2048, 500, True), (4096, 4096, 590, False)])
 def test_grids_of_two_and_three_ctas_per_sm(bits, g, cols, rows, bf16):
     # every kernel family at grids whose CTAs are spread over the SMs by their shared memory (two and three to an SM)
