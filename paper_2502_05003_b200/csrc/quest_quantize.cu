@@ -172,11 +172,10 @@ struct QuantTensor {
 // with the neighbour leaves more to wait for: 16384 x 4096 63.3 -> 60.3 us, 4096 x 4096 18.3 -> 17.6; narrower blocks gain 2 %
 // at 16384 rows and lose 5 % at 1024, binary32 loses 8 %.
 __host__ __device__ constexpr int wide_threads(bool bf16, bool g4096) { return bf16 && g4096 ? 640 : 512; }
-// quantize_direct128_kernel: 56 registers with run-time row lengths, so that six CTAs of 192 threads (rows of 5152 .. 6144)
-// fit an SM, not five: 8192 x 5504 + 2048 x 5504 at 8 bits 63.7 -> 60.8 us, without masks 59.0 -> 56.9, cached weights of two
-// bits 4096 x 2048 x 5504 46.7 -> 45.7; 1 % slower on some shorter rows (8192 x 640).  The fixed row lengths, which fill an SM
-// either way, lose 5 % with 48 registers.
-__host__ __device__ constexpr int direct_threads(int cols) { return cols ? 65536 / 64 : 65536 / 56; }
+// quantize_direct128_kernel: 56 registers in place of 64 let six CTAs of 192 threads (rows of 5152 .. 6144) on an SM, not
+// five: 8192 x 5504 + 2048 x 5504 at 8 bits 63.7 -> 60.8 us, without masks 59.0 -> 56.9, cached weights of two bits 4096 x
+// 2048 x 5504 46.7 -> 45.7.  Shorter rows, whose CTAs of 128 threads fill an SM either way, lose 1 .. 9 %.
+constexpr int direct_threads(int regs) { return 65536 / regs; }
 constexpr int WIDE32_THREADS = 768, ROWS32_THREADS = 1024, ROWS64_THREADS = 512;
 constexpr int MAX_QUANT_TENSORS = 4;   // tensors one launch of the block kernel can serve (the other kernels: two)
 struct QuantArgs {
@@ -1025,8 +1024,8 @@ static cudaError_t launch_wide(bool bf16, int cb, int grid, int threads, size_t 
 // their own with run-time row length (6144 x 2048, g = 64, every output, against the general kernel: 13.6 -> 11.9 us;
 // a whole layer of 777 x 2048 x 5504 without masks 21.8 -> 21.1 us).
 template <int CB, int GRID = GRID_UNIFORM, bool RS = false, int COLS = 0, int HB = 128, bool OPT = false,
-          bool DECODE = false>
-__global__ void __maxnreg__(COLS ? 64 : 56)
+          bool DECODE = false, int REGS = 64>
+__global__ void __maxnreg__(REGS)
 quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
     constexpr int CS = COLS / 32;
     const int S = CS ? CS : a.S, R = CS ? 128 / CS : a.R, cols = COLS ? COLS : a.cols;
@@ -1318,12 +1317,12 @@ static cudaError_t launch_block128(int cb, dim3 grid, int threads, size_t smem, 
     return launch_block128_ct<GRID, 0>(cb, grid, threads, smem, st, a);
 }
 
-template <int GRID, int COLS, int HB, bool OPT, bool DECODE = false>
+template <int GRID, int COLS, int HB, bool OPT, bool DECODE = false, int REGS = 64>
 static cudaError_t launch_direct128_cols(int cb, dim3 grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                          bool rowsums) {
 #define QUEST_LAUNCH(CBV, RSV)                                                                              \
-    return launch_quantizer<quantize_direct128_kernel<CBV, GRID, RSV, COLS, HB, OPT, DECODE>>(grid, threads, smem, st, a)
-    smem = even_share_smem(grid.x, direct_threads(COLS) / threads, smem);
+    return launch_quantizer<quantize_direct128_kernel<CBV, GRID, RSV, COLS, HB, OPT, DECODE, REGS>>(grid, threads, smem, st, a)
+    smem = even_share_smem(grid.x, direct_threads(REGS) / threads, smem);
     if constexpr (GRID == GRID_FP4) {
         QUEST_LAUNCH(4, false);
     } else {
@@ -1345,6 +1344,11 @@ static cudaError_t launch_direct128(int cb, dim3 grid, int threads, size_t smem,
         if (for_decode)
             return a.had_block == 64 ? launch_direct128_cols<GRID, 0, 64, true, true>(cb, grid, threads, smem, st, a, rowsums)
                                      : launch_direct128_cols<GRID, 0, 128, true, true>(cb, grid, threads, smem, st, a, rowsums);
+    }
+    if (threads == 192) {
+        if (a.had_block == 64) return launch_direct128_cols<GRID, 0, 64, true, false, 56>(cb, grid, threads, smem, st, a, rowsums);
+        return every_output ? launch_direct128_cols<GRID, 0, 128, false, false, 56>(cb, grid, threads, smem, st, a, rowsums)
+                            : launch_direct128_cols<GRID, 0, 128, true, false, 56>(cb, grid, threads, smem, st, a, rowsums);
     }
     if (a.had_block == 64) return launch_direct128_cols<GRID, 0, 64, true>(cb, grid, threads, smem, st, a, rowsums);
     if (!every_output) return launch_direct128_cols<GRID, 0, 128, true>(cb, grid, threads, smem, st, a, rowsums);
