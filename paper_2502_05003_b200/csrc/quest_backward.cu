@@ -14,6 +14,8 @@
 //   3. iht_wide / iht_rows    block Hadamard transform, 1/sqrt(g), store in the output type
 //      (for blocks of up to 128 stages 2 and 3 are one kernel: the transform runs in the GEMM epilogue,
 //      where a thread holds 128 aligned columns of its output row)
+//   A product whose output is small and whose sum is long runs in parts of the contraction index, or it would leave most
+//   SMs idle; then stage 3 adds the parts (in order) and applies the mask, at any block size.
 #include <cuda_bf16.h>
 #include <math.h>
 
@@ -97,9 +99,11 @@ dequant_codes_kernel(DequantTensor t0, DequantTensor t1, int blocks0, int rpb, i
 // stored as out_dtype with row stride ld.  Every thread owns 32 contiguous elements; descending
 // stride: partners in other warps through shared memory, partners in this warp through shuffles,
 // the rest in registers.  A row of T = cols/32 threads occupies S slots as in the quantizer.
+// PARTS: d is `parts` matrices `part_stride` elements apart, whose sum, where `mask` [rows x cols/8] keeps it, is the input.
+template <bool PARTS>
 __global__ void __launch_bounds__(512)
-iht_rows_kernel(const void *__restrict__ d, int in_dtype, long long ld_in, long long rows, int cols, int had_block,
-                float inv_sqrt_g, void *__restrict__ out, int out_dtype, long long ld, int S, int R) {
+iht_rows_kernel(const float *__restrict__ d, long long rows, int cols, int had_block, float inv_sqrt_g, void *__restrict__ out,
+                int out_dtype, int S, int R, int parts, long long part_stride, const uint8_t *__restrict__ mask) {
     extern __shared__ float xsm[];                 // [32][blockDim.x] exchange
     pdl_launch_dependents();
     pdl_wait();
@@ -109,24 +113,26 @@ iht_rows_kernel(const void *__restrict__ d, int in_dtype, long long ld_in, long 
     const long long row = (long long)blockIdx.x * R + r_local;
     const bool active = row < rows && tr < cols / 32;
     float v[32];
-    if (active && in_dtype == QUEST_F32) {
-        const float4 *src = reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(d) + row * ld_in + (long long)tr * 32);
+    if (active) {
+        const float4 *src = reinterpret_cast<const float4 *>(d + row * cols + (long long)tr * 32);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const float4 w = __ldg(src + q);
             v[4 * q] = w.x; v[4 * q + 1] = w.y; v[4 * q + 2] = w.z; v[4 * q + 3] = w.w;
         }
-    } else if (active) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(d) + row * ld_in + (long long)tr * 32);
+        if constexpr (PARTS) {
+            const uint32_t keep = __ldg(reinterpret_cast<const uint32_t *>(mask + row * (cols >> 3)) + tr);
+#pragma unroll 2
+            for (int q2 = 1; q2 < parts; ++q2) {
+                src += part_stride / 4;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint4 w = __ldg(src + q);
-            const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                v[8 * q + 2 * j] = __uint_as_float(ww[j] << 16);
-                v[8 * q + 2 * j + 1] = __uint_as_float(ww[j] & 0xFFFF0000u);
+                for (int q = 0; q < 8; ++q) {
+                    const float4 w = __ldg(src + q);
+                    v[4 * q] += w.x; v[4 * q + 1] += w.y; v[4 * q + 2] += w.z; v[4 * q + 3] += w.w;
+                }
             }
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] = (keep >> i) & 1u ? v[i] : 0.0f;
         }
     } else {
 #pragma unroll
@@ -168,13 +174,13 @@ iht_rows_kernel(const void *__restrict__ d, int in_dtype, long long ld_in, long 
     }
     if (!active) return;
     if (out_dtype == QUEST_F32) {
-        float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(out) + row * ld + (long long)tr * 32);
+        float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(out) + row * cols + (long long)tr * 32);
 #pragma unroll
         for (int q = 0; q < 8; ++q)
             dst[q] = make_float4(v[4 * q] * inv_sqrt_g, v[4 * q + 1] * inv_sqrt_g, v[4 * q + 2] * inv_sqrt_g,
                                  v[4 * q + 3] * inv_sqrt_g);
     } else {
-        uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(out) + row * ld + (long long)tr * 32);
+        uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(out) + row * cols + (long long)tr * 32);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             uint32_t w[4];
@@ -195,10 +201,10 @@ iht_rows_kernel(const void *__restrict__ d, int in_dtype, long long ld_in, long 
 // goes back through the same shared memory so that it leaves in consecutive 16-byte stores.  The order of the stages
 // and every operand are those of the kernel above: identical results.
 // Bound by memory traffic (the masked product is read from L2, where the contraction left it).
-template <int L>
+template <int L, bool PARTS>
 __global__ void __launch_bounds__(128, 4)
 iht_wide_kernel(const float *__restrict__ d, long long rows, int cols, float inv_sqrt_g, void *__restrict__ out,
-                int out_dtype, long long ld, int S, int R) {
+                int out_dtype, int S, int R, int parts, long long part_stride, const uint8_t *__restrict__ mask) {
     extern __shared__ __align__(16) float tbuf[];              // [R][cols + cols / 16]
     constexpr int NA = L == 12 ? 5 : L - 6;                    // strides of phase A
     constexpr int NL = 5 - NA;
@@ -223,6 +229,21 @@ iht_wide_kernel(const float *__restrict__ d, long long rows, int cols, float inv
 #pragma unroll
         for (int j = 0; j < 32; ++j)
             v[j] = __ldg(reinterpret_cast<const float2 *>(src + (j >> NL) * HI + 2 * ((j & ((1 << NL) - 1)) << NA)));
+        if constexpr (PARTS) {
+            for (int q = 1; q < parts; ++q) {
+                src += part_stride;
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    v[j] = __fadd2_rn(v[j], __ldg(reinterpret_cast<const float2 *>(src + (j >> NL) * HI + 2 * ((j & ((1 << NL) - 1)) << NA))));
+            }
+            const uint8_t *mrow = mask + row * (cols >> 3);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                const int e = i0 + (j >> NL) * HI + 2 * ((j & ((1 << NL) - 1)) << NA);
+                const uint32_t keep = (uint32_t)__ldg(mrow + (e >> 3)) >> (e & 7);
+                v[j] = make_float2(keep & 1u ? v[j].x : 0.0f, keep & 2u ? v[j].y : 0.0f);
+            }
+        }
 #pragma unroll
         for (int s = 16; s >= (1 << NL); s >>= 1)
 #pragma unroll
@@ -297,7 +318,7 @@ iht_wide_kernel(const float *__restrict__ d, long long rows, int cols, float inv
     const int chunks = cols >> (6 - sh);
     const long long left = rows - row0;
     const int rows_here = left < R ? (int)left : R;
-    const size_t row_bytes = (size_t)ld * (out_dtype == QUEST_F32 ? 4 : 2);
+    const size_t row_bytes = (size_t)cols * (out_dtype == QUEST_F32 ? 4 : 2);
     for (int r = 0; r < rows_here; ++r) {
         uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(out) + (size_t)(row0 + r) * row_bytes);
         const float *from = tbuf + (size_t)r * pitch;
@@ -324,36 +345,74 @@ BwdWorkspace carve_bwd(void *base, int64_t M, int64_t N, int64_t K) {
     return w;
 }
 
-template <int L>
-cudaError_t launch_iht_wide(const float *d, int64_t rows, int64_t cols, int had_block, void *out, int out_dtype, int64_t ld,
-                            cudaStream_t st) {
-    const int T = (int)(cols >> 6);                            // at most 128 (cols <= 8192)
-    int S = 1;
-    while (S < T) S <<= 1;
-    const int R = 128 / S;
-    const size_t smem = sizeof(float) * (size_t)R * (size_t)(cols + cols / 16);      // at most 34 KB
+// Rows per CTA of a transform whose rows take S threads: CTAs of 128 threads where a row fits.  Adding parts is bound by the
+// reads in flight, so there the rows are dealt out until every SM has several CTAs.
+int transform_rows_per_cta(int64_t rows, int S, int parts) {
+    int R = S <= 128 ? 128 / S : 1;
+    while (parts > 1 && R > 1 && R * S > 32 && rows < 4ll * num_sms() * R) R >>= 1;
+    return R;
+}
+
+// A transform launched ahead of its predecessor's end, or (adding parts, and where launch_iht_wide says so) plainly.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_transform(void (*kernel)(KArgs...), int64_t grid, int threads, size_t smem, cudaStream_t st, bool ahead, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)((rows + R - 1) / R));
-    cfg.blockDim = dim3(128);
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = attr;
+    cfg.numAttrs = ahead ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    return e == cudaSuccess ? cudaGetLastError() : e;
+}
+
+template <int L>
+cudaError_t launch_iht_wide(const float *d, int64_t rows, int64_t cols, int had_block, void *out, int out_dtype, int parts,
+                            const uint8_t *mask, cudaStream_t st) {
+    const int T = (int)(cols >> 6);                            // at most 128 (cols <= 8192)
+    int S = 1;
+    while (S < T) S <<= 1;
+    const int R = transform_rows_per_cta(rows, S, parts);
+    const size_t smem = sizeof(float) * (size_t)R * (size_t)(cols + cols / 16);      // at most 34 KB
     // Launched ahead, the CTAs settle on the few SMs that the gradient product leaves free and run there several to an SM
     // while the others idle: an input gradient of 0.3 to 5 Mi elements launched plainly takes 0.72 .. 0.93 of the time
     // (204 shapes, at most 1.02).  A grid of a few waves levels that and gains the launch, 0.96 from 6 Mi elements on, and so
     // does one that fits those SMs.
     const int64_t elements = rows * cols;
-    cfg.numAttrs = elements < (300 << 10) || elements >= (5 << 20);
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, iht_wide_kernel<L>, d, (long long)rows, (int)cols, 1.0f / sqrtf((float)had_block),
-                                             out, out_dtype, (long long)ld, S, R);
-    return e == cudaSuccess ? cudaGetLastError() : e;
+    const bool ahead = parts == 1 && (elements < (300 << 10) || elements >= (5 << 20));
+    return launch_transform(parts > 1 ? iht_wide_kernel<L, true> : iht_wide_kernel<L, false>, (rows + R - 1) / R, R * S, smem, st, ahead, d,
+                            (long long)rows, (int)cols, 1.0f / sqrtf((float)had_block), out, out_dtype, S, R, parts,
+                            (long long)((rows + 255) / 256 * 256 * cols), mask);
 }
 
-int launch_iht(const float *d, int64_t rows, int64_t cols, int had_block, void *out, int out_dtype, int64_t ld,
-               cudaStream_t st) {
+// Any block size, one thread per 32 elements.
+int launch_iht_rows(const float *d, int64_t rows, int64_t cols, int had_block, void *out, int out_dtype, int parts,
+                    const uint8_t *mask, cudaStream_t st) {
+    const int T = (int)(cols / 32);
+    int S;
+    if (T < 32) { S = 1; while (S < T) S <<= 1; } else { S = (T + 31) / 32 * 32; }
+    const int R = transform_rows_per_cta(rows, S, parts);
+    const int threads = R * S;
+    const size_t smem = had_block >= 2048 ? sizeof(float) * 32 * (size_t)threads : 0;
+    if (smem > 48 * 1024) {
+        static DynamicSmemOnce whole, divided;
+        cudaError_t e = parts > 1 ? divided.set(iht_rows_kernel<true>, 72 * 1024) : whole.set(iht_rows_kernel<false>, 72 * 1024);
+        if (e != cudaSuccess) return cuda_fail(e);
+    }
+    const cudaError_t e = launch_transform(parts > 1 ? iht_rows_kernel<true> : iht_rows_kernel<false>, (rows + R - 1) / R, threads, smem, st,
+                                           parts == 1, d, (long long)rows, (int)cols, had_block, 1.0f / sqrtf((float)had_block), out,
+                                           out_dtype, S, R, parts, (long long)((rows + 255) / 256 * 256 * cols), mask);
+    return e == cudaSuccess ? QUEST_OK : cuda_fail(e);
+}
+
+// Inverse transform of d [rows x cols], binary32 and dense, or (parts > 1) of the sum of the parts that
+// launch_gemm_bf16_parts left there, where `mask` keeps it; `out` is dense too.
+int launch_iht(const float *d, int64_t rows, int64_t cols, int had_block, void *out, int out_dtype, int parts,
+               const uint8_t *mask, cudaStream_t st) {
     // blocks of 256 .. 4096 in rows that one CTA holds with 64 elements per thread.  Small outputs of narrow blocks stay
     // with the general kernel: its CTAs are many and short, and the fewer strides leave a thread the less there is to gain.
     // General kernel's time over this one's, contraction and dequantisation included: g = 256 0.7 .. 0.95 below
@@ -363,43 +422,16 @@ int launch_iht(const float *d, int64_t rows, int64_t cols, int had_block, void *
     if (rows * cols >= few && had_block >= 256 && had_block <= 4096 && cols <= 8192) {
         cudaError_t e;
         switch (had_block) {
-            case 256: e = launch_iht_wide<8>(d, rows, cols, had_block, out, out_dtype, ld, st); break;
-            case 512: e = launch_iht_wide<9>(d, rows, cols, had_block, out, out_dtype, ld, st); break;
-            case 1024: e = launch_iht_wide<10>(d, rows, cols, had_block, out, out_dtype, ld, st); break;
-            case 2048: e = launch_iht_wide<11>(d, rows, cols, had_block, out, out_dtype, ld, st); break;
-            default: e = launch_iht_wide<12>(d, rows, cols, had_block, out, out_dtype, ld, st); break;
+            case 256: e = launch_iht_wide<8>(d, rows, cols, had_block, out, out_dtype, parts, mask, st); break;
+            case 512: e = launch_iht_wide<9>(d, rows, cols, had_block, out, out_dtype, parts, mask, st); break;
+            case 1024: e = launch_iht_wide<10>(d, rows, cols, had_block, out, out_dtype, parts, mask, st); break;
+            case 2048: e = launch_iht_wide<11>(d, rows, cols, had_block, out, out_dtype, parts, mask, st); break;
+            default: e = launch_iht_wide<12>(d, rows, cols, had_block, out, out_dtype, parts, mask, st); break;
         }
         return e == cudaSuccess ? QUEST_OK : cuda_fail(e);
     }
-    return launch_hadamard_rows(d, QUEST_F32, cols, rows, cols, had_block, out, out_dtype, ld, st);
+    return launch_iht_rows(d, rows, cols, had_block, out, out_dtype, parts, mask, st);
 }
-
-}  // namespace
-
-// Orthonormal block Hadamard transform (its own inverse) of every row: in [rows x cols] with row
-// stride ld_in (16-byte aligned rows), out with row stride ld; cols % 32 == 0.
-int launch_hadamard_rows(const void *in, int in_dtype, int64_t ld_in, int64_t rows, int64_t cols, int had_block,
-                         void *out, int out_dtype, int64_t ld, cudaStream_t st) {
-    if (rows == 0) return QUEST_OK;
-    const int T = (int)(cols / 32);
-    int S;
-    if (T < 32) { S = 1; while (S < T) S <<= 1; } else { S = (T + 31) / 32 * 32; }
-    const int R = S <= 128 ? 128 / S : 1;      // CTAs of 128 threads where a row fits
-    const int threads = R * S;
-    const size_t smem = had_block >= 2048 ? sizeof(float) * 32 * (size_t)threads : 0;
-    if (smem > 48 * 1024) {
-        static DynamicSmemOnce smem_attr;
-        cudaError_t e = smem_attr.set(iht_rows_kernel, 72 * 1024);
-        if (e != cudaSuccess) return cuda_fail(e);
-    }
-    const long long grid = (rows + R - 1) / R;
-    cudaError_t e = launch_pdl(iht_rows_kernel, dim3((unsigned)grid), dim3(threads), smem, st, 1, in, in_dtype, (long long)ld_in,
-                               (long long)rows, (int)cols, had_block, 1.0f / sqrtf((float)had_block), out, out_dtype,
-                               (long long)ld, S, R);
-    return e == cudaSuccess ? QUEST_OK : cuda_fail(e);
-}
-
-namespace {
 
 bool bwd_shape_ok(int64_t M, int64_t N, int64_t K) {
     return M > 0 && N > 0 && K >= 32 && K % 32 == 0 && K <= 16384 && M % 8 == 0 && N % 8 == 0 &&
@@ -476,25 +508,22 @@ extern "C" int quest_linear_bwd(const void *dy, int64_t M, int64_t N, int64_t K,
     // blocks of up to 128 in rows of whole 128-column groups: the inverse transform runs in the contraction's epilogue,
     // the masked product never reaches memory
     const bool fuse = had_block <= 128 && K % 128 == 0;
-    if (dx) {
+    // one gradient: masked product of a and b (see launch_gemm_bf16_masked), then the inverse transform
+    const int64_t rows_free = (int64_t)(((uint8_t *)workspace + ws.bytes - (uint8_t *)ws.d1) / (K * 4));
+    auto gradient = [&](const void *a, const void *b, int64_t I, int64_t Kc, const uint8_t *mask, void *out, float *d, int opl) {
         Stage gemm_stage(QUEST_STAGE_GEMM, st);
-        // activation gradient of Algorithm 2 with its trust mask: d1[m][k] = M_x[m][k] * sum_n dy[m][n] wq_h[n][k]
-        if (fuse) {
-            if ((s = launch_gemm_bf16_masked(dy, ws.wh, M, K, N, mx, dx, out_dtype, had_block, 1, st))) return s;
-        } else {
-            if ((s = launch_gemm_bf16_masked(dy, ws.wh, M, K, N, mx, ws.d1, QUEST_F32, 0, 1, st))) return s;
-            if ((s = launch_iht(ws.d1, M, K, had_block, dx, out_dtype, K, st))) return s;
+        const int parts = divide_contraction(I, K, Kc, rows_free);
+        if (parts > 1) {                                     // the products run one after the other: both may use d1 and d2
+            const int e = launch_gemm_bf16_parts(a, b, I, K, Kc, ws.d1, parts, opl, st);
+            return e ? e : launch_iht(ws.d1, I, K, had_block, out, out_dtype, parts, mask, st);
         }
-    }
-    if (dw) {
-        Stage gemm_stage(QUEST_STAGE_GEMM, st);
-        // weight gradient of Algorithm 2 with its trust mask: d2[n][k] = M_w[n][k] * sum_m dy[m][n] xq_h[m][k]
-        if (fuse) {
-            if ((s = launch_gemm_bf16_masked(dy, ws.xh, N, K, M, mw, dw, out_dtype, had_block, 2, st))) return s;
-        } else {
-            if ((s = launch_gemm_bf16_masked(dy, ws.xh, N, K, M, mw, ws.d2, QUEST_F32, 0, 2, st))) return s;
-            if ((s = launch_iht(ws.d2, N, K, had_block, dw, out_dtype, K, st))) return s;
-        }
-    }
+        if (fuse) return launch_gemm_bf16_masked(a, b, I, K, Kc, mask, out, out_dtype, had_block, opl, st);
+        const int e = launch_gemm_bf16_masked(a, b, I, K, Kc, mask, d, QUEST_F32, 0, opl, st);
+        return e ? e : launch_iht(d, I, K, had_block, out, out_dtype, 1, nullptr, st);
+    };
+    // activation gradient of Algorithm 2 with its trust mask: d1[m][k] = M_x[m][k] * sum_n dy[m][n] wq_h[n][k]
+    if (dx && (s = gradient(dy, ws.wh, M, N, mx, dx, ws.d1, 1))) return s;
+    // weight gradient of Algorithm 2 with its trust mask: d2[n][k] = M_w[n][k] * sum_m dy[m][n] xq_h[m][k]
+    if (dw && (s = gradient(dy, ws.xh, N, M, mw, dw, ws.d2, 2))) return s;
     return QUEST_OK;
 }

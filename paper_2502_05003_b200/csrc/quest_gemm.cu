@@ -77,6 +77,8 @@ struct GemmParams {
     // index the gate rows, sw2 the up rows (rs_b is one array over all rows of B)
     const float *sw2;
     int up_row0;
+    // divided contraction (MODE 7): parts, k-blocks per part, rows between the parts of the output
+    int parts = 1, part_kb = 0, part_rows = 0;
     // fused inverse transform (MODE 6): block size, at most 128, and 1 / sqrt of it
     int iht_g = 0;
     float iht_scale = 0.0f;
@@ -315,7 +317,8 @@ struct SmemLayout {
 // transaction) instead of per-thread 16-byte stores, which write every 32-byte sector twice.
 // MODE 0: int8 operands, scaled output.  MODE 1: int8 operands with the exact correction for 8-bit
 // codes.  MODE 2 (backward pass, Algorithm 2): bfloat16 operands (kind::f16, binary32 accumulators);
-// the epilogue zeroes the elements the trust mask rejects and stores binary32.  MODE 3: MODE 2 plus
+// the epilogue zeroes the elements the trust mask rejects and stores binary32.  MODE 7: the contraction index is divided
+// into parts, every tile computes one part of its sum and stores the bare binary32 accumulators (see divide_contraction).  MODE 3: MODE 2 plus
 // the inverse Hadamard transform for blocks of 128 fused into the epilogue (the 128 columns a
 // thread holds are exactly one block), output in the caller's type.  MODE 6: the same for smaller blocks
 // (several to a thread); an instantiation of its own because the branches around the stages that a smaller block does
@@ -344,7 +347,8 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                const __grid_constant__ CUtensorMap tmY, GemmParams p) {
     using L = SmemLayout<BN, MODE == 1>;
     constexpr bool CORR = MODE == 1;
-    constexpr bool BWD = MODE == 2 || MODE == 3 || MODE == 6;
+    constexpr bool PART = MODE == 7;
+    constexpr bool BWD = MODE == 2 || MODE == 3 || MODE == 6 || PART;
     constexpr bool F16 = MODE >= 2;               // bfloat16 operands, binary32 accumulators
     constexpr bool WO = MODE == 4;
     constexpr bool MX = MODE == 5;
@@ -458,7 +462,8 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
     const int num_m = (p.M + TILE_M - 1) / TILE_M;
     const int num_n = (p.N + BN_OUT - 1) / BN_OUT;
-    const int num_tiles = num_m * num_n;
+    const int tiles_mn = num_m * num_n;
+    const int num_tiles = PART ? tiles_mn * p.parts : tiles_mn;
     const int num_kb = (p.K + BK - 1) / BK;
     // SHORT, leaving: a CTA must stay until its peer can no longer signal its barriers or read its shared and tensor
     // memory.  An epilogue warp arrives at the cluster barrier right after handing back its last accumulator buffer
@@ -472,11 +477,13 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             bool ok = true;
             for (int tile = unit; tile < num_tiles && ok; tile += num_units) {
                 int tm, tn;
-                tile_coords(tile, num_m, num_n, tm, tn);
+                const int part = PART ? tile / tiles_mn : 0;
+                tile_coords(PART ? tile - part * tiles_mn : tile, num_m, num_n, tm, tn);
+                const int kb0 = PART ? part * p.part_kb : 0, kb1 = PART ? min(num_kb, kb0 + p.part_kb) : num_kb;
                 const int m0 = tm * TILE_M + (int)rank * BM;                     // this CTA's rows of A
                 // this CTA's rows of B (SwiGLU pair: the leader stages the gate rows, its peer the up rows)
                 const int n0 = SWIGLU ? tn * BN_OUT + (int)rank * p.up_row0 : tn * BN + (int)rank * L::B_ROWS;
-                for (int kb = 0; kb < num_kb; ++kb) {
+                for (int kb = kb0; kb < kb1; ++kb) {
                     ok = mbar_wait(smem_u32(&empty_bar[stage]), phase ^ 1u, abort_flag, p.status, ST_PRODUCER);
                     if (!ok) break;
                     const uint32_t fb = smem_u32(&full_bar[stage]);
@@ -529,7 +536,8 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * BN);
-                for (int kb = 0; kb < num_kb; ++kb) {
+                const int kb0 = PART ? tile / tiles_mn * p.part_kb : 0, kb1 = PART ? min(num_kb, kb0 + p.part_kb) : num_kb;
+                for (int kb = kb0; kb < kb1; ++kb) {
                     ok = mbar_wait(smem_u32(&full_bar[stage]), phase, abort_flag, p.status, ST_MMA);
                     if (!ok) break;
                     tc_fence_after();
@@ -542,7 +550,7 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                         // MN-major 16 k = two 1024-byte atoms further (+128)
                         const uint64_t ad = a_desc + (uint64_t)(kk * (AMN ? 128 : (UMMA_K >> 4)));
                         const uint64_t bd = b_desc + (uint64_t)(kk * (BMN ? 128 : (UMMA_K >> 4)));
-                        const uint32_t accum = (kb | kk) != 0 ? 1u : 0u;
+                        const uint32_t accum = kb != kb0 || kk != 0 ? 1u : 0u;
                         if constexpr (MX) {       // 32 bytes of K = 64 E2M1 per instruction
                             umma_mxf4_pair(d_tmem, ad, bd, idesc, accum, tmem_base + SF_COL, tmem_base + SF_COL + 16);
                         } else if constexpr (F16) {      // 32 bytes of K = 16 bfloat16 per instruction
@@ -578,8 +586,9 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         int slab_count = 0;                            // slabs this warp has handed to TMA
         for (int tile = unit + t * num_units; tile < num_tiles && ok; tile += TILE_STEP * num_units, t += TILE_STEP) {
             int tm, tn;
-            tile_coords(tile, num_m, num_n, tm, tn);
-            const int m0 = tm * TILE_M + (int)rank * BM;
+            const int part = PART ? tile / tiles_mn : 0;
+            tile_coords(PART ? tile - part * tiles_mn : tile, num_m, num_n, tm, tn);
+            const int m0 = tm * TILE_M + (int)rank * BM + (PART ? part * p.part_rows : 0);
             const int n0 = tn * BN_OUT;
             const int buf = NBUF == 2 ? (t & 1) : 0;
             const uint32_t bphase = (uint32_t)(NBUF == 2 ? (t >> 1) : t) & 1u;
@@ -767,8 +776,8 @@ gemm_i8_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 if (col0 < p.N) {                      // uniform across the warp
                     const bool full = col0 + 32 <= p.N;
                     uint32_t *rc = &r[c0];
-                    if constexpr (IHT128) {
-                        // already masked and transformed above
+                    if constexpr (IHT128 || PART) {
+                        // already masked and transformed above, or left to the kernel that adds the parts
                     } else if constexpr (BWD) {
                         // trust estimator: keep the gradient only where the forward mask trusts the element
                         const uint32_t mbits = row_ok ? __ldg(reinterpret_cast<const uint32_t *>(
@@ -1214,7 +1223,7 @@ int launch_gemm_bn(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtenso
         if (e != cudaSuccess) return cuda_fail(e);
     }
     const int bn_out = SWIGLU ? BN / 2 : BN;
-    const int tiles = ((p.M + 2 * BM - 1) / (2 * BM)) * ((p.N + bn_out - 1) / bn_out);
+    const int tiles = ((p.M + 2 * BM - 1) / (2 * BM)) * ((p.N + bn_out - 1) / bn_out) * p.parts;
     const int pairs = std::min(tiles, num_sms() / 2);
     cudaError_t e = launch_pdl(gemm_i8_kernel<BN, MODE, YT, OPL, SWIGLU, SHORT>, dim3((unsigned)(2 * pairs)), dim3(NUM_THREADS),
                                (size_t)L::TOTAL, st, 2, tmA, tmB, tmY, p);
@@ -1433,6 +1442,43 @@ int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, 
     if (out_dtype != QUEST_F32) return QUEST_ERR_DTYPE;
     return QUEST_GEMM_BWD(2);
 #undef QUEST_GEMM_BWD
+}
+
+// Parts into which the contraction of a gradient product is divided so that a small output with a long sum does not leave
+// most pairs idle: 1 where it would not pay.  A k-block of the 256 x 128 tiles takes about 0.19 us; adding the parts costs a
+// launch and reads them back from L2, about 2.5 us and a microsecond for 3 MB.  `rows_free`: rows of J binary32 numbers
+// that the parts may take, each of them whole tiles high.
+int divide_contraction(int64_t I, int64_t J, int64_t Kc, int64_t rows_free) {
+    const int64_t pairs = num_sms() / 2, tall = (I + 255) / 256, tiles = tall * ((J + 127) / 128), kb = (2 * Kc + BK - 1) / BK;
+    int64_t parts = pairs / tiles;
+    if (parts > kb / 4) parts = kb / 4;
+    if (parts > rows_free / (tall * 256)) parts = rows_free / (tall * 256);
+    if (parts < 2) return 1;
+    const int64_t per = (kb + parts - 1) / parts;
+    parts = (kb + per - 1) / per;
+    const double gain = 0.19 * (double)(kb - per), cost = 2.5 + (double)(parts * I * J * 4) / 3e6;
+    return gain > cost + 1.0 ? (int)parts : 1;
+}
+
+// The parts of such a product: part q, [tall * 256 x J] binary32 from row q * tall * 256 of `out`, without mask and transform.
+int launch_gemm_bf16_parts(const void *a, const void *b, int64_t I, int64_t J, int64_t Kc, float *out, int parts, int opl,
+                           cudaStream_t st) {
+    GemmParams p = {};
+    const int64_t tall = (I + 255) / 256 * 256;
+    p.M = (int)I; p.N = (int)J; p.K = (int)(2 * Kc);
+    p.mul = 1;
+    p.y = out; p.y_dtype = QUEST_F32; p.ldy = J;
+    p.parts = parts; p.part_kb = ((p.K + BK - 1) / BK + parts - 1) / parts; p.part_rows = (int)tall;
+    p.status = device_status_word();
+    if (!p.status) return QUEST_ERR_CUDA;
+    CUtensorMap tmA, tmB, tmY;
+    int s;
+    if (opl == 2) s = make_operand_map(&tmA, reinterpret_cast<const int8_t *>(a), Kc, 2 * I, 64);
+    else s = make_operand_map(&tmA, reinterpret_cast<const int8_t *>(a), I, 2 * Kc, BM);
+    if (s) return s;
+    if ((s = make_operand_map(&tmB, reinterpret_cast<const int8_t *>(b), Kc, 2 * J, 64))) return s;
+    if ((s = make_output_map(&tmY, out, parts * tall, J * 4, J * 4))) return s;
+    return opl == 2 ? launch_gemm_bn<128, 7, true, 2>(tmA, tmB, tmY, p, st) : launch_gemm_bn<128, 7, true, 1>(tmA, tmB, tmY, p, st);
 }
 
 // Contraction of E2M1 nibble operands xq [M x K/2], wq [N x K/2] on the FP4 tensor-core path:

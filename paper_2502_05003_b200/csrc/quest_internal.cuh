@@ -184,14 +184,17 @@ void stage_end(void *scope);
 int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, int64_t Kc,
                             const uint8_t *mask, void *out, int out_dtype, int fuse_iht, int opl, cudaStream_t st);
 
+// The same product in `parts` parts of the contraction index (divide_contraction says how many): bare binary32 sums, part q
+// from row q * ((I + 255) / 256 * 256) of `out`.
+int divide_contraction(int64_t I, int64_t J, int64_t Kc, int64_t rows_free);
+int launch_gemm_bf16_parts(const void *a, const void *b, int64_t I, int64_t J, int64_t Kc, float *out, int parts, int opl,
+                           cudaStream_t st);
+
 // Contraction of E2M1 nibble operands (tcgen05 kind::mxf4, unit block scales): acc = acc_mul * sum v_x v_w
 // (int32, exact), y = sx sw sum v_x v_w.  xq, wq 16-byte aligned, K % 32 == 0.  Serves the FP4 grid
 // (acc_mul = 4) and, inside launch_gemm, the one- and two-bit uniform grids (acc_mul = 1).
 int launch_gemm_e2m1(const uint8_t *xq, const uint8_t *wq, const float *sx, const float *sw, int64_t M, int64_t N,
                      int64_t K, void *y, int y_dtype, int64_t ldy, int32_t *acc, int acc_mul, cudaStream_t st);
-// Orthonormal block Hadamard transform of every row (binary32 or bfloat16 in, binary32 or bfloat16 out).
-int launch_hadamard_rows(const void *in, int in_dtype, int64_t ld_in, int64_t rows, int64_t cols, int had_block,
-                         void *out, int out_dtype, int64_t ld, cudaStream_t st);
 // Weight-only contraction: y[m][n] = sw[n] * sum_k a[m][k] b[n][k], bfloat16 operands (dense, K contiguous),
 // binary32 accumulation.
 int launch_gemm_bf16_scaled(const void *a, const void *b, const float *sw, int64_t M, int64_t N, int64_t K,

@@ -113,6 +113,15 @@ def test_hadamard_block_sizes(g):
     run_case(gauss(200, 2048, 5), gauss(256, 2048, 6, 0.02), 4, g, seed=g)
 
 
+@pytest.mark.parametrize("M,N,K,g", [(2048, 64, 128, 128),      # small outputs of long sums: the contraction runs in parts
+                                     (4104, 72, 160, 32),       # a k-block that is nearly empty, half a tile of columns
+                                     (40, 4096, 512, 512), (72, 3000, 96, 1), (4096, 264, 256, 256), (4104, 520, 768, 256),
+                                     (2304, 136, 2048, 2048), (1800, 16, 4096, 4096), (1800, 24, 8192, 8192)])
+@pytest.mark.parametrize("out_dtype", [torch.float32, torch.bfloat16])
+def test_small_outputs_of_long_sums(M, N, K, g, out_dtype):
+    run_case(gauss(M, K, 41), gauss(N, K, 42, 0.02), 4, g, seed=M + K, out_dtype=out_dtype)
+
+
 @pytest.mark.parametrize("M,N,K,g", [(40, 24, 768, 256),        # eight rows per CTA of the transform, four slots of padding
                                      (24, 136, 2560, 512),      # one row per CTA, 40 of 64 threads
                                      (136, 8, 3072, 1024), (48, 40, 6144, 2048), (8, 72, 4096, 4096), (24, 16, 8192, 4096)])
