@@ -74,6 +74,46 @@ __device__ __forceinline__ void pdl_begin() {
     if (HOLD) pdl_launch_dependents();
 }
 
+// 32 bytes in one access of a thread (both ends 32-byte aligned).  Threads that own 32 or 64 consecutive bytes touch whole
+// sectors this way; with 16-byte accesses every sector is touched twice.
+__device__ __forceinline__ void load32B(const void *p, uint32_t *w) {
+    asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                 : "l"(p));
+}
+__device__ __forceinline__ void store32B(void *p, const uint32_t *w) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
+}
+__device__ __forceinline__ bool aligned32B(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 31) == 0; }
+// N words (a multiple of 8) from or to a pointer that is only known to be 16-byte aligned.
+template <int N>
+__device__ __forceinline__ void load_words(const void *p, uint32_t (&w)[N]) {
+    const uint8_t *b = reinterpret_cast<const uint8_t *>(p);
+    if (aligned32B(p)) {
+#pragma unroll
+        for (int i = 0; i < N; i += 8) load32B(b + 4 * i, &w[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(b + 4 * i));
+            w[i] = v.x; w[i + 1] = v.y; w[i + 2] = v.z; w[i + 3] = v.w;
+        }
+    }
+}
+template <int N>
+__device__ __forceinline__ void store_words(void *p, const uint32_t (&w)[N]) {
+    uint8_t *b = reinterpret_cast<uint8_t *>(p);
+    if (aligned32B(p)) {
+#pragma unroll
+        for (int i = 0; i < N; i += 8) store32B(b + 4 * i, &w[i]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; i += 4) *reinterpret_cast<uint4 *>(b + 4 * i) = make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]);
+    }
+}
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                               int cluster_x, Args &&...args) {

@@ -365,17 +365,17 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
         if (tn.rot) {                                           // uniform over the CTA
             if (active) {
                 const float2 ig = make_float2(a.inv_sqrt_g, a.inv_sqrt_g);
-                uint4 *dst = reinterpret_cast<uint4 *>(tn.rot + row * (long long)cols + (long long)tr * E);
+                uint8_t *dst = reinterpret_cast<uint8_t *>(tn.rot + row * (long long)cols + (long long)tr * E);
 #pragma unroll
-                for (int q = 0; q < E / 8; ++q) {
-                    uint32_t o[4];
+                for (int q = 0; q < E / 16; ++q) {
+                    uint32_t o[8];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float2 p = __fmul2_rn(v[q * 4 + j], ig);
+                    for (int j = 0; j < 8; ++j) {
+                        const float2 p = __fmul2_rn(v[q * 8 + j], ig);
                         const __nv_bfloat162 h = __floats2bfloat162_rn(p.x, p.y);
                         o[j] = *reinterpret_cast<const uint32_t *>(&h);
                     }
-                    dst[q] = make_uint4(o[0], o[1], o[2], o[3]);
+                    store_words(dst + q * 32, o);
                 }
             }
             if (!tn.codes && !tn.scales && !tn.mask && !tn.op8 && !tn.rowsum && !tn.cbf) return;   // nothing else asked for
@@ -498,8 +498,7 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
             if (!OPT || tn.codes) {
                 uint8_t *dst = tn.codes + row * (long long)(cols * CB / 8) + ((long long)tr * (E / 32) + g32) * (4 * CB);
                 if constexpr (CB == 8) {
-                    reinterpret_cast<uint4 *>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-                    reinterpret_cast<uint4 *>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+                    store_words(dst, w);
                 } else if constexpr (CB == 4) {
                     reinterpret_cast<uint4 *>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
                 } else if constexpr (CB == 2) {
@@ -512,19 +511,19 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                 if (tn.cbf) {                                   // uniform over the CTA
                     // a small integer as bfloat16 is the upper half of its binary32 pattern (|c| <= 255: exact)
                     const int L1 = (1 << a.bits) - 1;
-                    uint4 *dst = reinterpret_cast<uint4 *>(tn.cbf + row * (long long)cols + (long long)tr * E + g32 * 32);
+                    uint8_t *dst = reinterpret_cast<uint8_t *>(tn.cbf + row * (long long)cols + (long long)tr * E + g32 * 32);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        uint32_t o[4];
+                    for (int q = 0; q < 2; ++q) {
+                        uint32_t o[8];
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const int e0 = 8 * q + 2 * j, e1 = e0 + 1;
+                        for (int j = 0; j < 8; ++j) {
+                            const int e0 = 16 * q + 2 * j, e1 = e0 + 1;
                             const int k0 = (int)((w[e0 / PER] >> ((e0 % PER) * CB)) & ((1u << CB) - 1u));
                             const int k1 = (int)((w[e1 / PER] >> ((e1 % PER) * CB)) & ((1u << CB) - 1u));
                             o[j] = (__float_as_uint((float)(2 * k0 - L1)) >> 16) |
                                    (__float_as_uint((float)(2 * k1 - L1)) & 0xFFFF0000u);
                         }
-                        dst[q] = make_uint4(o[0], o[1], o[2], o[3]);
+                        store_words(dst + q * 32, o);
                     }
                 }
             }
@@ -534,9 +533,7 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                 if (DECODE && tn.op8) {                         // uniform over the CTA; the decoding kernel multiplies bytes
                     uint32_t o[8];
                     operand_from_code_words<CB>(w, a.bits, o);
-                    uint4 *dst = reinterpret_cast<uint4 *>(tn.op8 + row * (long long)cols + (long long)tr * E + g32 * 32);
-                    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-                    dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+                    store32B(tn.op8 + row * (long long)cols + (long long)tr * E + g32 * 32, o);
                 } else if (tn.op8) {
                     uint32_t o[4];
                     e2m1_operand_from_code_words<CB>(w, o);
@@ -546,9 +543,7 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
             } else if (tn.op8) {
                 uint32_t o[8];
                 operand_from_code_words<CB>(w, a.bits, o);
-                uint4 *dst = reinterpret_cast<uint4 *>(tn.op8 + row * (long long)cols + (long long)tr * E + g32 * 32);
-                dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-                dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+                store32B(tn.op8 + row * (long long)cols + (long long)tr * E + g32 * 32, o);
                 if ((RS || !FAST) && tn.rowsum) {
 #pragma unroll
                     for (int q = 0; q < 8; ++q) rsum += sum_bytes_s8(o[q]);
@@ -594,23 +589,15 @@ quantize_rows_kernel(const __grid_constant__ QuantArgs a) {
     float2 v[H];
     if (active) {
         if (BF16) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(tn.x) + row * tn.ld + (long long)tr * E);
+            uint32_t w[H];
+            load_words(reinterpret_cast<const uint16_t *>(tn.x) + row * tn.ld + (long long)tr * E, w);
 #pragma unroll
-            for (int q = 0; q < E / 8; ++q) {
-                const uint4 w = __ldg(src + q);
-                const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    v[q * 4 + j] = make_float2(__uint_as_float(ww[j] << 16), __uint_as_float(ww[j] & 0xFFFF0000u));
-            }
+            for (int i = 0; i < H; ++i) v[i] = make_float2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u));
         } else {
-            const float4 *src = reinterpret_cast<const float4 *>(reinterpret_cast<const float *>(tn.x) + row * tn.ld + (long long)tr * E);
+            uint32_t w[E];
+            load_words(reinterpret_cast<const float *>(tn.x) + row * tn.ld + (long long)tr * E, w);
 #pragma unroll
-            for (int q = 0; q < E / 4; ++q) {
-                const float4 w = __ldg(src + q);
-                v[q * 2] = make_float2(w.x, w.y);
-                v[q * 2 + 1] = make_float2(w.z, w.w);
-            }
+            for (int i = 0; i < H; ++i) v[i] = make_float2(__uint_as_float(w[2 * i]), __uint_as_float(w[2 * i + 1]));
         }
     } else {
 #pragma unroll
@@ -1041,15 +1028,10 @@ quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
     const bool active = row < tn.rows && tr < (cols >> 5);     // slots past the row end hold zeros
     float2 v[16];
     if (active) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(reinterpret_cast<const uint16_t *>(tn.x) + row * tn.ld + (long long)tr * 32);
+        uint32_t w[16];
+        load_words(reinterpret_cast<const uint16_t *>(tn.x) + row * tn.ld + (long long)tr * 32, w);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint4 w = __ldg(src + q);
-            const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                v[q * 4 + j] = make_float2(__uint_as_float(ww[j] << 16), __uint_as_float(ww[j] & 0xFFFF0000u));
-        }
+        for (int i = 0; i < 16; ++i) v[i] = make_float2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u));
     } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = make_float2(0.0f, 0.0f);
