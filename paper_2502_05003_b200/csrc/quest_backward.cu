@@ -114,22 +114,22 @@ iht_rows_kernel(const float *__restrict__ d, long long rows, int cols, int had_b
     const bool active = row < rows && tr < cols / 32;
     float v[32];
     if (active) {
-        const float4 *src = reinterpret_cast<const float4 *>(d + row * cols + (long long)tr * 32);
+        // d is in the workspace (256-byte aligned), rows are multiples of 128 bytes
+        const float *src = d + row * cols + (long long)tr * 32;
+        uint32_t w[32];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const float4 w = __ldg(src + q);
-            v[4 * q] = w.x; v[4 * q + 1] = w.y; v[4 * q + 2] = w.z; v[4 * q + 3] = w.w;
-        }
+        for (int q = 0; q < 4; ++q) load32B(src + 8 * q, &w[8 * q]);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(w[i]);
         if constexpr (PARTS) {
             const uint32_t keep = __ldg(reinterpret_cast<const uint32_t *>(mask + row * (cols >> 3)) + tr);
 #pragma unroll 2
             for (int q2 = 1; q2 < parts; ++q2) {
-                src += part_stride / 4;
+                src += part_stride;
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const float4 w = __ldg(src + q);
-                    v[4 * q] += w.x; v[4 * q + 1] += w.y; v[4 * q + 2] += w.z; v[4 * q + 3] += w.w;
-                }
+                for (int q = 0; q < 4; ++q) load32B(src + 8 * q, &w[8 * q]);
+#pragma unroll
+                for (int i = 0; i < 32; ++i) v[i] += __uint_as_float(w[i]);
             }
 #pragma unroll
             for (int i = 0; i < 32; ++i) v[i] = (keep >> i) & 1u ? v[i] : 0.0f;
@@ -174,22 +174,16 @@ iht_rows_kernel(const float *__restrict__ d, long long rows, int cols, int had_b
     }
     if (!active) return;
     if (out_dtype == QUEST_F32) {
-        float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(out) + row * cols + (long long)tr * 32);
+        uint32_t w[32];
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-            dst[q] = make_float4(v[4 * q] * inv_sqrt_g, v[4 * q + 1] * inv_sqrt_g, v[4 * q + 2] * inv_sqrt_g,
-                                 v[4 * q + 3] * inv_sqrt_g);
+        for (int i = 0; i < 32; ++i) w[i] = __float_as_uint(v[i] * inv_sqrt_g);
+        store_words(reinterpret_cast<float *>(out) + row * cols + (long long)tr * 32, w);
     } else {
-        uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<uint16_t *>(out) + row * cols + (long long)tr * 32);
+        uint32_t w[16];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uint32_t w[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                w[j] = (uint32_t)bf16_bits(v[8 * q + 2 * j] * inv_sqrt_g) |
-                       ((uint32_t)bf16_bits(v[8 * q + 2 * j + 1] * inv_sqrt_g) << 16);
-            dst[q] = make_uint4(w[0], w[1], w[2], w[3]);
-        }
+        for (int i = 0; i < 16; ++i)
+            w[i] = (uint32_t)bf16_bits(v[2 * i] * inv_sqrt_g) | ((uint32_t)bf16_bits(v[2 * i + 1] * inv_sqrt_g) << 16);
+        store_words(reinterpret_cast<uint16_t *>(out) + row * cols + (long long)tr * 32, w);
     }
 }
 

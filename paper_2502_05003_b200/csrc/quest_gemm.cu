@@ -968,9 +968,7 @@ __global__ void unpack_codes_kernel(const uint8_t *__restrict__ codes, int bits,
         for (int i = 0; i < CB; ++i) w[i] = __ldg(src + i);
         uint32_t o[8];
         operand_from_code_words<CB>(w, bits, o);
-        uint4 *dst = reinterpret_cast<uint4 *>(out + g * 32);
-        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+        store32B(out + g * 32, o);                             // the workspace is 256-byte aligned
     }
 }
 
@@ -1007,9 +1005,7 @@ __device__ __forceinline__ void unpack_group(const uint8_t *codes, int bits, lon
     }
     uint32_t o[8];
     operand_from_code_words<CB>(w, bits, o);
-    uint4 *dst = reinterpret_cast<uint4 *>(out + g * 32);
-    dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
-    dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
+    store32B(out + g * 32, o);
 }
 __global__ void __launch_bounds__(128)
 unpack_pair_kernel(const uint8_t *__restrict__ codes_x, int bits_x, long long groups_x, uint8_t *__restrict__ out_x,

@@ -427,6 +427,8 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
     const float top = a.qc.top, hh = a.qc.h;
     int rsum = 0;
     if (active) {
+        // 64 elements: codes and mask of both halves leave together (halves of sectors, written twice, otherwise)
+        [[maybe_unused]] uint32_t mwords[E / 32], cwords[E == 64 ? 2 * CB : 1];
 #pragma unroll
         for (int g32 = 0; g32 < E / 32; ++g32) {
             uint32_t mbits = 0;
@@ -478,8 +480,11 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                 }
                 mbits = ~mbits;
             }
-            if (!OPT || tn.mask)
-                reinterpret_cast<uint32_t *>(tn.mask + row * (long long)(cols >> 3))[tr * (E / 32) + g32] = mbits;
+            if constexpr (E == 32) {
+                if (!OPT || tn.mask) reinterpret_cast<uint32_t *>(tn.mask + row * (long long)(cols >> 3))[tr] = mbits;
+            } else {
+                mwords[g32] = mbits;
+            }
             constexpr int PER = 32 / CB;
             if constexpr (!FAST && GRID != GRID_FP4) {
                 // pack 32/CB codes per word: sum_j (MAGIC_BITS + k_j) * 2^(CB*j), minus the constant part
@@ -495,17 +500,17 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                 }
             }
 
-            if (!OPT || tn.codes) {
-                uint8_t *dst = tn.codes + row * (long long)(cols * CB / 8) + ((long long)tr * (E / 32) + g32) * (4 * CB);
-                if constexpr (CB == 8) {
-                    store_words(dst, w);
-                } else if constexpr (CB == 4) {
-                    reinterpret_cast<uint4 *>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-                } else if constexpr (CB == 2) {
-                    reinterpret_cast<uint2 *>(dst)[0] = make_uint2(w[0], w[1]);
-                } else {
-                    reinterpret_cast<uint32_t *>(dst)[0] = w[0];
+            if constexpr (E == 32) {
+                if (!OPT || tn.codes) {
+                    uint8_t *dst = tn.codes + row * (long long)(cols * CB / 8) + (long long)tr * (4 * CB);
+                    if constexpr (CB == 8) store_words(dst, w);
+                    else if constexpr (CB == 4) *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+                    else if constexpr (CB == 2) *reinterpret_cast<uint2 *>(dst) = make_uint2(w[0], w[1]);
+                    else *reinterpret_cast<uint32_t *>(dst) = w[0];
                 }
+            } else {
+#pragma unroll
+                for (int q = 0; q < CB; ++q) cwords[g32 * CB + q] = w[q];
             }
             if constexpr (GRID == GRID_UNIFORM) {
                 if (tn.cbf) {                                   // uniform over the CTA
@@ -549,6 +554,38 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                     for (int q = 0; q < 8; ++q) rsum += sum_bytes_s8(o[q]);
                 }
             }
+            }
+        }
+        if constexpr (E == 64) {
+            if (!OPT || tn.mask) {
+                uint32_t *dst = reinterpret_cast<uint32_t *>(tn.mask + row * (long long)(cols >> 3)) + 2 * tr;
+                if ((reinterpret_cast<uintptr_t>(dst) & 7) == 0) {
+                    *reinterpret_cast<uint2 *>(dst) = make_uint2(mwords[0], mwords[1]);
+                } else {
+                    dst[0] = mwords[0];
+                    dst[1] = mwords[1];
+                }
+            }
+            if (!OPT || tn.codes) {                            // 8 CB bytes per thread
+                uint8_t *dst = tn.codes + row * (long long)(cols * CB / 8) + (long long)tr * (8 * CB);
+                if constexpr (CB >= 4) {
+                    store_words(dst, cwords);
+                } else {                                       // the weight-only layer takes codes at any multiple of four bytes
+                    const bool whole = (reinterpret_cast<uintptr_t>(dst) & (8 * CB - 1)) == 0;
+                    if constexpr (CB == 2) {
+                        if (whole) {
+                            *reinterpret_cast<uint4 *>(dst) = make_uint4(cwords[0], cwords[1], cwords[2], cwords[3]);
+                        } else {
+                            reinterpret_cast<uint2 *>(dst)[0] = make_uint2(cwords[0], cwords[1]);
+                            reinterpret_cast<uint2 *>(dst)[1] = make_uint2(cwords[2], cwords[3]);
+                        }
+                    } else if (whole) {
+                        *reinterpret_cast<uint2 *>(dst) = make_uint2(cwords[0], cwords[1]);
+                    } else {
+                        reinterpret_cast<uint32_t *>(dst)[0] = cwords[0];
+                        reinterpret_cast<uint32_t *>(dst)[1] = cwords[1];
+                    }
+                }
             }
         }
     }

@@ -69,6 +69,25 @@ def test_blocks_of_64(bits, cols, trust):
     check(x, bits, 64, trust)
 
 
+@pytest.mark.parametrize("bits", [1, 2, 4, 8])
+@pytest.mark.parametrize("g,cols,rows,bf16", [(128, 1024, 40, True), (32, 320, 40, True), (64, 192, 40, False), (256, 768, 40, False),
+                                              (2048, 2048, 2100, True), (1024, 2048, 2100, False)])
+def test_buffers_at_the_least_alignment(bits, g, cols, rows, bf16):
+    # rows at an odd multiple of 16 bytes, codes too, the mask at an odd multiple of 4: the wide accesses do not serve
+    import paper_2502_05003_b200 as quest
+    x_np = rows_of("student", rows, cols, bits + g, bf16)
+    ref = qo.quantize(x_np, bits, g, 1.0)
+    dt, off = (torch.bfloat16, 8) if bf16 else (torch.float32, 4)
+    x = torch.empty(rows * cols + off, dtype=dt, device="cuda")[off:].view(rows, cols)
+    x.copy_(to_dev(x_np))
+    nc = cols * quest.container_bits(bits) // 8
+    codes = torch.empty(rows * nc + 16, dtype=torch.uint8, device="cuda")[16:].view(rows, nc)
+    mask = torch.empty(rows * cols // 8 + 4, dtype=torch.uint8, device="cuda")[4:].view(rows, cols // 8)
+    assert x.data_ptr() % 32 == 16 and codes.data_ptr() % 32 == 16 and mask.data_ptr() % 8 == 4
+    quest.quest_quantize(x, bits, g, 1.0, codes=codes, mask=mask)
+    assert np.array_equal(codes.cpu().numpy(), ref["codes"]) and np.array_equal(mask.cpu().numpy(), ref["mask"])
+
+
 @pytest.mark.parametrize("bits", [1, 4, 8])
 @pytest.mark.parametrize("g,cols,rows,bf16", [(128, 1024, 1200, True), (64, 1344, 700, True), (32, 1024, 1000, True),
                                               (128, 512, 3600, True), (2048, 2048, 500, True), (4096, 4096, 590, False)])
