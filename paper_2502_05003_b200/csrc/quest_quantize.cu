@@ -275,14 +275,14 @@ __device__ __forceinline__ void project32_trusting(const float2 *v, float inv, c
 // applied by the caller), RMS, projection, trust test, packing and stores for the E elements this
 // thread holds.  GFULL: had_block >= E, so every in-register stage runs.  FAST: the common case
 // fixed at compile time -- had_block = 128 with the first stage already applied, rows of at least
-// one warp, codes, scales and mask requested (the GEMM operand and the bfloat16 outputs of the
+// one warp (SHORT_ROWS: of any length), codes, scales and mask requested (the GEMM operand and the bfloat16 outputs of the
 // weight-only variant are optional; a tensor may also ask for the rotation alone), no row sums,
 // trust_factor >= 1 -- so that no per-row loop and only a few uniform branches remain.
 // OPT: any of codes, scales and mask may be missing (FAST without OPT: all are there).
 // DECODE: the launch precedes the decoding kernel (see launch_quantize).
 // CS, CCOLS: threads per row and row length when the kernel is instantiated for one row length (0 = run-time values).
 template <int CB, int E, bool GFULL, bool FAST, int GRID = GRID_UNIFORM, bool XDONE = false, bool RS = false, int CS = 0, int CCOLS = 0,
-          bool OPT = !FAST, bool DECODE = false>
+          bool OPT = !FAST, bool DECODE = false, bool SHORT_ROWS = false>
 __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const QuantArgs &a, const QuantTensor &tn,
                                                      bool active, long long row, int tr, int r_local, float *xsm,
                                                      int s_start) {
@@ -397,10 +397,11 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
             for (int i = 0; i < n; ++i) q[i] = __fadd_rn(q[2 * i], q[2 * i + 1]);
         ss = q[0];
     }
-    const int lanes_per_row = (FAST || S >= 32) ? 32 : S;
+    const int lanes_per_row = ((FAST && !SHORT_ROWS) || S >= 32) ? 32 : S;
     if constexpr (FAST) {
 #pragma unroll
-        for (int m = 1; m < 32; m <<= 1) ss = __fadd_rn(ss, __shfl_xor_sync(0xffffffffu, ss, m));
+        for (int m = 1; m < 32; m <<= 1)
+            if (!SHORT_ROWS || m < lanes_per_row) ss = __fadd_rn(ss, __shfl_xor_sync(0xffffffffu, ss, m));
     } else {
         for (int m = 1; m < lanes_per_row; m <<= 1) ss = __fadd_rn(ss, __shfl_xor_sync(0xffffffffu, ss, m));
     }
@@ -1048,7 +1049,7 @@ static cudaError_t launch_wide(bool bf16, int cb, int grid, int threads, size_t 
 // their own with run-time row length (6144 x 2048, g = 64, every output, against the general kernel: 13.6 -> 11.9 us;
 // a whole layer of 777 x 2048 x 5504 without masks 21.8 -> 21.1 us).
 template <int CB, int GRID = GRID_UNIFORM, bool RS = false, int COLS = 0, int HB = 128, bool OPT = false,
-          bool DECODE = false, int REGS = 64>
+          bool DECODE = false, int REGS = 64, bool BF16 = true, bool SHORT_ROWS = false>
 __global__ void __maxnreg__(REGS)
 quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
     constexpr int CS = COLS / 32;
@@ -1065,10 +1066,17 @@ quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
     const bool active = row < tn.rows && tr < (cols >> 5);     // slots past the row end hold zeros
     float2 v[16];
     if (active) {
-        uint32_t w[16];
-        load_words(reinterpret_cast<const uint16_t *>(tn.x) + row * tn.ld + (long long)tr * 32, w);
+        if constexpr (BF16) {
+            uint32_t w[16];
+            load_words(reinterpret_cast<const uint16_t *>(tn.x) + row * tn.ld + (long long)tr * 32, w);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = make_float2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u));
+            for (int i = 0; i < 16; ++i) v[i] = make_float2(__uint_as_float(w[i] << 16), __uint_as_float(w[i] & 0xFFFF0000u));
+        } else {
+            uint32_t w[32];
+            load_words(reinterpret_cast<const float *>(tn.x) + row * tn.ld + (long long)tr * 32, w);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = make_float2(__uint_as_float(w[2 * i]), __uint_as_float(w[2 * i + 1]));
+        }
     } else {
 #pragma unroll
         for (int i = 0; i < 16; ++i) v[i] = make_float2(0.0f, 0.0f);
@@ -1084,7 +1092,7 @@ quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
             v[i] = __ffma2_rn(v[i], sgn, p);
         }
     }
-    rotate_project_store<CB, 32, true, true, GRID, false, RS, CS, COLS, OPT, DECODE>(v, a, tn, active, row, tr, r_local, xsm, 32);
+    rotate_project_store<CB, 32, true, true, GRID, false, RS, CS, COLS, OPT, DECODE, SHORT_ROWS>(v, a, tn, active, row, tr, r_local, xsm, 32);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1336,11 +1344,11 @@ static cudaError_t launch_block128(int cb, dim3 grid, int threads, size_t smem, 
     return launch_block128_ct<GRID, 0>(cb, grid, threads, smem, st, a);
 }
 
-template <int GRID, int COLS, int HB, bool OPT, bool DECODE = false, int REGS = 64>
+template <int GRID, int COLS, int HB, bool OPT, bool DECODE = false, int REGS = 64, bool BF16 = true, bool SHORT_ROWS = false>
 static cudaError_t launch_direct128_cols(int cb, dim3 grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                          bool rowsums) {
 #define QUEST_LAUNCH(CBV, RSV)                                                                              \
-    return launch_quantizer<quantize_direct128_kernel<CBV, GRID, RSV, COLS, HB, OPT, DECODE, REGS>>(grid, threads, smem, st, a)
+    return launch_quantizer<quantize_direct128_kernel<CBV, GRID, RSV, COLS, HB, OPT, DECODE, REGS, BF16, SHORT_ROWS>>(grid, threads, smem, st, a)
     smem = even_share_smem(grid.x, direct_threads(REGS) / threads, smem);
     if constexpr (GRID == GRID_FP4) {
         QUEST_LAUNCH(4, false);
@@ -1358,7 +1366,13 @@ static cudaError_t launch_direct128_cols(int cb, dim3 grid, int threads, size_t 
 
 template <int GRID>
 static cudaError_t launch_direct128(int cb, dim3 grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
-                                    bool rowsums, bool every_output, bool for_decode) {
+                                    bool rowsums, bool every_output, bool for_decode, bool bf16) {
+    if (!bf16)
+        return a.had_block == 64 ? launch_direct128_cols<GRID, 0, 64, true, false, 64, false, true>(cb, grid, threads, smem, st, a, rowsums)
+                                 : launch_direct128_cols<GRID, 0, 128, true, false, 64, false, true>(cb, grid, threads, smem, st, a, rowsums);
+    if (a.S < 32 && !for_decode)
+        return a.had_block == 64 ? launch_direct128_cols<GRID, 0, 64, true, false, 64, true, true>(cb, grid, threads, smem, st, a, rowsums)
+                                 : launch_direct128_cols<GRID, 0, 128, true, false, 64, true, true>(cb, grid, threads, smem, st, a, rowsums);
     if constexpr (GRID == GRID_UNIFORM) {
         if (for_decode)
             return a.had_block == 64 ? launch_direct128_cols<GRID, 0, 64, true, true>(cb, grid, threads, smem, st, a, rowsums)
@@ -1502,7 +1516,8 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
     if (cols % 32 == 0) {
         // 32 elements per thread (64 registers, twice the resident warps) for bfloat16 rows up to 8192 elements;
         // wider rows keep 64 per thread
-        const bool e32 = dtype == QUEST_BF16 && had_block >= 64 && cols <= 8192;
+        const bool direct_block = (had_block == 128 || had_block == 64) && trust_factor >= 1.0f;
+        const bool e32 = had_block >= 64 && cols <= 8192 && (dtype == QUEST_BF16 || (direct_block && !for_decode));
         // wide rotation blocks, 64 elements per thread: rows of whole spans, and enough of them that a CTA's latency (longer
         // than with 32 elements per thread: 3.5 against 2.9 us for 300 rows of 2048) does not show
         bool wide = had_block >= 256 && had_block <= 4096 && cols % 2048 == 0 && (had_block < 4096 || cols % 4096 == 0) &&
@@ -1551,7 +1566,7 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
             cudaError_t e;
             // the specialised tail (trust_factor >= 1): with codes, scales and masks requested (or the rotation alone), with
             // row sums besides, or with any of the outputs; the FP4 grid has no separate GEMM operand
-            const bool fast_tail_opt = trust_factor >= 1.0f && S >= 32;
+            const bool fast_tail_opt = trust_factor >= 1.0f && S >= 32, direct_rows = S >= 32 || !for_decode;
             bool every_output = true, any_rowsum = false;
             for (int j = 0; j < 2; ++j) {
                 const QuantTensor &t = a.t[j];
@@ -1583,11 +1598,12 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
                 else
                     e = fast_tail ? launch_wide32<GRID_UNIFORM, true>(cb, g, threads, smem2, st, a, exchange)
                                   : launch_wide32<GRID_UNIFORM, false>(cb, g, threads, smem2, st, a, exchange);
-            } else if (e32 && (had_block == 128 || had_block == 64) && fast_tail_opt && (!any_rowsum || (cb == 8 && grid_kind == GRID_UNIFORM)) &&
+            } else if (e32 && direct_block && direct_rows && (!any_rowsum || (cb == 8 && grid_kind == GRID_UNIFORM)) &&
                        threads <= 256) {
                 // the common case: direct loads, one CTA per row group
-                e = grid_kind == GRID_FP4 ? launch_direct128<GRID_FP4>(cb, grid, threads, smem, st, a, false, every_output, false)
-                                          : launch_direct128<GRID_UNIFORM>(cb, grid, threads, smem, st, a, any_rowsum, every_output, for_decode);
+                e = grid_kind == GRID_FP4 ? launch_direct128<GRID_FP4>(cb, grid, threads, smem, st, a, false, every_output, false, dtype == QUEST_BF16)
+                                          : launch_direct128<GRID_UNIFORM>(cb, grid, threads, smem, st, a, any_rowsum, every_output, for_decode,
+                                                                     dtype == QUEST_BF16);
             } else if (streaming) {
                 // rows wider than 8192: persistent streaming kernel, 64 elements per thread, as many CTAs as fit
                 const int exchange = (int)((smem + 15) / 16 * 16);

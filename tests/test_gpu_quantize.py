@@ -69,6 +69,17 @@ def test_blocks_of_64(bits, cols, trust):
     check(x, bits, 64, trust)
 
 
+@pytest.mark.parametrize("bits", [1, 2, 3, 4, 8])
+@pytest.mark.parametrize("g,cols", [(64, 64), (64, 192), (128, 128), (128, 384), (64, 448), (128, 896), (128, 2048), (64, 5504), (128, 8192),
+                                    (128, 8320)])
+@pytest.mark.parametrize("bf16,trust", [(False, 1.0), (False, 1.3), (False, 0.5), (True, 1.3)])
+def test_narrow_blocks_of_either_type(bits, g, cols, bf16, trust):
+    # rows of less than a warp, of one, of several; binary32 beside bfloat16
+    x = rows_of("outliers", 37, cols, bits + cols, bf16)
+    x[3] = 0
+    check(x, bits, g, trust, repeat=1)
+
+
 @pytest.mark.parametrize("bits", [1, 2, 4, 8])
 @pytest.mark.parametrize("g,cols,rows,bf16", [(128, 1024, 40, True), (32, 320, 40, True), (64, 192, 40, False), (256, 768, 40, False),
                                               (2048, 2048, 2100, True), (1024, 2048, 2100, False)])
