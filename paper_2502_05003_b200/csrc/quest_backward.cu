@@ -31,10 +31,10 @@ __device__ __forceinline__ uint16_t bf16_bits(float v) {
 
 // Packed level indices and per-row scales -> dequantised values bf16(scale[r] * c) [rows x K], dense, up to two
 // tensors per launch (CTAs from blocks0 on work on the second).  A CTA converts `rpb` whole rows, or (SPLIT)
-// `piece` octets of one row, gridDim.y of them: a few long rows would leave most SMs without a CTA.  Eight consecutive
-// elements (one 16-byte store; K % 32 == 0 keeps them in one row) per thread and step, four steps in flight.  Bound by
-// the writes (2 B/element) once the arithmetic is out of the way: the row of an octet comes from a multiplication
-// (`magic` = ceil(2^32 / octets), exact below 2^20 octets per CTA) instead of a 64-bit division, and 2k - (2^b - 1) from
+// `piece` units of one row, gridDim.y of them: a few long rows would leave most SMs without a CTA.  A unit is sixteen
+// consecutive elements (one 32-byte store; K % 32 == 0 keeps them in one row); two per thread and step are in flight.  Bound by
+// the writes (2 B/element) once the arithmetic is out of the way: the row of a unit comes from a multiplication
+// (`magic` = ceil(2^32 / units), exact below 2^20 units per CTA) instead of a 64-bit division, and 2k - (2^b - 1) from
 // a packed multiply-add on 2^22 + k (the level in the low bits) instead of integer conversions, both exact.
 // 4096 x 2048 + 2048 x 2048 elements at four bits: 10.4 -> 6.9 us.
 struct DequantTensor {
@@ -45,7 +45,7 @@ struct DequantTensor {
 };
 template <int CB, bool SPLIT>
 __global__ void __launch_bounds__(256)
-dequant_codes_kernel(DequantTensor t0, DequantTensor t1, int blocks0, int rpb, int piece, int octets, uint32_t magic, int bits) {
+dequant_codes_kernel(DequantTensor t0, DequantTensor t1, int blocks0, int rpb, int piece, int units, uint32_t magic, int bits) {
     pdl_launch_dependents();
     pdl_wait();
     const bool second = (int)blockIdx.x >= blocks0;
@@ -53,36 +53,39 @@ dequant_codes_kernel(DequantTensor t0, DequantTensor t1, int blocks0, int rpb, i
     const long long row0 = (long long)(second ? (int)blockIdx.x - blocks0 : (int)blockIdx.x) * rpb;
     const int rows_here = t.rows - row0 < rpb ? (int)(t.rows - row0) : rpb;
     const int begin = SPLIT ? (int)blockIdx.y * piece : 0;
-    const int n = SPLIT ? min(octets - begin, piece) : rows_here * octets;
-    const long long first = row0 * octets + begin;           // the CTA's first octet
+    const int n = SPLIT ? min(units - begin, piece) : rows_here * units;
+    const long long first = row0 * units + begin;            // the CTA's first unit
     const uint32_t *c32 = reinterpret_cast<const uint32_t *>(t.codes);
     const float off = -(8388608.0f + (float)((1 << bits) - 1));
     const float2 two = make_float2(2.0f, 2.0f), off2 = make_float2(off, off);
-    for (int i0 = threadIdx.x; i0 < n; i0 += 4 * 256) {
-        float sc[4];
-        uint32_t lo[4], hi[CB == 8 ? 4 : 1];                 // the 8 * CB bits of an octet's levels
+    constexpr int NW = CB >= 2 ? CB / 2 : 1;                 // words that hold the levels of a unit
+    for (int i0 = threadIdx.x; i0 < n; i0 += 2 * 256) {
+        float sc[2];
+        uint32_t lv[2][NW];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 2; ++u) {
             const int i = i0 + 256 * u;
             if (i < n) {
                 const long long o = first + i;
                 sc[u] = __ldg(t.scales + row0 + __umulhi((uint32_t)i, magic));
-                if constexpr (CB == 8) { lo[u] = __ldg(c32 + 2 * o); hi[u] = __ldg(c32 + 2 * o + 1); }
-                else if constexpr (CB == 4) lo[u] = __ldg(c32 + o);
-                else if constexpr (CB == 2) lo[u] = (__ldg(c32 + (o >> 1)) >> (16 * (int)(o & 1))) & 0xFFFFu;
-                else lo[u] = (__ldg(c32 + (o >> 2)) >> (8 * (int)(o & 3))) & 0xFFu;
+                if constexpr (CB == 1) {
+                    lv[u][0] = (__ldg(c32 + (o >> 1)) >> (16 * (int)(o & 1))) & 0xFFFFu;
+                } else {
+#pragma unroll
+                    for (int q = 0; q < NW; ++q) lv[u][q] = __ldg(c32 + NW * o + q);
+                }
             }
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 2; ++u) {
             const int i = i0 + 256 * u;
             if (i >= n) break;
             const float2 sc2 = make_float2(sc[u], sc[u]);
-            uint32_t r[4];
+            uint32_t r[8];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t w = CB == 8 && j >= 2 ? hi[CB == 8 ? u : 0] : lo[u];
-                const int s0 = CB == 8 ? 16 * (j & 1) : 2 * j * CB;
+            for (int j = 0; j < 8; ++j) {
+                const uint32_t w = lv[u][(2 * j * CB) / 32];
+                const int s0 = (2 * j * CB) % 32;
                 const uint32_t mask = ((1u << CB) - 1u) << 1;    // the level one bit up: 2^22 + k
                 const float2 k = make_float2(__uint_as_float(((s0 ? w >> (s0 - 1) : w << 1) & mask) | 0x4A800000u),
                                              __uint_as_float(((w >> (s0 + CB - 1)) & mask) | 0x4A800000u));
@@ -90,7 +93,7 @@ dequant_codes_kernel(DequantTensor t0, DequantTensor t1, int blocks0, int rpb, i
                 const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
                 r[j] = *reinterpret_cast<const uint32_t *>(&h);
             }
-            *reinterpret_cast<uint4 *>(t.out + (first + i) * 8) = make_uint4(r[0], r[1], r[2], r[3]);
+            store32B(t.out + (first + i) * 16, r);
         }
     }
 }
@@ -473,22 +476,22 @@ extern "C" int quest_linear_bwd(const void *dy, int64_t M, int64_t N, int64_t K,
         // both dequantised operands in one launch, then the two products back to back
         Stage prep(QUEST_STAGE_UNPACK, st);
         const DequantTensor tw = {wq, sw, ws.wh, dx ? (long long)N : 0}, tx = {xq, sx, ws.xh, dw ? (long long)M : 0};
-        const int octets = (int)(K / 8);                     // at most 2048
-        // about four octets per thread, fewer while that would leave an SM less than about eight CTAs (7016 x 512 + 768 x 512
-        // elements: 1.1 us slower with four than with fewer)
-        int per_cta = 1024;
-        while (per_cta > 256 && (tw.rows + tx.rows) * octets < 1184ll * per_cta) per_cta >>= 1;
-        const int rpb = (per_cta + octets - 1) / octets;
+        const int units = (int)(K / 16);                     // at most 1024
+        // about two units per thread, fewer while that would leave an SM less than about eight CTAs (7016 x 512 + 768 x 512
+        // elements: 1.1 us slower with two than with fewer)
+        int per_cta = 512;
+        while (per_cta > 128 && (tw.rows + tx.rows) * units < 1184ll * per_cta) per_cta >>= 1;
+        const int rpb = (per_cta + units - 1) / units;
         const int blocks0 = (int)((tw.rows + rpb - 1) / rpb);
         const int blocks = blocks0 + (int)((tx.rows + rpb - 1) / rpb);
         // rows shared by several CTAs only where there are fewer rows than two per SM (64 x 8192: 0.7 us; 1536 x 5504 would
         // take 2.9 us longer)
-        const int parts = rpb == 1 && blocks < 2 * num_sms() ? (octets + 255) / 256 : 1;
-        const int piece = (octets + parts - 1) / parts;
+        const int parts = rpb == 1 && blocks < 2 * num_sms() ? (units + 127) / 128 : 1;
+        const int piece = (units + parts - 1) / parts;
         const dim3 grid((unsigned)blocks, (unsigned)parts);
-        const uint32_t magic = (uint32_t)((((uint64_t)1 << 32) + octets - 1) / octets);
+        const uint32_t magic = (uint32_t)((((uint64_t)1 << 32) + units - 1) / units);
         auto dequant = [&](auto whole, auto split) {
-            return launch_pdl(parts > 1 ? split : whole, grid, dim3(256), 0, st, 1, tw, tx, blocks0, rpb, piece, octets, magic, bits);
+            return launch_pdl(parts > 1 ? split : whole, grid, dim3(256), 0, st, 1, tw, tx, blocks0, rpb, piece, units, magic, bits);
         };
         cudaError_t e;
         switch (container_bits(bits)) {
