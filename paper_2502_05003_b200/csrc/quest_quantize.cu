@@ -1045,7 +1045,7 @@ static cudaError_t launch_wide(bool bf16, int cb, int grid, int threads, size_t 
 // RS: the row sums of the 8-bit GEMM operand are wanted (kept out of the common instantiation).
 // COLS: the row length when it is one of the common ones (1024, 2048, 4096: threads per row, rows per CTA and every
 // row pitch become constants, worth 6 % of the kernel); 0 takes them from the arguments.
-// HB, OPT: blocks of 64 (stride 64 is left out) and launches that do not ask for every output take instantiations of
+// HB, OPT: blocks of 64 and 32 (the strides they do not have are left out) and launches that do not ask for every output take instantiations of
 // their own with run-time row length (6144 x 2048, g = 64, every output, against the general kernel: 13.6 -> 11.9 us;
 // a whole layer of 777 x 2048 x 5504 without masks 21.8 -> 21.1 us).
 template <int CB, int GRID = GRID_UNIFORM, bool RS = false, int COLS = 0, int HB = 128, bool OPT = false,
@@ -1092,7 +1092,7 @@ quantize_direct128_kernel(const __grid_constant__ QuantArgs a) {
             v[i] = __ffma2_rn(v[i], sgn, p);
         }
     }
-    rotate_project_store<CB, 32, true, true, GRID, false, RS, CS, COLS, OPT, DECODE, SHORT_ROWS>(v, a, tn, active, row, tr, r_local, xsm, 32);
+    rotate_project_store<CB, 32, true, true, GRID, HB == 32, RS, CS, COLS, OPT, DECODE, SHORT_ROWS>(v, a, tn, active, row, tr, r_local, xsm, 32);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1367,6 +1367,9 @@ static cudaError_t launch_direct128_cols(int cb, dim3 grid, int threads, size_t 
 template <int GRID>
 static cudaError_t launch_direct128(int cb, dim3 grid, int threads, size_t smem, cudaStream_t st, const QuantArgs &a,
                                     bool rowsums, bool every_output, bool for_decode, bool bf16) {
+    if (a.had_block == 32)
+        return bf16 ? launch_direct128_cols<GRID, 0, 32, true, false, 64, true, true>(cb, grid, threads, smem, st, a, rowsums)
+                    : launch_direct128_cols<GRID, 0, 32, true, false, 64, false, true>(cb, grid, threads, smem, st, a, rowsums);
     if (!bf16)
         return a.had_block == 64 ? launch_direct128_cols<GRID, 0, 64, true, false, 64, false, true>(cb, grid, threads, smem, st, a, rowsums)
                                  : launch_direct128_cols<GRID, 0, 128, true, false, 64, false, true>(cb, grid, threads, smem, st, a, rowsums);
@@ -1516,8 +1519,8 @@ int launch_quantize(const QuantJob *jobs, int njobs, int dtype, int64_t cols, in
     if (cols % 32 == 0) {
         // 32 elements per thread (64 registers, twice the resident warps) for bfloat16 rows up to 8192 elements;
         // wider rows keep 64 per thread
-        const bool direct_block = (had_block == 128 || had_block == 64) && trust_factor >= 1.0f;
-        const bool e32 = had_block >= 64 && cols <= 8192 && (dtype == QUEST_BF16 || (direct_block && !for_decode));
+        const bool direct_block = (had_block == 128 || had_block == 64 || (had_block == 32 && !for_decode)) && trust_factor >= 1.0f;
+        const bool e32 = cols <= 8192 && ((dtype == QUEST_BF16 && had_block >= 64) || (direct_block && !for_decode));
         // wide rotation blocks, 64 elements per thread: rows of whole spans, and enough of them that a CTA's latency (longer
         // than with 32 elements per thread: 3.5 against 2.9 us for 300 rows of 2048) does not show
         bool wide = had_block >= 256 && had_block <= 4096 && cols % 2048 == 0 && (had_block < 4096 || cols % 4096 == 0) &&

@@ -71,7 +71,7 @@ def test_blocks_of_64(bits, cols, trust):
 
 @pytest.mark.parametrize("bits", [1, 2, 3, 4, 8])
 @pytest.mark.parametrize("g,cols", [(64, 64), (64, 192), (128, 128), (128, 384), (64, 448), (128, 896), (128, 2048), (64, 5504), (128, 8192),
-                                    (128, 8320)])
+                                    (128, 8320), (32, 32), (32, 96), (32, 480), (32, 1376), (32, 8160)])
 @pytest.mark.parametrize("bf16,trust", [(False, 1.0), (False, 1.3), (False, 0.5), (True, 1.3)])
 def test_narrow_blocks_of_either_type(bits, g, cols, bf16, trust):
     # rows of less than a warp, of one, of several; binary32 beside bfloat16
