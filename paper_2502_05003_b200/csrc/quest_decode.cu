@@ -24,6 +24,8 @@
 // stated in quest_quantize.cu bit for bit (rows with NaN or infinities included).
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "quest_internal.cuh"
 #include "quest_operand.cuh"
 
@@ -294,18 +296,20 @@ __device__ __forceinline__ void quantize_rows_in_cta(const DecodeArgs &a, int8_t
     }
 }
 
-template <bool FUSED, int MT, int NT> struct Ring {
+// DEEP: the CTA has an SM to itself.
+template <bool FUSED, int MT, int NT, bool DEEP> struct Ring {
     static constexpr int UNITS = 2 * MT + (FUSED ? 0 : NT);            // 16-byte slots per thread and chunk
     static constexpr int STAGE = UNITS * THREADS * 16;
-    static constexpr int DEPTH = 24 / UNITS > 8 ? 8 : 24 / UNITS;      // chunks in flight: at most 96 KB, so that two CTAs share an SM
+    static constexpr int MOST = DEEP ? 48 : 24;                        // chunks in flight: at most 96 KB where two CTAs share an SM
+    static constexpr int DEPTH = MOST / UNITS > 8 ? 8 : MOST / UNITS;
     static constexpr int RED = WARPS * 8 * NT * 16 * MT * 4;           // the partial sums take the ring's place
     static constexpr int BYTES = DEPTH * STAGE > RED ? DEPTH * STAGE : RED;
 };
 
-template <int SRC, bool FUSED, int MT, int NT>
-__global__ void __launch_bounds__(THREADS, 2)
+template <int SRC, bool FUSED, int MT, int NT, bool DEEP>
+__global__ void __launch_bounds__(THREADS, DEEP ? 1 : 2)
 decode_kernel(const __grid_constant__ DecodeArgs a) {
-    using L = Ring<FUSED, MT, NT>;
+    using L = Ring<FUSED, MT, NT, DEEP>;
     constexpr int ROWS = 16 * MT;
     constexpr int NW = SrcWords<SRC>::N;
     constexpr int D = L::DEPTH;
@@ -479,21 +483,16 @@ decode_kernel(const __grid_constant__ DecodeArgs a) {
     }
 }
 
-template <int SRC, bool FUSED, int MT, int NT>
+template <int SRC, bool FUSED, int MT, int NT, bool DEEP = false>
 cudaError_t launch_one(const DecodeArgs &a, cudaStream_t st) {
-    size_t smem = Ring<FUSED, MT, NT>::BYTES;
+    size_t smem = Ring<FUSED, MT, NT, DEEP>::BYTES;
     const int ctas = (a.N + 16 * MT - 1) / (16 * MT);
     if (FUSED) smem += (size_t)a.M * a.pitch + (a.g >= 512 ? (size_t)a.M * ((a.K + 255) / 256) * 1024 : 0);
-    // One CTA per SM where there are no more of them: started while the quantizer drains, two would share each SM that is
-    // free first.  Bytes of w from the operand or 4- and 8-bit codes: 24 x 2048 x 5504 9.5 -> 7.8 us, from packed codes 12.8
-    // -> 9.3, 24 x 4096 x 4096 at 8 bits 11.0 -> 9.0; equal on short rows.  One and two bits are held by unpacking and lose
-    // a little (24 x 4096 x 4096 at two bits 8.5 -> 8.7); the fused form, whose CTAs are short, gains nothing.
-    constexpr bool BYTES_OR_NIBBLES = SRC == SRC_OP8 || SRC == SRC_CODES4 || SRC == SRC_CODES8;
-    if (!FUSED && BYTES_OR_NIBBLES && ctas <= num_sms() && smem < 116 * 1024) smem = 116 * 1024;
+    if ((DEEP || (SRC == SRC_CODES8 && !FUSED && ctas <= num_sms())) && smem < 116 * 1024) smem = 116 * 1024;      // one CTA per SM
     static DynamicSmemOnce once;
-    const cudaError_t e = once.set(decode_kernel<SRC, FUSED, MT, NT>, 144 * 1024);
+    const cudaError_t e = once.set(decode_kernel<SRC, FUSED, MT, NT, DEEP>, DEEP ? 200 * 1024 : 144 * 1024);
     if (e != cudaSuccess) return e;
-    return launch_pdl(decode_kernel<SRC, FUSED, MT, NT>, dim3((unsigned)ctas), dim3(THREADS), smem, st, 1, a);
+    return launch_pdl(decode_kernel<SRC, FUSED, MT, NT, DEEP>, dim3((unsigned)ctas), dim3(THREADS), smem, st, 1, a);
 }
 
 template <int SRC, bool FUSED>
@@ -501,6 +500,23 @@ cudaError_t launch_src(const DecodeArgs &a, bool two, cudaStream_t st) {
     if constexpr (FUSED) {
         return two ? launch_one<SRC, true, 2, 1>(a, st) : launch_one<SRC, true, 1, 1>(a, st);
     } else {
+        // One CTA per SM, with up to twice the chunks in flight, where 16, 32 or 48 rows of w a CTA allow it: started while the
+        // quantizer drains, two would share each SM that is free first, and a second CTA on some SMs is what all wait for.
+        // 24 x 5504 x 2048 from packed codes 9.6 -> 7.8 us, with w's operand prepared 7.8 -> 7.1; 24 x 2048 x 5504 12.8 -> 8.9 and
+        // 9.5 -> 7.8; 5 x 5504 x 2048 from codes 6.7 -> 5.8; equal on short rows.  Packed codes of 8 bits gain the single CTA
+        // only (5 x 5504 x 2048 with 48 rows 7.6 -> 8.2); one and two bits are held by unpacking and lose a little even there
+        // (24 x 4096 x 4096 at two bits 8.5 -> 8.7).
+        if constexpr (SRC == SRC_OP8 || SRC == SRC_CODES4) {
+            const int mt = (a.N + 16 * num_sms() - 1) / (16 * num_sms());
+            auto deep = [&](auto nt) {
+                constexpr int NT = decltype(nt)::value;
+                return mt == 1 ? launch_one<SRC, false, 1, NT, true>(a, st) : mt == 2 ? launch_one<SRC, false, 2, NT, true>(a, st)
+                                                                                    : launch_one<SRC, false, 3, NT, true>(a, st);
+            };
+            if (mt <= 3)
+                return a.M <= 8 ? deep(std::integral_constant<int, 1>()) : a.M <= 16 ? deep(std::integral_constant<int, 2>())
+                                                                                     : deep(std::integral_constant<int, 4>());
+        }
         if (a.M <= 8) return two ? launch_one<SRC, false, 2, 1>(a, st) : launch_one<SRC, false, 1, 1>(a, st);
         if (a.M <= 16) return two ? launch_one<SRC, false, 2, 2>(a, st) : launch_one<SRC, false, 1, 2>(a, st);
         return two ? launch_one<SRC, false, 2, 4>(a, st) : launch_one<SRC, false, 1, 4>(a, st);

@@ -55,6 +55,13 @@ def test_shapes_and_blocks(M, N, K, g):
     check(M, N, K, 4, g, seed=M + N)
 
 
+@pytest.mark.parametrize("M", [5, 16, 32])
+@pytest.mark.parametrize("N,K,bits", [(4744, 544, 4), (7104, 160, 3), (7112, 160, 4), (2368, 2080, 5), (2376, 1056, 4), (4736, 288, 8), (4744, 288, 8)])
+def test_rows_of_w_per_cta(M, N, K, bits):
+    # either side of 16, 32 and 48 rows of w to a CTA that has an SM to itself
+    check(M, N, K, bits, 32, seed=M + N)
+
+
 @pytest.mark.parametrize("M,N,K,bits", [(1, 9472, 256, 4), (1, 9480, 256, 4), (4, 9480, 1024, 2), (2, 4728, 2048, 4),
                                         (2, 4744, 2048, 1), (1, 2048, 3072, 4), (8, 9480, 3104, 1), (16, 9480, 1568, 2),
                                         (16, 14216, 64, 1), (17, 1192, 2080, 1), (24, 2376, 1056, 2), (24, 9480, 992, 4),
