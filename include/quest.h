@@ -304,7 +304,8 @@ int quest_linear_fwd_fp4(const void *x, const void *w, int dtype, int64_t M, int
  *                          16-byte aligned rows; K a multiple of 32, 32 <= K <= 16384
  *   y [M x N]              device, y_dtype, row stride ldy elements
  *   xh                     optional device output [M x K] bfloat16, dense, 16-byte aligned
- *   wq, sw, mw             optional device outputs as in quest_quantize
+ *   wq, sw, mw             optional device outputs as in quest_quantize (codes of one bit may be 4-byte and those of
+ *                          two bits 8-byte aligned)
  *   workspace              device scratch of at least quest_weight_only_workspace_bytes(M, N, K)
  *                          bytes, 256-byte aligned; nothing is allocated by the call
  * Errors as for quest_linear_fwd; M = 0 or N = 0 is QUEST_OK and launches nothing.

@@ -571,7 +571,7 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                 uint8_t *dst = tn.codes + row * (long long)(cols * CB / 8) + (long long)tr * (8 * CB);
                 if constexpr (CB >= 4) {
                     store_words(dst, cwords);
-                } else {                                       // the weight-only layer takes codes at any multiple of four bytes
+                } else {                                       // the weight-only layer takes codes at any multiple of 4 CB bytes
                     const bool whole = (reinterpret_cast<uintptr_t>(dst) & (8 * CB - 1)) == 0;
                     if constexpr (CB == 2) {
                         if (whole) {

@@ -8,6 +8,8 @@
 //   y[m][n] = sw[n] sum_k x_h[m][k] c_w[n][k]    tcgen05 kind::f16 contraction, binary32 accumulators
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "quest_internal.cuh"
 
 namespace quest {
@@ -63,8 +65,10 @@ extern "C" int quest_linear_fwd_weight_only(const void *x, int x_dtype, int64_t 
     if (!(trust_factor >= 0.0f)) return QUEST_ERR_TRUST;
     auto al = [](const void *p, size_t a) { return reinterpret_cast<uintptr_t>(p) % a == 0; };
     const size_t xes = x_dtype == QUEST_F32 ? 4 : 2, wes = w_dtype == QUEST_F32 ? 4 : 2, yes = y_dtype == QUEST_F32 ? 4 : 2;
+    // the quantizer stores the codes of 32 elements in one access, up to 16 bytes of them, and the mask in 4-byte words
+    const size_t wq_store = std::min(4 * container_bits(bits_w), 16);
     if (!al(x, 16) || (size_t)ldx * xes % 16 != 0 || !al(w, 16) || (size_t)ldw * wes % 16 != 0 || !al(y, yes) ||
-        (xh && !al(xh, 16)) || (wq && !al(wq, 4)) || (sw && !al(sw, 4)))
+        (xh && !al(xh, 16)) || (wq && !al(wq, wq_store)) || (sw && !al(sw, 4)) || (mw && !al(mw, 4)))
         return QUEST_ERR_ALIGN;
     if (!workspace || !al(workspace, 256) || workspace_bytes < quest_weight_only_workspace_bytes(M, N, K))
         return QUEST_ERR_WORKSPACE;

@@ -153,3 +153,17 @@ def test_fp4_entry_points_validate_on_the_host(lib):
     assert g(xq=None) == 1 and g(K=100) == 2 and g(yd=4) == 5
     # the packed codes are read by TMA: 16-byte alignment; the scratch arguments are unused (no workspace error)
     assert g(xq=ctypes.c_void_p(FAKE.value + 8)) == 6 and g(ws=None) != 8
+
+
+@pytest.mark.parametrize("bits,stored", [(1, 4), (2, 8), (3, 16), (4, 16), (5, 16), (8, 16)])
+def test_weight_only_outputs_aligned_to_their_stores(lib, bits, stored):
+    # codes leave in stores of up to 16 bytes, masks in stores of four: what they cannot serve is refused, what they can
+    # is taken.  No workspace is given, so no call gets past the checks.
+    def call(wq=FAKE.value, mw=FAKE.value):
+        return lib.quest_linear_fwd_weight_only(FAKE, 1, 128, FAKE, 1, 128, 64, 64, 128, bits, 128, F(1.0), FAKE, 1, 64, FAKE,
+                                                ctypes.c_void_p(wq), FAKE, ctypes.c_void_p(mw), None, 0, None)
+    for off in (1, 2, 4, 8, 12, 16):
+        assert call(wq=FAKE.value + off) == (8 if off % stored == 0 else 6), off
+    for off in (1, 2, 4, 6):
+        assert call(mw=FAKE.value + off) == (8 if off % 4 == 0 else 6), off
+    assert call(wq=None, mw=None) == 8
