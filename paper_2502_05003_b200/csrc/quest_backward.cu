@@ -99,10 +99,11 @@ dequant_codes_kernel(DequantTensor t0, DequantTensor t1, int blocks0, int rpb, i
 }
 
 // Inverse orthonormal block Hadamard transform of every row of d [rows x cols] (binary32, dense),
-// stored as out_dtype with row stride ld.  Every thread owns 32 contiguous elements; descending
+// stored as out_dtype, dense.  Every thread owns 32 contiguous elements; descending
 // stride: partners in other warps through shared memory, partners in this warp through shuffles,
 // the rest in registers.  A row of T = cols/32 threads occupies S slots as in the quantizer.
-// PARTS: d is `parts` matrices `part_stride` elements apart, whose sum, where `mask` [rows x cols/8] keeps it, is the input.
+// PARTS: d is `parts` matrices `part_stride` elements apart, whose sum, where `mask` [rows x cols/8] keeps it, is the input
+// (blocks of up to 1024: see transform_adds_parts).
 template <bool PARTS>
 __global__ void __launch_bounds__(512)
 iht_rows_kernel(const float *__restrict__ d, long long rows, int cols, int had_block, float inv_sqrt_g, void *__restrict__ out,
@@ -141,16 +142,18 @@ iht_rows_kernel(const float *__restrict__ d, long long rows, int cols, int had_b
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] = 0.0f;
     }
-    for (int s = had_block >> 1; s >= 1024; s >>= 1) {        // partner thread is in another warp
-        const int dist = s >> 5;
-        __syncthreads();
+    if constexpr (!PARTS) {
+        for (int s = had_block >> 1; s >= 1024; s >>= 1) {     // partner thread is in another warp
+            const int dist = s >> 5;
+            __syncthreads();
 #pragma unroll
-        for (int i = 0; i < 32; ++i) xsm[i * nthreads + tid] = v[i];
-        __syncthreads();
-        const float sg = (tid & dist) ? -1.0f : 1.0f;
-        const int pt = tid ^ dist;
+            for (int i = 0; i < 32; ++i) xsm[i * nthreads + tid] = v[i];
+            __syncthreads();
+            const float sg = (tid & dist) ? -1.0f : 1.0f;
+            const int pt = tid ^ dist;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = fmaf(v[i], sg, xsm[i * nthreads + pt]);
+            for (int i = 0; i < 32; ++i) v[i] = fmaf(v[i], sg, xsm[i * nthreads + pt]);
+        }
     }
     {
         int s0 = had_block >> 1;
@@ -396,8 +399,8 @@ int launch_iht_rows(const float *d, int64_t rows, int64_t cols, int had_block, v
     const int threads = R * S;
     const size_t smem = had_block >= 2048 ? sizeof(float) * 32 * (size_t)threads : 0;
     if (smem > 48 * 1024) {
-        static DynamicSmemOnce whole, divided;
-        cudaError_t e = parts > 1 ? divided.set(iht_rows_kernel<true>, 72 * 1024) : whole.set(iht_rows_kernel<false>, 72 * 1024);
+        static DynamicSmemOnce once;
+        const cudaError_t e = once.set(iht_rows_kernel<false>, 72 * 1024);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     const cudaError_t e = launch_transform(parts > 1 ? iht_rows_kernel<true> : iht_rows_kernel<false>, (rows + R - 1) / R, threads, smem, st,
@@ -405,6 +408,11 @@ int launch_iht_rows(const float *d, int64_t rows, int64_t cols, int had_block, v
                                            out_dtype, S, R, parts, (long long)((rows + 255) / 256 * 256 * cols), mask);
     return e == cudaSuccess ? QUEST_OK : cuda_fail(e);
 }
+
+// Whether a transform that adds parts serves these rows.  It has no exchange between warps for the general kernel, which
+// blocks of 8192 and more take, and blocks of 2048 and 4096 in rows above 8192 columns; their 64 column tiles and more
+// leave 74 pairs nothing to divide among anyway.
+bool transform_adds_parts(int64_t cols, int had_block) { return had_block <= 1024 || (had_block <= 4096 && cols <= 8192); }
 
 // Inverse transform of d [rows x cols], binary32 and dense, or (parts > 1) of the sum of the parts that
 // launch_gemm_bf16_parts left there, where `mask` keeps it; `out` is dense too.
@@ -509,7 +517,7 @@ extern "C" int quest_linear_bwd(const void *dy, int64_t M, int64_t N, int64_t K,
     const int64_t rows_free = (int64_t)(((uint8_t *)workspace + ws.bytes - (uint8_t *)ws.d1) / (K * 4));
     auto gradient = [&](const void *a, const void *b, int64_t I, int64_t Kc, const uint8_t *mask, void *out, float *d, int opl) {
         Stage gemm_stage(QUEST_STAGE_GEMM, st);
-        const int parts = divide_contraction(I, K, Kc, rows_free);
+        const int parts = transform_adds_parts(K, had_block) ? divide_contraction(I, K, Kc, rows_free) : 1;
         if (parts > 1) {                                     // the products run one after the other: both may use d1 and d2
             const int e = launch_gemm_bf16_parts(a, b, I, K, Kc, ws.d1, parts, opl, st);
             return e ? e : launch_iht(ws.d1, I, K, had_block, out, out_dtype, parts, mask, st);

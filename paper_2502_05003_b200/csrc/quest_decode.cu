@@ -516,10 +516,13 @@ cudaError_t launch_src(const DecodeArgs &a, bool two, cudaStream_t st) {
             if (mt <= 3)
                 return a.M <= 8 ? deep(std::integral_constant<int, 1>()) : a.M <= 16 ? deep(std::integral_constant<int, 2>())
                                                                                      : deep(std::integral_constant<int, 4>());
+            return a.M <= 8 ? launch_one<SRC, false, 2, 1>(a, st) : a.M <= 16 ? launch_one<SRC, false, 2, 2>(a, st)
+                                                                              : launch_one<SRC, false, 2, 4>(a, st);
+        } else {
+            if (a.M <= 8) return two ? launch_one<SRC, false, 2, 1>(a, st) : launch_one<SRC, false, 1, 1>(a, st);
+            if (a.M <= 16) return two ? launch_one<SRC, false, 2, 2>(a, st) : launch_one<SRC, false, 1, 2>(a, st);
+            return two ? launch_one<SRC, false, 2, 4>(a, st) : launch_one<SRC, false, 1, 4>(a, st);
         }
-        if (a.M <= 8) return two ? launch_one<SRC, false, 2, 1>(a, st) : launch_one<SRC, false, 1, 1>(a, st);
-        if (a.M <= 16) return two ? launch_one<SRC, false, 2, 2>(a, st) : launch_one<SRC, false, 1, 2>(a, st);
-        return two ? launch_one<SRC, false, 2, 4>(a, st) : launch_one<SRC, false, 1, 4>(a, st);
     }
 }
 
