@@ -50,3 +50,42 @@ def assert_output_close(got, ref, out_is_bf16):
     if out_is_bf16 and ref.size >= 4096:
         rel = np.linalg.norm(got - ref) / max(np.linalg.norm(ref), 1e-300)
         assert rel <= BF16_OUT_NORM_RTOL, f"norm-wise relative error {rel:.2e}"
+
+
+def kernels_of(fn):
+    """Mangled names of the kernels that fn() launches, in order: the kernel nodes of a graph that captures it.  Call fn
+    once before: what it allocates or looks up the first time is not capturable."""
+    import ctypes
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        keep = fn()
+    driver = ctypes.CDLL("libcuda.so.1")
+    handle = ctypes.c_void_p(graph.raw_cuda_graph())
+
+    def call(name, *args):
+        status = getattr(driver, name)(*args)
+        assert status == 0, (name, status)
+
+    class KernelNode(ctypes.Structure):                  # CUDA_KERNEL_NODE_PARAMS
+        _fields_ = [("func", ctypes.c_void_p), ("sizes", ctypes.c_uint * 7), ("params", ctypes.c_void_p),
+                    ("extra", ctypes.c_void_p), ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+    count = ctypes.c_size_t(0)
+    call("cuGraphGetNodes", handle, None, ctypes.byref(count))
+    nodes = (ctypes.c_void_p * count.value)()
+    call("cuGraphGetNodes", handle, nodes, ctypes.byref(count))
+    names = []
+    for node in nodes:
+        kind = ctypes.c_int(-1)
+        call("cuGraphNodeGetType", ctypes.c_void_p(node), ctypes.byref(kind))
+        if kind.value != 0:                              # CU_GRAPH_NODE_TYPE_KERNEL
+            continue
+        p, name = KernelNode(), ctypes.c_char_p()
+        call("cuGraphKernelNodeGetParams_v2", ctypes.c_void_p(node), ctypes.byref(p))
+        if p.func:
+            call("cuFuncGetName", ctypes.byref(name), ctypes.c_void_p(p.func))
+        else:
+            call("cuKernelGetName", ctypes.byref(name), ctypes.c_void_p(p.kern))
+        names.append(name.value.decode())
+    del keep
+    return names

@@ -30,7 +30,7 @@ import torch
 from oracle import backward as ob
 from oracle import quest_oracle as qo
 from paper_2502_05003_b200 import synth
-from tests.gpu_util import to_dev
+from tests.gpu_util import kernels_of, to_dev
 
 pytestmark = pytest.mark.gpu
 
@@ -89,7 +89,7 @@ def run_case(x_np, w_np, bits, g, seed=0, out_dtype=torch.float32, rows_x=None, 
             # no rotation: a masked element is an exact zero
             dropped = (mbx if name == "dx" else mbw) == 0
             assert np.all(got[dropped] == 0.0), f"{name}: masked elements are not exact zeros"
-    return out
+    return {**out, "fwd": fwd}
 
 
 def gauss(rows, cols, seed, std=1.0, bf16=True):
@@ -113,13 +113,22 @@ def test_hadamard_block_sizes(g):
     run_case(gauss(200, 2048, 5), gauss(256, 2048, 6, 0.02), 4, g, seed=g)
 
 
-@pytest.mark.parametrize("M,N,K,g", [(2048, 64, 128, 128),      # small outputs of long sums: the contraction runs in parts
-                                     (4104, 72, 160, 32),       # a k-block that is nearly empty, half a tile of columns
-                                     (40, 4096, 512, 512), (72, 3000, 96, 1), (4096, 264, 256, 256), (4104, 520, 768, 256),
-                                     (2304, 136, 2048, 2048), (1800, 16, 4096, 4096), (1800, 24, 8192, 8192)])
+# small outputs of long sums: on 148 SMs the contraction of one of the two gradients runs in parts, which `transform` adds
+@pytest.mark.parametrize("M,N,K,g,transform", [
+    (2048, 64, 128, 128, "iht_rows"),
+    (4104, 72, 160, 32, "iht_rows"),                            # a k-block that is nearly empty, half a tile of columns
+    (40, 4096, 512, 512, "iht_rows"), (72, 3000, 96, 1, "iht_rows"), (4096, 264, 256, 256, "iht_rows"),
+    (4104, 520, 768, 256, "iht_rows"), (520, 4104, 1280, 256, "iht_wide8"), (4104, 520, 1280, 256, "iht_wide8"),
+    (4104, 520, 1536, 512, "iht_wide9"), (4104, 520, 1024, 1024, "iht_wide10"), (2304, 136, 2048, 2048, "iht_wide11"),
+    (3000, 72, 4096, 4096, "iht_wide12"), (3000, 8, 4608, 512, "iht_wide9")])
 @pytest.mark.parametrize("out_dtype", [torch.float32, torch.bfloat16])
-def test_small_outputs_of_long_sums(M, N, K, g, out_dtype):
-    run_case(gauss(M, K, 41), gauss(N, K, 42, 0.02), 4, g, seed=M + K, out_dtype=out_dtype)
+def test_small_outputs_of_long_sums(M, N, K, g, transform, out_dtype):
+    import paper_2502_05003_b200 as quest
+    fwd = run_case(gauss(M, K, 41), gauss(N, K, 42, 0.02), 4, g, seed=M + K, out_dtype=out_dtype)["fwd"]
+    dy = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda")
+    names = kernels_of(lambda: quest.quest_linear_bwd(dy, fwd, 4, g, K, out_dtype=out_dtype))
+    want = "iht_rows_kernelILb1E" if transform == "iht_rows" else f"iht_wide_kernelILi{transform[8:]}ELb1E"
+    assert sum("gemm_i8_kernelILi128ELi7E" in n for n in names) == 1 and sum(want in n for n in names) == 1, names
 
 
 @pytest.mark.parametrize("M,N,K,g", [(40, 24, 768, 256),        # eight rows per CTA of the transform, four slots of padding

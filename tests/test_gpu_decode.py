@@ -56,9 +56,11 @@ def test_shapes_and_blocks(M, N, K, g):
 
 
 @pytest.mark.parametrize("M", [5, 16, 32])
-@pytest.mark.parametrize("N,K,bits", [(4744, 544, 4), (7104, 160, 3), (7112, 160, 4), (2368, 2080, 5), (2376, 1056, 4), (4736, 288, 8), (4744, 288, 8)])
+@pytest.mark.parametrize("N,K,bits", [(4744, 544, 4), (7104, 160, 3), (7112, 160, 4), (2368, 2080, 5), (2376, 1056, 4), (4736, 288, 8), (4744, 288, 8),
+                                      (5504, 5504, 4), (4744, 6176, 3)])
 def test_rows_of_w_per_cta(M, N, K, bits):
-    # either side of 16, 32 and 48 rows of w to a CTA that has an SM to itself
+    # either side of 16, 32 and 48 rows of w to a CTA that has an SM to itself; rows of w that go round its ring of 4 or 6
+    # chunks more than once
     check(M, N, K, bits, 32, seed=M + N)
 
 

@@ -101,9 +101,11 @@ def test_buffers_at_the_least_alignment(bits, g, cols, rows, bf16):
 
 @pytest.mark.parametrize("bits", [1, 4, 8])
 @pytest.mark.parametrize("g,cols,rows,bf16", [(128, 1024, 1200, True), (64, 1344, 700, True), (32, 1024, 1000, True),
-                                              (128, 512, 3600, True), (2048, 2048, 500, True), (4096, 4096, 590, False)])
+                                              (128, 512, 3600, True), (2048, 2048, 500, True), (4096, 4096, 590, False),
+                                              (256, 768, 1500, True), (128, 5504, 400, True), (4096, 4096, 1100, True)])
 def test_grids_of_two_and_three_ctas_per_sm(bits, g, cols, rows, bf16):
-    # every kernel family at grids whose CTAs are spread over the SMs by their shared memory (two and three to an SM)
+    # the kernels that take one CTA to a group of rows, at grids whose CTAs are spread over the SMs by their shared memory (two
+    # and three to an SM; the last one four, where five would fit)
     check(rows_of("outliers", rows, cols, bits + cols, bf16), bits, g, repeat=1)
 
 
