@@ -353,7 +353,7 @@ int transform_rows_per_cta(int64_t rows, int S, int parts) {
     return R;
 }
 
-// A transform launched ahead of its predecessor's end, or (adding parts, and where launch_iht_wide says so) plainly.
+// A transform launched ahead of its predecessor's end, or (adding parts, and where its launcher says so) plainly.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_transform(void (*kernel)(KArgs...), int64_t grid, int threads, size_t smem, cudaStream_t st, bool ahead, Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -403,8 +403,13 @@ int launch_iht_rows(const float *d, int64_t rows, int64_t cols, int had_block, v
         const cudaError_t e = once.set(iht_rows_kernel<false>, 72 * 1024);
         if (e != cudaSuccess) return cuda_fail(e);
     }
+    // Launched ahead, the CTAs gather on the SMs that the gradient product leaves free, as in launch_iht_wide; eight of them
+    // fit on an SM.  Plainly an output of 0.5 to 0.9 Mi elements takes 0.4 .. 0.8 us less, of 1 to 3 Mi 1.2 .. 2.1 us less,
+    // below 0.3 and above 4 Mi elements up to 0.6 us more (300 backward passes).
+    const int64_t elements = rows * cols;
+    const bool ahead = parts == 1 && (elements < (400 << 10) || elements >= (4 << 20));
     const cudaError_t e = launch_transform(parts > 1 ? iht_rows_kernel<true> : iht_rows_kernel<false>, (rows + R - 1) / R, threads, smem, st,
-                                           parts == 1, d, (long long)rows, (int)cols, had_block, 1.0f / sqrtf((float)had_block), out,
+                                           ahead, d, (long long)rows, (int)cols, had_block, 1.0f / sqrtf((float)had_block), out,
                                            out_dtype, S, R, parts, (long long)((rows + 255) / 256 * 256 * cols), mask);
     return e == cudaSuccess ? QUEST_OK : cuda_fail(e);
 }
