@@ -522,7 +522,7 @@ extern "C" int quest_linear_bwd(const void *dy, int64_t M, int64_t N, int64_t K,
     const int64_t rows_free = (int64_t)(((uint8_t *)workspace + ws.bytes - (uint8_t *)ws.d1) / (K * 4));
     auto gradient = [&](const void *a, const void *b, int64_t I, int64_t Kc, const uint8_t *mask, void *out, float *d, int opl) {
         Stage gemm_stage(QUEST_STAGE_GEMM, st);
-        const int parts = transform_adds_parts(K, had_block) ? divide_contraction(I, K, Kc, rows_free) : 1;
+        const int parts = transform_adds_parts(K, had_block) ? divide_contraction(I, K, Kc, rows_free, fuse) : 1;
         if (parts > 1) {                                     // the products run one after the other: both may use d1 and d2
             const int e = launch_gemm_bf16_parts(a, b, I, K, Kc, ws.d1, parts, opl, st);
             return e ? e : launch_iht(ws.d1, I, K, had_block, out, out_dtype, parts, mask, st);

@@ -1443,8 +1443,11 @@ int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, 
 // Parts into which the contraction of a gradient product is divided so that a small output with a long sum does not leave
 // most pairs idle: 1 where it would not pay.  A k-block of the 256 x 128 tiles takes about 0.19 us; adding the parts costs a
 // launch and reads them back from L2, about 2.5 us and a microsecond for 3 MB.  `rows_free`: rows of J binary32 numbers
-// that the parts may take, each of them whole tiles high.
-int divide_contraction(int64_t I, int64_t J, int64_t Kc, int64_t rows_free) {
+// that the parts may take, each of them whole tiles high.  `own_launch`: undivided, the product needs no transform after
+// it.  Then fewer than 32 rows, whose transform is a few CTAs that each wait for the parts in turn, cost 1.2 us more (120
+// passes with 8 to 64 rows, 1500 to 3000 terms and 1024 to 4096 columns, divided without this: 8 x 2432 over 1856 terms
+// 26.2 -> 27.7 us, 8 x 3072 28.5 -> 29.9; gains of up to 0.7 us are given away, those above it kept).
+int divide_contraction(int64_t I, int64_t J, int64_t Kc, int64_t rows_free, bool own_launch) {
     const int64_t pairs = num_sms() / 2, tall = (I + 255) / 256, tiles = tall * ((J + 127) / 128), kb = (2 * Kc + BK - 1) / BK;
     int64_t parts = pairs / tiles;
     if (parts > kb / 4) parts = kb / 4;
@@ -1452,7 +1455,7 @@ int divide_contraction(int64_t I, int64_t J, int64_t Kc, int64_t rows_free) {
     if (parts < 2) return 1;
     const int64_t per = (kb + parts - 1) / parts;
     parts = (kb + per - 1) / per;
-    const double gain = 0.19 * (double)(kb - per), cost = 2.5 + (double)(parts * I * J * 4) / 3e6;
+    const double gain = 0.19 * (double)(kb - per), cost = (own_launch && I < 32 ? 3.7 : 2.5) + (double)(parts * I * J * 4) / 3e6;
     return gain > cost + 1.0 ? (int)parts : 1;
 }
 

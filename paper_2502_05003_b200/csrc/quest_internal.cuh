@@ -226,7 +226,7 @@ int launch_gemm_bf16_masked(const void *a, const void *b, int64_t I, int64_t J, 
 
 // The same product in `parts` parts of the contraction index (divide_contraction says how many): bare binary32 sums, part q
 // from row q * ((I + 255) / 256 * 256) of `out`.
-int divide_contraction(int64_t I, int64_t J, int64_t Kc, int64_t rows_free);
+int divide_contraction(int64_t I, int64_t J, int64_t Kc, int64_t rows_free, bool own_launch);
 int launch_gemm_bf16_parts(const void *a, const void *b, int64_t I, int64_t J, int64_t Kc, float *out, int parts, int opl,
                            cudaStream_t st);
 

@@ -131,6 +131,16 @@ def test_small_outputs_of_long_sums(M, N, K, g, transform, out_dtype):
     assert sum("gemm_i8_kernelILi128ELi7E" in n for n in names) == 1 and sum(want in n for n in names) == 1, names
 
 
+@pytest.mark.parametrize("M,N,K,whole", [(1856, 8, 2432, True), (16, 1736, 2304, True), (2304, 64, 128, False)])
+def test_few_rows_are_divided_later(M, N, K, whole):
+    # a product that transforms in its epilogue is divided for fewer than 32 rows only where that gains a transform's wait too
+    import paper_2502_05003_b200 as quest
+    fwd = run_case(gauss(M, K, 43), gauss(N, K, 44, 0.02), 4, 128, seed=M + K)["fwd"]
+    dy = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda")
+    names = kernels_of(lambda: quest.quest_linear_bwd(dy, fwd, 4, 128, K))
+    assert any("gemm_i8_kernelILi128ELi7E" in n for n in names) != whole, names
+
+
 @pytest.mark.parametrize("M,N,K,g", [(40, 24, 768, 256),        # eight rows per CTA of the transform, four slots of padding
                                      (24, 136, 2560, 512),      # one row per CTA, 40 of 64 threads
                                      (136, 8, 3072, 1024), (48, 40, 6144, 2048), (8, 72, 4096, 4096), (24, 16, 8192, 4096)])
