@@ -273,16 +273,17 @@ __device__ __forceinline__ void project32_trusting(const float2 *v, float inv, c
 
 // Everything after the load: rotation from stride s_start downwards (larger strides already
 // applied by the caller), RMS, projection, trust test, packing and stores for the E elements this
-// thread holds.  GFULL: had_block >= E, so every in-register stage runs.  FAST: the common case
-// fixed at compile time -- had_block = 128 with the first stage already applied, rows of at least
-// one warp (SHORT_ROWS: of any length), codes, scales and mask requested (the GEMM operand and the bfloat16 outputs of the
-// weight-only variant are optional; a tensor may also ask for the rotation alone), no row sums,
-// trust_factor >= 1 -- so that no per-row loop and only a few uniform branches remain.
+// thread holds.  GFULL: had_block >= E, so every in-register stage runs.  FAST: the common cases
+// fixed at compile time -- no stride left above E (with 32 elements stride 32 is done here unless XDONE), rows of at
+// least one warp (SHORT_ROWS: of any length), trust_factor >= 1, codes, scales and mask requested (the GEMM operand and the
+// bfloat16 outputs of the weight-only variant are optional; a tensor may also ask for the rotation alone), row sums only
+// with RS -- so that no per-row loop and only a few uniform branches remain.
+// XDONE: the caller has applied every stride that pairs two threads.
 // OPT: any of codes, scales and mask may be missing (FAST without OPT: all are there).
-// DECODE: the launch precedes the decoding kernel (see launch_quantize).
+// DECODE: the launch precedes the decoding kernel (see launch_quantize).  STREAM: called by the streaming kernel.
 // CS, CCOLS: threads per row and row length when the kernel is instantiated for one row length (0 = run-time values).
 template <int CB, int E, bool GFULL, bool FAST, int GRID = GRID_UNIFORM, bool XDONE = false, bool RS = false, int CS = 0, int CCOLS = 0,
-          bool OPT = !FAST, bool DECODE = false, bool SHORT_ROWS = false>
+          bool OPT = !FAST, bool DECODE = false, bool SHORT_ROWS = false, bool STREAM = false>
 __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const QuantArgs &a, const QuantTensor &tn,
                                                      bool active, long long row, int tr, int r_local, float *xsm,
                                                      int s_start) {
@@ -428,8 +429,11 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
     const float top = a.qc.top, hh = a.qc.h;
     int rsum = 0;
     if (active) {
-        // 64 elements: codes and mask of both halves leave together (halves of sectors, written twice, otherwise)
-        [[maybe_unused]] uint32_t mwords[E / 32], cwords[E == 64 ? 2 * CB : 1];
+        // 64 elements: codes and mask of both halves leave together (halves of sectors, written twice, otherwise).  8-bit codes
+        // fill a sector per half and leave at once: 0.97 of the time where they waited for the second half in the general
+        // kernel on binary32 rows, 0.99 in the wide one, but 1.01 in the streaming one.
+        constexpr bool CODES_AT_ONCE = E == 32 || (CB == 8 && !STREAM);
+        [[maybe_unused]] uint32_t mwords[E / 32], cwords[CODES_AT_ONCE ? 1 : 2 * CB];
 #pragma unroll
         for (int g32 = 0; g32 < E / 32; ++g32) {
             uint32_t mbits = 0;
@@ -501,10 +505,15 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                 }
             }
 
-            if constexpr (E == 32) {
+            if constexpr (CODES_AT_ONCE) {
                 if (!OPT || tn.codes) {
-                    uint8_t *dst = tn.codes + row * (long long)(cols * CB / 8) + (long long)tr * (4 * CB);
-                    if constexpr (CB == 8) store_words(dst, w);
+                    uint8_t *dst = tn.codes + row * (long long)(cols * CB / 8) + ((long long)tr * (E / 32) + g32) * (4 * CB);
+                    if constexpr (CB == 8 && !FAST) {
+                        // not store_words: its choice costs short rows of the general kernel more than half sectors do
+                        // (188 x 640, g = 4: 2.89 us with it, 2.79 without)
+                        reinterpret_cast<uint4 *>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+                        reinterpret_cast<uint4 *>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+                    } else if constexpr (CB == 8) store_words(dst, w);
                     else if constexpr (CB == 4) *reinterpret_cast<uint4 *>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
                     else if constexpr (CB == 2) *reinterpret_cast<uint2 *>(dst) = make_uint2(w[0], w[1]);
                     else *reinterpret_cast<uint32_t *>(dst) = w[0];
@@ -567,7 +576,9 @@ __device__ __forceinline__ void rotate_project_store(float2 (&v)[E / 2], const Q
                     dst[1] = mwords[1];
                 }
             }
-            if (!OPT || tn.codes) {                            // 8 CB bytes per thread
+            if constexpr (CODES_AT_ONCE) {
+                // gone already
+            } else if (!OPT || tn.codes) {                     // 8 CB bytes per thread
                 uint8_t *dst = tn.codes + row * (long long)(cols * CB / 8) + (long long)tr * (8 * CB);
                 if constexpr (CB >= 4) {
                     store_words(dst, cwords);
@@ -736,7 +747,7 @@ quantize_stream_kernel(const __grid_constant__ QuantArgs a, int total_groups, in
 #pragma unroll
             for (int q = 0; q < E / 8; ++q) widen(own[q], &v[q * 4]);
         }
-        rotate_project_store<CB, E, true, FAST, GRID, false, false, 0, 0, DECODE || !FAST, DECODE>(v, a, tn, active, row, tr, r_local, xsm, s_start);
+        rotate_project_store<CB, E, true, FAST, GRID, false, false, 0, 0, DECODE || !FAST, DECODE, false, true>(v, a, tn, active, row, tr, r_local, xsm, s_start);
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
