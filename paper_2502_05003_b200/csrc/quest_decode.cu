@@ -3,15 +3,15 @@
 // The tensor-core kernel of quest_gemm.cu gives such a layer 256 x 128 tiles of CTA pairs, of which 8 to 32 rows are wanted:
 // 16 pairs for 2048 columns (8.2 us with the quantizer; 11.7 with the single-CTA 128 x 256 tiles it had when this was
 // written).  What bounds the work is reading w once
-// (4 MB at 2048 x 2048: under a microsecond from HBM) and latency, so here a CTA takes 16 or 32 rows of w, its eight
+// (4 MB at 2048 x 2048: under a microsecond from HBM) and latency, so here a CTA takes 16, 32 or 48 rows of w, its eight
 // warps split K, and every warp multiplies with mma.sync m16n8k32 (w is the 16-row operand, the rows of x are the 8
 // columns): integer sums are exact in any order, so the K positions a lane holds are simply 16 consecutive bytes of
 // its row.  A lane copies its own bytes with cp.async into its own slots of a ring (no barrier in the main loop, up
 // to eight chunks in flight: loads into registers left the warps waiting for every chunk in turn, 14.6 us for 30 MB
 // of w against 9.0).  The partial sums of the eight warps meet in shared memory.  tcgen05 would need 128-row tiles,
 // tensor memory and descriptors for a product whose arithmetic is not what takes the time.
-// Whole layer at 2048 x 2048, device time back to back: one row 11.7 -> 4.1 us, 32 rows 12.0 -> 5.6 us; 24 rows x
-// 5504 x 2048 from packed codes 16.6 -> 10.0 us.
+// Whole layer at 2048 x 2048, device time back to back over eight layers: one row 11.7 -> 3.7 us, 32 rows 12.0 -> 5.2 us;
+// 24 rows x 5504 x 2048 from packed codes 16.6 -> 8.8 us.
 //
 // Two forms.  FUSED (few rows): the CTA rotates and quantizes x itself while its first loads of w are in flight;
 // every CTA repeats that work, one launch does the layer.  Otherwise the quantizer is a launch of its own, and this
@@ -502,8 +502,9 @@ cudaError_t launch_src(const DecodeArgs &a, bool two, cudaStream_t st) {
     } else {
         // One CTA per SM, with up to twice the chunks in flight, where 16, 32 or 48 rows of w a CTA allow it: started while the
         // quantizer drains, two would share each SM that is free first, and a second CTA on some SMs is what all wait for.
-        // 24 x 5504 x 2048 from packed codes 9.6 -> 7.8 us, with w's operand prepared 7.8 -> 7.1; 24 x 2048 x 5504 12.8 -> 8.9 and
-        // 9.5 -> 7.8; 5 x 5504 x 2048 from codes 6.7 -> 5.8; equal on short rows.  Packed codes of 8 bits gain the single CTA
+        // 24 x 5504 x 2048 from packed codes 10.9 -> 8.9 us, with w's operand prepared 9.2 -> 8.3; 24 x 2048 x 5504 10.0 -> 9.4 and
+        // 8.7 -> 8.3 .. 8.7; 5 x 5504 x 2048 from codes 8.0 -> 6.7; 32 x 5504 x 5504 15.0 -> 13.2 (back to back over 40 layers); equal
+        // up to 160 elements a row.  Packed codes of 8 bits gain the single CTA
         // only (5 x 5504 x 2048 with 48 rows 7.6 -> 8.2); one and two bits are held by unpacking and lose a little even there
         // (24 x 4096 x 4096 at two bits 8.5 -> 8.7).
         if constexpr (SRC == SRC_OP8 || SRC == SRC_CODES4) {
@@ -541,7 +542,9 @@ cudaError_t launch_form(int src, const DecodeArgs &a, bool two, cudaStream_t st)
 }  // namespace
 
 // Where the decoding path serves.  Its time grows in steps with N, with the CTAs that share an SM (a CTA takes 16 rows of
-// w, 32 above 16 per SM; from 32 rows per SM on CTAs begin to share one, above 64 there is a second round), with the
+// w, 32 above 16 per SM; from 32 rows per SM on CTAs begin to share one, above 64 there is a second round; from the byte
+// operand and 4-bit codes a CTA of 16, 32 or 48 rows has an SM to itself up to 48 rows per SM, and these limits, measured
+// when it had not, were not moved), with the
 // groups of eight rows of x, and at one and two bits with the unpacking of w to bytes, which the FP4 contraction of
 // quest_gemm.cu need not do.  Against that contraction (device time back to back, us, here / there):
 //    4 bits, operand: 8 x 32768 x 4096 27.1 / 41.0; 32 x 4096 x 4096 10.0 / 10.5, 32 x 11008 x 512 1.09 of it, 32 x 16384 x
@@ -599,8 +602,8 @@ int launch_decode(const QuantJob &jx, int dtype, bool fused, const uint8_t *wq, 
         const int cb = container_bits(bits);
         src = cb == 1 ? SRC_CODES1 : cb == 2 ? SRC_CODES2 : cb == 4 ? SRC_CODES4 : SRC_CODES8;
     }
-    // 32 rows of w per CTA once 16 would give more CTAs than there are SMs: half the reads (or quantizations) of x
-    // (32 x 2048 x 2048: 5.7 us with 16 rows, 6.9 with 32; 32 x 5504 x 5504: 15.1 and 14.7 us)
+    // 32 rows of w per CTA once 16 would give more CTAs than there are SMs: half the reads (or quantizations) of x.  (The
+    // byte operand and 4-bit codes behind a quantizer launch follow launch_src instead, up to 48 rows per SM.)
     const bool two = N > 16ll * num_sms();
     const cudaError_t e = fused ? launch_form<true>(src, a, two, st) : launch_form<false>(src, a, two, st);
     return e == cudaSuccess ? QUEST_OK : cuda_fail(e);

@@ -168,7 +168,7 @@ struct QuantTensor {
     uint16_t *cbf;         // grid values c = 2k - (2^b - 1) as bfloat16 (weight-only variant)
 };
 // Threads that an SM holds of a kernel, by the registers its launch bounds leave.
-// quantize_wide_kernel: five CTAs (96 registers, up to five words spilled) pay for bfloat16 blocks of 4096, whose exchange
+// quantize_wide_kernel: five CTAs (96 registers; two words spilled on the FP4 grid, none elsewhere) pay for bfloat16 blocks of 4096, whose exchange
 // with the neighbour leaves more to wait for: 16384 x 4096 63.3 -> 60.3 us, 4096 x 4096 18.3 -> 17.6; narrower blocks gain 2 %
 // at 16384 rows and lose 5 % at 1024, binary32 loses 8 %.
 __host__ __device__ constexpr int wide_threads(bool bf16, bool g4096) { return bf16 && g4096 ? 640 : 512; }
@@ -1049,11 +1049,12 @@ static cudaError_t launch_wide(bool bf16, int cb, int grid, int threads, size_t 
                 : launch_wide_g<false, GRID, false>(cb, grid, threads, smem, st, a, exchange_bytes, rowsums);
 }
 
-// The specialised case (bfloat16 rows, had_block = 128, 32 elements per thread) with direct loads and
+// Blocks of 128, 64 and 32 with 32 elements per thread, trust_factor >= 1, rows of up to 8192 columns (bfloat16; binary32
+// with BF16 = false; SHORT_ROWS: rows of less than a warp too, binary32 and blocks of 32 always) with direct loads and
 // one CTA per row group: at sizes whose whole input is a few waves of CTAs the hardware's own CTA
 // scheduling balances better than the persistent loop of the streaming kernel and there is no
 // staging to set up.  Stride 64 pairs this thread with lane ^ 2 (shuffles); the rest is the common tail.
-// RS: the row sums of the 8-bit GEMM operand are wanted (kept out of the common instantiation).
+// RS: the row sums of the 8-bit GEMM operand are wanted (kept out of the common instantiation).  REGS: see direct_threads.
 // COLS: the row length when it is one of the common ones (1024, 2048, 4096: threads per row, rows per CTA and every
 // row pitch become constants, worth 6 % of the kernel); 0 takes them from the arguments.
 // HB, OPT: blocks of 64 and 32 (the strides they do not have are left out) and launches that do not ask for every output take instantiations of
