@@ -52,9 +52,10 @@ def assert_output_close(got, ref, out_is_bf16):
         assert rel <= BF16_OUT_NORM_RTOL, f"norm-wise relative error {rel:.2e}"
 
 
-def kernels_of(fn):
-    """Mangled names of the kernels that fn() launches, in order: the kernel nodes of a graph that captures it.  Call fn
-    once before: what it allocates or looks up the first time is not capturable."""
+def kernels_of(fn, ahead=False):
+    """Mangled names of the kernels that fn() launches, in order: the kernel nodes of a graph that captures it.  With `ahead`
+    pairs of a name and whether the kernel may start before its predecessor has ended (a programmatic edge leads to it).
+    Call fn once before: what it allocates or looks up the first time is not capturable."""
     import ctypes
     graph = torch.cuda.CUDAGraph(keep_graph=True)
     with torch.cuda.graph(graph):
@@ -74,6 +75,11 @@ def kernels_of(fn):
     call("cuGraphGetNodes", handle, None, ctypes.byref(count))
     nodes = (ctypes.c_void_p * count.value)()
     call("cuGraphGetNodes", handle, nodes, ctypes.byref(count))
+    n = ctypes.c_size_t(0)
+    call("cuGraphGetEdges_v2", handle, None, None, None, ctypes.byref(n))
+    source, target, data = (ctypes.c_void_p * n.value)(), (ctypes.c_void_p * n.value)(), (ctypes.c_ubyte * (8 * n.value))()
+    call("cuGraphGetEdges_v2", handle, source, target, data, ctypes.byref(n))
+    early = {target[i] for i in range(n.value) if data[8 * i + 2] == 1}      # CU_GRAPH_DEPENDENCY_TYPE_PROGRAMMATIC
     names = []
     for node in nodes:
         kind = ctypes.c_int(-1)
@@ -86,6 +92,6 @@ def kernels_of(fn):
             call("cuFuncGetName", ctypes.byref(name), ctypes.c_void_p(p.func))
         else:
             call("cuKernelGetName", ctypes.byref(name), ctypes.c_void_p(p.kern))
-        names.append(name.value.decode())
+        names.append((name.value.decode(), node in early) if ahead else name.value.decode())
     del keep
     return names

@@ -141,6 +141,17 @@ def test_few_rows_are_divided_later(M, N, K, whole):
     assert any("gemm_i8_kernelILi128ELi7E" in n for n in names) != whole, names
 
 
+@pytest.mark.parametrize("M,K,ahead", [(120, 2912, True), (168, 2912, False), (1400, 2976, False), (1440, 2976, True)])
+def test_general_transform_ahead_of_the_product(M, K, ahead):
+    # either side of 0.39 and 4 Mi elements of an input gradient that the epilogue does not transform
+    import paper_2502_05003_b200 as quest
+    fwd = run_case(gauss(M, K, 45), gauss(64, K, 46, 0.02), 4, 32, seed=M)["fwd"]
+    dy = torch.zeros((M, 64), dtype=torch.bfloat16, device="cuda")
+    found = kernels_of(lambda: quest.quest_linear_bwd(dy, fwd, 4, 32, K), ahead=True)
+    transforms = [early for name, early in found if "iht_rows_kernelILb0E" in name]
+    assert transforms and transforms[0] == ahead, found
+
+
 @pytest.mark.parametrize("M,N,K,g", [(40, 24, 768, 256),        # eight rows per CTA of the transform, four slots of padding
                                      (24, 136, 2560, 512),      # one row per CTA, 40 of 64 threads
                                      (136, 8, 3072, 1024), (48, 40, 6144, 2048), (8, 72, 4096, 4096), (24, 16, 8192, 4096)])
